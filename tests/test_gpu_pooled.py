@@ -131,3 +131,44 @@ def test_pooled_predictions_rank_held_out_programs_like_the_reference(env):
                 checked += 1
     assert checked > 500
     assert int(cnt.cpu()[0]) == n
+
+
+@pytest.mark.parametrize("feat", [1, 7, 16, 17, 33, 255, 512])
+def test_pooled_factor_at_the_edges_of_its_panels(env, feat):
+    """Feature widths around the factorisation's 16-column panels and its largest, the refined fit
+    and its predictions (one warp per version, with fewer versions than a block takes).  The bound
+    is that of the test above: the BF16 x 3 Gram's delta, refined once."""
+    rs, ctx = env
+    batch = synth.make_batch(30, versions=(5, 64), feat=feat, dtype=np.float64, seed=300 + feat)
+    r = oracle.cv_batch(batch, synth.make_splits(batch, "all"))
+    train = range(29) if feat > 64 else range(20)
+    use = np.zeros(batch.n_programs, dtype=np.uint8)
+    use[list(train)] = 1
+    lam = 1.0              # keeps kappa moderate where a width exceeds the pairs
+    ref = _pooled_reference(batch, r.Z, train, lam)
+    zb = rs.DeviceBatch.from_host(batch).with_X(ctx.standardize(rs.DeviceBatch.from_host(batch)))
+    coef, st = ctx.fit_pooled(zb, torch.from_numpy(use).cuda(), lam=lam, flags=rs.RS_REFINE_X)
+    n = batch.n_rows
+    code = torch.empty(n, dtype=torch.int32, device="cuda")
+    pa = torch.empty(n * 6, dtype=torch.float64, device="cuda")
+    cnt = torch.zeros(16, dtype=torch.int64, device="cuda")
+    ctx.predict_pooled(zb, coef, st, code, pred_all=pa, counters=cnt)
+    torch.cuda.synchronize()
+    ctx.check_device_status()
+    coef, st, pa = coef.cpu().numpy(), st.cpu().numpy(), pa.cpu().numpy().reshape(n, 6)
+    delta, eps = 2.0 ** -17, np.finfo(float).eps
+    for j, (s_ref, b_ref, beta_ref, _, kappa) in enumerate(ref):
+        assert s_ref == oracle.FIT_OK and st[j] == oracle.FIT_OK
+        bound = (10 * kappa * delta) ** 2 + 100 * kappa * eps
+        err = np.abs(coef[j, 1:] - beta_ref).max() / np.abs(beta_ref).max()
+        assert err <= bound, (feat, j, err, bound)
+    for row in range(n):
+        p = int(np.searchsorted(batch.row_offsets, row, side="right")) - 1
+        z = r.Z[int(batch.x_offsets[p]) + (row - int(batch.row_offsets[p])) * feat:][:feat]
+        for j in range(6):
+            if (int(batch.masks[row]) >> j) & 1:
+                assert np.isnan(pa[row, j])
+            else:          # the dot product of the returned coefficients, in another order
+                want = coef[j, 0] + z @ coef[j, 1:]
+                assert abs(pa[row, j] - want) <= 1e-11 + 4 * feat * eps * (np.abs(z) @ np.abs(coef[j, 1:])), (row, j)
+    assert int(cnt.cpu()[0]) == n
