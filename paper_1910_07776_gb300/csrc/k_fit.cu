@@ -534,7 +534,16 @@ struct SolveArgs {
     int max_feat;
     int order;            // 0: largest fits first; 1: alternate ranges from both ends
     unsigned long long* row_info;   // [R] the rank pass's row records (with predictions)
+    // Closed-form fits of a call that did not ask for them (rs_launch_fit_predict): *left fits
+    // remain for the direct solvers, those whose status is kLeft; NULL: all of them
+    unsigned long long* left;
 };
+constexpr uint8_t kLeft = 0xff;
+
+// No fit is left for the direct solvers (every thread of the block asks).
+__device__ __forceinline__ bool none_left(const SolveArgs& a) { return a.left && __ldcg(a.left) == 0ull; }
+// Fit f is this call's direct solvers' to do.
+__device__ __forceinline__ bool is_left(const SolveArgs& a, int64_t f) { return !a.left || a.status[f] == kLeft; }
 
 __device__ __forceinline__ bool pred_target_v(const SolveArgs& a, int64_t s, int j, int p, int V, PredTarget& pt) {
     if (!a.predbuf) return false;
@@ -708,6 +717,7 @@ template <int NLO, int NHI, int MINB>
 __global__ void __launch_bounds__(128, MINB)
 solve_small_kernel(const SolveArgs a, unsigned long long* work) {
     __shared__ long long start[kHist], cstart[kHist];
+    if (none_left(a)) return;
     bucket_tables(a.hist, start, cstart);
     const long long lo = start[NLO], hi = start[NHI + 1];
     const int lane = threadIdx.x & 31;
@@ -732,7 +742,7 @@ solve_small_kernel(const SolveArgs a, unsigned long long* work) {
         uint4 nrec = make_uint4(0, 0, 0, 0);
         if (next < hi && position(next) >= lo) nrec = a.recs[position(next)];
         const long long pos = position(base);
-        const bool active = pos >= lo;
+        const bool active = pos >= lo && is_left(a, rec.x);
         int st = RS_FIT_OK;
         if (active) {
             int n = NLO;
@@ -927,6 +937,7 @@ __global__ void __launch_bounds__(128)
 solve_mid_kernel(const SolveArgs a, int nmax, unsigned long long* work) {
     extern __shared__ __align__(16) double dsm[];
     __shared__ long long start[kHist], cstart[kHist];
+    if (none_left(a)) return;
     bucket_tables(a.hist, start, cstart);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int per = tri(nmax) + 3 * nmax;
@@ -938,12 +949,13 @@ solve_mid_kernel(const SolveArgs a, int nmax, unsigned long long* work) {
     while (base < hi) {
         got = take32(work);
         const long long pos = hi - 1 - (base - lo) - lane;
-        const bool active = pos >= lo;
+        uint4 rec = make_uint4(0, 0, 0, 0);
+        if (pos >= lo) rec = a.recs[pos];
+        const bool active = pos >= lo && is_left(a, rec.x);
         int st = RS_FIT_OK;
         if (active) {
             int n = kNReg + 1;
             while (start[n + 1] <= pos) ++n;
-            const uint4 rec = a.recs[pos];
             const int64_t f = rec.x;
             const int64_t s = f / RS_NOPT;
             const int j = (int)(f - s * RS_NOPT);
@@ -1338,6 +1350,7 @@ solve_wide_kernel(const SolveArgs a, unsigned long long* work) {
     __shared__ long long start[kHist], cstart[kHist];
     __shared__ uint16_t tri_rc[tri(RS_MAXPAIRS - 1)];         // packed-triangle entry -> row, column
     extern __shared__ __align__(16) double wsm[];
+    if (none_left(a)) return;
     for (int i = threadIdx.x >> 5; i < RS_MAXPAIRS - 1; i += kWideWarps)
         for (int j = threadIdx.x & 31; j <= i; j += 32) tri_rc[tri(i) + j] = (uint16_t)(i << 8 | j);
     bucket_tables(a.hist, start, cstart);                      // (ends with a barrier)
@@ -1356,13 +1369,13 @@ solve_wide_kernel(const SolveArgs a, unsigned long long* work) {
         if (lane == 0) got = atomicAdd(work, (unsigned long long)kWideGroups);
         const long long pos = lo + (long long)__shfl_sync(0xffffffffu, got, 0) + g;
         if (__shfl_sync(0xffffffffu, pos, 0) >= hi) break;
-        const bool active = pos < hi;
         int n = 0;
         uint4 rec = make_uint4(0, 0, 0, 0);
+        if (pos < hi) rec = a.recs[pos];
+        const bool active = pos < hi && is_left(a, rec.x);
         if (active) {
             n = kNMid + 1;
             while (start[n + 1] <= pos) ++n;
-            rec = a.recs[pos];
         }
         const int nw = __reduce_max_sync(0xffffffffu, n);
         const int64_t f = rec.x;
@@ -1523,108 +1536,175 @@ constexpr int kLooW1 = kLooWy + RS_MAXPAIRS;
 constexpr int kLooSum = kLooW1 + RS_MAXPAIRS;
 constexpr int kLooTab = kLooSum + 4;                                   // doubles per (p, j)
 constexpr int kLooFitThreads = 256;
+// Largest q = max M_ii max (M^-1)_ii for which a call that did not ask for the closed form takes
+// it: the condition number is then at most n^2 q = 4e6, an error of the inverse below 5e-10 even
+// at that bound.  (Typical systems: q of tens; it passes the limit near as many features as pairs.)
+constexpr float kLooLimit = 4096.f;
 
-// One warp per (program, optimization): Gauss-Jordan elimination of [M | y | 1] without
-// pivoting (M is symmetric positive definite), lane i holding row i in registers, padded
-// with the identity past n (inert: a padded row or column meets only zeros), so that every
-// index is static.  Step k: every row i != k subtracts A_ik / p_k times row k (p_k = A_kk,
-// the pivot; row k reaches the others through shared memory) and stores -A_ik / p_k in
-// column k, the right block's column that column k's elimination has made; row k stays and
-// stores 1 there.  The left block ends diagonal, diag(p), so M^-1 is each row of the right
-// block divided by its pivot.  Row k needs no scaling inside the loop, so every lane runs the
-// same instructions.  Writes the symmetrized inverse, w_y, w_1 and their sums to tab, and
-// ok = 1 when every pivot was positive and finite.  A non-finite label enters y as 0 and sets
-// its pair's bit in bad: a fit that trains on that pair is non-finite, and one that leaves it
-// out does not depend on its label (the deletion formula above holds for any value in
-// position i).
-__global__ void __launch_bounds__(32)
+// One block per (program, optimization): the symmetric sweep operator over the lower triangle of
+//   [ M  . ]        with M = K_PP + lambda I of its n pairs (symmetric positive definite, no
+//   [ yt 0 ]        pivoting); rows 32 and 33 are the right-hand sides y and 1.
+//   [ 1t 0 ]
+// Sweeping pivot k (d = A_kk): A_ij -= A_ik (A_kj / d) for i, j != k, A_ik = A_ik / d, A_kk =
+// -1 / d.  After all n pivots the triangle holds -M^-1 and the two rows M^-1 y and M^-1 1.  The 592
+// entries are dealt flat to 128 threads (5 each, in registers; 4 in warp 0), so every FP64
+// instruction has its 32 lanes full and only half of the square is formed: 25 FP64 warp
+// instructions a pivot on four schedulers.  Per pivot two barriers: one warp scales the published
+// column by 1 / d; then every entry is updated, warp 0 first moving its copy of the diagonal ahead
+// so that the next pivot's reciprocal is ready when the column is.  Pivots past n are not swept.
+// (One warp per system with full rows in registers -- Gauss-Jordan, 38 instructions a pivot on one
+// scheduler: 256 programs 125 us, and the step of 2 programs 128 us; this form 115 and 104 us.)
+// Writes the inverse, w_y, w_1 and their sums to tab, and
+// ok = 1 when every pivot was positive and finite -- and, with limit > 0, when q = max_i M_ii
+// max_i (M^-1)_ii is at most limit (q bounds the condition number: q <= cond(M) <= n^2 q for a
+// symmetric positive definite M; taken from the values' high words, rounded up).  A non-finite label
+// enters y as 0 and sets its pair's bit in bad: a fit that trains on that pair is non-finite, and
+// one that leaves it out does not depend on its label (the deletion formula above holds for any
+// value in position i).
+constexpr int kLooThreads = 128;
+constexpr int kLooEntries = tri(RS_MAXPAIRS) + 2 * RS_MAXPAIRS;
+constexpr int kLooPer = 5;
+static_assert(kLooEntries <= 4 * kLooThreads + (kLooThreads - 32), "4 entries in warp 0's threads, 5 in the others'");
+
+__global__ void __launch_bounds__(kLooThreads)
 loo_inv_kernel(const int64_t* __restrict__ row_off, const double* __restrict__ K,
                const uint8_t* __restrict__ pb, const double* __restrict__ ylab,
-               const int* __restrict__ npair, const double* __restrict__ dlam, double* tab, uint8_t* ok,
-               uint32_t* bad) {
-    __shared__ __align__(16) double rowk[RS_MAXPAIRS + 2];     // the pivot row and its right-hand sides
-    __shared__ double S[RS_MAXPAIRS][RS_MAXPAIRS + 1];          // the inverse, for the symmetrized store
-    __shared__ int vs[RS_MAXPAIRS];
-    const int pj = blockIdx.x, p = pj / RS_NOPT, i = threadIdx.x;
+               const int* __restrict__ npair, const double* __restrict__ dlam, float limit, double* tab,
+               uint8_t* ok, uint32_t* bad) {
+    __shared__ double col[2][RS_MAXPAIRS + 2];                  // column k as it stands, by row
+    __shared__ double w[RS_MAXPAIRS + 2];                       // the column / d
+    __shared__ double rk;                                       // 1 / d of the next pivot; 0: not positive
+    __shared__ double rhs[2][RS_MAXPAIRS];
+    __shared__ int vs[RS_MAXPAIRS], umax;
+    const int pj = blockIdx.x, p = pj / RS_NOPT, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int V = (int)(row_off[p + 1] - row_off[p]);
     const int n = V >= 1 && V <= RS_MAXV ? npair[pj] : 0;
     if (n < 1 || n > RS_MAXPAIRS) {
-        if (i == 0) {
+        if (tid == 0) {
             ok[pj] = 0;
             bad[pj] = 0;
         }
         return;
     }
     const double* Kp = K + (int64_t)p * RS_GRAM_LD * RS_GRAM_LD;
-    const bool row = i < n;
-    if (row) vs[i] = pb[(int64_t)pj * RS_MAXPAIRS + i];
-    __syncwarp();
-    double A[RS_MAXPAIRS], y = 0.0, one = 0.0;
-    const int vi = row ? vs[i] : 0;
+    if (tid < n) vs[tid] = pb[(int64_t)pj * RS_MAXPAIRS + tid];
+    if (tid == 0) umax = 0;
+    __syncthreads();
+    double A[kLooPer];
+    int ri[kLooPer], ci[kLooPer];                               // row 0..33, column 0..31; -1: none
 #pragma unroll
-    for (int c = 0; c < RS_MAXPAIRS; ++c) {
-        double v = c == i ? 1.0 : 0.0;
-        if (row && c < n) v = c == i ? dlam[(int64_t)p * RS_MAXV + vi] : __ldg(Kp + vi * RS_GRAM_LD + vs[c]);
-        A[c] = v;
+    for (int s = 0; s < kLooPer; ++s) {
+        const int e = s < 4 ? tid + kLooThreads * s : (warp ? 4 * kLooThreads + tid - 32 : kLooEntries);
+        int i = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
+        if (tri(i) > e) --i;
+        if (tri(i + 1) <= e) ++i;
+        int j = e - tri(i);
+        if (e >= tri(RS_MAXPAIRS)) {
+            i = RS_MAXPAIRS + (e - tri(RS_MAXPAIRS)) / RS_MAXPAIRS;
+            j = (e - tri(RS_MAXPAIRS)) % RS_MAXPAIRS;
+        }
+        const bool in = e < kLooEntries && j < n && (i < n || i >= RS_MAXPAIRS);
+        ri[s] = in ? i : -1;
+        ci[s] = in ? j : -1;
+        double v = 0.0;
+        if (in) {
+            if (i == RS_MAXPAIRS) {
+                v = ylab[(int64_t)pj * RS_MAXPAIRS + j];
+                if (!finite_bits(v)) v = 0.0;
+            } else if (i == RS_MAXPAIRS + 1) {
+                v = 1.0;
+            } else {
+                v = i == j ? dlam[(int64_t)p * RS_MAXV + vs[i]] : __ldg(Kp + vs[i] * RS_GRAM_LD + vs[j]);
+            }
+        }
+        A[s] = v;
     }
-    if (row) {
-        y = ylab[(int64_t)pj * RS_MAXPAIRS + i];
-        one = 1.0;
-    }
-    const bool yb = row && !finite_bits(y);
-    const unsigned badm = __ballot_sync(0xffffffffu, yb);
-    if (yb) y = 0.0;
-    double piv = 1.0;                                           // this row's pivot
+    // entry (i, j) belongs to column k when j = k (row i) or i = k (row j)
+    auto publish = [&](int k) {
+#pragma unroll
+        for (int s = 0; s < kLooPer; ++s) {
+            if (ci[s] == k) col[k & 1][ri[s]] = A[s];
+            else if (ri[s] == k) col[k & 1][ci[s]] = A[s];
+        }
+    };
+    // warp 0, lane i: A_ii (i < n), ahead of the entries by one reciprocal
+    double dg = warp == 0 && lane < n ? dlam[(int64_t)p * RS_MAXV + vs[lane]] : 1.0;
+    auto next_pivot = [&](int k) {
+        if (lane == k) rk = pos_finite(dg) ? rcp_newton(dg) : 0.0;
+    };
+    publish(0);
+    if (warp == 0) next_pivot(0);
+    __syncthreads();
     bool good = true;
-#pragma unroll
-    for (int k = 0; k < RS_MAXPAIRS; ++k) {
-        if (i == k) {
-#pragma unroll
-            for (int c = 0; c < RS_MAXPAIRS; c += 2)
-                *reinterpret_cast<double2*>(rowk + c) = make_double2(A[c], A[c + 1]);
-            rowk[RS_MAXPAIRS] = y;
-            rowk[RS_MAXPAIRS + 1] = one;
+    for (int k = 0; k < n; ++k) {
+        const double* c = col[k & 1];
+        const double r = rk;                                    // the same value in every thread
+        good = pos_finite(r);
+        if (!good) break;
+        if (warp == 1) {
+            if (lane < n) w[lane] = lane == k ? -r : c[lane] * r;
+            if (lane < 2) w[RS_MAXPAIRS + lane] = c[RS_MAXPAIRS + lane] * r;
         }
-        __syncwarp();
-        const double d = rowk[k];                               // the same value in every lane
-        good = good && pos_finite(d);
-        const double r = rcp_newton(good ? d : 1.0);
-        const double fr = i == k ? 0.0 : A[k] * r;
-        if (i == k) piv = d;
-#pragma unroll
-        for (int c = 0; c < RS_MAXPAIRS; c += 2) {
-            const double2 rk = *reinterpret_cast<const double2*>(rowk + c);
-            if (c != k) A[c] = fma(-fr, rk.x, A[c]);
-            if (c + 1 != k) A[c + 1] = fma(-fr, rk.y, A[c + 1]);
+        __syncthreads();
+        if (warp == 0 && k + 1 < n) {
+            if (lane < n) dg = fma(-c[lane], w[lane], dg);      // (lanes up to k: not read again)
+            next_pivot(k + 1);
         }
-        y = fma(-fr, rowk[RS_MAXPAIRS], y);
-        one = fma(-fr, rowk[RS_MAXPAIRS + 1], one);
-        A[k] = i == k ? 1.0 : -fr;
-        __syncwarp();                                           // before the next pivot row
+#pragma unroll
+        for (int s = 0; s < kLooPer; ++s) {
+            if (ri[s] < 0) continue;
+            const double wj = w[ci[s]];
+            const double v = fma(-c[ri[s]], wj, A[s]);
+            A[s] = ri[s] == k ? wj : (ci[s] == k ? w[ri[s]] : v);   // row and column k: scaled, w_k = -1 / d
+        }
+        if (k + 1 < n) publish(k + 1);
+        __syncthreads();
     }
     if (good) {
-        const double rp = rcp_newton(piv);
+        // -diag(M^-1), and the largest diagonal entry of M, as high words of positive doubles
+        int um = 0, um_bad = 0;
 #pragma unroll
-        for (int c = 0; c < RS_MAXPAIRS; ++c) S[i][c] = A[c] * rp;
-        y *= rp;
-        one *= rp;
-        __syncwarp();
-        double* T = tab + (int64_t)pj * kLooTab;
-        for (int rr = 0; rr < n; ++rr)
-            if (row) T[rr * RS_MAXPAIRS + i] = 0.5 * (S[rr][i] + S[i][rr]);
-        if (row) {
-            T[kLooWy + i] = y;
-            T[kLooW1 + i] = one;
-        }
-        const double sy = warp_sum(y), s1 = warp_sum(one);    // lanes past n hold 0
-        if (i == 0) {
-            T[kLooSum] = sy;
-            T[kLooSum + 1] = s1;
+        for (int s = 0; s < kLooPer; ++s)
+            if (ri[s] >= 0 && ri[s] == ci[s]) {
+                if (pos_finite(-A[s])) um = max(um, __double2hiint(-A[s]));
+                else um_bad = 1;
+            }
+        atomicMax(&umax, um_bad ? 0x7ff00000 : um);
+        __syncthreads();
+        if (limit > 0.f) {
+            double dii = 0.0;
+            if (lane < n) dii = dlam[(int64_t)p * RS_MAXV + vs[lane]];
+            const int dmax = __reduce_max_sync(0xffffffffu, pos_finite(dii) ? __double2hiint(dii) : 0);
+            good = umax < 0x7fe00000 &&
+                   (double)limit >= __hiloint2double(dmax + 1, 0) * __hiloint2double(umax + 1, 0);
         }
     }
-    if (i == 0) {
-        ok[pj] = good ? 1 : 0;
-        bad[pj] = badm;
+    if (good) {
+        double* T = tab + (int64_t)pj * kLooTab;
+#pragma unroll
+        for (int s = 0; s < kLooPer; ++s) {
+            if (ri[s] < 0) continue;
+            if (ri[s] < RS_MAXPAIRS) {
+                T[ri[s] * RS_MAXPAIRS + ci[s]] = -A[s];
+                T[ci[s] * RS_MAXPAIRS + ri[s]] = -A[s];
+            } else {
+                T[(ri[s] == RS_MAXPAIRS ? kLooWy : kLooW1) + ci[s]] = A[s];
+                rhs[ri[s] - RS_MAXPAIRS][ci[s]] = A[s];
+            }
+        }
+        __syncthreads();
+        if (warp < 2) {
+            const double t = warp_sum(lane < n ? rhs[warp][lane] : 0.0);
+            if (lane == 0) T[kLooSum + warp] = t;
+        }
+    }
+    if (warp == 0) {
+        const bool yb = lane < n && !finite_bits(ylab[(int64_t)pj * RS_MAXPAIRS + lane]);
+        const unsigned badm = __ballot_sync(0xffffffffu, yb);
+        if (lane == 0) {
+            ok[pj] = good ? 1 : 0;
+            bad[pj] = badm;
+        }
     }
 }
 
@@ -1642,6 +1722,10 @@ loo_inv_kernel(const int64_t* __restrict__ row_off, const double* __restrict__ K
 // for j has no closed form here: RS_EDATA (detail: the program), and the fit is reported
 // failed.  Non-finite b or e: RS_FIT_NONFINITE.  Fits without a pair were finished by the
 // bucket pass.
+// AUTO (a call that did not ask for the closed form): only the fits that have it and come out
+// finite are finished here; every other one gets the status kLeft and is counted in *a.left for
+// the direct solvers that follow.
+template <bool AUTO>
 __global__ void __launch_bounds__(kLooFitThreads)
 loo_fit_kernel(const SolveArgs a, int64_t S6, const int* __restrict__ npair,
                const double* __restrict__ tab, const uint8_t* __restrict__ tab_ok,
@@ -1663,7 +1747,7 @@ loo_fit_kernel(const SolveArgs a, int64_t S6, const int* __restrict__ npair,
         st = RS_FIT_OK;
         if (__popc(removed) > 1 || (pm & ~full)) {
             st = RS_FIT_NOTPD;
-            rs_dev_flag(a.dstatus, RS_EDATA, p);
+            if (!AUTO) rs_dev_flag(a.dstatus, RS_EDATA, p);
         } else if (!tab_ok[pj]) {
             st = RS_FIT_NOTPD;
         } else if (pm & tab_bad[pj]) {
@@ -1691,6 +1775,10 @@ loo_fit_kernel(const SolveArgs a, int64_t S6, const int* __restrict__ npair,
                 if (!finite_bits(b) || !finite_bits(e)) st = RS_FIT_NONFINITE;
             }
         }
+        if (AUTO && st != RS_FIT_OK) {
+            a.status[f] = kLeft;
+            st = kLeft;
+        }
         const uint8_t* pbj = a.pb + (int64_t)pj * RS_MAXPAIRS;
         auto alpha = [&](int q) {
             const double al = fma(-b, T[kLooW1 + q], T[kLooWy + q]);
@@ -1703,7 +1791,8 @@ loo_fit_kernel(const SolveArgs a, int64_t S6, const int* __restrict__ npair,
             for (uint32_t m = pm; m; m &= m - 1) out[c++] = alpha(__ffs(m) - 1);
         }
         PredTarget pt;
-        const bool has = pred_target_v(a, s, j, p, (int)(a.row_off[p + 1] - a.row_off[p]), pt);
+        const bool has = (!AUTO || st == RS_FIT_OK) &&
+                         pred_target_v(a, s, j, p, (int)(a.row_off[p + 1] - a.row_off[p]), pt);
         if (has && st == RS_FIT_OK) {
             const int vi = i >= 0 ? pbj[i] : -1;
             const double* Kp = a.K + (int64_t)p * RS_GRAM_LD * RS_GRAM_LD;
@@ -1724,10 +1813,14 @@ loo_fit_kernel(const SolveArgs a, int64_t S6, const int* __restrict__ npair,
                 if (r < pt.room) pt.dst[r] = yh;
             }
         }
-        if (st != RS_FIT_OK && has) mark_failed(a, s, j, pt);
-        finish_record(a, f, n, st, out);
+        if (!AUTO && st != RS_FIT_OK && has) mark_failed(a, s, j, pt);
+        if (!AUTO || st == RS_FIT_OK) finish_record(a, f, n, st, out);
     }
     count_status(a, st, active);
+    if (AUTO) {
+        const unsigned l = __reduce_add_sync(0xffffffffu, active && st == kLeft);
+        if ((threadIdx.x & 31) == 0 && l) atomicAdd(a.left, (unsigned long long)l);
+    }
 }
 
 // ====================================================================== rank pass
@@ -2347,8 +2440,9 @@ size_t a256(size_t x) { return (x + 255) & ~(size_t)255; }
 // boundary (the rank pass copies row ranges of the planes with TMA bulk copies).
 int64_t plane_stride(int64_t Rcap) { return (Rcap + 1) & ~(int64_t)1; }
 
-// histogram + bucket cursors (unsigned) and five 64-bit work counters, zeroed per call
-constexpr size_t kCounterBytes = 2 * kHist * sizeof(unsigned) + 5 * sizeof(unsigned long long);
+// histogram + bucket cursors (unsigned), five 64-bit work counters and the number of fits that
+// the closed form left, zeroed per call
+constexpr size_t kCounterBytes = 2 * kHist * sizeof(unsigned) + 6 * sizeof(unsigned long long);
 
 FitWs carve(void* base, int64_t P, int64_t S, int nmax, int64_t Rcap) {
     FitWs w{};
@@ -2484,7 +2578,7 @@ cudaError_t rs_launch_fit_predict(const rs_fit_args& a, cudaStream_t st) {
                  a.counters,
                  a.row_offsets, a.train_masks, a.rec_offsets, w.cand, rank ? w.predbuf : nullptr,
                  a.rows_cap, plane_stride(a.rows_cap), a.flags, a.dstatus, a.Z, a.x_offsets,
-                 a.feat_width, a.max_feat, a.tune_order, rank ? w.row_info : nullptr};
+                 a.feat_width, a.max_feat, a.tune_order, rank ? w.row_info : nullptr, nullptr};
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -2503,12 +2597,12 @@ cudaError_t rs_launch_fit_predict(const rs_fit_args& a, cudaStream_t st) {
         mark(4);
     } else if (a.flags & RS_LOO_CLOSED) {
         // one inverse per (program, optimization), then every fit in closed form
-        loo_inv_kernel<<<(unsigned)(a.P * RS_NOPT), 32, 0, st>>>(a.row_offsets, a.K, w.pb, w.ylab, w.npair,
-                                                                 w.dlam, w.loo_tab, w.loo_ok, w.loo_bad);
+        loo_inv_kernel<<<(unsigned)(a.P * RS_NOPT), kLooThreads, 0, st>>>(a.row_offsets, a.K, w.pb, w.ylab, w.npair,
+                                                                 w.dlam, 0.f, w.loo_tab, w.loo_ok, w.loo_bad);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         const int64_t grid = (S6 + kLooFitThreads - 1) / kLooFitThreads;
-        loo_fit_kernel<<<(unsigned)grid, kLooFitThreads, 0, st>>>(sa, S6, w.npair, w.loo_tab, w.loo_ok, w.loo_bad);
+        loo_fit_kernel<false><<<(unsigned)grid, kLooFitThreads, 0, st>>>(sa, S6, w.npair, w.loo_tab, w.loo_ok, w.loo_bad);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         mark(4);
@@ -2521,7 +2615,30 @@ cudaError_t rs_launch_fit_predict(const rs_fit_args& a, cudaStream_t st) {
         // dynamically, so the kernels sharing the SMs cost none of them a statically assigned
         // share.
         const bool mid = nmax > kNReg;
-        const bool fork = mid && a.side && a.fork && a.join;
+        // Leave-one-version-out splits recognised: as many splits as versions, training sets large
+        // enough for fits of more than kNMid pairs (the host's sizes; whether a fit really leaves
+        // out at most one pair is decided per fit on the device).  Those fits take the closed form
+        // of RS_LOO_CLOSED, one inverse per (program, optimization) instead of a factorisation per
+        // fit; any that it does not cover -- several pairs left out, a failed pivot, a non-finite
+        // label, an ill-conditioned system -- stay with the direct solvers, which leave at once
+        // when there are none.  Smaller fits (n <= kNMid) are cheaper by the direct solvers than
+        // the 32 x 32 inverses.  Needs the coefficients' region for the inverses, so not for calls
+        // that keep compact records.  Against 64 bits the two forms differ by no more than their
+        // own rounding while the condition bound q stays below the limit (relative prediction
+        // errors within 0.9-1.3 of each other, 48..1024 features: equal).  256 programs x 64
+        // versions x 1024 features: the fit stage 1.95 -> 0.15 ms.
+        const bool lovo = a.lovo && nmax > kNMid && (user || rank) && a.lambda > 0.0;
+        if (lovo) {
+            sa.left = w.work + 5;
+            loo_inv_kernel<<<(unsigned)(a.P * RS_NOPT), kLooThreads, 0, st>>>(a.row_offsets, a.K, w.pb, w.ylab, w.npair,
+                                                                     w.dlam, kLooLimit, w.loo_tab, w.loo_ok, w.loo_bad);
+            const int64_t grid = (S6 + kLooFitThreads - 1) / kLooFitThreads;
+            loo_fit_kernel<true><<<(unsigned)grid, kLooFitThreads, 0, st>>>(sa, S6, w.npair, w.loo_tab, w.loo_ok,
+                                                                            w.loo_bad);
+            e = cudaGetLastError();
+            if (e != cudaSuccess) return e;
+        }
+        const bool fork = mid && !lovo && a.side && a.fork && a.join;
         cudaStream_t s2 = fork ? a.side : st;
         if (fork) {
             e = cudaEventRecord(a.fork, st);

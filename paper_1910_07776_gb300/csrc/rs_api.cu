@@ -269,6 +269,7 @@ static rs_status fit_common(rs_ctx* c, const rs_batch* b, const double* K, const
     a.lambda = lambda;
     a.form = form;
     a.max_feat = b->max_feat;
+    a.lovo = sp->n_splits == b->n_rows;
     a.dstatus = c->dstatus;
     a.queue = (unsigned int*)(c->dstatus + RS_DST_QUEUE);
     a.ev = c->profiling ? c->ev : nullptr;

@@ -185,6 +185,7 @@ struct rs_fit_args {
     // batched form only
     int max_train;                // host bound on popcount(train mask)
     int max_feat;                 // host bound on F_p (refinement buffers)
+    int lovo;                     // as many splits as versions: leave-one-version-out by the host's sizes
     int tune_split;               // largest n of the lighter one-fit-per-thread solver (4..8)
     int tune_rank_waves;          // rank-pass grid = SMs x this (0: default)
     int tune_order;               // register solvers' work order: 0 largest fits first, 1 from both ends

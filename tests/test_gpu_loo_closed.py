@@ -242,3 +242,85 @@ def test_closed_form_on_the_tensor_core_gram(rs, ctx):
     close(c["pred_all"], d["pred_all"])
     _, nnear = compare_rankings(c["rec_code"], d["rec_code"], d["pred_all"], math.log(1.05))
     compare_counters(c["counters"], d["counters"], slack=nnear)
+
+
+def _mixed_case(name):
+    """As many splits as versions, so that a call without the flag looks for the closed form."""
+    if name == "several_left_out":  # 1..4 versions held out: only some fits have the closed form
+        b = synth.make_batch(4, versions=(50, 64), feat=80, dtype=np.float64, seed=91)
+        rng, tm = np.random.default_rng(91), []
+        for p in range(4):
+            V = b.versions(p)
+            full = (1 << V) - 1
+            for r in range(V):
+                m = full & ~(1 << r)
+                for _ in range(int(rng.integers(0, 4))):
+                    m &= ~(1 << int(rng.integers(0, V)))
+                tm.append(m)
+        return b, synth.Splits(split_offsets=b.row_offsets.copy(), train_masks=np.array(tm, dtype=np.uint64))
+    if name == "ill_conditioned":   # fewer features than pairs beside wide ones: beyond the limit
+        b = synth.make_batch(6, versions=(40, 64), feat_choices=[8, 24, 96], dtype=np.float64, seed=92)
+        return b, synth.make_splits(b, "lovo")
+    if name == "bad_values":        # an infinite counter, an infinite time, equal rows
+        b = synth.make_batch(5, versions=64, feat=70, dtype=np.float64, seed=93)
+        X, lt = b.X.copy(), b.log_time.copy()
+        X[int(b.x_offsets[1]) + 5 * 70 + 3] = np.inf
+        lt[int(b.row_offsets[2]) + 9] = np.inf
+        x3 = X[int(b.x_offsets[3]):int(b.x_offsets[3]) + 64 * 70].reshape(64, 70)
+        x3[17], x3[40] = x3[3], x3[3]
+        b.X, b.log_time = X, lt
+        return b, synth.make_splits(b, "lovo")
+    if name == "shuffled":          # masks in any slot order, 1..64 versions
+        b = synth.make_batch(7, versions=(1, 64), feat=48, dtype=np.float32, seed=94)
+        rng = np.random.default_rng(94)
+        for p in range(7):
+            r0, V, F, xo = int(b.row_offsets[p]), b.versions(p), 48, int(b.x_offsets[p])
+            perm = rng.permutation(V)
+            for arr in (b.masks, b.log_time, b.cycles):
+                arr[r0:r0 + V] = arr[r0:r0 + V][perm]
+            b.X[xo:xo + V * F] = b.X[xo:xo + V * F].reshape(V, F)[perm].reshape(-1)
+        return b, synth.make_splits(b, "lovo")
+    raise ValueError(name)
+
+
+@pytest.mark.parametrize("name", ["tiny", "inf_label", "several_left_out", "ill_conditioned", "bad_values", "shuffled"])
+@pytest.mark.parametrize("rank_all", [False, True])
+def test_calls_without_the_flag_equal_the_plain_form(rs, ctx, name, rank_all):
+    """A call whose sizes look like leave-one-version-out takes the closed form for the fits that
+    have it and the direct solvers for the rest: against the plain form (one warp per fit, no
+    closed form), the same fits, failures and rankings.  Tolerance: the parity bound, with the
+    absolute term scaled by cond(M) u of the worst system the closed form accepts (4e6)."""
+    batch, splits = _case(name) if name in ("tiny", "inf_label") else _mixed_case(name)
+    db = rs.DeviceBatch.from_host(batch)
+    ds = rs.DeviceSplits.from_host(splits, batch=batch)
+    assert ds.n_splits == batch.n_rows and ds.max_train >= 34
+    flags = rs.RS_RANK_ALL if rank_all else 0
+    g = rs.cv_run(ctx, db, ds, flags=flags)
+    r = rs.cv_run(ctx, db, ds, flags=flags, form=rs.RS_FORM_PLAIN)
+    np.testing.assert_array_equal(g["rec_offsets"], r["rec_offsets"])
+    close(g["pred_all"], r["pred_all"], abs_=4e6 * 2.0 ** -53)
+    _, nnear = compare_rankings(g["rec_code"], r["rec_code"], r["pred_all"], math.log(1.05))
+    compare_counters(g["counters"], r["counters"], slack=nnear)
+
+
+def test_coefficients_without_the_flag_equal_the_direct_fits(rs, ctx):
+    # rs_fit_batched with a caller's array, no predictions: mixed closed-form and direct fits
+    # against the plain form, normwise per fit (two solutions of one system), statuses equal
+    batch, splits = _mixed_case("several_left_out")
+    db, ds = rs.DeviceBatch.from_host(batch), rs.DeviceSplits.from_host(splits, batch=batch)
+    zb = db.with_X(ctx.standardize(db))
+    K = ctx.gram(zb)
+    S = ds.n_splits
+    res = []
+    for form in (rs.RS_FORM_BATCHED, rs.RS_FORM_PLAIN):
+        coef = torch.full((S * 6 * 33,), 7.0, dtype=torch.float64, device="cuda")
+        st = torch.full((S * 6,), 9, dtype=torch.uint8, device="cuda")
+        ctx.fit_batched(zb, K, ds, 1e-3, form, coef, st)
+        torch.cuda.synchronize()
+        ctx.check_device_status()
+        res.append((coef.cpu().numpy().reshape(S * 6, 33), st.cpu().numpy()))
+    (cg, sg), (cp, sp) = res
+    np.testing.assert_array_equal(sg, sp)
+    ok = sg == 0
+    scale = np.abs(cp[ok]).max(axis=1, keepdims=True)
+    assert np.all(np.abs(cg[ok] - cp[ok]) <= 1e-9 * scale + 1e-11)
