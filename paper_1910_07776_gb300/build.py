@@ -39,25 +39,27 @@ def _stale(srcs, target) -> bool:
 
 
 def write_log_table(path: str) -> None:
-    """Constants of the table-driven logarithm of the standardization kernel, correctly
-    rounded to FP64 from exact decimal arithmetic (the same values on every build machine):
-    log F_i and 1 / F_i for the centres F_i = 1 + (2 i + 1) / 512 of the 256 intervals of
-    width 1/256 that split the mantissa range [1, 2); ln 2; and log(1e-30), the clamp value."""
+    """Constants of the standardization's fixed-point logarithm, rounded from exact decimal
+    arithmetic (the same values on every build machine).  For the centres F_i = 1 + (2 i + 1) / 512
+    of the 256 intervals of width 1/256 that split the mantissa range [1, 2): the 11-bit integer c_i
+    nearest 2^11 / F_i, and -log(c_i / 2^11) in units of 2^-63; ln 2 in units of 2^-63 as two signed
+    32-bit halves; and log(1e-30), the clamp value, in units of 2^-53."""
     from decimal import Decimal, getcontext
     getcontext().prec = 60
-    lines = ["// generated by build.py (write_log_table): do not edit", "#pragma once", ""]
-    logs, invs = [], []
+    logs, rcps = [], []
     for i in range(256):
-        F = Decimal(1) + Decimal(2 * i + 1) / Decimal(512)
-        logs.append(float(F.ln()).hex())
-        invs.append(float(Decimal(1) / F).hex())
-    ln2 = Decimal(2).ln()
-    eps = Decimal(1e-30)                 # the FP64 value nearest 1e-30, exactly
-    lines.append("__device__ const double kLogTabF[256] = {" + ", ".join(logs) + "};")
-    lines.append("__device__ const double kLogTabInv[256] = {" + ", ".join(invs) + "};")
-    lines.append(f"constexpr double kLn2 = {float(ln2).hex()};")
-    lines.append(f"constexpr double kLogClamp = {float(eps.ln()).hex()};   // log(1e-30)")
-    txt = "\n".join(lines) + "\n"
+        c = int((Decimal(2048) / (Decimal(1) + Decimal(2 * i + 1) / Decimal(512))).to_integral_value())
+        rcps.append(str(c))
+        logs.append(f"{int((-(Decimal(c) / Decimal(2048)).ln() * 2 ** 63).to_integral_value())}ll")
+    ln2 = int((Decimal(2).ln() * 2 ** 63).to_integral_value())
+    lo = (ln2 + 2 ** 31) % 2 ** 32 - 2 ** 31
+    clamp = int((Decimal(1e-30).ln() * 2 ** 53).to_integral_value())   # the FP64 value nearest 1e-30
+    txt = "\n".join([
+        "// generated by build.py (write_log_table): do not edit", "#pragma once", "#include <stdint.h>", "",
+        "__device__ const long long kFixLogTab[256] = {" + ", ".join(logs) + "};",
+        "__device__ const uint16_t kFixRcpTab[256] = {" + ", ".join(rcps) + "};",
+        f"constexpr int kFixLn2Hi = {(ln2 - lo) // 2 ** 32}, kFixLn2Lo = {lo};",
+        f"constexpr long long kFixClamp = {clamp}ll;", ""])
     if not os.path.exists(path) or open(path).read() != txt:
         with open(path, "w") as f:
             f.write(txt)

@@ -1,10 +1,13 @@
 // K1: feature vectors (Sec. 2: counters normalised by the cycle count), followed by the
 // library's log / per-program z-score reading.  One read of X, one write of Z.
 //
-// The logarithm runs once per element on this part's narrow FP64 pipe, so it is written
-// here to need few FP64 instructions (log_pos below, 9 of them); X is read once, spread
-// over sixteen row groups per feature, in blocks small enough (16 features) that programs
-// of different sizes spread evenly over the SMs.
+// This part's FP64 pipe takes 64 cycles for a warp instruction, its integer multiplier 2 to 4, so
+// the logarithms, their mean and the centring run in 64-bit fixed point (53 fraction bits, |log q|
+// < 1024) and FP64 is left with two instructions per element: the square that the deviation sums
+// and the product that scales it.  log(x / c) is log x - log c, the second taken once per version.
+// 256 programs x 64 versions x 1024 FP64 counters: 562 -> 149 us (the two passes over
+// memory alone take 40 us); 64 programs x 40 x 256 FP32: 41 -> 16 us.
+#include "rank_row.cuh"
 #include "rs_internal.cuh"
 #include "rs_log_table.h"
 
@@ -12,135 +15,226 @@ namespace {
 
 constexpr long long kClampBits = 0x39b4484bfeebc2a0ll;   // bit pattern of 1e-30
 constexpr long long kInfBits = 0x7ff0000000000000ll;
+constexpr long long kFixInf = 0x7fffffffffffffffll;       // log of +inf
+constexpr long long kFixNone = -0x7fffffffffffffffll - 1; // a cycle count outside the fast range
 
-// log q for a positive, normal, finite q, table-driven (after P. T. P. Tang, "Table-driven
-// implementation of the logarithm function in IEEE floating-point arithmetic", ACM TOMS
-// 16(4), 1990): q = 2^e m with m in [1, 2); F = the centre of m's interval of width 1/256
-// (index i = the top eight fraction bits of m); r = m (1/F) - 1 in one FMA, |r| <= 2^-9;
-//     log q = e ln2 + (log F + log1p(r)),
-// log1p(r) by its Taylor series up to r^5 (the first term left out, r^6 / 6, is below
-// 2^-56), e ln2 as one FMA with ln 2 rounded to FP64.  9 FP64 instructions.  Against an
-// extended-precision log over 3e7 arguments (1e-29 .. 1e31, exponents -1000 .. 1000, and
-// q within 0.5 % of 1) the error is at most 2.4 units of 2^-53 max(1, |log q|), rms 0.52 --
-// the same as Tang's exact reduction m - F and split ln 2 (2.2, rms 0.51), which took three
-// more FP64 instructions.
-__device__ __forceinline__ double log_pos(double q, const double* tlog, const double* tinv) {
-    const long long b = __double_as_longlong(q);
-    const int i = (int)((b >> 44) & 0xff);
-    const double m = __longlong_as_double((b & 0x000fffffffffffffll) | 0x3ff0000000000000ll);
-    const double r = fma(m, tinv[i], -1.0);
-    double p = fma(r, 0.2, -0.25);
-    p = fma(p, r, 1.0 / 3.0);
-    p = fma(p, r, -0.5);
-    const double l1p = fma(r * r, p, r);
-    // e as a double without a conversion instruction: 2^52 + 2048 + e, minus 2^52 + 2048
-    const long long eb = (b >> 52) - 1023 + 2048;
-    const double ed = __longlong_as_double(0x4330000000000000ll | eb) - 4503599627372544.0;
-    return fma(ed, kLn2, tlog[i] + l1p);
+// log q in units of 2^-53 for the bit pattern of a positive, normal, finite q = 2^e m, m in
+// [1, 2).  After P. T. P. Tang's table-driven method (ACM TOMS 16(4), 1990), in integers: the top
+// eight fraction bits of m pick an 11-bit c with m c / 2^11 = 1 + r, |r| < 1.26 2^-9, so r is exact
+// in 63 fraction bits; log q = e ln2 - log(c / 2^11) + r - r^2/2 + r^3/3 - r^4/4 + r^5/5 - r^6/6.
+// r^2 comes from r's 39-bit and 24-bit halves (78 fraction bits), r^3/3 from 31-bit pieces, the
+// terms from r^4 on (below 2^-36) in FP32 with the 2^23-offset conversion; ln2 and the logarithms
+// have 63 fraction bits.  Against an 80-bit logarithm over 8e7 arguments (exponents -511 .. 510,
+// and q within 2^-50 .. 1 of 1): error at most 0.625 units of 2^-53, rms 0.27 (the FP64 form it
+// replaces: 2.4 units of 2^-53 max(1, |log q|), rms 0.52, and 9 FP64 instructions).
+__device__ __forceinline__ long long fix_log(unsigned hi, unsigned lo, const long long* tl, const uint16_t* tc) {
+    const int e = (int)(hi >> 20) - 1023;
+    const unsigned mh = (hi & 0xfffffu) | 0x100000u;
+    const int i = (int)(mh >> 12) & 0xff;
+    const unsigned c = tc[i];
+    const long long r = (long long)(((unsigned long long)(mh * c - 0x80000000u) << 32) + (unsigned long long)lo * c);
+    const int rh = (int)((r + (1 << 23)) >> 24);                       // 39 fraction bits
+    const int rl = (int)(r - ((long long)rh << 24));
+    const long long r2 = (long long)rh * rh + (((long long)rh * rl) >> 23);        // 78
+    const int r23 = (int)(((long long)(int)(r2 >> 30) * 0x55555555) >> 31);        // r^2 / 3: 49
+    const long long t3 = (long long)r23 * rh;                          // 88
+    const float rf = (float)rh * 0x1p-39f, q = rf * rf;
+    const float t = fmaf(q * q * 0x1p58f, fmaf(q, -1.0f / 6.0f, fmaf(rf, 0.2f, -0.25f)), 12582912.0f);
+    const int ti = __float_as_int(t) - 0x4B400000;                     // 58
+    const long long s = tl[i] + r - (r2 >> 16) + (t3 >> 25) + ((long long)ti << 5);
+    return ((long long)e * kFixLn2Hi << 22) + (((long long)e * kFixLn2Lo + s + 512) >> 10);
 }
 
-// log(max(q, 1e-30)) with the branches of the plain definition: q above the clamp and finite
-// -> log_pos (subnormal q never reach it); +inf -> +inf; q <= 1e-30 or NaN -> log(1e-30).
-__device__ __forceinline__ double log_clamped(double q, const double* tlog, const double* tinv) {
-    const long long b = __double_as_longlong(q);
-    if (b > kClampBits && b < kInfBits) return log_pos(q, tlog, tinv);
-    return b == kInfBits ? q : kLogClamp;
+// The value 2^-53 v as a double, rounded to nearest, by integer operations.
+__device__ __forceinline__ double fix_double(long long v) {
+    const unsigned long long a = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+    if (a == 0) return 0.0;
+    const int lz = __clzll((long long)a);
+    const unsigned long long m = a << lz;
+    const unsigned long long b = ((unsigned long long)(1023 - 53 + 63 - 1 - lz) << 52) + (m >> 11) + ((m >> 10) & 1ull);
+    return __longlong_as_double((long long)(b | ((unsigned long long)v & 0x8000000000000000ull)));
 }
 
-// An input element as a double: FP32 values are re-packed with integer operations (exact for
-// normal numbers); zeros, subnormals, infinities and NaNs take the conversion instruction.
-__device__ __forceinline__ double as_double(float x) {
+__device__ __forceinline__ long long fix_log(double q, const long long* tl, const uint16_t* tc) {
+    const long long b = __double_as_longlong(q);
+    return fix_log((unsigned)(b >> 32), (unsigned)b, tl, tc);
+}
+
+// log(max(q, 1e-30)) with the branches of the plain definition: above the clamp and finite -> its
+// logarithm (subnormal q never reach it); +inf -> +inf; q <= 1e-30 or NaN -> log(1e-30).
+__device__ __forceinline__ long long fix_log_clamped(double q, const long long* tl, const uint16_t* tc) {
+    const long long b = __double_as_longlong(q);
+    if (b > kClampBits && b < kInfBits) return fix_log(q, tl, tc);
+    return b == kInfBits ? kFixInf : kFixClamp;
+}
+
+// A version's cycle count: its logarithm, or kFixNone unless it is positive with an exponent in
+// -511 .. 511 (then the difference of two logarithms of that range fits the fixed point).
+__device__ __forceinline__ bool fast_hi(unsigned hi) { return hi - (512u << 20) < (1023u << 20); }
+__device__ __forceinline__ long long cycle_log(double c, const long long* tl, const uint16_t* tc) {
+    return fast_hi((unsigned)__double2hiint(c)) ? fix_log(c, tl, tc) : kFixNone;
+}
+
+// log(max(x / c, 1e-30)) of an element; lc = cycle_log(c).  Any value outside the fast range (zeros,
+// subnormals, negatives, infinities, NaN, extreme exponents) takes the plain definition's division.
+__device__ __forceinline__ long long elem_log(double x, bool cyc, double c, long long lc, const long long* tl,
+                                              const uint16_t* tc) {
+    const unsigned hi = (unsigned)__double2hiint(x);
+    if (!fast_hi(hi) || (cyc && lc == kFixNone)) return fix_log_clamped(cyc ? x * (1.0 / c) : x, tl, tc);
+    const long long l = fix_log(hi, (unsigned)__double2loint(x), tl, tc) - (cyc ? lc : 0ll);
+    return l > kFixClamp ? l : kFixClamp;
+}
+__device__ __forceinline__ long long elem_log(float x, bool cyc, double c, long long lc, const long long* tl,
+                                              const uint16_t* tc) {
     const unsigned u = __float_as_uint(x);
-    const unsigned ex = (u >> 23) & 0xff;
-    if (ex == 0 || ex == 0xff) return (double)x;
-    return __longlong_as_double(((long long)(u & 0x80000000u) << 32) |
-                                ((long long)(ex - 127 + 1023) << 52) | ((long long)(u & 0x7fffff) << 29));
+    if (u - (1u << 23) >= (254u << 23) || (cyc && lc == kFixNone))     // not a positive normal number
+        return fix_log_clamped(cyc ? (double)x * (1.0 / c) : (double)x, tl, tc);
+    const long long l = fix_log((u >> 3) + (896u << 20), u << 29, tl, tc) - (cyc ? lc : 0ll);
+    return l > kFixClamp ? l : kFixClamp;
 }
-__device__ __forceinline__ double as_double(double x) { return x; }
 
-constexpr int kFeat = 16;                    // features per block
-constexpr int kGroups = 16;                  // row groups per block
-constexpr int kThreads = kFeat * kGroups;
+__device__ __forceinline__ void load_log_tables(long long* tl, uint16_t* tc, int threads) {
+    for (int t = threadIdx.x; t < 256; t += threads) {
+        tl[t] = kFixLogTab[t];
+        tc[t] = kFixRcpTab[t];
+    }
+}
 
-// Block = (program, 16-feature slice); thread (g, f) takes rows g, g + 16, ... of feature f.
-// A warp reads 16 consecutive features of two rows (64-byte segments).  The log values stay in
-// shared memory; per-feature sums are combined from the 16 row groups in a fixed order.
-template <typename T>
+constexpr int kThreads = 256;
+
+// The mean of n logarithms from the sums of their halves (v >> 24 and v & 0xffffff), rounded to
+// the fixed point.
+__device__ __forceinline__ long long fix_mean(long long hs, long long ls, int n) {
+    const long long q = hs / n;
+    const long long rem = ((hs - q * n) << 24) + ls;
+    return (q << 24) + (rem + (rem >= 0 ? n / 2 : -(n / 2))) / n;
+}
+
+// What the two kernels below do once a thread holds its ROWS logarithms of feature fl (rows g,
+// g + GROUPS, ..., those below n): the mean and the deviation over the n rows of the block's
+// feature, then the centred values (as doubles) and 1 / sigma (0: a constant or non-finite feature).
+template <int FEAT, int ROWS>
+struct StdSmem {
+    static constexpr int kGroups = kThreads / FEAT;
+    long long ph[kGroups][FEAT], mean[FEAT];
+    double pq[kGroups][FEAT], rs[FEAT];
+    unsigned pl[kGroups][FEAT];
+    int inf[FEAT];
+    long long tl[256];
+    uint16_t tc[256];
+};
+
+template <int FEAT, int ROWS>
+__device__ __forceinline__ double centre(StdSmem<FEAT, ROWS>& S, const long long (&l)[ROWS], double (&d)[ROWS], int n,
+                                         bool active, double* mu, double* sigma) {
+    constexpr int G = kThreads / FEAT;
+    const int fl = threadIdx.x % FEAT, g = threadIdx.x / FEAT;
+    long long hs = 0;
+    unsigned ls = 0;
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q)
+        if (active && g + G * q < n) {
+            if (l[q] == kFixInf) S.inf[fl] = 1;
+            hs += l[q] >> 24;
+            ls += (unsigned)l[q] & 0xffffffu;
+        }
+    S.ph[g][fl] = hs;
+    S.pl[g][fl] = ls;
+    __syncthreads();
+    if (threadIdx.x < FEAT) {
+        hs = 0;
+        long long lt = 0;
+#pragma unroll
+        for (int q = 0; q < G; ++q) {
+            hs += S.ph[q][fl];
+            lt += S.pl[q][fl];
+        }
+        S.mean[fl] = fix_mean(hs, lt, n);
+    }
+    __syncthreads();
+    const long long m = S.mean[fl];
+    double q2 = 0.0;
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q) {
+        d[q] = 0.0;
+        if (active && g + G * q < n) {
+            d[q] = fix_double(l[q] - m);
+            q2 = fma(d[q], d[q], q2);
+        }
+    }
+    S.pq[g][fl] = q2;
+    __syncthreads();
+    if (threadIdx.x < FEAT) {
+        double t = 0.0;
+#pragma unroll
+        for (int q = 0; q < G; ++q) t += S.pq[q][fl];
+        t = t * rcp_newton((double)n);
+        const bool inf = S.inf[fl] != 0;
+        const bool ok = !inf && t > 1e-24;                   // sigma > 1e-12
+        const double r = ok ? rsqrt_newton(t) : 0.0;
+        S.rs[fl] = r;
+        if (active && mu) *mu = inf ? __longlong_as_double(kInfBits) : fix_double(m);
+        if (active && sigma) *sigma = inf ? nan_d() : sqrt(t);
+    }
+    __syncthreads();
+    return S.rs[fl];
+}
+
+// Block = (program, FEAT-feature slice); thread (g, f) takes rows g, g + GROUPS, ... of feature f
+// and keeps them in registers.  A half-warp's or a warp's lanes read consecutive features.  32
+// features (8 rows a thread) halve the narrow per-feature work of the statistics per element and
+// are taken once the grid fills the chip (256 programs x 1024 features: 149 us against 177 with 16;
+// 64 x 256: 15.9 against 17.9); 16 (4 rows a thread) leave the shorter chain for few programs (2
+// programs x 96 features: 8.4 us against 9.9 with 32).
+template <typename T, int FEAT>
 __global__ void __launch_bounds__(kThreads)
 standardize_kernel(int P, const int64_t* __restrict__ row_off, const int32_t* __restrict__ fw,
                    const int64_t* __restrict__ xo, const int64_t* __restrict__ fo,
                    const T* __restrict__ X, const double* __restrict__ cycles,
                    double* __restrict__ Z, double* __restrict__ mu, double* __restrict__ sigma,
                    int* dstatus) {
-    __shared__ double lv[RS_MAXV][kFeat];
-    __shared__ double part[kGroups][kFeat];
-    __shared__ double stat[2][kFeat];
-    __shared__ double inv_c[RS_MAXV];
-    __shared__ double tlog[256], tinv[256];
+    constexpr int G = kThreads / FEAT, ROWS = RS_MAXV / G;
+    __shared__ StdSmem<FEAT, ROWS> S;
+    __shared__ double cyc_s[RS_MAXV];
+    __shared__ long long lc_s[RS_MAXV];
     const int p = blockIdx.x;
     const int64_t r0 = row_off[p];
     const int V = (int)(row_off[p + 1] - r0);
     const int F = fw[p];
-    const int fl = threadIdx.x % kFeat, g = threadIdx.x / kFeat;
-    const int f = blockIdx.y * kFeat + fl;
-    if (blockIdx.y * kFeat >= F) return;
+    const int fl = threadIdx.x % FEAT, g = threadIdx.x / FEAT;
+    const int f = blockIdx.y * FEAT + fl;
+    if (blockIdx.y * FEAT >= F) return;
     if (V < 1 || V > RS_MAXV) {
         if (threadIdx.x == 0 && blockIdx.y == 0) rs_dev_flag(dstatus, RS_EDATA, p);
         return;
     }
     const int64_t base = xo[p];
     const bool active = f < F;
-    // one reciprocal per version instead of a division per element (FP64 divisions are
-    // expensive on this part's narrow FP64 pipe)
-    if (cycles && threadIdx.x < V) inv_c[threadIdx.x] = 1.0 / cycles[r0 + threadIdx.x];
-    for (int t = threadIdx.x; t < 256; t += kThreads) {
-        tlog[t] = kLogTabF[t];
-        tinv[t] = kLogTabInv[t];
+    T x[ROWS];
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q) x[q] = active && g + G * q < V ? X[base + (int64_t)(g + G * q) * F + f] : (T)1;
+    load_log_tables(S.tl, S.tc, kThreads);
+    if (threadIdx.x < FEAT) S.inf[threadIdx.x] = 0;
+    __syncthreads();
+    if (cycles && threadIdx.x < V) {
+        const double c = cycles[r0 + threadIdx.x];
+        cyc_s[threadIdx.x] = c;
+        lc_s[threadIdx.x] = cycle_log(c, S.tl, S.tc);
     }
     __syncthreads();
-    double s = 0.0;
-    if (active)
-        for (int r = g; r < V; r += kGroups) {
-            double x = as_double(X[base + (int64_t)r * F + f]);
-            if (cycles) x = x * inv_c[r];
-            const double l = log_clamped(x, tlog, tinv);
-            lv[r][fl] = l;
-            s += l;
-        }
-    part[g][fl] = s;
-    __syncthreads();
-    if (g == 0) {
-        double t = 0.0;
-        for (int q = 0; q < kGroups; ++q) t += part[q][fl];
-        stat[0][fl] = t / V;
+    long long l[ROWS];
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q) {
+        const int r = g + G * q;
+        l[q] = r < V ? elem_log(x[q], cycles != nullptr, cyc_s[r], lc_s[r], S.tl, S.tc) : 0;
     }
-    __syncthreads();
-    const double m = stat[0][fl];
-    double q2 = 0.0;
-    if (active)
-        for (int r = g; r < V; r += kGroups) {
-            const double d = lv[r][fl] - m;
-            lv[r][fl] = d;                     // kept for the output
-            q2 += d * d;
-        }
-    part[g][fl] = q2;
-    __syncthreads();
-    if (g == 0) {
-        double t = 0.0;
-        for (int q = 0; q < kGroups; ++q) t += part[q][fl];
-        stat[1][fl] = sqrt(t / V);
-    }
-    __syncthreads();
+    double d[ROWS];
+    const double rs = centre(S, l, d, V, active, mu && active ? mu + fo[p] + f : nullptr,
+                             sigma && active ? sigma + fo[p] + f : nullptr);
     if (!active) return;
-    const double sd = stat[1][fl];
-    const bool ok = sd > 1e-12;
-    const double rs = ok ? 1.0 / sd : 0.0;
-    for (int r = g; r < V; r += kGroups)
-        Z[base + (int64_t)r * F + f] = ok ? lv[r][fl] * rs : 0.0;
-    if (g == 0) {
-        if (mu) mu[fo[p] + f] = m;
-        if (sigma) sigma[fo[p] + f] = sd;
-    }
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q)
+        if (g + G * q < V) Z[base + (int64_t)(g + G * q) * F + f] = rs > 0.0 ? d[q] * rs : 0.0;
 }
 
 // Standardization of the training side of a transfer (Table 2): problem q trains on the runs
@@ -149,8 +243,10 @@ standardize_kernel(int P, const int64_t* __restrict__ row_off, const int32_t* __
 // the vectors of all of them -- into Z in X's layout; mu, sigma at q * stat_stride + f.
 // Block = (problem, 16-feature slice), as standardize_kernel with up to kGroupRows rows.
 constexpr int kGroupRows = RS_MAXV * RS_MAXRUNS;
+constexpr int kFeat = 16;                    // features per block
+constexpr int kGroups = kThreads / kFeat;    // row groups per block
 
-template <typename T>
+template <typename T, int RUNS>
 __global__ void __launch_bounds__(kThreads)
 group_standardize_kernel(const int64_t* __restrict__ group_off, int max_runs, int64_t n_runs,
                          const int64_t* __restrict__ row_off,
@@ -158,12 +254,11 @@ group_standardize_kernel(const int64_t* __restrict__ group_off, int max_runs, in
                          const T* __restrict__ X, const double* __restrict__ cycles,
                          const int32_t* __restrict__ fw_test, int stat_stride, double* __restrict__ Z,
                          double* __restrict__ mu, double* __restrict__ sigma, int* dstatus) {
-    __shared__ double lv[kGroupRows][kFeat];
-    __shared__ double part[kGroups][kFeat];
-    __shared__ double stat[2][kFeat];
-    __shared__ double inv_c[kGroupRows];
-    __shared__ int64_t rowx[kGroupRows];
-    __shared__ double tlog[256], tinv[256];
+    constexpr int ROWS = RS_MAXV * RUNS / kGroups;           // RUNS >= max_runs
+    __shared__ StdSmem<kFeat, ROWS> S;
+    __shared__ double cyc_s[RS_MAXV * RUNS];
+    __shared__ long long lc_s[RS_MAXV * RUNS];
+    __shared__ int64_t rowx[RS_MAXV * RUNS];
     const int q = blockIdx.x;
     int start[RS_MAXRUNS + 1], F = 0;
     const int N = rs_group_layout(q, group_off, max_runs, n_runs, row_off, fw, fw_test, stat_stride, start, F);
@@ -176,59 +271,36 @@ group_standardize_kernel(const int64_t* __restrict__ group_off, int max_runs, in
     const int f = blockIdx.y * kFeat + fl;
     const bool active = f < F;
     const int64_t g0 = group_off[q];
+    load_log_tables(S.tl, S.tc, kThreads);
+    if (threadIdx.x < kFeat) S.inf[threadIdx.x] = 0;
+    __syncthreads();
     for (int u = threadIdx.x; u < N; u += kThreads) {
         int r = 0;
         while (u >= start[r + 1]) ++r;
         const int v = u - start[r];
         rowx[u] = xo[g0 + r] + (int64_t)v * F;
-        if (cycles) inv_c[u] = 1.0 / cycles[row_off[g0 + r] + v];
-    }
-    for (int t = threadIdx.x; t < 256; t += kThreads) {
-        tlog[t] = kLogTabF[t];
-        tinv[t] = kLogTabInv[t];
-    }
-    __syncthreads();
-    double s = 0.0;
-    if (active)
-        for (int u = g; u < N; u += kGroups) {
-            double x = as_double(X[rowx[u] + f]);
-            if (cycles) x = x * inv_c[u];
-            const double l = log_clamped(x, tlog, tinv);
-            lv[u][fl] = l;
-            s += l;
+        if (cycles) {
+            cyc_s[u] = cycles[row_off[g0 + r] + v];
+            lc_s[u] = cycle_log(cyc_s[u], S.tl, S.tc);
         }
-    part[g][fl] = s;
-    __syncthreads();
-    if (g == 0) {
-        double t = 0.0;
-        for (int i = 0; i < kGroups; ++i) t += part[i][fl];
-        stat[0][fl] = t / N;
     }
     __syncthreads();
-    const double m = stat[0][fl];
-    double q2 = 0.0;
-    if (active)
-        for (int u = g; u < N; u += kGroups) {
-            const double d = lv[u][fl] - m;
-            lv[u][fl] = d;                     // kept for the output
-            q2 += d * d;
-        }
-    part[g][fl] = q2;
-    __syncthreads();
-    if (g == 0) {
-        double t = 0.0;
-        for (int i = 0; i < kGroups; ++i) t += part[i][fl];
-        stat[1][fl] = sqrt(t / N);
+    T x[ROWS];
+#pragma unroll
+    for (int e = 0; e < ROWS; ++e) x[e] = active && g + kGroups * e < N ? X[rowx[g + kGroups * e] + f] : (T)1;
+    long long l[ROWS];
+#pragma unroll
+    for (int e = 0; e < ROWS; ++e) {
+        const int u = g + kGroups * e;
+        l[e] = u < N ? elem_log(x[e], cycles != nullptr, cyc_s[u], lc_s[u], S.tl, S.tc) : 0;
     }
-    __syncthreads();
+    double d[ROWS];
+    const double rs = centre(S, l, d, N, active, mu + (int64_t)q * stat_stride + f, sigma + (int64_t)q * stat_stride + f);
     if (!active) return;
-    const double sd = stat[1][fl];
-    const bool ok = sd > 1e-12;
-    const double rs = ok ? 1.0 / sd : 0.0;
-    for (int u = g; u < N; u += kGroups) Z[rowx[u] + f] = ok ? lv[u][fl] * rs : 0.0;
-    if (g == 0) {
-        mu[(int64_t)q * stat_stride + f] = m;
-        sigma[(int64_t)q * stat_stride + f] = sd;
+#pragma unroll
+    for (int e = 0; e < ROWS; ++e) {
+        const int u = g + kGroups * e;
+        if (u < N) Z[rowx[u] + f] = rs > 0.0 ? d[e] * rs : 0.0;
     }
 }
 
@@ -240,8 +312,11 @@ standardize_apply_kernel(const int64_t* __restrict__ row_off, const int32_t* __r
                          const int64_t* __restrict__ xo, const T* __restrict__ X,
                          const double* __restrict__ cycles, const double* __restrict__ mu,
                          const double* __restrict__ sigma, int stat_stride, double* __restrict__ Z) {
-    __shared__ double inv_c[RS_MAXV];
-    __shared__ double tlog[256], tinv[256];
+    __shared__ double cyc_s[RS_MAXV];
+    __shared__ long long lc_s[RS_MAXV], tl[256];
+    __shared__ uint16_t tc[256];
+    __shared__ double rs_s[kFeat];
+    __shared__ long long mf_s[kFeat];
     const int p = blockIdx.x;
     const int64_t r0 = row_off[p];
     const int V = (int)(row_off[p + 1] - r0);
@@ -250,23 +325,53 @@ standardize_apply_kernel(const int64_t* __restrict__ row_off, const int32_t* __r
     const int f = blockIdx.y * kFeat + fl;
     // a bad program was reported by group_standardize_kernel
     if (blockIdx.y * kFeat >= F || V < 1 || V > RS_MAXV || F > stat_stride) return;
-    if (cycles && threadIdx.x < V) inv_c[threadIdx.x] = 1.0 / cycles[r0 + threadIdx.x];
-    for (int t = threadIdx.x; t < 256; t += kThreads) {
-        tlog[t] = kLogTabF[t];
-        tinv[t] = kLogTabInv[t];
+    load_log_tables(tl, tc, kThreads);
+    if (threadIdx.x < kFeat && f < F) {      // the feature's statistics: 1 / sigma, mu in fixed point
+        const double sd = sigma[(int64_t)p * stat_stride + f];
+        const bool ok = sd > 1e-12;          // (not for the NaN of a feature with an infinite value)
+        rs_s[threadIdx.x] = ok ? 1.0 / sd : 0.0;
+        mf_s[threadIdx.x] = ok ? __double2ll_rn(mu[(int64_t)p * stat_stride + f] * 9007199254740992.0) : 0;
+    }
+    __syncthreads();
+    if (cycles && threadIdx.x < V) {
+        cyc_s[threadIdx.x] = cycles[r0 + threadIdx.x];
+        lc_s[threadIdx.x] = cycle_log(cyc_s[threadIdx.x], tl, tc);
     }
     __syncthreads();
     if (f >= F) return;
-    const double m = mu[(int64_t)p * stat_stride + f], sd = sigma[(int64_t)p * stat_stride + f];
-    const bool ok = sd > 1e-12;
-    const double rs = ok ? 1.0 / sd : 0.0;
+    const double rs = rs_s[fl];
+    const long long m = mf_s[fl];
     const int64_t base = xo[p];
-    for (int r = g; r < V; r += kGroups) {
-        double x = as_double(X[base + (int64_t)r * F + f]);
-        if (cycles) x = x * inv_c[r];
-        const double l = log_clamped(x, tlog, tinv);
-        Z[base + (int64_t)r * F + f] = ok ? (l - m) * rs : 0.0;
+#pragma unroll
+    for (int q = 0; q < RS_MAXV / kGroups; ++q) {
+        const int r = g + kGroups * q;
+        if (r >= V) break;
+        const long long l = elem_log(X[base + (int64_t)r * F + f], cycles != nullptr, cyc_s[r], lc_s[r], tl, tc);
+        const double d = l == kFixInf ? __longlong_as_double(kInfBits) : fix_double(l - m);
+        Z[base + (int64_t)r * F + f] = rs > 0.0 ? d * rs : 0.0;
     }
+}
+
+template <typename T>
+void launch_group(int runs, dim3 grid, cudaStream_t st, const int64_t* group_off, const rs_batch* train,
+                  const rs_batch* test, int max_runs, int stat_stride, double* ZA, double* mu, double* sigma,
+                  int* dstatus) {
+    auto go = [&](auto kern) {
+        kern<<<grid, kThreads, 0, st>>>(group_off, max_runs, train->n_programs, train->row_offsets, train->feat_width,
+                                        train->x_offsets, (const T*)train->X, train->cycles, test->feat_width,
+                                        stat_stride, ZA, mu, sigma, dstatus);
+    };
+    if (runs <= 1) go(group_standardize_kernel<T, 1>);
+    else if (runs <= 2) go(group_standardize_kernel<T, 2>);
+    else go(group_standardize_kernel<T, RS_MAXRUNS>);
+}
+
+template <typename T, int FEAT>
+void launch_standardize(const rs_batch* b, double* Z, double* mu, double* sigma, int* dstatus, cudaStream_t st) {
+    dim3 grid((unsigned)b->n_programs, (unsigned)((b->max_feat + FEAT - 1) / FEAT));
+    standardize_kernel<T, FEAT><<<grid, kThreads, 0, st>>>(b->n_programs, b->row_offsets, b->feat_width, b->x_offsets,
+                                                           b->feat_offsets, (const T*)b->X, b->cycles, Z, mu, sigma,
+                                                           dstatus);
 }
 
 }  // namespace
@@ -277,15 +382,9 @@ cudaError_t rs_launch_transfer_standardize(const rs_batch* train, const rs_batch
     const int Q = test->n_programs;
     dim3 ga((unsigned)Q, (unsigned)((stat_stride + kFeat - 1) / kFeat));
     if (train->dtype == RS_F32)
-        group_standardize_kernel<float><<<ga, kThreads, 0, st>>>(
-            group_off, max_runs, train->n_programs, train->row_offsets, train->feat_width, train->x_offsets,
-            (const float*)train->X,
-            train->cycles, test->feat_width, stat_stride, ZA, mu, sigma, dstatus);
+        launch_group<float>(max_runs, ga, st, group_off, train, test, max_runs, stat_stride, ZA, mu, sigma, dstatus);
     else
-        group_standardize_kernel<double><<<ga, kThreads, 0, st>>>(
-            group_off, max_runs, train->n_programs, train->row_offsets, train->feat_width, train->x_offsets,
-            (const double*)train->X,
-            train->cycles, test->feat_width, stat_stride, ZA, mu, sigma, dstatus);
+        launch_group<double>(max_runs, ga, st, group_off, train, test, max_runs, stat_stride, ZA, mu, sigma, dstatus);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     dim3 gb((unsigned)Q, (unsigned)((test->max_feat + kFeat - 1) / kFeat));
@@ -302,14 +401,14 @@ cudaError_t rs_launch_transfer_standardize(const rs_batch* train, const rs_batch
 
 cudaError_t rs_launch_standardize(const rs_batch* b, double* Z, double* mu, double* sigma,
                                   int* dstatus, cudaStream_t st) {
-    dim3 grid((unsigned)b->n_programs, (unsigned)((b->max_feat + kFeat - 1) / kFeat));
-    if (b->dtype == RS_F32)
-        standardize_kernel<float><<<grid, kThreads, 0, st>>>(
-            b->n_programs, b->row_offsets, b->feat_width, b->x_offsets, b->feat_offsets,
-            (const float*)b->X, b->cycles, Z, mu, sigma, dstatus);
-    else
-        standardize_kernel<double><<<grid, kThreads, 0, st>>>(
-            b->n_programs, b->row_offsets, b->feat_width, b->x_offsets, b->feat_offsets,
-            (const double*)b->X, b->cycles, Z, mu, sigma, dstatus);
+    // 32-feature blocks once they give every SM two blocks
+    const bool wide = (int64_t)b->n_programs * ((b->max_feat + 31) / 32) >= 304;
+    if (b->dtype == RS_F32) {
+        if (wide) launch_standardize<float, 32>(b, Z, mu, sigma, dstatus, st);
+        else launch_standardize<float, 16>(b, Z, mu, sigma, dstatus, st);
+    } else {
+        if (wide) launch_standardize<double, 32>(b, Z, mu, sigma, dstatus, st);
+        else launch_standardize<double, 16>(b, Z, mu, sigma, dstatus, st);
+    }
     return cudaGetLastError();
 }
