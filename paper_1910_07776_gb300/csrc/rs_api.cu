@@ -897,6 +897,22 @@ rs_status rs_cv_graph_create(rs_ctx* c, const rs_batch* b, const rs_splits* sp, 
     cudaStream_t orig = c->stream, cap = nullptr;
     cudaError_t e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
     if (e != cudaSuccess) return cuda_fail(c, e, "rs_cv_graph_create");
+    // the eager pass below uses the caller's workspace and outputs on a stream of its own: behind
+    // whatever the caller has enqueued on the context's stream (which may be using them)
+    cudaStreamCaptureStatus busy = cudaStreamCaptureStatusNone;
+    e = cudaStreamIsCapturing(orig, &busy);
+    if (e == cudaSuccess && busy == cudaStreamCaptureStatusNone) {
+        if (c->fork) {
+            e = cudaEventRecord(c->fork, orig);
+            if (e == cudaSuccess) e = cudaStreamWaitEvent(cap, c->fork, 0);
+        } else {
+            e = cudaStreamSynchronize(orig);
+        }
+    }
+    if (e != cudaSuccess) {
+        cudaStreamDestroy(cap);
+        return cuda_fail(c, e, "rs_cv_graph_create (ordering)");
+    }
     c->stream = cap;
     // one eager pass first: function attributes and driver entry points are set up outside
     // the capture, and argument errors are reported before anything is recorded
