@@ -1,5 +1,5 @@
-// K2 (FP64 form): per-program Gram block K_p = Z_p Z_p^T of the standardized feature
-// vectors.  It is the only contraction of the method: every ridge fit of every split of
+// K2 (FP64 form, few programs): per-program Gram block K_p = Z_p Z_p^T of the standardized feature
+// vectors, and the blocks of squared distances and of transfer problems.  It is the only contraction of the method: every ridge fit of every split of
 // program p reads its kernel entries K_p[v_a][v_b] from this block (dual form of the
 // regression family of Sec. 3.4), so it is formed once per program, not once per fit.
 //
@@ -293,6 +293,15 @@ cudaError_t rs_launch_transfer_blocks(const rs_batch* train_std, const rs_batch*
 #define RS_GRAM_MAXB 4
 #endif
 cudaError_t rs_launch_gram_f64(const rs_batch* b, double* K, int* dstatus, cudaStream_t st) {
+    // The tensor-core form (k_gram_split.cu) takes about 10 + 0.05 F us per program and SM whatever
+    // its versions; this one 32 F ns per block of 128 entries and SM, plus 6 us.  So the latter keeps
+    // the grids that fit the SMs once, and small products (64 versions x 96 features: 26 programs
+    // 14.7 against 16.4 us, 40 programs 22.6 against 16.4; 256 features: 8 programs 18.6 against
+    // 20.0, 12 programs 22.6 against 20.5; 30 versions x 96: 76 programs 12.9 against 14.5, 300
+    // programs 30.9 against 24.7).
+    const int64_t v = b->n_rows / b->n_programs < RS_MAXV ? b->n_rows / b->n_programs : RS_MAXV;
+    const int64_t blocks = b->n_programs * ((v * (v + 1) / 2 + kGramThreads - 1) / kGramThreads);
+    if (blocks > 152 && blocks * b->max_feat >= 44000) return rs_launch_gram_split(b, K, dstatus, st);
     dim3 grid((unsigned)b->n_programs, kGramChunks);
     const size_t pad = rs_residency_pad(RS_GRAM_MAXB, sizeof(double) * 2 * RS_MAXV * kGramLd);
     if (pad) cudaFuncSetAttribute(gram_f64_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pad);

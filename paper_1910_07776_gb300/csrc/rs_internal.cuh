@@ -98,6 +98,7 @@ __device__ __forceinline__ int rs_group_layout(int q, const int64_t* group_off, 
 cudaError_t rs_launch_standardize(const rs_batch* b, double* Z, double* mu, double* sigma,
                                   int* dstatus, cudaStream_t st);
 cudaError_t rs_launch_gram_f64(const rs_batch* b, double* K, int* dstatus, cudaStream_t st);
+cudaError_t rs_launch_gram_split(const rs_batch* b, double* K, int* dstatus, cudaStream_t st);
 cudaError_t rs_launch_dist2_f64(const rs_batch* b, double* K, int* dstatus, cudaStream_t st);
 cudaError_t rs_launch_transfer_standardize(const rs_batch* train, const rs_batch* test, const int64_t* group_off,
                                            int max_runs, int stat_stride, double* ZA, double* ZB, double* mu,
