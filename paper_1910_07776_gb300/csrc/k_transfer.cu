@@ -49,26 +49,34 @@ __device__ void load_group(GroupSmem& G, const int64_t* __restrict__ a_row, cons
     __syncthreads();
 }
 
-// The pairs of optimization j (one thread): group version of each before side, and labels.
-// Returns their number; more than kTrPairs (only possible with repeated masks) is reported.
-__device__ int build_pairs(const GroupSmem& G, int j, int R, const int (&start)[RS_MAXRUNS + 1], uint16_t* pu,
+// The pairs of optimization j (one warp, 32 of the group's versions at a time): group version of
+// each before side, and labels, run by run in ascending slot order.  Returns their number; more than
+// kTrPairs (only possible with repeated masks) is reported.
+__device__ int build_pairs(const GroupSmem& G, int j, int R, int N, const int (&start)[RS_MAXRUNS + 1], uint16_t* pu,
                            double* yl, int* dstatus, int q) {
+    const int lane = threadIdx.x & 31;
     int np = 0;
-    for (int r = 0; r < R; ++r)
-        for (int u = start[r]; u < start[r + 1]; ++u) {
+    for (int u0 = 0; u0 < N; u0 += 32) {
+        const int u = u0 + lane;
+        int r = 0, w = -1;
+        if (u < N) {
+            while (u >= start[r + 1]) ++r;
             const int m = G.msk[u];
-            if ((m >> j) & 1) continue;
-            const int w = G.slot[r][m | (1 << j)];
-            if (w < 0) continue;
-            if (np == kTrPairs) {
-                rs_dev_flag(dstatus, RS_EDATA, q);
-                continue;
-            }
-            pu[np] = (uint16_t)u;
-            yl[np] = G.lt[u] - G.lt[start[r] + w];
-            ++np;
+            w = (m >> j) & 1 ? -1 : G.slot[r][m | (1 << j)];
         }
-    return np;
+        const unsigned b = __ballot_sync(0xffffffffu, w >= 0);
+        const int at = np + __popc(b & ((1u << lane) - 1u));
+        if (w >= 0) {
+            if (at < kTrPairs) {
+                pu[at] = (uint16_t)u;
+                yl[at] = G.lt[u] - G.lt[start[r] + w];
+            } else {
+                rs_dev_flag(dstatus, RS_EDATA, q);
+            }
+        }
+        np += __popc(b);
+    }
+    return np < kTrPairs ? np : kTrPairs;
 }
 
 struct M5Tree;
@@ -91,6 +99,7 @@ struct TransferArgs {
     double lambda;
     double* coef;                        // [Q][6][kTrCoef] ridge fits (written by the fit kernel)
     uint8_t* fst;                        // [Q][6] their status
+    double* pred;                        // [Q][64][6] predictions (transfer_predict_kernel)
     int ibk, opt_mask, rank_all;
     int m5p;                             // the M5P model tree instead of ridge
     M5Tree* trees;                       // [Q][6] M5P trees
@@ -135,7 +144,10 @@ transfer_fit_kernel(const TransferArgs a, int nmax) {
     const int64_t g0 = a.group_off[q];
     const int R = (int)(a.group_off[q + 1] - g0);
     load_group(G, a.a_row, a.a_masks, a.a_lt, g0, start, N);
-    if (tid == 0) np_s = build_pairs(G, j, R, start, pu, yl, nullptr, q);
+    if (tid < 32) {
+        const int np = build_pairs(G, j, R, N, start, pu, yl, nullptr, q);
+        if (tid == 0) np_s = np;
+    }
     __syncthreads();
     const int n = np_s;
     double* out = a.coef + ((int64_t)q * RS_NOPT + j) * kTrCoef;
@@ -239,12 +251,31 @@ transfer_fit_kernel(const TransferArgs a, int nmax) {
 // in its subtree as pruned so far (children are modelled and pruned first), simplified by
 // greedy elimination, bottom-up pruning by estimated error, and smoothing on the way up at
 // prediction time (k = 15).
+//
+// One block per fit.  What decides the tree is computed with the reference's own roundings (label
+// sums in order, SDRs by IEEE division and square root), but only where it can matter: an SDR takes
+// over a hundred FP64 instructions of 64 cycles each, and a node has up to 127 F candidate splits.  So
+// every candidate is first bounded in FP32 (prefix sums by shuffles, an explicit error bound), and
+// only those whose interval reaches the best one are evaluated exactly; a single survivor needs no
+// evaluation.  The tree grows a level at a time: the (node, attribute) scans and partitions of a
+// whole level are dealt to the eight warps, five block barriers a level instead of seven a node.
+// Greedy elimination keeps the inverse H of the normal equations, the residuals and T = C H (C the
+// centred attributes): dropping attribute d changes every residual by (w_d / H_dd) T_ad, so all the
+// drop-one errors of a round cost m ns operations, and the round's winner is taken out by rank-one
+// updates of H, w and T; the model that stays is solved again from scratch.  (Before: one thread per
+// attribute walking every candidate's SDR, an inverse per round and every drop-one model applied to
+// every instance, all serial over the nodes.)  Small nodes' models take one warp each.
+// 36 problems x 3 runs x 37 attributes (96 instances a fit): 5532 -> 1976 us.
 constexpr int kM5MaxN = kTrPairs;                 // instances of one fit
 constexpr int kM5MaxNodes = 2 * kM5MaxN - 1;
 constexpr int kM5MaxTerms = 64;
-constexpr int kM5MaxFeat = 256;                   // attributes (one thread each in the split search)
+constexpr int kM5MaxFeat = 256;
 constexpr int kM5Threads = 256;
-constexpr int kM5Ld = kM5MaxTerms + 1;
+constexpr int kM5Warps = kM5Threads / 32;
+constexpr int kM5WarpTerms = 16, kM5WarpN = 32;   // models up to this size take one warp
+constexpr int kM5WarpLd = kM5WarpTerms + 1;
+constexpr int kM5WarpBuf = 2 * kM5WarpTerms * kM5WarpLd + kM5WarpN * kM5WarpLd;   // G, H, C
+constexpr int kM5Surv = 512;                      // candidate splits kept for exact evaluation, per level
 constexpr double kM5SdFrac = 0.05, kM5Smooth = 15.0, kM5Ridge = 1e-8;
 
 struct M5Tree {
@@ -257,107 +288,489 @@ struct M5Tree {
     double term_w[kM5MaxNodes][kM5MaxTerms];
 };
 
+// Per group of threads (a warp, or the block): the vectors of one node's model.
+template <int N>
+struct M5Vec {
+    double colk[N], rowk[N], zbar[N], r[N], w[N], fac[N];
+    int16_t cand[N];
+    uint8_t sel[N];
+    double e_cur, b;
+    int drop;
+};
+
 struct M5Smem {
-    union {                                       // the growing pass, then the models' pass
-        struct {
-            uint8_t sorted[kM5MaxFeat][kM5MaxN];  // per attribute: instances in (value, index) order
-            uint8_t scratch[kM5Threads][kM5MaxN];
-        } gr;
-        struct {
-            double G[kM5MaxTerms * kM5Ld];        // centred normal equations of the node's candidates
-            double H[kM5MaxTerms * kM5Ld];        // inverse of the current subset's system
-        } mo;
-    };
-    double colk[kM5MaxTerms], rowk[kM5MaxTerms];
-    double zbar[kM5MaxTerms], r[kM5MaxTerms], w[kM5MaxTerms], cand_err[kM5MaxTerms];
-    double res[kM5MaxN];
-    double y[kM5MaxN];
+    double y[kM5MaxN], y2[kM5MaxN];               // labels and their rounded squares
     const double* zp[kM5MaxN];                    // each instance's standardized row
+    float yf[kM5MaxN];                            // labels less the root's mean, in FP32
     double thr[kM5MaxNodes], est[kM5MaxNodes];
     unsigned long long tested[kM5MaxNodes][kM5MaxFeat / 64];
-    int16_t attr[kM5MaxNodes], left[kM5MaxNodes], right[kM5MaxNodes];
+    int16_t attr[kM5MaxNodes], left[kM5MaxNodes], right[kM5MaxNodes], parent[kM5MaxNodes];
     uint8_t lo[kM5MaxNodes], hi[kM5MaxNodes];
-    uint8_t ids[kM5MaxN];
-    uint8_t side[kM5MaxN];
-    uint8_t sel[kM5MaxTerms];                     // current subset: positions in the candidate list
-    int16_t cand[kM5MaxTerms];
-    double red_v[kM5Threads / 32];
-    int red_i[kM5Threads / 32];
-    int stack_node[kM5MaxNodes], stack_lo[kM5MaxNodes], stack_hi[kM5MaxNodes];
-    int sp, nn, cur, cur_lo, cur_hi, ncand, nsel, split_attr, drop;
-    double split_thr, sd_root, e_cur, bval;
+    uint8_t ids[kM5MaxN], side[kM5MaxN];
+    int level[kM5MaxN + 2];                       // first node of each level
+    int nn, task, nsurv;
+    double sd_root;
+    // the level's nodes (at most kM5MaxN / 2 that split), by node - first of the level
+    float mean[kM5MaxN], tot[kM5MaxN], tot2[kM5MaxN], amax2[kM5MaxN], sda[kM5MaxN];
+    unsigned best_hi[kM5MaxN];                    // smallest upper bound of Q, as FP32 bits
+    unsigned long long best_red[kM5MaxN];         // largest exact SDR, as FP64 bits
+    unsigned best_key[kM5MaxN];                   // attribute << 8 | count of the chosen split
+    int cnt[kM5MaxN];                             // survivors; -1: a leaf, -2: by the exact scan
+    double s1[kM5MaxN], s2[kM5MaxN];              // exact label sums, in instance order
+    unsigned surv[kM5Surv];                       // node << 16 | attribute << 8 | count
+    double red[kM5Surv];                          // their SDRs
+    double errp[kM5Warps][kM5MaxTerms];
+    union {
+        M5Vec<kM5MaxTerms> blk;
+        M5Vec<kM5WarpTerms> wv[kM5Warps];
+    } v;
 };
 
 // The standard deviation from a count, sum and sum of squares: sqrt(max(0, (s2 - s1 s1 / c) / c)),
 // with one rounding per operation (the reference's arithmetic).
-__device__ __forceinline__ double m5_sd(int c, double s1, double s2) {
+__device__ __noinline__ double m5_sd(int c, double s1, double s2) {
     const double cd = (double)c;
     const double v = __ddiv_rn(__dsub_rn(s2, __ddiv_rn(__dmul_rn(s1, s1), cd)), cd);
     return __dsqrt_rn(v > 0.0 ? v : 0.0);
 }
 
-// In-place inverse of the nb x nb leading block of M (row stride kM5Ld) by Gauss-Jordan
-// elimination without pivoting (the systems are symmetric positive definite).  Block-wide.
-__device__ void m5_invert(M5Smem& S, double* M, int nb) {
-    const int tid = threadIdx.x;
-    for (int k = 0; k < nb; ++k) {
-        const double piv = 1.0 / M[k * kM5Ld + k];
-        for (int i = tid; i < nb; i += kM5Threads) {
-            S.colk[i] = M[i * kM5Ld + k];
-            S.rowk[i] = M[k * kM5Ld + i] * piv;
+__device__ __forceinline__ double m5_warp_sum(double x) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+}
+
+// Bounds of Q = sqrt(c l2 - l1^2) + sqrt((m - c) r2 - r1^2) (SDR = sd - Q / m) from FP32 prefix
+// sums.  Each radicand's error is below 1e-5 n^2 A^2 for n labels of magnitude at most A: labels
+// rounded to FP32 and shifted (1.8e-7 A each), sums by at most 12 additions (7e-7 each way), products.
+__device__ __forceinline__ void m5_bounds(int c, int m, float l1, float l2, float t1, float t2, float a2, float& lo,
+                                          float& hi) {
+    const float cl = (float)c, cr = (float)(m - c);
+    const float r1 = t1 - l1, r2 = t2 - l2;
+    const float L = cl * l2 - l1 * l1, R = cr * r2 - r1 * r1;
+    const float dl = 1e-5f * a2 * cl * cl, dr = 1e-5f * a2 * cr * cr;
+    hi = (sqrtf(fmaxf(L, 0.f) + dl) + sqrtf(fmaxf(R, 0.f) + dr)) * 1.00001f;
+    lo = (sqrtf(fmaxf(L - dl, 0.f)) + sqrtf(fmaxf(R - dr, 0.f))) * 0.99999f;
+}
+
+// One warp scans attribute f of a node (rank lo.., m instances, level slot q): SURVIVORS false
+// lowers the node's best upper bound, true lists the candidates whose lower bound reaches it.
+template <bool SURVIVORS>
+__device__ __forceinline__ void m5_scan(M5Smem& S, const uint8_t* srt, const uint8_t* rk, int f, int lo, int m, int q) {
+    const int lane = threadIdx.x & 31;
+    const float mean = S.mean[q], t1 = S.tot[q], t2 = S.tot2[q], a2 = S.amax2[q];
+    float c1 = 0.f, c2 = 0.f, best = __int_as_float(0x7f800000);
+    const float lim = SURVIVORS ? __uint_as_float(S.best_hi[q]) : 0.f;
+    for (int base = 0; base < m; base += 32) {
+        const int e = base + lane;
+        const bool in = e < m;
+        const int id = in ? srt[lo + e] : 0;
+        const int nx = e + 1 < m ? srt[lo + e + 1] : id;
+        const float v = in ? S.yf[id] - mean : 0.f;
+        float s = v, w = v * v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const float a = __shfl_up_sync(0xffffffffu, s, o), b = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) {
+                s += a;
+                w += b;
+            }
         }
-        __syncthreads();
-        for (int e = tid; e < nb * nb; e += kM5Threads) {
-            const int i = e / nb, j = e - i * nb;
-            if (i == k && j == k) M[k * kM5Ld + k] = piv;
-            else if (i == k) M[k * kM5Ld + j] = S.rowk[j];
-            else if (j == k) M[i * kM5Ld + k] = -S.colk[i] * piv;
-            else M[i * kM5Ld + j] = fma(-S.colk[i], S.rowk[j], M[i * kM5Ld + j]);
+        s += c1;
+        w += c2;
+        c1 = __shfl_sync(0xffffffffu, s, 31);
+        c2 = __shfl_sync(0xffffffffu, w, 31);
+        const int c = e + 1;
+        if (in && c >= 2 && m - c >= 2 && rk[nx] != rk[id]) {
+            float ql, qh;
+            m5_bounds(c, m, s, w, t1, t2, a2, ql, qh);
+            if (!SURVIVORS) {
+                best = fminf(best, qh);
+            } else if (ql <= lim) {
+                const int k = atomicAdd(&S.nsurv, 1);
+                atomicAdd(&S.cnt[q], 1);
+                if (k < kM5Surv) S.surv[k] = (unsigned)q << 16 | (unsigned)f << 8 | (unsigned)c;
+            }
         }
-        __syncthreads();
+    }
+    if (!SURVIVORS) {
+        const unsigned b = __reduce_min_sync(0xffffffffu, __float_as_uint(best));
+        if (lane == 0) atomicMin(&S.best_hi[q], b);
     }
 }
 
-// Estimated error of a model (b, w on the selected candidates) over the node's instances:
-// mean |y - prediction| * (m + v) / (m - v), v = terms + 1; DBL_MAX when m <= v.  One warp.
-__device__ double m5_warp_err(const M5Smem& S, int lo, int m, const double* w, double b, int nsel,
-                              const uint8_t* selpos, int skip) {
+// Every candidate of attribute f by the reference's arithmetic, one thread (labels that are not
+// finite, or more survivors than fit): the best SDR > 0 of the attribute goes to best / key.
+__device__ __noinline__ void m5_exact_scan(const M5Smem& S, const uint8_t* o, const uint8_t* rk, int f, int lo, int m,
+                                           int q, double sd, double& best, unsigned& key) {
+    double l1 = 0.0, l2 = 0.0;
+    for (int c = 1; c < m; ++c) {
+        const int ia = o[lo + c - 1], ib = o[lo + c];
+        l1 = __dadd_rn(l1, S.y[ia]);
+        l2 = __dadd_rn(l2, S.y2[ia]);
+        if (rk[ia] == rk[ib] || c < 2 || m - c < 2) continue;
+        const double sdl = m5_sd(c, l1, l2), sdr = m5_sd(m - c, __dsub_rn(S.s1[q], l1), __dsub_rn(S.s2[q], l2));
+        const double red = __dsub_rn(sd, __ddiv_rn(__dadd_rn(__dmul_rn((double)c, sdl), __dmul_rn((double)(m - c), sdr)),
+                                                   (double)m));
+        if (red > best) {
+            best = red;
+            key = (unsigned)f << 8 | (unsigned)c;
+        }
+    }
+}
+
+// A group of threads working on one node's model: a warp, or the whole block.
+template <bool WARP>
+struct M5Group {
+    static constexpr int kNT = WARP ? 32 : kM5Threads;
+    static __device__ __forceinline__ int tid() { return WARP ? (int)(threadIdx.x & 31) : (int)threadIdx.x; }
+    static __device__ __forceinline__ void sync() {
+        if (WARP) __syncwarp();
+        else __syncthreads();
+    }
+};
+
+// In-place inverse of the nb x nb leading block of M (row stride ld) by Gauss-Jordan elimination
+// without pivoting (the systems are symmetric positive definite).
+template <bool WARP, class Vec>
+__device__ void m5_invert(Vec& V, double* M, int ld, int nb) {
+    using Gp = M5Group<WARP>;
+    const int tid = Gp::tid();
+    for (int k = 0; k < nb; ++k) {
+        const double piv = rcp_newton_any(M[k * ld + k]);
+        for (int i = tid; i < nb; i += Gp::kNT) {
+            V.colk[i] = M[i * ld + k];
+            V.rowk[i] = M[k * ld + i] * piv;
+        }
+        Gp::sync();
+        for (int e = tid; e < nb * nb; e += Gp::kNT) {
+            const int i = e / nb, j = e - i * nb;
+            if (i == k && j == k) M[k * ld + k] = piv;
+            else if (i == k) M[k * ld + j] = V.rowk[j];
+            else if (j == k) M[i * ld + k] = -V.colk[i] * piv;
+            else M[i * ld + j] = fma(-V.colk[i], V.rowk[j], M[i * ld + j]);
+        }
+        Gp::sync();
+    }
+}
+
+// Estimated error of the node's model (V.b, V.w on V.sel) over its instances: mean |y - prediction|
+// (m + v) / (m - v), v = terms + 1; DBL_MAX when m <= v.  One warp.
+template <class Vec>
+__device__ double m5_warp_err(const M5Smem& S, const Vec& V, int lo, int m, int nsel) {
     const int lane = threadIdx.x & 31;
     double acc = 0.0;
     for (int a = lane; a < m; a += 32) {
         const int i = S.ids[lo + a];
         const double* z = S.zp[i];
-        double p = b;
-        for (int q = 0; q < nsel; ++q) {
-            if (q == skip) continue;
-            p = fma(w[q], __ldg(z + S.cand[selpos[q]]), p);
-        }
+        double p = V.b;
+        for (int q = 0; q < nsel; ++q) p = fma(V.w[q], __ldg(z + V.cand[V.sel[q]]), p);
         acc += fabs(S.y[i] - p);
     }
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    const int v = nsel - (skip >= 0 ? 1 : 0) + 1;
+    acc = m5_warp_sum(acc);
+    const int v = nsel + 1;
     if (m <= v) return DBL_MAX;
     return acc / m * ((double)(m + v) / (double)(m - v));
 }
 
-__global__ void __launch_bounds__(kM5Threads, 1)
-m5p_fit_kernel(const TransferArgs a) {
+// w = H r, the intercept and e_cur of the model on V.sel[0 .. ns), H = inverse of its system.
+template <bool WARP, class Vec>
+__device__ void m5_solve(M5Smem& S, Vec& V, const double* G, double* H, int ld, int ns, int lo, int m, double ybar) {
+    using Gp = M5Group<WARP>;
+    const int tid = Gp::tid();
+    for (int e = tid; e < ns * ns; e += Gp::kNT) {
+        const int i = e / ns, k = e - i * ns;
+        H[i * ld + k] = G[V.sel[i] * ld + V.sel[k]];
+    }
+    Gp::sync();
+    m5_invert<WARP>(V, H, ld, ns);
+    for (int i = tid; i < ns; i += Gp::kNT) {
+        double s = 0.0;
+        for (int k = 0; k < ns; ++k) s = fma(H[i * ld + k], V.r[V.sel[k]], s);
+        V.w[i] = s;
+    }
+    Gp::sync();
+    if (tid == 0) {
+        double b = ybar;
+        for (int i = 0; i < ns; ++i) b -= V.w[i] * V.zbar[V.sel[i]];
+        V.b = b;
+    }
+    Gp::sync();
+    if (WARP || threadIdx.x < 32) {
+        const double e = m5_warp_err(S, V, lo, m, ns);
+        if (tid == 0) V.e_cur = e;
+    }
+    Gp::sync();
+}
+
+// The model of internal node t on the attributes tested below it (the lowest kM5MaxTerms of them),
+// greedily simplified, and the pruning decision.  G, H: tmax x ld; C: m x ld.
+template <bool WARP, class Vec>
+__device__ __noinline__ void m5_model(M5Smem& S, Vec& V, M5Tree* T, int t, int F, double* G, double* H, double* C, int ld) {
+    using Gp = M5Group<WARP>;
+    const int tid = Gp::tid(), lane = threadIdx.x & 31;
+    const int wp = WARP ? 0 : (int)(threadIdx.x >> 5), nw = WARP ? 1 : kM5Warps;
+    const int lo = S.lo[t], m = S.hi[t] - S.lo[t];
+    // candidates: the attributes tested in the subtree, ascending
+    int nc = 0;
+    for (int w = 0; w < kM5MaxFeat / 64; ++w) {
+        const unsigned long long bits = S.tested[t][w];
+        for (int f = tid; f < 64; f += Gp::kNT)
+            if ((bits >> f) & 1ull) {
+                const int pos = nc + __popcll(bits & ((1ull << f) - 1ull));
+                if (pos < kM5MaxTerms) V.cand[pos] = (int16_t)(64 * w + f);
+            }
+        nc += __popcll(bits);
+    }
+    nc = nc < kM5MaxTerms ? nc : kM5MaxTerms;
+    double ybar = 0.0;
+    for (int a = lane; a < m; a += 32) ybar += S.y[S.ids[lo + a]];
+    ybar = m5_warp_sum(ybar) / m;
+    Gp::sync();
+    for (int e = tid; e < m * nc; e += Gp::kNT) {
+        const int a = e / nc, k = e - a * nc;
+        C[a * ld + k] = __ldg(S.zp[S.ids[lo + a]] + V.cand[k]);
+    }
+    Gp::sync();
+    for (int k = wp; k < nc; k += nw) {            // a warp centres a column
+        double s = 0.0, d = 0.0;
+        for (int a = lane; a < m; a += 32) s += C[a * ld + k];
+        s = m5_warp_sum(s) / m;
+        for (int a = lane; a < m; a += 32) {
+            const double c = C[a * ld + k] - s;
+            C[a * ld + k] = c;
+            d = fma(c, S.y[S.ids[lo + a]] - ybar, d);
+        }
+        d = m5_warp_sum(d);
+        if (lane == 0) {
+            V.zbar[k] = s;
+            V.r[k] = d;
+            V.sel[k] = (uint8_t)k;
+        }
+    }
+    Gp::sync();
+    for (int e = tid; e < nc * (nc + 1) / 2; e += Gp::kNT) {
+        int f = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
+        while (f * (f + 1) / 2 > e) --f;
+        while ((f + 1) * (f + 2) / 2 <= e) ++f;
+        const int g = e - f * (f + 1) / 2;
+        double s = 0.0;
+        for (int a = 0; a < m; ++a) s = fma(C[a * ld + f], C[a * ld + g], s);
+        if (f == g) s += kM5Ridge;
+        G[f * ld + g] = s;
+        G[g * ld + f] = s;
+    }
+    Gp::sync();
+    m5_solve<WARP>(S, V, G, H, ld, nc, lo, m, ybar);
+    // residuals (kept by row owners) and T = C H in C's place
+    double res[WARP ? 1 : kM5MaxN / kM5Warps];
+    unsigned long long alive = nc >= 64 ? ~0ull : (1ull << nc) - 1ull;
+    int ns = nc;
+    bool dropped = false;
+    if (nc > 0 && m > nc) {                        // else no model with one attribute fewer has an estimate
+        if constexpr (WARP) {                      // lane = instance
+            double c[kM5WarpTerms];
+            res[0] = 0.0;
+            if (lane < m) {
+                double p = ybar;
+#pragma unroll
+                for (int i = 0; i < kM5WarpTerms; ++i) {
+                    c[i] = i < nc ? C[lane * ld + i] : 0.0;
+                    if (i < nc) p = fma(c[i], V.w[i], p);
+                }
+                res[0] = S.y[S.ids[lo + lane]] - p;
+                for (int k = 0; k < nc; ++k) {
+                    double s = 0.0;
+#pragma unroll
+                    for (int i = 0; i < kM5WarpTerms; ++i)
+                        if (i < nc) s = fma(c[i], H[i * ld + k], s);
+                    C[lane * ld + k] = s;
+                }
+            }
+        } else {                                   // a warp takes instances wp, wp + 8, ...
+#pragma unroll
+            for (int x = 0; x < kM5MaxN / kM5Warps; ++x) {
+                const int a = wp + kM5Warps * x;
+                res[x] = 0.0;
+                if (a >= m) continue;
+                double p = 0.0, s0 = 0.0, s1 = 0.0;
+                if (lane < nc) p = C[a * ld + lane] * V.w[lane];
+                if (lane + 32 < nc) p = fma(C[a * ld + lane + 32], V.w[lane + 32], p);
+                res[x] = S.y[S.ids[lo + a]] - (ybar + m5_warp_sum(p));
+                for (int i = 0; i < nc; ++i) {
+                    const double ci = C[a * ld + i];
+                    if (lane < nc) s0 = fma(ci, H[i * ld + lane], s0);
+                    if (lane + 32 < nc) s1 = fma(ci, H[i * ld + lane + 32], s1);
+                }
+                __syncwarp();
+                if (lane < nc) C[a * ld + lane] = s0;
+                if (lane + 32 < nc) C[a * ld + lane + 32] = s1;
+            }
+        }
+        Gp::sync();
+        for (;;) {
+            // w_d / H_dd, then sum_a |res_a + fac_d T_ad| of every attribute still there
+            for (int d = tid; d < nc; d += Gp::kNT)
+                V.fac[d] = (alive >> d) & 1ull ? V.w[d] * rcp_newton_any(H[d * ld + d]) : 0.0;
+            Gp::sync();
+            double bd = DBL_MAX;
+            int drop = -1;
+            if constexpr (WARP) {                  // lane d and lane d + 16 share attribute d's instances
+                const int d = lane & 15, h = lane >> 4;
+                double s = 0.0;
+                for (int a = 0; a < m; ++a) {
+                    const double ra = __shfl_sync(0xffffffffu, res[0], a);
+                    if (d < nc && (a & 1) == h) s += fabs(fma(V.fac[d], C[a * ld + d], ra));
+                }
+                s += __shfl_xor_sync(0xffffffffu, s, 16);
+                if (d < nc && ((alive >> d) & 1ull) && s < DBL_MAX) {
+                    bd = s;
+                    drop = d;
+                }
+            } else {
+                double s0 = 0.0, s1 = 0.0;
+                const double f0 = lane < nc ? V.fac[lane] : 0.0, f1 = lane + 32 < nc ? V.fac[lane + 32] : 0.0;
+#pragma unroll
+                for (int x = 0; x < kM5MaxN / kM5Warps; ++x) {
+                    const int a = wp + kM5Warps * x;
+                    if (a >= m) continue;
+                    if (lane < nc) s0 += fabs(fma(f0, C[a * ld + lane], res[x]));
+                    if (lane + 32 < nc) s1 += fabs(fma(f1, C[a * ld + lane + 32], res[x]));
+                }
+                S.errp[wp][lane] = s0;
+                S.errp[wp][lane + 32] = s1;
+                __syncthreads();
+                if (wp == 0)
+                    for (int d = lane; d < nc; d += 32) {
+                        double s = 0.0;
+#pragma unroll
+                        for (int w = 0; w < kM5Warps; ++w) s += S.errp[w][d];
+                        if (((alive >> d) & 1ull) && s < bd) {
+                            bd = s;
+                            drop = d;
+                        }
+                    }
+            }
+            if (WARP || wp == 0) {
+#pragma unroll
+                for (int o = 16; o >= 1; o >>= 1) {
+                    const double ob = __shfl_xor_sync(0xffffffffu, bd, o);
+                    const int od = __shfl_xor_sync(0xffffffffu, drop, o);
+                    if (od >= 0 && (drop < 0 || ob < bd || (ob == bd && od < drop))) {
+                        bd = ob;
+                        drop = od;
+                    }
+                }
+                if (tid == 0) {
+                    const int v = ns;              // terms + 1 of the smaller model
+                    const double e = m <= v ? DBL_MAX : bd / m * ((double)(m + v) / (double)(m - v));
+                    V.drop = drop >= 0 && e < DBL_MAX && e <= V.e_cur ? drop : -1;
+                    if (V.drop >= 0) V.e_cur = e;
+                }
+            }
+            Gp::sync();
+            const int d = V.drop;
+            if (d < 0) break;
+            dropped = true;
+            --ns;
+            alive &= ~(1ull << d);
+            if (ns == 0) break;
+            // take d out: H -= H_d H_d^T / H_dd, w -= H_d fac_d, T -= T_d H_d^T / H_dd, res += fac_d T_d
+            const double fd = V.fac[d], hi = rcp_newton_any(H[d * ld + d]);
+            for (int i = tid; i < nc; i += Gp::kNT) {
+                V.colk[i] = H[i * ld + d];
+                V.rowk[i] = H[i * ld + d] * hi;
+                if (i != d) V.w[i] = fma(-H[i * ld + d], fd, V.w[i]);
+            }
+            Gp::sync();
+            for (int e = tid; e < nc * nc; e += Gp::kNT) {
+                const int i = e / nc, j = e - i * nc;
+                if (i != d && j != d) H[i * ld + j] = fma(-V.colk[i], V.rowk[j], H[i * ld + j]);
+            }
+            if constexpr (WARP) {
+                if (lane < m) {
+                    const double td = C[lane * ld + d];
+                    res[0] = fma(fd, td, res[0]);
+                    for (int k = 0; k < nc; ++k)
+                        if (k != d) C[lane * ld + k] = fma(-td, V.rowk[k], C[lane * ld + k]);
+                }
+            } else {
+#pragma unroll
+                for (int x = 0; x < kM5MaxN / kM5Warps; ++x) {
+                    const int a = wp + kM5Warps * x;
+                    if (a >= m) continue;
+                    const double td = C[a * ld + d];
+                    res[x] = fma(fd, td, res[x]);
+                    if (lane < nc && lane != d) C[a * ld + lane] = fma(-td, V.rowk[lane], C[a * ld + lane]);
+                    if (lane + 32 < nc && lane + 32 != d)
+                        C[a * ld + lane + 32] = fma(-td, V.rowk[lane + 32], C[a * ld + lane + 32]);
+                }
+            }
+            Gp::sync();
+        }
+    }
+    if (dropped) {                                 // the model that stays, from its own normal equations
+        if (tid < nc && ((alive >> tid) & 1ull)) V.sel[__popcll(alive & ((1ull << tid) - 1ull))] = (uint8_t)tid;
+        Gp::sync();
+        m5_solve<WARP>(S, V, G, H, ld, ns, lo, m, ybar);
+    }
+    // the node's model and the pruning decision
+    for (int k = tid; k < ns; k += Gp::kNT) {
+        T->term_attr[t][k] = V.cand[V.sel[k]];
+        T->term_w[t][k] = V.w[k];
+    }
+    if (tid == 0) {
+        T->nterm[t] = ns;
+        T->b[t] = V.b;
+        T->count[t] = m;
+        const double e = V.e_cur;
+        const int l = S.left[t], r = S.right[t];
+        const int ml = S.hi[l] - S.lo[l], mr = S.hi[r] - S.lo[r];
+        const double keep = (ml * S.est[l] + mr * S.est[r]) / m;
+        if (!(e <= keep)) {
+            S.est[t] = keep;
+        } else {                                   // a leaf: its parent's candidates get no test
+            S.attr[t] = -1;                        // from here down
+            S.est[t] = e;
+            for (int k = 0; k < kM5MaxFeat / 64; ++k) S.tested[t][k] = 0;
+        }
+    }
+    Gp::sync();
+}
+
+// Dynamic shared memory behind M5Smem: while growing, per attribute the instances in (value, index)
+// order and each instance's rank among the attribute's distinct values; then the models' matrices.
+__host__ __device__ __forceinline__ size_t m5_dyn_bytes(int F) {
+    const int nmax = kM5MaxN;
+    const size_t grow = 2 * (size_t)F * nmax;
+    const int tm = F < kM5MaxTerms ? F : kM5MaxTerms, ld = tm | 1;
+    const size_t blk = ((size_t)2 * tm * ld + (size_t)nmax * ld) * sizeof(double);
+    const size_t wrp = (size_t)kM5Warps * kM5WarpBuf * sizeof(double);
+    const size_t mo = blk > wrp ? blk : wrp;
+    return grow > mo ? grow : mo;
+}
+
+__global__ void __launch_bounds__(kM5Threads)
+m5p_fit_kernel(const TransferArgs a, int fmax) {
+    constexpr int nmax = kM5MaxN;
     extern __shared__ __align__(16) unsigned char m5sm[];
     M5Smem& S = *reinterpret_cast<M5Smem*>(m5sm);
+    unsigned char* dyn = m5sm + ((sizeof(M5Smem) + 15) & ~(size_t)15);
     __shared__ GroupSmem G;
     __shared__ uint16_t pu[kTrPairs];
     __shared__ double yl[kTrPairs];
     __shared__ int np_s;
     const int q = blockIdx.x, j = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int nwarps = kM5Threads / 32;
     int start[RS_MAXRUNS + 1], F = 0;
     const int N = rs_group_layout(q, a.group_off, a.max_runs, a.n_runs, a.a_row, a.a_fw, a.b_fw, a.stat_stride, start, F);
-    if (N < 0 || N > a.ld || F > kM5MaxFeat) return;   // reported by the predict / rank kernel
+    if (N < 0 || N > a.ld || F > kM5MaxFeat || F > fmax) return;   // reported by the predict / rank kernel
     const int64_t g0 = a.group_off[q];
     const int R = (int)(a.group_off[q + 1] - g0);
     load_group(G, a.a_row, a.a_masks, a.a_lt, g0, start, N);
-    if (tid == 0) np_s = build_pairs(G, j, R, start, pu, yl, nullptr, q);
+    if (warp == 0) {
+        const int np = build_pairs(G, j, R, N, start, pu, yl, nullptr, q);
+        if (lane == 0) np_s = np;
+    }
     __syncthreads();
     const int n = np_s;
     M5Tree* T = a.trees + ((int64_t)q * RS_NOPT + j);
@@ -366,319 +779,326 @@ m5p_fit_kernel(const TransferArgs a) {
         if (tid == 0) *st_out = RS_FIT_EMPTY;
         return;
     }
+    uint8_t* srt = dyn;                                           // [F][nmax]
+    uint8_t* rk = dyn + (size_t)fmax * nmax;                      // [F][nmax]
     for (int i = tid; i < n; i += kM5Threads) {
         const int u = pu[i];
         int r = 0;
         while (u >= start[r + 1]) ++r;
         S.zp[i] = a.ZA + a.a_xo[g0 + r] + (int64_t)(u - start[r]) * F;
         S.y[i] = yl[i];
+        S.y2[i] = __dmul_rn(yl[i], yl[i]);
         S.ids[i] = (uint8_t)i;
     }
     __syncthreads();
-    // presort: attribute f's instances by (value, index)
-    for (int f = tid; f < F; f += kM5Threads) {
-        uint8_t* o = S.gr.sorted[f];
-        for (int i = 0; i < n; ++i) {
-            const double v = __ldg(S.zp[i] + f);
-            int p = i;
-            while (p > 0) {
-                const int w = o[p - 1];
-                const double u = __ldg(S.zp[w] + f);
-                if (u > v || (u == v && w > i)) {
-                    o[p] = (uint8_t)w;
-                    --p;
-                } else {
-                    break;
+    // presort, a warp per attribute: an instance's place is the number before it by (value, index),
+    // its rank the number of smaller values (a label of its group of equals); integer order keys
+    for (int f = warp; f < F; f += kM5Warps) {
+        long long key[kM5MaxN / 32];
+        int pos[kM5MaxN / 32], less[kM5MaxN / 32];
+#pragma unroll
+        for (int x = 0; x < kM5MaxN / 32; ++x) {
+            const int i = lane + 32 * x;
+            key[x] = i < n ? okey(__ldg(S.zp[i] + f)) : 0x7fffffffffffffffll;
+            pos[x] = less[x] = 0;
+        }
+#pragma unroll
+        for (int x = 0; x < kM5MaxN / 32; ++x)
+            for (int s = 0; s < 32 && 32 * x + s < n; ++s) {
+                const long long k = __shfl_sync(0xffffffffu, key[x], s);
+                const int i = 32 * x + s;
+#pragma unroll
+                for (int z = 0; z < kM5MaxN / 32; ++z) {
+                    less[z] += k < key[z];
+                    pos[z] += k < key[z] || (k == key[z] && i < lane + 32 * z);
                 }
             }
-            o[p] = (uint8_t)i;
+#pragma unroll
+        for (int x = 0; x < kM5MaxN / 32; ++x) {
+            const int i = lane + 32 * x;
+            if (i < n) {
+                srt[f * nmax + pos[x]] = (uint8_t)i;
+                rk[f * nmax + i] = (uint8_t)less[x];
+            }
         }
     }
-    if (tid == 0) {
-        S.nn = 1;
-        S.sp = 1;
-        S.stack_node[0] = 0;
-        S.stack_lo[0] = 0;
-        S.stack_hi[0] = n;
-        double s1 = 0.0, s2 = 0.0;
-        for (int i = 0; i < n; ++i) {
-            s1 = __dadd_rn(s1, S.y[i]);
-            s2 = __dadd_rn(s2, __dmul_rn(S.y[i], S.y[i]));
+    if (warp == 0) {                               // the root's exact sums: lane 0 s1, lane 1 s2, one chain
+        double s = 0.0;
+        for (int i = 0; i < n; ++i) s = __dadd_rn(s, lane == 1 ? S.y2[i] : S.y[i]);
+        const double s1 = __shfl_sync(0xffffffffu, s, 0), s2 = __shfl_sync(0xffffffffu, s, 1);
+        const double sd = m5_sd(n, s1, s2);
+        if (lane == 0) {
+            S.sd_root = sd;
+            S.nn = 1;
+            S.level[0] = 0;
+            S.level[1] = 1;
+            S.lo[0] = 0;
+            S.hi[0] = (uint8_t)n;
+            S.parent[0] = -1;
         }
-        S.sd_root = m5_sd(n, s1, s2);
+        const double mean = s1 / n;
+        for (int i = lane; i < n; i += 32) S.yf[i] = (float)(S.y[i] - mean);
     }
     __syncthreads();
-    // ---- grow (depth first, left child first: the reference's node numbering).  Thread 0 pops
-    // the next node; every path through the body ends at a barrier before the next pop.
-    for (;;) {
+    // ---- grow, level by level (children get larger numbers than their parents)
+    int depth = 0;
+    for (;; ++depth) {
+        const int n0 = S.level[depth], nl = S.level[depth + 1] - n0;
         if (tid == 0) {
-            if (S.sp > 0) {
-                --S.sp;
-                S.cur = S.stack_node[S.sp];
-                S.cur_lo = S.stack_lo[S.sp];
-                S.cur_hi = S.stack_hi[S.sp];
-            } else {
-                S.cur = -1;
+            S.task = 0;
+            S.nsurv = 0;
+        }
+        // per node: FP32 statistics, and leaves by size or deviation (near the line, or with labels
+        // that FP32 does not hold: by the exact deviation)
+        for (int k = warp; k < nl; k += kM5Warps) {
+            const int t = n0 + k, lo = S.lo[t], m = S.hi[t] - lo;
+            float s = 0.f, am = 0.f;
+            for (int e = lane; e < m; e += 32) {
+                const float v = S.yf[S.ids[lo + e]];
+                s += v;
+                am = fmaxf(am, fabsf(v));
             }
-        }
-        __syncthreads();
-        const int t = S.cur, lo = S.cur_lo, hi = S.cur_hi, m = hi - lo;
-        if (t < 0) break;
-        if (tid == 0) {
-            S.attr[t] = -1;
-            S.lo[t] = (uint8_t)lo;
-            S.hi[t] = (uint8_t)hi;
-        }
-        // the node's label sums in instance order
-        double s1 = 0.0, s2 = 0.0;
-        for (int a2 = lo; a2 < hi; ++a2) {
-            const double yv = S.y[S.ids[a2]];
-            s1 = __dadd_rn(s1, yv);
-            s2 = __dadd_rn(s2, __dmul_rn(yv, yv));
-        }
-        const double sd = m5_sd(m, s1, s2);
-        if (m < 4 || sd <= __dmul_rn(kM5SdFrac, S.sd_root)) {
-            __syncthreads();
-            continue;
-        }
-        // split search: one thread per attribute, candidates in sorted order
-        double best = 0.0, bthr = 0.0;
-        int battr = -1;
-        for (int f = tid; f < F; f += kM5Threads) {
-            const uint8_t* o = S.gr.sorted[f];
-            double l1 = 0.0, l2 = 0.0;
-            for (int c = 1; c < m; ++c) {
-                const int ia = o[lo + c - 1], ib = o[lo + c];
-                const double yv = S.y[ia];
-                l1 = __dadd_rn(l1, yv);
-                l2 = __dadd_rn(l2, __dmul_rn(yv, yv));
-                const double va = __ldg(S.zp[ia] + f), vb = __ldg(S.zp[ib] + f);
-                if (!(va < vb) || c < 2 || m - c < 2) continue;
-                const double sdl = m5_sd(c, l1, l2), sdr = m5_sd(m - c, __dsub_rn(s1, l1), __dsub_rn(s2, l2));
-                const double red = __dsub_rn(sd, __ddiv_rn(__dadd_rn(__dmul_rn((double)c, sdl),
-                                                                     __dmul_rn((double)(m - c), sdr)),
-                                                           (double)m));
-                if (red > best) {
-                    best = red;
-                    battr = f;
-                    bthr = __dmul_rn(__dadd_rn(va, vb), 0.5);
-                }
-            }
-        }
-        // block argmax: largest SDR, ties to the lower attribute
 #pragma unroll
-        for (int o2 = 16; o2 >= 1; o2 >>= 1) {
-            const double ob = __shfl_xor_sync(0xffffffffu, best, o2);
-            const int oa = __shfl_xor_sync(0xffffffffu, battr, o2);
-            const double ot = __shfl_xor_sync(0xffffffffu, bthr, o2);
-            if (oa >= 0 && (battr < 0 || ob > best || (ob == best && oa < battr))) {
-                best = ob;
-                battr = oa;
-                bthr = ot;
+            for (int o = 16; o > 0; o >>= 1) {
+                s += __shfl_xor_sync(0xffffffffu, s, o);
+                am = fmaxf(am, __shfl_xor_sync(0xffffffffu, am, o));
             }
-        }
-        if (lane == 0) {
-            S.red_v[warp] = best;
-            S.red_i[warp] = battr;
-            S.colk[warp] = bthr;
-        }
-        __syncthreads();
-        if (tid == 0) {
-            double bb = 0.0, bt = 0.0;
-            int ba = -1;
-            for (int w2 = 0; w2 < nwarps; ++w2) {
-                const int oa = S.red_i[w2];
-                if (oa >= 0 && (ba < 0 || S.red_v[w2] > bb || (S.red_v[w2] == bb && oa < ba))) {
-                    bb = S.red_v[w2];
-                    ba = oa;
-                    bt = S.colk[w2];
+            const float mean = s / (float)m;
+            float t1 = 0.f, t2 = 0.f;
+            for (int e = lane; e < m; e += 32) {
+                const float v = S.yf[S.ids[lo + e]] - mean;
+                t1 += v;
+                t2 = fmaf(v, v, t2);
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                t1 += __shfl_xor_sync(0xffffffffu, t1, o);
+                t2 += __shfl_xor_sync(0xffffffffu, t2, o);
+            }
+            // the exact label sums in instance order: lane 0 s1, lane 1 s2
+            double xs = 0.0;
+            bool leaf = m < 4;
+            const float sda = sqrtf(t2 / (float)m), lim = (float)(kM5SdFrac * S.sd_root);
+            const bool fp32 = t2 < 1e30f && am < 1e15f && lim > 1e-15f;
+            const float slack = 1e-3f * lim + 4e-6f * am;
+            if (!leaf && fp32 && sda < lim - slack) leaf = true;
+            int cnt = leaf ? -1 : 0;
+            if (!leaf) {
+                for (int e = 0; e < m; ++e) {
+                    const int i = S.ids[lo + e];
+                    xs = __dadd_rn(xs, lane == 1 ? S.y2[i] : S.y[i]);
+                }
+                const double s1 = __shfl_sync(0xffffffffu, xs, 0), s2 = __shfl_sync(0xffffffffu, xs, 1);
+                if (!fp32 || sda <= lim + slack) {
+                    if (m5_sd(m, s1, s2) <= __dmul_rn(kM5SdFrac, S.sd_root)) cnt = -1;
+                    else if (!fp32) cnt = -2;
+                }
+                if (lane == 0) {
+                    S.s1[k] = s1;
+                    S.s2[k] = s2;
                 }
             }
-            S.split_attr = ba;
-            S.split_thr = bt;
+            if (lane == 0) {
+                S.attr[t] = -1;
+                S.cnt[k] = cnt;
+                S.mean[k] = mean;
+                S.tot[k] = t1;
+                S.tot2[k] = t2;
+                S.amax2[k] = am * am;
+                S.sda[k] = sda;
+                S.best_hi[k] = 0x7f800000u;
+                S.best_red[k] = 0ull;
+                S.best_key[k] = 0xffffffffu;
+            }
         }
         __syncthreads();
-        const int sa = S.split_attr;
-        if (sa < 0) {                              // no admissible split: a leaf (uniform)
+        // the attributes' scans of every splitting node, dealt to the warps: the best upper bound
+        for (int x = warp; x < nl * F; x += kM5Warps) {
+            const int k = x / F, f = x - k * F;
+            if (S.cnt[k] < 0) continue;
+            m5_scan<false>(S, srt + f * nmax, rk + f * nmax, f, S.lo[n0 + k], S.hi[n0 + k] - S.lo[n0 + k], k);
+        }
+        __syncthreads();
+        for (int x = warp; x < nl * F; x += kM5Warps) {
+            const int k = x / F, f = x - k * F;
+            if (S.cnt[k] < 0 || S.best_hi[k] == 0x7f800000u) continue;
+            m5_scan<true>(S, srt + f * nmax, rk + f * nmax, f, S.lo[n0 + k], S.hi[n0 + k] - S.lo[n0 + k], k);
+        }
+        __syncthreads();
+        const bool over = S.nsurv > kM5Surv;       // then every node of the level by the exact scan
+        const int nsv = over ? 0 : S.nsurv;
+        // exact SDRs of the survivors, two threads each (left and right); a node's only survivor
+        // whose SDR is positive beyond doubt needs none
+        for (int x = tid >> 1; x < ((nsv + kM5Threads / 2 - 1) & ~(kM5Threads / 2 - 1)); x += kM5Threads / 2) {
+            const unsigned sv = x < nsv ? S.surv[x] : 0u;
+            const int k = (int)(sv >> 16), f = (int)(sv >> 8) & 0xff, c = (int)(sv & 0xff);
+            const int t = n0 + k, lo = S.lo[t], m = S.hi[t] - lo;
+            const bool sure = x < nsv && S.cnt[k] == 1 && __uint_as_float(S.best_hi[k]) < 0.999f * (float)m * S.sda[k] - 1e-5f * (float)m * sqrtf(S.amax2[k]);
+            const bool work = x < nsv && !sure;
+            double sdx = 0.0;
+            if (work) {
+                const uint8_t* o = srt + f * nmax + lo;
+                double l1 = 0.0, l2 = 0.0;
+                for (int e = 0; e < c; ++e) {
+                    l1 = __dadd_rn(l1, S.y[o[e]]);
+                    l2 = __dadd_rn(l2, S.y2[o[e]]);
+                }
+                if (tid & 1) {
+                    l1 = __dsub_rn(S.s1[k], l1);
+                    l2 = __dsub_rn(S.s2[k], l2);
+                }
+                const int cc = (tid & 1) ? m - c : c;
+                sdx = __dmul_rn((double)cc, m5_sd(cc, l1, l2));
+            }
+            const double other = __shfl_xor_sync(0xffffffffu, sdx, 1);
+            if (x < nsv && !(tid & 1)) {
+                double red = 1.0;
+                if (work) red = __dsub_rn(m5_sd(m, S.s1[k], S.s2[k]), __ddiv_rn(__dadd_rn(sdx, other), (double)m));
+                S.red[x] = red;
+                if (red > 0.0) atomicMax(&S.best_red[k], (unsigned long long)__double_as_longlong(red));
+            }
+        }
+        // nodes for the exact scan: one thread per attribute
+        for (int k = 0; k < nl; ++k) {
+            const int c = S.cnt[k];
+            if (c != -2 && !(over && c >= 0)) continue;      // (uniform)
+            const int t = n0 + k, lo = S.lo[t], m = S.hi[t] - lo;
+            const double sd = m5_sd(m, S.s1[k], S.s2[k]);
+            double best = 0.0;
+            unsigned key = 0xffffffffu;
+            for (int f = tid; f < F; f += kM5Threads)
+                m5_exact_scan(S, srt + f * nmax, rk + f * nmax, f, lo, m, k, sd, best, key);
+            if (best > 0.0) atomicMax(&S.best_red[k], (unsigned long long)__double_as_longlong(best));
             __syncthreads();
-            continue;
-        }
-        const double sthr = S.split_thr;
-        for (int a2 = lo + tid; a2 < hi; a2 += kM5Threads) {
-            const int i = S.ids[a2];
-            S.side[i] = __ldg(S.zp[i] + sa) <= sthr ? 0 : 1;
+            if (best > 0.0 && (unsigned long long)__double_as_longlong(best) == S.best_red[k]) atomicMin(&S.best_key[k], key);
+            __syncthreads();
         }
         __syncthreads();
-        // stable partition of the node's instance list and of every attribute's sorted list
-        int nl = 0;
-        for (int f = tid; f < F + 1; f += kM5Threads) {
-            uint8_t* o = f < F ? S.gr.sorted[f] : S.ids;
-            uint8_t* sc = S.gr.scratch[tid];
-            int k = 0;
-            for (int a2 = lo; a2 < hi; ++a2)
-                if (S.side[o[a2]] == 0) sc[k++] = o[a2];
-            nl = k;
-            for (int a2 = lo; a2 < hi; ++a2)
-                if (S.side[o[a2]] == 1) sc[k++] = o[a2];
-            for (int a2 = 0; a2 < m; ++a2) o[lo + a2] = sc[a2];
+        // ties: the lowest attribute, then the lowest count
+        for (int x = tid; x < nsv; x += kM5Threads) {
+            const int k = (int)(S.surv[x] >> 16);
+            const double red = S.red[x];
+            if (red > 0.0 && (unsigned long long)__double_as_longlong(red) == S.best_red[k])
+                atomicMin(&S.best_key[k], S.surv[x] & 0xffffu);
+        }
+        __syncthreads();
+        // thresholds, sides and the number of instances going left, a warp per splitting node
+        for (int k = warp; k < nl; k += kM5Warps) {
+            const unsigned key = S.best_key[k];
+            if (key == 0xffffffffu) {
+                if (lane == 0) S.cnt[k] = -1;
+                continue;
+            }
+            const int t = n0 + k, lo = S.lo[t], m = S.hi[t] - lo, f = (int)(key >> 8), c = (int)(key & 0xff);
+            const uint8_t* o = srt + f * nmax + lo;
+            const double thr = __dmul_rn(__dadd_rn(__ldg(S.zp[o[c - 1]] + f), __ldg(S.zp[o[c]] + f)), 0.5);
+            int left = 0;
+            for (int e0 = 0; e0 < m; e0 += 32) {
+                const int e = e0 + lane;
+                const int i = e < m ? S.ids[lo + e] : 0;
+                const bool lf = e < m && __ldg(S.zp[i] + f) <= thr;
+                if (e < m) S.side[i] = lf ? 0 : 1;
+                left += __popc(__ballot_sync(0xffffffffu, lf));
+            }
+            // (two neighbouring doubles may have the upper one as their rounded mean: a side without
+            // instances is no split)
+            if (lane == 0) {
+                const bool two = left > 0 && left < m;
+                S.attr[t] = two ? (int16_t)f : (int16_t)-1;
+                S.thr[t] = thr;
+                S.cnt[k] = two ? left : -1;
+            }
         }
         __syncthreads();
         if (tid == 0) {
-            int cnt = 0;
-            for (int a2 = lo; a2 < hi; ++a2) cnt += S.side[S.ids[a2]] == 0;
-            const int l = S.nn, r = S.nn + 1;
-            S.nn += 2;
-            S.attr[t] = (int16_t)sa;
-            S.thr[t] = sthr;
-            S.left[t] = (int16_t)l;
-            S.right[t] = (int16_t)r;
-            T->parent[l] = T->parent[r] = (int16_t)t;
-            S.stack_node[S.sp] = r;
-            S.stack_lo[S.sp] = lo + cnt;
-            S.stack_hi[S.sp] = hi;
-            ++S.sp;
-            S.stack_node[S.sp] = l;
-            S.stack_lo[S.sp] = lo;
-            S.stack_hi[S.sp] = lo + cnt;
-            ++S.sp;
+            int nn = S.nn;
+            for (int k = 0; k < nl; ++k) {
+                if (S.cnt[k] < 0) continue;
+                const int t = n0 + k;
+                S.left[t] = (int16_t)nn;
+                S.right[t] = (int16_t)(nn + 1);
+                S.parent[nn] = S.parent[nn + 1] = (int16_t)t;
+                S.lo[nn] = S.lo[t];
+                S.hi[nn] = S.lo[nn + 1] = (uint8_t)(S.lo[t] + S.cnt[k]);
+                S.hi[nn + 1] = S.hi[t];
+                nn += 2;
+            }
+            S.nn = nn;
+            S.level[depth + 2] = nn;
         }
-        (void)nl;
+        // stable partition of each splitting node's range of every attribute's list and of the
+        // instance list, a warp per list
+        for (int x = warp; x < nl * (F + 1); x += kM5Warps) {
+            const int k = x / (F + 1), f = x - k * (F + 1);
+            if (S.cnt[k] < 0) continue;
+            const int t = n0 + k, lo = S.lo[t], m = S.hi[t] - lo;
+            uint8_t* o = (f < F ? srt + f * nmax : S.ids) + lo;
+            int id[kM5MaxN / 32], at[kM5MaxN / 32], l = 0, r = S.cnt[k];
+#pragma unroll
+            for (int z = 0; z < kM5MaxN / 32; ++z) {
+                const int e = 32 * z + lane;
+                id[z] = e < m ? o[e] : -1;
+                const bool lf = e < m && S.side[id[z]] == 0, rt = e < m && !lf;
+                const unsigned bl = __ballot_sync(0xffffffffu, lf), br = __ballot_sync(0xffffffffu, rt);
+                at[z] = lf ? l + __popc(bl & ((1u << lane) - 1u)) : r + __popc(br & ((1u << lane) - 1u));
+                l += __popc(bl);
+                r += __popc(br);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int z = 0; z < kM5MaxN / 32; ++z)
+                if (id[z] >= 0) o[at[z]] = (uint8_t)id[z];
+        }
         __syncthreads();
+        if (S.level[depth + 2] == S.level[depth + 1]) break;
     }
+    // ---- models and pruning.  Leaves (the label mean) first, a warp each; then the internal nodes
+    // level by level from the deepest, small ones a warp each, the others by the block
     const int nn = S.nn;
-    // ---- models and pruning, children before parents (children have larger node numbers)
-    for (int t = nn - 1; t >= 0; --t) {
-        const int lo = S.lo[t], m = S.hi[t] - S.lo[t];
-        const bool internal = S.attr[t] >= 0;
-        if (tid < kM5MaxFeat / 64) {
-            unsigned long long bits = 0;
-            if (internal) {
-                bits = S.tested[S.left[t]][tid] | S.tested[S.right[t]][tid];
-                if (S.attr[t] / 64 == tid) bits |= 1ull << (S.attr[t] % 64);
-            }
-            S.tested[t][tid] = bits;
-        }
-        __syncthreads();
-        if (tid == 0) {
-            int nc = 0;
-            for (int f = 0; f < F && nc < kM5MaxTerms; ++f)
-                if ((S.tested[t][f / 64] >> (f % 64)) & 1ull) S.cand[nc++] = (int16_t)f;
-            S.ncand = nc;
-            S.nsel = nc;
-            for (int k = 0; k < nc; ++k) S.sel[k] = (uint8_t)k;
-            double yb = 0.0;
-            for (int a2 = 0; a2 < m; ++a2) yb += S.y[S.ids[lo + a2]];
-            S.bval = yb / m;                       // the label mean, for now
-        }
-        __syncthreads();
-        const int nc = S.ncand;
-        const double ybar = S.bval;
-        for (int f = tid; f < nc; f += kM5Threads) {
-            double s = 0.0;
-            for (int a2 = 0; a2 < m; ++a2) s += __ldg(S.zp[S.ids[lo + a2]] + S.cand[f]);
-            S.zbar[f] = s / m;
-        }
-        __syncthreads();
-        for (int e = tid; e < nc * (nc + 1); e += kM5Threads) {
-            const int f = e / (nc + 1), g = e - f * (nc + 1);
-            double s = 0.0;
-            if (g < nc) {
-                if (g > f) continue;
-                for (int a2 = 0; a2 < m; ++a2) {
-                    const double* z = S.zp[S.ids[lo + a2]];
-                    s += (__ldg(z + S.cand[f]) - S.zbar[f]) * (__ldg(z + S.cand[g]) - S.zbar[g]);
-                }
-                S.mo.G[f * kM5Ld + g] = s + (f == g ? kM5Ridge : 0.0);
-                S.mo.G[g * kM5Ld + f] = s + (f == g ? kM5Ridge : 0.0);
-            } else {
-                for (int a2 = 0; a2 < m; ++a2) {
-                    const int i = S.ids[lo + a2];
-                    s += (__ldg(S.zp[i] + S.cand[f]) - S.zbar[f]) * (S.y[i] - ybar);
-                }
-                S.r[f] = s;
-            }
-        }
-        __syncthreads();
-        // greedy elimination
-        for (;;) {
-            const int ns = S.nsel;
-            for (int e = tid; e < ns * ns; e += kM5Threads) {
-                const int i = e / ns, k = e - i * ns;
-                S.mo.H[i * kM5Ld + k] = S.mo.G[S.sel[i] * kM5Ld + S.sel[k]];
-            }
-            __syncthreads();
-            m5_invert(S, S.mo.H, ns);
-            for (int i = tid; i < ns; i += kM5Threads) {
-                double s = 0.0;
-                for (int k = 0; k < ns; ++k) s = fma(S.mo.H[i * kM5Ld + k], S.r[S.sel[k]], s);
-                S.w[i] = s;
-            }
-            __syncthreads();
-            if (tid == 0) {
-                double b = ybar;
-                for (int i = 0; i < ns; ++i) b -= S.w[i] * S.zbar[S.sel[i]];
-                S.rowk[0] = b;                     // the model's intercept
-            }
-            __syncthreads();
-            if (warp == 0) {
-                const double e_full = m5_warp_err(S, lo, m, S.w, S.rowk[0], ns, S.sel, -1);
-                if (lane == 0) S.e_cur = e_full;
-            }
-            // drop-one candidates: w' = w - H[:, d] w_d / H_dd, one warp each
-            for (int d = warp; d < ns; d += nwarps) {
-                const double fac = S.w[d] / S.mo.H[d * kM5Ld + d];
-                double wd[kM5MaxTerms];
-                double b = ybar;
-                for (int i = 0; i < ns; ++i) {
-                    wd[i] = i == d ? 0.0 : fma(-S.mo.H[i * kM5Ld + d], fac, S.w[i]);
-                    if (i != d) b -= wd[i] * S.zbar[S.sel[i]];
-                }
-                const double ed = m5_warp_err(S, lo, m, wd, b, ns, S.sel, d);
-                if (lane == 0) S.cand_err[d] = ed;
-            }
-            __syncthreads();
-            if (tid == 0) {
-                double bestd = DBL_MAX;
-                int drop = -1;
-                for (int d = 0; d < ns; ++d)
-                    if (S.cand_err[d] < bestd) {
-                        bestd = S.cand_err[d];
-                        drop = d;
-                    }
-                S.drop = (ns > 0 && drop >= 0 && bestd <= S.e_cur) ? drop : -1;
-                if (S.drop >= 0) {
-                    for (int k = S.drop; k < ns - 1; ++k) S.sel[k] = S.sel[k + 1];
-                    S.nsel = ns - 1;
-                }
-            }
-            __syncthreads();
-            if (S.drop < 0) break;
-        }
-        // the node's model and the pruning decision
-        if (tid == 0) {
-            const int ns = S.nsel;
-            T->nterm[t] = ns;
-            for (int k = 0; k < ns; ++k) {
-                T->term_attr[t][k] = S.cand[S.sel[k]];
-                T->term_w[t][k] = S.w[k];
-            }
-            T->b[t] = S.rowk[0];
+    for (int t = warp; t < nn; t += kM5Warps) {
+        if (S.attr[t] >= 0) continue;
+        const int lo = S.lo[t], m = S.hi[t] - lo;
+        double s = 0.0, e = 0.0;
+        for (int x = lane; x < m; x += 32) s += S.y[S.ids[lo + x]];
+        s = m5_warp_sum(s) / m;
+        for (int x = lane; x < m; x += 32) e += fabs(S.y[S.ids[lo + x]] - s);
+        e = m5_warp_sum(e);
+        if (lane == 0) {
+            T->nterm[t] = 0;
+            T->b[t] = s;
             T->count[t] = m;
-            const double e = S.e_cur;
-            double keep = DBL_MAX;
-            if (internal) {
-                const int l = S.left[t], r = S.right[t];
-                const int ml = S.hi[l] - S.lo[l], mr = S.hi[r] - S.lo[r];
-                keep = (ml * S.est[l] + mr * S.est[r]) / m;
-            }
-            if (internal && !(e <= keep)) {
-                S.est[t] = keep;
-            } else {                               // a leaf: its parent's candidates get no test
-                S.attr[t] = -1;                    // from here down
-                S.est[t] = e;
-                for (int k = 0; k < kM5MaxFeat / 64; ++k) S.tested[t][k] = 0;
-            }
+            S.est[t] = m <= 1 ? DBL_MAX : e / m * ((double)(m + 1) / (double)(m - 1));
+            for (int k = 0; k < kM5MaxFeat / 64; ++k) S.tested[t][k] = 0;
         }
+    }
+    const int tm = fmax < kM5MaxTerms ? fmax : kM5MaxTerms, ld = tm | 1;
+    double* buf = reinterpret_cast<double*>(dyn);
+    __syncthreads();
+    for (int dp = depth; dp >= 0; --dp) {
+        const int n0 = S.level[dp], n1 = S.level[dp + 1];
+        for (int t = n0 + tid; t < n1; t += kM5Threads)      // (the children's are final)
+            if (S.attr[t] >= 0)
+                for (int k = 0; k < kM5MaxFeat / 64; ++k)
+                    S.tested[t][k] = S.tested[S.left[t]][k] | S.tested[S.right[t]][k] |
+                                     (S.attr[t] / 64 == k ? 1ull << (S.attr[t] % 64) : 0ull);
+        __syncthreads();
+        // which nodes of the level a warp can take (decided before any of them is pruned)
+        for (int t = n0 + tid; t < n1; t += kM5Threads) {
+            int nc = 0;
+            for (int k = 0; k < kM5MaxFeat / 64; ++k) nc += __popcll(S.tested[t][k]);
+            S.cnt[t - n0] = S.attr[t] < 0 ? 0 : (nc <= kM5WarpTerms && S.hi[t] - S.lo[t] <= kM5WarpN ? 1 : 2);
+        }
+        __syncthreads();
+        int turn = 0;
+        for (int t = n0; t < n1; ++t)
+            if (S.cnt[t - n0] == 1 && (turn++ & (kM5Warps - 1)) == warp) {
+                double* wb = buf + warp * kM5WarpBuf;
+                m5_model<true>(S, S.v.wv[warp], T, t, F, wb, wb + kM5WarpTerms * kM5WarpLd,
+                               wb + 2 * kM5WarpTerms * kM5WarpLd, kM5WarpLd);
+            }
+        __syncthreads();
+        for (int t = n0; t < n1; ++t)
+            if (S.cnt[t - n0] == 2) m5_model<false>(S, S.v.blk, T, t, F, buf, buf + tm * ld, buf + 2 * tm * ld, ld);
         __syncthreads();
     }
     for (int t = tid; t < nn; t += kM5Threads) {
@@ -686,10 +1106,10 @@ m5p_fit_kernel(const TransferArgs a) {
         T->thr[t] = S.thr[t];
         T->left[t] = S.left[t];
         T->right[t] = S.right[t];
+        T->parent[t] = S.parent[t];
     }
     if (tid == 0) {
         T->n_nodes = nn;
-        T->parent[0] = -1;
         *st_out = RS_FIT_OK;
     }
 }
@@ -737,23 +1157,71 @@ __device__ __forceinline__ double ibk_nearest_mean_n(int n, const double* __rest
     return sum / (double)kIbkK;
 }
 
-// One block per problem, one thread per version t of the test program: the pairs of the six
-// optimizations (the fits' order), the predictions (ridge: the fits of transfer_fit_kernel;
-// IBK: the neighbour lists), and rank_row.
-struct RankSmem {
-    GroupSmem G;
-    double yl[RS_NOPT][kTrPairs];
-    double lt_b[RS_MAXV];
-    uint16_t pu[RS_NOPT][kTrPairs];
-    uint8_t msk_b[RS_MAXV];
-    int8_t slot_b[RS_MAXV];
-    int np[RS_NOPT], st[RS_NOPT];
-};
+// The predictions of one (problem, optimization) for every candidate version of its test program, by
+// the fit of transfer_fit_kernel (four lanes a version), the neighbour list of IBK or the M5P tree
+// (one lane a version), into pred [Q][64][6] for transfer_rank_kernel.  One block per problem used to
+// walk the six optimizations in turn (101 us at 90 problems of 96 pairs; the two kernels: 27 us).
+template <int SUB>
+__global__ void __launch_bounds__(RS_MAXV * SUB)
+transfer_predict_kernel(const TransferArgs a) {
+    __shared__ GroupSmem G;
+    __shared__ uint16_t pu[kTrPairs];
+    __shared__ double yl[kTrPairs];
+    __shared__ int np_s;
+    const int q = blockIdx.x, j = blockIdx.y, tid = threadIdx.x;
+    int start[RS_MAXRUNS + 1], F = 0;
+    const int N = rs_group_layout(q, a.group_off, a.max_runs, a.n_runs, a.a_row, a.a_fw, a.b_fw, a.stat_stride, start, F);
+    const int64_t rb = a.b_row[q];
+    const int VB = (int)(a.b_row[q + 1] - rb);
+    if (N < 0 || N > a.ld || VB < 1 || VB > RS_MAXV) return;       // reported by transfer_rank_kernel
+    const int64_t g0 = a.group_off[q];
+    load_group(G, a.a_row, a.a_masks, a.a_lt, g0, start, N);
+    if (tid < 32) {
+        const int np = build_pairs(G, j, (int)(a.group_off[q + 1] - g0), N, start, pu, yl, a.r.dstatus, q);
+        if (tid == 0) np_s = np;
+    }
+    __syncthreads();
+    const int n = np_s;
+    uint8_t* st = a.fst + (int64_t)q * RS_NOPT + j;
+    if (a.ibk) {
+        if (tid == 0) *st = n > 0 ? RS_FIT_OK : RS_FIT_EMPTY;
+        if (n == 0) return;
+    } else if (*st != RS_FIT_OK) {
+        return;
+    }
+    const int t = tid / SUB, sub = tid % SUB;
+    const bool cand = t < VB && ((a.opt_mask >> j) & 1) && (a.rank_all || !((a.b_masks[rb + (t < VB ? t : 0)] >> j) & 1));
+    const double* Kt = a.Kx + ((int64_t)q * RS_MAXV + t) * a.ld;
+    double yh = 0.0;
+    if (SUB == 1) {
+        if (!cand) return;
+        if (a.m5p) {
+            yh = m5_predict(a.trees + ((int64_t)q * RS_NOPT + j), a.ZB + a.b_xo[q] + (int64_t)t * F);
+        } else if (n <= kIbkK) {
+            for (int i = 0; i < n; ++i) yh += yl[i];
+            yh /= (double)n;
+        } else {
+            yh = ibk_nearest_mean_n(n, Kt, pu, yl);
+        }
+    } else {
+        const double* cf = a.coef + ((int64_t)q * RS_NOPT + j) * kTrCoef;
+        if (cand && n > 1)
+            for (int i = sub; i < n; i += SUB) yh = fma(cf[1 + i], __ldg(Kt + pu[i]), yh);
+#pragma unroll
+        for (int o = 1; o < SUB; o <<= 1) yh += __shfl_xor_sync(0xffffffffu, yh, o);
+        if (!cand || sub) return;
+        yh += cf[0];
+    }
+    a.pred[((int64_t)q * RS_MAXV + t) * RS_NOPT + j] = yh;
+}
 
+// One block per problem, one thread per version t of the test program: its predictions through
+// rank_row, the problem's fit statuses and the counters.
 __global__ void __launch_bounds__(RS_MAXV)
 transfer_rank_kernel(const TransferArgs a) {
-    extern __shared__ __align__(16) unsigned char tsm[];
-    RankSmem& S = *reinterpret_cast<RankSmem*>(tsm);
+    __shared__ double lt_b[RS_MAXV];
+    __shared__ uint8_t msk_b[RS_MAXV];
+    __shared__ int8_t slot_b[RS_MAXV];
     const int q = blockIdx.x, tid = threadIdx.x;
     int start[RS_MAXRUNS + 1], F = 0;
     const int N = rs_group_layout(q, a.group_off, a.max_runs, a.n_runs, a.a_row, a.a_fw, a.b_fw, a.stat_stride, start, F);
@@ -763,57 +1231,28 @@ transfer_rank_kernel(const TransferArgs a) {
         if (tid == 0) rs_dev_flag(a.r.dstatus, RS_EDATA, q);
         return;
     }
-    const int64_t g0 = a.group_off[q];
-    const int R = (int)(a.group_off[q + 1] - g0);
-    S.slot_b[tid] = -1;
+    slot_b[tid] = -1;
+    __syncthreads();
     if (tid < VB) {
-        S.msk_b[tid] = a.b_masks[rb + tid] & 63;
-        S.lt_b[tid] = a.b_lt[rb + tid];
-    }
-    load_group(S.G, a.a_row, a.a_masks, a.a_lt, g0, start, N);
-    if (tid < VB) S.slot_b[S.msk_b[tid]] = (int8_t)tid;
-    if (tid < RS_NOPT) {
-        const int j = tid;
-        const int np = build_pairs(S.G, j, R, start, S.pu[j], S.yl[j], a.r.dstatus, q);
-        S.np[j] = np;
-        S.st[j] = a.ibk ? (np > 0 ? RS_FIT_OK : RS_FIT_EMPTY) : a.fst[(int64_t)q * RS_NOPT + j];
-        if (a.m5p && np > kM5MaxN) S.st[j] = RS_FIT_NOTPD;
+        msk_b[tid] = a.b_masks[rb + tid] & 63;
+        lt_b[tid] = a.b_lt[rb + tid];
+        slot_b[msk_b[tid]] = (int8_t)tid;
     }
     __syncthreads();
+    const uint8_t* fst = a.fst + (int64_t)q * RS_NOPT;
     RankTally c;
     const int t = tid;
     if (t < VB) {
-        const int mt = S.msk_b[t];
-        const uint32_t info = row_summary(t, VB, S.msk_b, S.lt_b, S.slot_b);
+        const int mt = msk_b[t];
+        const uint32_t info = row_summary(t, VB, msk_b, lt_b, slot_b);
         const int candm = (a.rank_all ? 63 : (~mt & 63)) & a.opt_mask;
         int okm = 0;
 #pragma unroll
-        for (int j = 0; j < RS_NOPT; ++j) okm |= (S.st[j] == RS_FIT_OK) << j;
-        const double* Kt = a.Kx + ((int64_t)q * RS_MAXV + t) * a.ld;
+        for (int j = 0; j < RS_NOPT; ++j) okm |= (fst[j] == RS_FIT_OK) << j;
+        const double* pr = a.pred + ((int64_t)q * RS_MAXV + t) * RS_NOPT;
         double pred[RS_NOPT];
 #pragma unroll
-        for (int j = 0; j < RS_NOPT; ++j) {
-            pred[j] = 0.0;
-            if (!(((candm & okm) >> j) & 1)) continue;
-            const int n = S.np[j];
-            if (a.m5p) {
-                pred[j] = m5_predict(a.trees + ((int64_t)q * RS_NOPT + j), a.ZB + a.b_xo[q] + (int64_t)t * F);
-            } else if (a.ibk) {
-                if (n <= kIbkK) {
-                    double sum = 0.0;
-                    for (int i = 0; i < n; ++i) sum += S.yl[j][i];
-                    pred[j] = sum / (double)n;
-                } else {
-                    pred[j] = ibk_nearest_mean_n(n, Kt, S.pu[j], S.yl[j]);
-                }
-            } else {
-                const double* cf = a.coef + ((int64_t)q * RS_NOPT + j) * kTrCoef;
-                double yh = cf[0];
-                if (n > 1)
-                    for (int i = 0; i < n; ++i) yh = fma(cf[1 + i], __ldg(Kt + S.pu[j][i]), yh);
-                pred[j] = yh;
-            }
-        }
+        for (int j = 0; j < RS_NOPT; ++j) pred[j] = ((candm & okm) >> j) & 1 ? pr[j] : 0.0;
         // rank_row's candidates are the optimizations outside the version-mask field: put the
         // excluded ones there (t's own unless all six are ranked, and those outside opt_mask);
         // the fits that are not OK go in the empty-fit field
@@ -823,7 +1262,7 @@ transfer_rank_kernel(const TransferArgs a) {
         rank_row(a.r, rb + t, info64, pred, c);
     }
     if (tid < RS_NOPT) {
-        const int st = S.st[tid];
+        const int st = fst[tid];
         if (a.fit_status) a.fit_status[(int64_t)q * RS_NOPT + tid] = (uint8_t)st;
         if (a.r.counters && st >= 0 && st <= RS_FIT_NONFINITE) atomicAdd(a.r.counters + 9 + st, 1ull);
     }
@@ -886,15 +1325,17 @@ cudaError_t rs_launch_transfer(const rs_transfer_args& t, cudaStream_t st) {
     a.ZA = t.ZA;
     a.a_xo = t.a_x_offsets;
     a.ZB = t.ZB;
+    a.pred = const_cast<double*>(t.KA);  // the group's Gram (at least 64 x 64 doubles a problem) is no
+                                         // longer read once the fits are made, nor at all without ridge
     a.b_xo = t.b_x_offsets;
     a.r = RankPassArgs{nullptr, 0, nullptr, 0, 0, nullptr, t.dstatus, t.k, okey_host(t.log_tau),
                        t.flags & ~RS_RANK_ALL, t.rec_code, t.rec_pred, t.pred_all, t.counters};
     cudaError_t e = cudaSuccess;
     if (t.m5p) {
-        const size_t msmem = sizeof(M5Smem);
+        const size_t msmem = ((sizeof(M5Smem) + 15) & ~(size_t)15) + m5_dyn_bytes(t.stat_stride);
         e = cudaFuncSetAttribute(m5p_fit_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)msmem);
         if (e != cudaSuccess) return e;
-        m5p_fit_kernel<<<dim3((unsigned)t.Q, RS_NOPT), kM5Threads, msmem, st>>>(a);
+        m5p_fit_kernel<<<dim3((unsigned)t.Q, RS_NOPT), kM5Threads, msmem, st>>>(a, t.stat_stride);
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     } else if (!t.ibk) {
@@ -906,9 +1347,11 @@ cudaError_t rs_launch_transfer(const rs_transfer_args& t, cudaStream_t st) {
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    const size_t smem = sizeof(RankSmem);
-    e = cudaFuncSetAttribute(transfer_rank_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const dim3 grid((unsigned)t.Q, RS_NOPT);
+    if (t.ibk || t.m5p) transfer_predict_kernel<1><<<grid, RS_MAXV, 0, st>>>(a);
+    else transfer_predict_kernel<4><<<grid, RS_MAXV * 4, 0, st>>>(a);
+    e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    transfer_rank_kernel<<<(unsigned)t.Q, RS_MAXV, smem, st>>>(a);
+    transfer_rank_kernel<<<(unsigned)t.Q, RS_MAXV, 0, st>>>(a);
     return cudaGetLastError();
 }
