@@ -265,7 +265,7 @@ transfer_fit_kernel(const TransferArgs a, int nmax) {
 // updates of H, w and T; the model that stays is solved again from scratch.  (Before: one thread per
 // attribute walking every candidate's SDR, an inverse per round and every drop-one model applied to
 // every instance, all serial over the nodes.)  Small nodes' models take one warp each.
-// 36 problems x 3 runs x 37 attributes (96 instances a fit): 5532 -> 1976 us.
+// 36 problems x 3 runs x 37 attributes (96 instances a fit): 5532 -> 1351 us.
 constexpr int kM5MaxN = kTrPairs;                 // instances of one fit
 constexpr int kM5MaxNodes = 2 * kM5MaxN - 1;
 constexpr int kM5MaxTerms = 64;
@@ -274,8 +274,9 @@ constexpr int kM5Threads = 256;
 constexpr int kM5Warps = kM5Threads / 32;
 constexpr int kM5WarpTerms = 16, kM5WarpN = 32;   // models up to this size take one warp
 constexpr int kM5WarpLd = kM5WarpTerms + 1;
-constexpr int kM5WarpBuf = 2 * kM5WarpTerms * kM5WarpLd + kM5WarpN * kM5WarpLd;   // G, H, C
-constexpr int kM5Surv = 512;                      // candidate splits kept for exact evaluation, per level
+constexpr int kM5WarpBuf = kM5WarpTerms * kM5WarpLd + kM5WarpN * kM5WarpLd +
+                           (kM5WarpN * kM5WarpLd + 1) / 2;                   // H, C, T (FP32)
+constexpr int kM5Surv = 1024;                     // candidate splits listed for exact evaluation, per level
 constexpr double kM5SdFrac = 0.05, kM5Smooth = 15.0, kM5Ridge = 1e-8;
 
 struct M5Tree {
@@ -291,10 +292,12 @@ struct M5Tree {
 // Per group of threads (a warp, or the block): the vectors of one node's model.
 template <int N>
 struct M5Vec {
-    double colk[N], rowk[N], zbar[N], r[N], w[N], fac[N];
+    double colk[N], rowk[N], zbar[N], r[N], w[N], wt[N], fac[N];
+    float fac32[N], rowk32[N];
     int16_t cand[N];
     uint8_t sel[N];
     double e_cur, b;
+    unsigned long long reach;                     // attributes whose drop may be the best
     int drop;
 };
 
@@ -318,19 +321,35 @@ struct M5Smem {
     int cnt[kM5MaxN];                             // survivors; -1: a leaf, -2: by the exact scan
     double s1[kM5MaxN], s2[kM5MaxN];              // exact label sums, in instance order
     unsigned surv[kM5Surv];                       // node << 16 | attribute << 8 | count
+    float ql[kM5Surv];                            // their lower bounds of Q
     double red[kM5Surv];                          // their SDRs
-    double errp[kM5Warps][kM5MaxTerms];
+    double rcp[kM5MaxN + 1];                      // 1 / c, rounded
+    float errp[2][kM5Warps][kM5MaxTerms];
+    double sump[kM5Warps];
+    float res32[kM5Warps * 32];
     union {
         M5Vec<kM5MaxTerms> blk;
         M5Vec<kM5WarpTerms> wv[kM5Warps];
     } v;
 };
 
+// a / c rounded to nearest, y = 1 / c rounded to nearest: q = a y is within a unit of the quotient,
+// its residual a - q c is exact in an FMA, and q + r y rounds to the quotient (P. Markstein,
+// "Computation of elementary functions on the IBM RISC System/6000 processor", IBM J. Res. Dev. 34,
+// 1990).  Three FP64 instructions; magnitudes whose residual could underflow, infinities and NaN take
+// the division.
+__device__ __forceinline__ double m5_div(double a, double c, double y) {
+    const int ex = (__double2hiint(a) >> 20) & 0x7ff;
+    if ((unsigned)(ex - 200) > 1600u && a != 0.0) return __ddiv_rn(a, c);
+    const double q = __dmul_rn(a, y);
+    return __fma_rn(__fma_rn(-q, c, a), y, q);
+}
+
 // The standard deviation from a count, sum and sum of squares: sqrt(max(0, (s2 - s1 s1 / c) / c)),
 // with one rounding per operation (the reference's arithmetic).
-__device__ __noinline__ double m5_sd(int c, double s1, double s2) {
+__device__ __noinline__ double m5_sd(int c, double y, double s1, double s2) {
     const double cd = (double)c;
-    const double v = __ddiv_rn(__dsub_rn(s2, __ddiv_rn(__dmul_rn(s1, s1), cd)), cd);
+    const double v = m5_div(__dsub_rn(s2, m5_div(__dmul_rn(s1, s1), cd, y)), cd, y);
     return __dsqrt_rn(v > 0.0 ? v : 0.0);
 }
 
@@ -353,49 +372,47 @@ __device__ __forceinline__ void m5_bounds(int c, int m, float l1, float l2, floa
     lo = (sqrtf(fmaxf(L - dl, 0.f)) + sqrtf(fmaxf(R - dr, 0.f))) * 0.99999f;
 }
 
-// One warp scans attribute f of a node (rank lo.., m instances, level slot q): SURVIVORS false
-// lowers the node's best upper bound, true lists the candidates whose lower bound reaches it.
-template <bool SURVIVORS>
-__device__ __forceinline__ void m5_scan(M5Smem& S, const uint8_t* srt, const uint8_t* rk, int f, int lo, int m, int q) {
-    const int lane = threadIdx.x & 31;
+// A segment of W lanes (W = 32, or at least m) scans attribute f of a node (instances lo .. lo + m,
+// level slot q; f < 0: no attribute for this segment): lowers the node's best upper bound of Q and
+// lists the candidates whose lower bound reaches it as it then stands.
+__device__ __forceinline__ void m5_scan(M5Smem& S, const uint8_t* srt, const uint8_t* rk, int f, int lo, int m, int q,
+                                        int W) {
+    const int lane = threadIdx.x & 31, sl = lane & (W - 1);
     const float mean = S.mean[q], t1 = S.tot[q], t2 = S.tot2[q], a2 = S.amax2[q];
-    float c1 = 0.f, c2 = 0.f, best = __int_as_float(0x7f800000);
-    const float lim = SURVIVORS ? __uint_as_float(S.best_hi[q]) : 0.f;
-    for (int base = 0; base < m; base += 32) {
-        const int e = base + lane;
-        const bool in = e < m;
+    float c1 = 0.f, c2 = 0.f;
+    for (int base = 0; base < m; base += W) {
+        const int e = base + sl;
+        const bool in = e < m && f >= 0;
         const int id = in ? srt[lo + e] : 0;
-        const int nx = e + 1 < m ? srt[lo + e + 1] : id;
+        const int nx = in && e + 1 < m ? srt[lo + e + 1] : id;
         const float v = in ? S.yf[id] - mean : 0.f;
         float s = v, w = v * v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const float a = __shfl_up_sync(0xffffffffu, s, o), b = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) {
+        for (int o = 1; o < W; o <<= 1) {
+            const float a = __shfl_up_sync(0xffffffffu, s, o, W), b = __shfl_up_sync(0xffffffffu, w, o, W);
+            if (sl >= o) {
                 s += a;
                 w += b;
             }
         }
         s += c1;
         w += c2;
-        c1 = __shfl_sync(0xffffffffu, s, 31);
+        c1 = __shfl_sync(0xffffffffu, s, 31);      // (carried on for W = 32 only)
         c2 = __shfl_sync(0xffffffffu, w, 31);
         const int c = e + 1;
-        if (in && c >= 2 && m - c >= 2 && rk[nx] != rk[id]) {
-            float ql, qh;
-            m5_bounds(c, m, s, w, t1, t2, a2, ql, qh);
-            if (!SURVIVORS) {
-                best = fminf(best, qh);
-            } else if (ql <= lim) {
-                const int k = atomicAdd(&S.nsurv, 1);
-                atomicAdd(&S.cnt[q], 1);
-                if (k < kM5Surv) S.surv[k] = (unsigned)q << 16 | (unsigned)f << 8 | (unsigned)c;
+        float ql = 0.f, qh = __int_as_float(0x7f800000);
+        const bool can = in && c >= 2 && m - c >= 2 && rk[nx] != rk[id];
+        if (can) m5_bounds(c, m, s, w, t1, t2, a2, ql, qh);
+        const unsigned low = __reduce_min_sync(0xffffffffu, __float_as_uint(qh));
+        unsigned lim = 0;
+        if (lane == 0) lim = low < 0x7f800000u ? atomicMin(&S.best_hi[q], low) : 0u;
+        lim = __shfl_sync(0xffffffffu, lim, 0);
+        if (can && ql <= __uint_as_float(lim < low ? lim : low)) {
+            const int k = atomicAdd(&S.nsurv, 1);
+            if (k < kM5Surv) {
+                S.surv[k] = (unsigned)q << 16 | (unsigned)f << 8 | (unsigned)c;
+                S.ql[k] = ql;
             }
         }
-    }
-    if (!SURVIVORS) {
-        const unsigned b = __reduce_min_sync(0xffffffffu, __float_as_uint(best));
-        if (lane == 0) atomicMin(&S.best_hi[q], b);
     }
 }
 
@@ -409,9 +426,10 @@ __device__ __noinline__ void m5_exact_scan(const M5Smem& S, const uint8_t* o, co
         l1 = __dadd_rn(l1, S.y[ia]);
         l2 = __dadd_rn(l2, S.y2[ia]);
         if (rk[ia] == rk[ib] || c < 2 || m - c < 2) continue;
-        const double sdl = m5_sd(c, l1, l2), sdr = m5_sd(m - c, __dsub_rn(S.s1[q], l1), __dsub_rn(S.s2[q], l2));
-        const double red = __dsub_rn(sd, __ddiv_rn(__dadd_rn(__dmul_rn((double)c, sdl), __dmul_rn((double)(m - c), sdr)),
-                                                   (double)m));
+        const double sdl = m5_sd(c, S.rcp[c], l1, l2);
+        const double sdr = m5_sd(m - c, S.rcp[m - c], __dsub_rn(S.s1[q], l1), __dsub_rn(S.s2[q], l2));
+        const double red = __dsub_rn(sd, m5_div(__dadd_rn(__dmul_rn((double)c, sdl), __dmul_rn((double)(m - c), sdr)),
+                                                (double)m, S.rcp[m]));
         if (red > best) {
             best = red;
             key = (unsigned)f << 8 | (unsigned)c;
@@ -473,14 +491,21 @@ __device__ double m5_warp_err(const M5Smem& S, const Vec& V, int lo, int m, int 
     return acc / m * ((double)(m + v) / (double)(m - v));
 }
 
-// w = H r, the intercept and e_cur of the model on V.sel[0 .. ns), H = inverse of its system.
+// H = inverse of the normal equations of V.sel[0 .. ns), w = H r, the intercept and e_cur.
 template <bool WARP, class Vec>
-__device__ void m5_solve(M5Smem& S, Vec& V, const double* G, double* H, int ld, int ns, int lo, int m, double ybar) {
+__device__ void m5_solve(M5Smem& S, Vec& V, const double* C, double* H, int ld, int ns, int lo, int m, double ybar) {
     using Gp = M5Group<WARP>;
     const int tid = Gp::tid();
-    for (int e = tid; e < ns * ns; e += Gp::kNT) {
-        const int i = e / ns, k = e - i * ns;
-        H[i * ld + k] = G[V.sel[i] * ld + V.sel[k]];
+    for (int e = tid; e < ns * (ns + 1) / 2; e += Gp::kNT) {
+        int f = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
+        while (f * (f + 1) / 2 > e) --f;
+        while ((f + 1) * (f + 2) / 2 <= e) ++f;
+        const int g = e - f * (f + 1) / 2, cf = V.sel[f], cg = V.sel[g];
+        double s = 0.0;
+        for (int a = 0; a < m; ++a) s = fma(C[a * ld + cf], C[a * ld + cg], s);
+        if (f == g) s += kM5Ridge;
+        H[f * ld + g] = s;
+        H[g * ld + f] = s;
     }
     Gp::sync();
     m5_invert<WARP>(V, H, ld, ns);
@@ -504,9 +529,9 @@ __device__ void m5_solve(M5Smem& S, Vec& V, const double* G, double* H, int ld, 
 }
 
 // The model of internal node t on the attributes tested below it (the lowest kM5MaxTerms of them),
-// greedily simplified, and the pruning decision.  G, H: tmax x ld; C: m x ld.
+// greedily simplified, and the pruning decision.  H: tmax x ld; C, T32: m x ld.
 template <bool WARP, class Vec>
-__device__ __noinline__ void m5_model(M5Smem& S, Vec& V, M5Tree* T, int t, int F, double* G, double* H, double* C, int ld) {
+__device__ __noinline__ void m5_model(M5Smem& S, Vec& V, M5Tree* T, int t, int F, double* H, double* C, float* T32, int ld) {
     using Gp = M5Group<WARP>;
     const int tid = Gp::tid(), lane = threadIdx.x & 31;
     const int wp = WARP ? 0 : (int)(threadIdx.x >> 5), nw = WARP ? 1 : kM5Warps;
@@ -549,170 +574,165 @@ __device__ __noinline__ void m5_model(M5Smem& S, Vec& V, M5Tree* T, int t, int F
         }
     }
     Gp::sync();
-    for (int e = tid; e < nc * (nc + 1) / 2; e += Gp::kNT) {
-        int f = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
-        while (f * (f + 1) / 2 > e) --f;
-        while ((f + 1) * (f + 2) / 2 <= e) ++f;
-        const int g = e - f * (f + 1) / 2;
-        double s = 0.0;
-        for (int a = 0; a < m; ++a) s = fma(C[a * ld + f], C[a * ld + g], s);
-        if (f == g) s += kM5Ridge;
-        G[f * ld + g] = s;
-        G[g * ld + f] = s;
-    }
-    Gp::sync();
-    m5_solve<WARP>(S, V, G, H, ld, nc, lo, m, ybar);
-    // residuals (kept by row owners) and T = C H in C's place
-    double res[WARP ? 1 : kM5MaxN / kM5Warps];
+    m5_solve<WARP>(S, V, C, H, ld, nc, lo, m, ybar);
     unsigned long long alive = nc >= 64 ? ~0ull : (1ull << nc) - 1ull;
     int ns = nc;
     bool dropped = false;
     if (nc > 0 && m > nc) {                        // else no model with one attribute fewer has an estimate
-        if constexpr (WARP) {                      // lane = instance
-            double c[kM5WarpTerms];
-            res[0] = 0.0;
-            if (lane < m) {
-                double p = ybar;
-#pragma unroll
-                for (int i = 0; i < kM5WarpTerms; ++i) {
-                    c[i] = i < nc ? C[lane * ld + i] : 0.0;
-                    if (i < nc) p = fma(c[i], V.w[i], p);
-                }
-                res[0] = S.y[S.ids[lo + lane]] - p;
-                for (int k = 0; k < nc; ++k) {
-                    double s = 0.0;
-#pragma unroll
-                    for (int i = 0; i < kM5WarpTerms; ++i)
-                        if (i < nc) s = fma(c[i], H[i * ld + k], s);
-                    C[lane * ld + k] = s;
-                }
-            }
-        } else {                                   // a warp takes instances wp, wp + 8, ...
-#pragma unroll
-            for (int x = 0; x < kM5MaxN / kM5Warps; ++x) {
-                const int a = wp + kM5Warps * x;
-                res[x] = 0.0;
-                if (a >= m) continue;
-                double p = 0.0, s0 = 0.0, s1 = 0.0;
-                if (lane < nc) p = C[a * ld + lane] * V.w[lane];
-                if (lane + 32 < nc) p = fma(C[a * ld + lane + 32], V.w[lane + 32], p);
-                res[x] = S.y[S.ids[lo + a]] - (ybar + m5_warp_sum(p));
-                for (int i = 0; i < nc; ++i) {
-                    const double ci = C[a * ld + i];
-                    if (lane < nc) s0 = fma(ci, H[i * ld + lane], s0);
-                    if (lane + 32 < nc) s1 = fma(ci, H[i * ld + lane + 32], s1);
-                }
-                __syncwarp();
-                if (lane < nc) C[a * ld + lane] = s0;
-                if (lane + 32 < nc) C[a * ld + lane + 32] = s1;
-            }
+        // residuals (lane = instance, kept by the warp that owns its 32 instances) and T = C H in FP32
+        const int row = WARP ? lane : (int)threadIdx.x;
+        double res = 0.0;
+        if (row < m) {
+            double p = ybar;
+            for (int i = 0; i < nc; ++i) p = fma(C[row * ld + i], V.w[i], p);
+            res = S.y[S.ids[lo + row]] - p;
         }
+        for (int e = tid; e < m * nc; e += Gp::kNT) {
+            const int a = e / nc, k = e - a * nc;
+            double s = 0.0;
+            for (int i = 0; i < nc; ++i) s = fma(C[a * ld + i], H[i * ld + k], s);
+            T32[a * ld + k] = (float)s;
+        }
+        float* res32 = S.res32 + (WARP ? 32 * (int)(threadIdx.x >> 5) : 0);
+        if (row < m) res32[row] = (float)res;
         Gp::sync();
         for (;;) {
-            // w_d / H_dd, then sum_a |res_a + fac_d T_ad| of every attribute still there
-            for (int d = tid; d < nc; d += Gp::kNT)
+            // w_d / H_dd, then sum_a |res_a + fac_d T_ad| of every attribute still there, in FP32
+            // with the size of its terms
+            for (int d = tid; d < nc; d += Gp::kNT) {
                 V.fac[d] = (alive >> d) & 1ull ? V.w[d] * rcp_newton_any(H[d * ld + d]) : 0.0;
+                V.fac32[d] = (float)V.fac[d];
+            }
             Gp::sync();
-            double bd = DBL_MAX;
-            int drop = -1;
-            if constexpr (WARP) {                  // lane d and lane d + 16 share attribute d's instances
-                const int d = lane & 15, h = lane >> 4;
-                double s = 0.0;
-                for (int a = 0; a < m; ++a) {
-                    const double ra = __shfl_sync(0xffffffffu, res[0], a);
-                    if (d < nc && (a & 1) == h) s += fabs(fma(V.fac[d], C[a * ld + d], ra));
-                }
-                s += __shfl_xor_sync(0xffffffffu, s, 16);
-                if (d < nc && ((alive >> d) & 1ull) && s < DBL_MAX) {
-                    bd = s;
-                    drop = d;
-                }
-            } else {
-                double s0 = 0.0, s1 = 0.0;
-                const double f0 = lane < nc ? V.fac[lane] : 0.0, f1 = lane + 32 < nc ? V.fac[lane + 32] : 0.0;
+            if constexpr (!WARP) {                 // lanes = attributes, warps = instances
+                float s[2] = {0.f, 0.f}, z[2] = {0.f, 0.f};
+                for (int a = wp; a < m; a += nw) {
+                    const float ra = res32[a];
 #pragma unroll
-                for (int x = 0; x < kM5MaxN / kM5Warps; ++x) {
-                    const int a = wp + kM5Warps * x;
-                    if (a >= m) continue;
-                    if (lane < nc) s0 += fabs(fma(f0, C[a * ld + lane], res[x]));
-                    if (lane + 32 < nc) s1 += fabs(fma(f1, C[a * ld + lane + 32], res[x]));
-                }
-                S.errp[wp][lane] = s0;
-                S.errp[wp][lane + 32] = s1;
-                __syncthreads();
-                if (wp == 0)
-                    for (int d = lane; d < nc; d += 32) {
-                        double s = 0.0;
-#pragma unroll
-                        for (int w = 0; w < kM5Warps; ++w) s += S.errp[w][d];
-                        if (((alive >> d) & 1ull) && s < bd) {
-                            bd = s;
-                            drop = d;
+                    for (int h = 0; h < 2; ++h)
+                        if (lane + 32 * h < nc) {
+                            const float x = V.fac32[lane + 32 * h] * T32[a * ld + lane + 32 * h];
+                            s[h] += fabsf(ra + x);
+                            z[h] += fabsf(ra) + fabsf(x);
                         }
-                    }
+                }
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    S.errp[0][wp][lane + 32 * h] = s[h];
+                    S.errp[1][wp][lane + 32 * h] = z[h];
+                }
+                __syncthreads();
             }
             if (WARP || wp == 0) {
+                float lo32[2] = {0.f, 0.f}, best = __int_as_float(0x7f800000);
+                bool on[2];
 #pragma unroll
-                for (int o = 16; o >= 1; o >>= 1) {
-                    const double ob = __shfl_xor_sync(0xffffffffu, bd, o);
-                    const int od = __shfl_xor_sync(0xffffffffu, drop, o);
-                    if (od >= 0 && (drop < 0 || ob < bd || (ob == bd && od < drop))) {
-                        bd = ob;
-                        drop = od;
+                for (int h = 0; h < 2; ++h) {
+                    const int d = lane + 32 * h;
+                    on[h] = d < nc && ((alive >> d) & 1ull);
+                    if (WARP && h == 1) continue;
+                    float s = 0.f, z = 0.f;
+                    if (on[h]) {
+                        if constexpr (WARP) {
+                            for (int a = 0; a < m; ++a) {
+                                const float ra = res32[a], x = V.fac32[d] * T32[a * ld + d];
+                                s += fabsf(ra + x);
+                                z += fabsf(ra) + fabsf(x);
+                            }
+                        } else {
+#pragma unroll
+                            for (int w = 0; w < kM5Warps; ++w) {
+                                s += S.errp[0][w][d];
+                                z += S.errp[1][w][d];
+                            }
+                        }
+                        lo32[h] = s - 1e-4f * z;
+                        best = fminf(best, s + 1e-4f * z);
+                        on[h] = s < 1e30f;         // (not for an estimate that is not finite)
                     }
                 }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
+                const unsigned b0 = __ballot_sync(0xffffffffu, on[0] && lo32[0] <= best);
+                const unsigned b1 = __ballot_sync(0xffffffffu, on[1] && lo32[1] <= best);
                 if (tid == 0) {
-                    const int v = ns;              // terms + 1 of the smaller model
-                    const double e = m <= v ? DBL_MAX : bd / m * ((double)(m + v) / (double)(m - v));
-                    V.drop = drop >= 0 && e < DBL_MAX && e <= V.e_cur ? drop : -1;
-                    if (V.drop >= 0) V.e_cur = e;
+                    V.reach = (unsigned long long)b1 << 32 | b0;
+                    V.drop = -1;
                 }
             }
             Gp::sync();
-            const int d = V.drop;
-            if (d < 0) break;
+            // the drops that may be the best, in FP64 from C (nearly always one): the lowest error
+            // wins, ties to the lower attribute
+            double be = DBL_MAX, bres = 0.0;
+            int drop = -1;
+            for (unsigned long long rc = V.reach; rc; rc &= rc - 1) {
+                const int d = __ffsll((long long)rc) - 1;
+                const double fd = V.fac[d];
+                for (int i = tid; i < nc; i += Gp::kNT)
+                    V.wt[i] = i != d && ((alive >> i) & 1ull) ? fma(-H[i * ld + d], fd, V.w[i]) : 0.0;
+                Gp::sync();
+                double rn = 0.0;
+                if (row < m) {
+                    double p = ybar;
+                    for (int i = 0; i < nc; ++i) p = fma(C[row * ld + i], V.wt[i], p);
+                    rn = S.y[S.ids[lo + row]] - p;
+                }
+                double e;
+                if constexpr (WARP) {
+                    e = m5_warp_sum(fabs(rn));
+                } else {
+                    if (32 * wp < m) {
+                        const double x = m5_warp_sum(fabs(rn));
+                        if (lane == 0) S.sump[wp] = x;
+                    }
+                    __syncthreads();
+                    e = 0.0;
+                    for (int w = 0; 32 * w < m; ++w) e += S.sump[w];
+                }
+                if (e < be) {                      // (the same in every thread)
+                    be = e;
+                    drop = d;
+                    bres = rn;
+                }
+                Gp::sync();
+            }
+            // estimate with ns - 1 terms (v = ns)
+            const double est = drop < 0 ? DBL_MAX : be * S.rcp[m] * ((double)(m + ns) * rcp_newton((double)(m - ns)));
+            if (m <= ns || drop < 0 || !(est <= V.e_cur)) break;
+            Gp::sync();                            // (every thread has compared with e_cur)
+            const int d = drop;
             dropped = true;
             --ns;
             alive &= ~(1ull << d);
+            if (tid == 0) V.e_cur = est;
             if (ns == 0) break;
-            // take d out: H -= H_d H_d^T / H_dd, w -= H_d fac_d, T -= T_d H_d^T / H_dd, res += fac_d T_d
+            // take d out: w and the residuals as just computed, H -= H_d H_d^T / H_dd, T -= T_d H_d^T / H_dd
             const double fd = V.fac[d], hi = rcp_newton_any(H[d * ld + d]);
             for (int i = tid; i < nc; i += Gp::kNT) {
                 V.colk[i] = H[i * ld + d];
                 V.rowk[i] = H[i * ld + d] * hi;
-                if (i != d) V.w[i] = fma(-H[i * ld + d], fd, V.w[i]);
+                V.rowk32[i] = (float)V.rowk[i];
+                V.w[i] = i != d && ((alive >> i) & 1ull) ? fma(-H[i * ld + d], fd, V.w[i]) : 0.0;
             }
+            res = bres;
+            if (row < m) res32[row] = (float)res;
             Gp::sync();
             for (int e = tid; e < nc * nc; e += Gp::kNT) {
                 const int i = e / nc, j = e - i * nc;
                 if (i != d && j != d) H[i * ld + j] = fma(-V.colk[i], V.rowk[j], H[i * ld + j]);
             }
-            if constexpr (WARP) {
-                if (lane < m) {
-                    const double td = C[lane * ld + d];
-                    res[0] = fma(fd, td, res[0]);
-                    for (int k = 0; k < nc; ++k)
-                        if (k != d) C[lane * ld + k] = fma(-td, V.rowk[k], C[lane * ld + k]);
-                }
-            } else {
-#pragma unroll
-                for (int x = 0; x < kM5MaxN / kM5Warps; ++x) {
-                    const int a = wp + kM5Warps * x;
-                    if (a >= m) continue;
-                    const double td = C[a * ld + d];
-                    res[x] = fma(fd, td, res[x]);
-                    if (lane < nc && lane != d) C[a * ld + lane] = fma(-td, V.rowk[lane], C[a * ld + lane]);
-                    if (lane + 32 < nc && lane + 32 != d)
-                        C[a * ld + lane + 32] = fma(-td, V.rowk[lane + 32], C[a * ld + lane + 32]);
-                }
+            for (int e = tid; e < m * nc; e += Gp::kNT) {
+                const int a = e / nc, k = e - a * nc;
+                if (k != d) T32[a * ld + k] = fmaf(-T32[a * ld + d], V.rowk32[k], T32[a * ld + k]);
             }
             Gp::sync();
         }
+        Gp::sync();
     }
     if (dropped) {                                 // the model that stays, from its own normal equations
         if (tid < nc && ((alive >> tid) & 1ull)) V.sel[__popcll(alive & ((1ull << tid) - 1ull))] = (uint8_t)tid;
         Gp::sync();
-        m5_solve<WARP>(S, V, G, H, ld, ns, lo, m, ybar);
+        m5_solve<WARP>(S, V, C, H, ld, ns, lo, m, ybar);
     }
     // the node's model and the pruning decision
     for (int k = tid; k < ns; k += Gp::kNT) {
@@ -744,7 +764,7 @@ __host__ __device__ __forceinline__ size_t m5_dyn_bytes(int F) {
     const int nmax = kM5MaxN;
     const size_t grow = 2 * (size_t)F * nmax;
     const int tm = F < kM5MaxTerms ? F : kM5MaxTerms, ld = tm | 1;
-    const size_t blk = ((size_t)2 * tm * ld + (size_t)nmax * ld) * sizeof(double);
+    const size_t blk = ((size_t)tm * ld + (size_t)nmax * ld) * sizeof(double) + (size_t)nmax * ld * sizeof(float);
     const size_t wrp = (size_t)kM5Warps * kM5WarpBuf * sizeof(double);
     const size_t mo = blk > wrp ? blk : wrp;
     return grow > mo ? grow : mo;
@@ -781,6 +801,7 @@ m5p_fit_kernel(const TransferArgs a, int fmax) {
     }
     uint8_t* srt = dyn;                                           // [F][nmax]
     uint8_t* rk = dyn + (size_t)fmax * nmax;                      // [F][nmax]
+    for (int c = tid; c <= kM5MaxN; c += kM5Threads) S.rcp[c] = __drcp_rn((double)(c ? c : 1));
     for (int i = tid; i < n; i += kM5Threads) {
         const int u = pu[i];
         int r = 0;
@@ -826,7 +847,7 @@ m5p_fit_kernel(const TransferArgs a, int fmax) {
         double s = 0.0;
         for (int i = 0; i < n; ++i) s = __dadd_rn(s, lane == 1 ? S.y2[i] : S.y[i]);
         const double s1 = __shfl_sync(0xffffffffu, s, 0), s2 = __shfl_sync(0xffffffffu, s, 1);
-        const double sd = m5_sd(n, s1, s2);
+        const double sd = m5_sd(n, __drcp_rn((double)n), s1, s2);
         if (lane == 0) {
             S.sd_root = sd;
             S.nn = 1;
@@ -890,7 +911,7 @@ m5p_fit_kernel(const TransferArgs a, int fmax) {
                 }
                 const double s1 = __shfl_sync(0xffffffffu, xs, 0), s2 = __shfl_sync(0xffffffffu, xs, 1);
                 if (!fp32 || sda <= lim + slack) {
-                    if (m5_sd(m, s1, s2) <= __dmul_rn(kM5SdFrac, S.sd_root)) cnt = -1;
+                    if (m5_sd(m, S.rcp[m], s1, s2) <= __dmul_rn(kM5SdFrac, S.sd_root)) cnt = -1;
                     else if (!fp32) cnt = -2;
                 }
                 if (lane == 0) {
@@ -912,29 +933,38 @@ m5p_fit_kernel(const TransferArgs a, int fmax) {
             }
         }
         __syncthreads();
-        // the attributes' scans of every splitting node, dealt to the warps: the best upper bound
-        for (int x = warp; x < nl * F; x += kM5Warps) {
-            const int k = x / F, f = x - k * F;
+        // the attributes' scans of every splitting node, dealt to the warps; a warp takes several
+        // attributes of a node that has few instances
+        int x0 = 0;
+        for (int k = 0; k < nl; ++k) {
             if (S.cnt[k] < 0) continue;
-            m5_scan<false>(S, srt + f * nmax, rk + f * nmax, f, S.lo[n0 + k], S.hi[n0 + k] - S.lo[n0 + k], k);
-        }
-        __syncthreads();
-        for (int x = warp; x < nl * F; x += kM5Warps) {
-            const int k = x / F, f = x - k * F;
-            if (S.cnt[k] < 0 || S.best_hi[k] == 0x7f800000u) continue;
-            m5_scan<true>(S, srt + f * nmax, rk + f * nmax, f, S.lo[n0 + k], S.hi[n0 + k] - S.lo[n0 + k], k);
+            const int lo = S.lo[n0 + k], m = S.hi[n0 + k] - lo;
+            const int W = m <= 8 ? 8 : m <= 16 ? 16 : 32, per = 32 / W, nt = (F + per - 1) / per;
+            for (int x = (warp - x0) & (kM5Warps - 1); x < nt; x += kM5Warps) {
+                const int f = x * per + lane / W;
+                m5_scan(S, srt + (f < F ? f : 0) * nmax, rk + (f < F ? f : 0) * nmax, f < F ? f : -1, lo, m, k, W);
+            }
+            x0 = (x0 + nt) & (kM5Warps - 1);       // the next node's first task to the next warp
         }
         __syncthreads();
         const bool over = S.nsurv > kM5Surv;       // then every node of the level by the exact scan
+        // of those listed early, the ones that still reach the final bound; how many a node has
+        for (int x = tid; x < (over ? 0 : S.nsurv); x += kM5Threads) {
+            const unsigned k = S.surv[x] >> 16;
+            if (S.ql[x] <= __uint_as_float(S.best_hi[k])) atomicAdd(&S.cnt[k], 1);
+            else S.surv[x] = 0xffffffffu;
+        }
+        __syncthreads();
         const int nsv = over ? 0 : S.nsurv;
         // exact SDRs of the survivors, two threads each (left and right); a node's only survivor
         // whose SDR is positive beyond doubt needs none
         for (int x = tid >> 1; x < ((nsv + kM5Threads / 2 - 1) & ~(kM5Threads / 2 - 1)); x += kM5Threads / 2) {
-            const unsigned sv = x < nsv ? S.surv[x] : 0u;
+            const unsigned sv = x < nsv && S.surv[x] != 0xffffffffu ? S.surv[x] : 0u;
+            const bool here = x < nsv && S.surv[x] != 0xffffffffu;
             const int k = (int)(sv >> 16), f = (int)(sv >> 8) & 0xff, c = (int)(sv & 0xff);
             const int t = n0 + k, lo = S.lo[t], m = S.hi[t] - lo;
-            const bool sure = x < nsv && S.cnt[k] == 1 && __uint_as_float(S.best_hi[k]) < 0.999f * (float)m * S.sda[k] - 1e-5f * (float)m * sqrtf(S.amax2[k]);
-            const bool work = x < nsv && !sure;
+            const bool sure = here && S.cnt[k] == 1 && __uint_as_float(S.best_hi[k]) < 0.999f * (float)m * S.sda[k] - 1e-5f * (float)m * sqrtf(S.amax2[k]);
+            const bool work = here && !sure;
             double sdx = 0.0;
             if (work) {
                 const uint8_t* o = srt + f * nmax + lo;
@@ -948,12 +978,13 @@ m5p_fit_kernel(const TransferArgs a, int fmax) {
                     l2 = __dsub_rn(S.s2[k], l2);
                 }
                 const int cc = (tid & 1) ? m - c : c;
-                sdx = __dmul_rn((double)cc, m5_sd(cc, l1, l2));
+                sdx = __dmul_rn((double)cc, m5_sd(cc, S.rcp[cc], l1, l2));
             }
             const double other = __shfl_xor_sync(0xffffffffu, sdx, 1);
-            if (x < nsv && !(tid & 1)) {
+            if (here && !(tid & 1)) {
                 double red = 1.0;
-                if (work) red = __dsub_rn(m5_sd(m, S.s1[k], S.s2[k]), __ddiv_rn(__dadd_rn(sdx, other), (double)m));
+                if (work)
+                    red = __dsub_rn(m5_sd(m, S.rcp[m], S.s1[k], S.s2[k]), m5_div(__dadd_rn(sdx, other), (double)m, S.rcp[m]));
                 S.red[x] = red;
                 if (red > 0.0) atomicMax(&S.best_red[k], (unsigned long long)__double_as_longlong(red));
             }
@@ -963,7 +994,7 @@ m5p_fit_kernel(const TransferArgs a, int fmax) {
             const int c = S.cnt[k];
             if (c != -2 && !(over && c >= 0)) continue;      // (uniform)
             const int t = n0 + k, lo = S.lo[t], m = S.hi[t] - lo;
-            const double sd = m5_sd(m, S.s1[k], S.s2[k]);
+            const double sd = m5_sd(m, S.rcp[m], S.s1[k], S.s2[k]);
             double best = 0.0;
             unsigned key = 0xffffffffu;
             for (int f = tid; f < F; f += kM5Threads)
@@ -976,6 +1007,7 @@ m5p_fit_kernel(const TransferArgs a, int fmax) {
         __syncthreads();
         // ties: the lowest attribute, then the lowest count
         for (int x = tid; x < nsv; x += kM5Threads) {
+            if (S.surv[x] == 0xffffffffu) continue;
             const int k = (int)(S.surv[x] >> 16);
             const double red = S.red[x];
             if (red > 0.0 && (unsigned long long)__double_as_longlong(red) == S.best_red[k])
@@ -1094,11 +1126,12 @@ m5p_fit_kernel(const TransferArgs a, int fmax) {
             if (S.cnt[t - n0] == 1 && (turn++ & (kM5Warps - 1)) == warp) {
                 double* wb = buf + warp * kM5WarpBuf;
                 m5_model<true>(S, S.v.wv[warp], T, t, F, wb, wb + kM5WarpTerms * kM5WarpLd,
-                               wb + 2 * kM5WarpTerms * kM5WarpLd, kM5WarpLd);
+                               reinterpret_cast<float*>(wb + (kM5WarpTerms + kM5WarpN) * kM5WarpLd), kM5WarpLd);
             }
         __syncthreads();
         for (int t = n0; t < n1; ++t)
-            if (S.cnt[t - n0] == 2) m5_model<false>(S, S.v.blk, T, t, F, buf, buf + tm * ld, buf + 2 * tm * ld, ld);
+            if (S.cnt[t - n0] == 2) m5_model<false>(S, S.v.blk, T, t, F, buf, buf + tm * ld,
+                                                            reinterpret_cast<float*>(buf + (tm + nmax) * ld), ld);
         __syncthreads();
     }
     for (int t = tid; t < nn; t += kM5Threads) {

@@ -157,3 +157,35 @@ def test_bad_group_is_reported_not_written(rs, ctx):
     assert (c[64:] == 0x7777).all() and (c[:64] != 0x7777).all()
     ref = oracle.transfer(train, synth.take_programs(b1, [1]), model="ibk")
     np.testing.assert_array_equal(c[:64].view(np.uint32), ref.rec_code)
+
+
+@pytest.mark.parametrize("feat,runs_per,versions,case", [
+    (1, 1, (3, 20), "plain"), (3, 2, (2, 64), "plain"), (17, 3, (10, 40), "ties"), (65, 1, (64, 64), "plain"),
+    (100, 4, (60, 64), "plain"), (256, 2, (50, 64), "plain"), (40, 2, (30, 64), "equal"), (24, 3, (64, 64), "labels"),
+    (70, 3, (64, 64), "many")])
+def test_m5p_at_its_edges(rs, ctx, feat, runs_per, versions, case):
+    """Trees of one to 128 instances, one to 256 attributes (more than a model takes terms), with equal
+    attribute values and equal labels (ties between splits and between dropped terms are decided by
+    the reference's own roundings), infinite labels, and labels that many attributes explain."""
+    b = synth.make_batch(4 * runs_per + 4, versions=versions, feat=feat, dtype=np.float64, seed=500 + feat)
+    rng = np.random.default_rng(feat)
+    if case == "ties":            # counters of few distinct values; whole columns constant or repeated
+        for p in range(b.n_programs):
+            X = b.program_X(p)
+            X[:] = np.exp(np.round(np.log(X / b.cycles[b.program_rows(p)][:, None])) * 0.5)
+            X[:, 3] = X[:, 5]
+            X[:, 7] = 2.0
+        b.cycles = np.ones_like(b.cycles)
+    if case == "equal":           # labels of two values only
+        b.log_time = np.round(b.log_time)
+    if case == "labels":
+        b.log_time[int(b.row_offsets[1]) + 5] = np.inf
+    if case == "many":            # every label a sum of many attributes' logs
+        for p in range(b.n_programs):
+            X = np.log(b.program_X(p) / b.cycles[b.program_rows(p)][:, None])
+            b.log_time[b.program_rows(p)] = X @ rng.standard_normal(feat) / feat
+    groups = np.arange(5, dtype=np.int64) * runs_per
+    train = synth.take_programs(b, list(range(4 * runs_per)))
+    test = synth.take_programs(b, list(range(4 * runs_per, 4 * runs_per + 4)))
+    g, r = _both(rs, ctx, train, test, groups, "m5p", flags=oracle.RANK_ALL)
+    _check(g, r, "m5p")
