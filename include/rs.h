@@ -450,8 +450,8 @@ rs_status rs_gemm_bf16(rs_ctx* ctx, const void* A, int64_t lda, const void* B, i
  * masks == NULL; threshold log(tau) compared in FP32; ties to the lower index; top k):
  * rec_code [n] and rec_pred [n][k] (double, nullable) in the rs_predict_rank format.
  * workspace: rs_surrogate_workspace_bytes(batch_rows) bytes, 256-byte aligned; inference
- * processes chunk_rows rows at a time (chunk_rows <= the batch_rows the workspace was
- * sized for).  RS_ETIMEOUT in the device status if a tensor-core pipeline wait gave up. */
+ * checks that chunk_rows <= the batch_rows the workspace was sized for, but keeps its
+ * activations on the chip and writes nothing there.  RS_ETIMEOUT in the device status if a tensor-core pipeline wait gave up. */
 typedef struct {
     int32_t batch_rows;
     int32_t use_graph;

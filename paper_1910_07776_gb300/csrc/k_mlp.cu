@@ -114,7 +114,7 @@ struct EpiOutput {           // out = acc + b3; training: residual, loss, dO, dO
     float log_tau;
     uint32_t* rec_code;      // [B]
     double* rec_pred;        // [B][k]
-    __device__ void rank_row(int row, const float (&o)[16]) const {
+    __device__ void rank_row(int64_t row, const float (&o)[16]) const {
         const int cand = (flags & RS_RANK_ALL) || !masks ? 63 : (~masks[row] & 63);
         int above = 0, bm[kOut];
 #pragma unroll
@@ -151,7 +151,7 @@ struct EpiOutput {           // out = acc + b3; training: residual, loss, dO, dO
             for (int x = 0; x < kOut; ++x)
                 if (x < k) rec_pred[(int64_t)row * k + x] = rp[x];
     }
-    __device__ void operator()(int row, int col0, const float (&v)[16]) const {
+    __device__ void operator()(int64_t row, int col0, const float (&v)[16]) const {
         if (col0 != 0) return;
         if (rec_code) {
             float o[16];
@@ -295,81 +295,7 @@ stage_kernel(const double* __restrict__ X, const double* __restrict__ Yin, int64
     }
 }
 
-// double -> BF16 and double -> float with integer operations only (this part's double
-// conversions run on its narrow FP64 pipe).  BF16: round to nearest, ties to even, on the 52
-// fraction bits; float: truncated fraction (used for the OOD score).  Values outside the
-// normal float range take the conversion instructions.
-__device__ __forceinline__ bool f32_normal_range(long long b) {
-    const int e = (int)((b >> 52) & 0x7ff);
-    return e > 1023 - 126 && e < 1023 + 127;
-}
-__device__ __forceinline__ __nv_bfloat16 bf16_of(double x) {
-    const long long b = __double_as_longlong(x);
-    if (!f32_normal_range(b)) return __float2bfloat16((float)x);
-    const unsigned long long u = (unsigned long long)b;
-    // keep 7 fraction bits: round on bit 45, ties to even on bit 45 of the kept part
-    const unsigned long long r = u + ((1ull << 44) - 1ull) + ((u >> 45) & 1ull);
-    const unsigned long long m = (r >> 45) & 0x7full;                // 7 fraction bits
-    const int e = (int)((r >> 52) & 0x7ff) - 1023 + 127;             // carry may bump the exponent
-    const unsigned short h = (unsigned short)(((u >> 63) << 15) | ((unsigned)e << 7) | (unsigned)m);
-    return __ushort_as_bfloat16(h);
-}
-__device__ __forceinline__ float f32_trunc_of(double x) {
-    const long long b = __double_as_longlong(x);
-    if (!f32_normal_range(b)) return (float)x;
-    const unsigned long long u = (unsigned long long)b;
-    const unsigned e = (unsigned)((u >> 52) & 0x7ff) - 1023u + 127u;
-    return __uint_as_float((unsigned)((u >> 63) << 31) | (e << 23) | (unsigned)((u >> 29) & 0x7fffff));
-}
-
-// Inference staging: rows of X (double [n][256]) -> BF16 X_s, one warp per row (lane l takes
-// features 8l .. 8l+7: 64 contiguous bytes in, 16 out), grid-stride over the chunk; with the
-// training statistics given, the same pass forms the out-of-distribution score (mean over
-// features of ((x - mean) / sd)^2, FP32) and the fallback flag of each row.
-__global__ void __launch_bounds__(256)
-infer_stage_kernel(const double* __restrict__ X, int64_t B, __nv_bfloat16* Xs, const float* __restrict__ mean,
-                   const float* __restrict__ sd, float thr, float* score, uint8_t* fallback) {
-    const int lane = threadIdx.x & 31;
-    const int64_t wstride = (int64_t)gridDim.x * (blockDim.x >> 5);
-    float mu[8], sinv[8];                    // per feature: mean and 1 / sd (0 where sd = 0)
-    if (mean) {
-#pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            mu[e] = mean[8 * lane + e];
-            const float d = sd[8 * lane + e];
-            sinv[e] = d > 0.f ? 1.0f / d : 0.f;
-        }
-    }
-    for (int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; r < B; r += wstride) {
-        const double2* src = reinterpret_cast<const double2*>(X + r * kIn + 8 * lane);
-        double x[8];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            const double2 v = __ldcs(src + e);       // read once: streaming
-            x[2 * e] = v.x;
-            x[2 * e + 1] = v.y;
-        }
-        alignas(16) __nv_bfloat16 hb[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e) hb[e] = bf16_of(x[e]);
-        *reinterpret_cast<uint4*>(Xs + r * kIn + 8 * lane) = *reinterpret_cast<const uint4*>(hb);
-        if (mean) {
-            float s = 0.f;
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const float d = (f32_trunc_of(x[e]) - mu[e]) * sinv[e];
-                s = fmaf(d, d, s);
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) {
-                s /= kIn;
-                if (score) score[r] = s;
-                if (fallback) fallback[r] = s > thr ? 1 : 0;
-            }
-        }
-    }
-}
+#include "k_mlp_infer.cuh"
 
 // Row sums of a transposed gradient [rows][B] (BF16) -> FP32 bias gradient; one warp per row.
 __global__ void __launch_bounds__(256)
@@ -724,37 +650,32 @@ cudaError_t rs_launch_surrogate_infer(const float* blob, const double* X, int64_
                                       int k, double tau, int flags, uint32_t* rec_code, double* rec_pred,
                                       void* ws, int64_t chunk, int* err, cudaStream_t st) {
     const __nv_bfloat16* bf = reinterpret_cast<const __nv_bfloat16*>(blob + Blob::oBf);
-    char* c = (char*)ws;
-    __nv_bfloat16* Xs = (__nv_bfloat16*)c;
-    __nv_bfloat16* H1 = (__nv_bfloat16*)(c + a256((size_t)chunk * kIn * 2));
-    __nv_bfloat16* H2 = (__nv_bfloat16*)(c + a256((size_t)chunk * kIn * 2) + a256((size_t)chunk * kHid * 2));
-    cudaError_t e = cudaSuccess;
-    for (int64_t r0 = 0; r0 < n && e == cudaSuccess; r0 += chunk) {
-        const int B = (int)((n - r0) < chunk ? (n - r0) : chunk);
-        CUtensorMap tX, tW1, tH1, tW2, tH2, tW3;
-        e = rs_make_tmap_bf16(&tX, Xs, B, kIn, kIn, 128);
-        if (e == cudaSuccess) e = rs_make_tmap_bf16(&tW1, bf + Blob::bW1, kHid, kIn, kIn, 128);
-        if (e == cudaSuccess) e = rs_make_tmap_bf16(&tH1, H1, B, kHid, kHid, 128);
-        if (e == cudaSuccess) e = rs_make_tmap_bf16(&tW2, bf + Blob::bW2, kHid, kHid, kHid, 128);
-        if (e == cudaSuccess) e = rs_make_tmap_bf16(&tH2, H2, B, kHid, kHid, 128);
-        if (e == cudaSuccess) e = rs_make_tmap_bf16(&tW3, bf + Blob::bW3, kOutP, kHid, kHid, 32);
-        if (e != cudaSuccess) break;
-        const bool ood = score || fallback;
-        const int sblocks = (int)((B + 7) / 8) < 4096 ? (int)((B + 7) / 8) : 4096;
-        infer_stage_kernel<<<sblocks, 256, 0, st>>>(X + r0 * kIn, B, Xs, ood ? blob + Blob::oStats : nullptr,
-                                                     blob + Blob::oStats + kIn, ood_thr,
-                                                     score ? score + r0 : nullptr,
-                                                     fallback ? fallback + r0 : nullptr);
-        e = gemm<128>(tX, tW1, B, kHid, kIn, EpiHidden{blob + Blob::ob1, nullptr, H1, nullptr, B}, err, st);
-        if (e == cudaSuccess)
-            e = gemm<128>(tH1, tW2, B, kHid, kHid, EpiHidden{blob + Blob::ob2, nullptr, H2, nullptr, B}, err, st);
-        if (e == cudaSuccess)
-            e = gemm<32>(tH2, tW3, B, kOutP, kHid,
-                         EpiOutput{blob + Blob::ob3, nullptr, nullptr, nullptr, nullptr, B, 0.f,
-                                   pred ? pred + r0 * kOut : nullptr, masks ? masks + r0 : nullptr, flags, k,
-                                   (float)log(tau), rec_code ? rec_code + r0 : nullptr,
-                                   rec_pred ? rec_pred + r0 * k : nullptr},
-                         err, st);
-    }
-    return e;
+    (void)ws;                     // the activations stay on the chip: neither the workspace nor its
+    (void)chunk;                  // chunks are needed
+    CUtensorMap tW1, tW2, tW3;
+    cudaError_t e = rs_make_tmap_bf16(&tW1, bf + Blob::bW1, kHid, kIn, kIn, 64);
+    if (e == cudaSuccess) e = rs_make_tmap_bf16(&tW2, bf + Blob::bW2, kHid, kHid, kHid, 64);
+    if (e == cudaSuccess) e = rs_make_tmap_bf16(&tW3, bf + Blob::bW3, kOutP, kHid, kHid, kOutP);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(mlp_infer_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kInfSmem);
+    int dev = 0, sms = 0;
+    if (e == cudaSuccess) e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    InferArgs a{};
+    a.X = X;
+    a.n = n;
+    a.b1 = blob + Blob::ob1;
+    a.b2 = blob + Blob::ob2;
+    a.mean = score || fallback ? blob + Blob::oStats : nullptr;
+    a.sd = blob + Blob::oStats + kIn;
+    a.thr = ood_thr;
+    a.score = score;
+    a.fallback = fallback;
+    a.out = EpiOutput{blob + Blob::ob3, nullptr, nullptr, nullptr, nullptr, 0, 0.f, pred, masks, flags, k,
+                      (float)log(tau), rec_code, rec_pred};
+    a.err = err;
+    const int64_t tiles = (n + 127) / 128;
+    mlp_infer_kernel<<<(unsigned)(tiles < sms ? tiles : sms), kInfThreads, kInfSmem, st>>>(tW1, tW2, tW3, a);
+    return cudaGetLastError();
 }

@@ -195,3 +195,57 @@ def test_checkpoint_resume_continues_the_run(env, tmp_path):
         with pytest.raises(rs.RsError) as e:
             c.restore(str(f))
         assert e.value.status == rs.RS_EINVAL
+
+
+@pytest.mark.parametrize("n", [1, 127, 128, 129, 152 * 128 + 1, 3 * 152 * 128 + 77])
+def test_inference_at_the_edges_of_its_tiles(env, n):
+    # Every row's outputs depend on that row alone: the same bits wherever it stands, beside rows of
+    # zeros, subnormals, infinities and NaN too; and they match the reference.
+    rs, ctx = env
+    rng = np.random.default_rng(n)
+    X = rng.normal(size=(n, 256)) * rng.choice([1e-3, 1.0, 30.0], size=(n, 1))
+    odd = {}
+    if n >= 127:
+        for i, v in enumerate([0.0, -0.0, 1e-310, 1e-40, -3e-39, 1e30]):
+            odd[7 * i] = v
+            X[7 * i, :] = v
+        X[50, 3], X[51, 200], X[126, 0] = np.inf, np.nan, 1e300
+    p = mlp.init_params(n % 97)
+    p["b1"] = rng.normal(size=512)
+    p["b2"] = rng.normal(size=512)
+    T = rng.normal(size=(256, 256)) + 0.5
+    sur = rs.Surrogate(ctx, 256)
+    sur.load(p)
+    sur.train(torch.from_numpy(T).cuda(), torch.zeros(256, 6, dtype=torch.float64, device="cuda"), steps=0)
+
+    def run(A, want=True):
+        d = torch.from_numpy(np.ascontiguousarray(A)).cuda()
+        m = len(A)
+        masks = torch.from_numpy((np.abs(np.nan_to_num(A[:, 9])) * 7).astype(np.int64).astype(np.uint8) & 63).cuda()
+        code = torch.zeros(m, dtype=torch.int32, device="cuda")
+        rp = torch.zeros(m * 2, dtype=torch.float64, device="cuda")
+        pred, score, fb = sur.infer(d, ood_threshold=2.0, want_ood=want, masks=masks, k=2, rec_code=code, rec_pred=rp)
+        torch.cuda.synchronize()
+        ctx.check_device_status()
+        out = [pred.cpu().numpy().view(np.uint32), code.cpu().numpy(), rp.cpu().numpy().view(np.uint64).reshape(m, 2)]
+        return out + ([score.cpu().numpy(), fb.cpu().numpy()] if want else [])
+
+    got = run(X)
+    pred, score = got[0].view(np.float32), got[3]
+    for a, b in zip(got, run(X, want=False)):                    # without the score: the same
+        np.testing.assert_array_equal(a, b)
+    order = rng.permutation(n)
+    for a, b in zip(got, run(X[order])):                         # in another order: the same
+        np.testing.assert_array_equal(a[order].view(np.uint8), b.view(np.uint8))
+    fine = np.isfinite(X).all(1) & (np.abs(X).max(1) < 1e25)
+    out, _ = mlp.forward(ref_params(p), bf16(X[fine].astype(np.float32)))
+    assert np.abs(pred[fine] - out).max() < 2e-2 * np.abs(out).max()
+    np.testing.assert_array_equal(got[4], (score > 2.0).astype(np.uint8))
+    # score: x truncated to 24 bits, (x - mean) / sd in FP32 (four roundings, mean and sd included), the
+    # sum over 256 squares in chains of 8 and 5 levels
+    mean, sd = T.mean(0), T.std(0)
+    d = (X[fine] - mean) / sd
+    ref = (d * d).mean(1)
+    eps = 2.0 ** -23
+    tol = (2 * np.abs(d) * (2 * np.abs(X[fine]) + 2 * np.abs(mean)) / sd).mean(1) * eps + (2 * 4 + 14) * eps * ref
+    assert (np.abs(score[fine] - ref) <= tol).all()
