@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(kSplThreads + 32, 1) gram_split_kernel(const S
     longlong2* xch = reinterpret_cast<longlong2*>(g + 2 * kStageBytes);
     // barriers: stage written [2] (8 warps), its products complete [2], accumulators read (8 warps)
     const uint32_t full = base + 2 * kStageBytes + 2 * kXchBytes, done = full + 16, drained = full + 32;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     if (tid == 0) {
         for (int i = 0; i < 2; ++i) {
             tc::mbar_init(full + 8 * i, 8);
@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(kSplThreads + 32, 1) gram_split_kernel(const S
     if (warp == 8) {                                       // ---- the products
         // f16 x f16 -> FP32, both operands K-major, 128 x 128
         constexpr uint32_t idesc = (1u << 4) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
-        if (lane == 0) {
+        if (tc::elect_one()) {
             int chunk = 0;
             for (; alive; ++it) {
                 const int buf = it & 1;

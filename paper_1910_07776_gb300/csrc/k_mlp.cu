@@ -4,15 +4,17 @@
 // FP32 accumulation; FP32 master weights with AdamW.
 //
 // One training step (a fixed sequence, captured once in a CUDA graph and replayed):
-//   stage    rows of X (double) -> BF16 X_s [B][256] and its transpose; labels -> Y_s
-//   fwd 1,2  U = X W^T + b (FP32 kept for the backward pass), H = gelu(U) (BF16) and H^T
-//   fwd 3    out = H2 W3^T + b3; residual; loss; dO = 2 (out - y) / (6B) (BF16) and dO^T
-//   dgrad    dU2 = (dO W3) * gelu'(U2);  dU1 = (dU2 W2) * gelu'(U1)   (BF16, and transposes)
-//   wgrad    dW3 = dO^T H2, dW2 = dU2^T H1, dW1 = dU1^T X_s             (FP32)
-//   bias     db = row sums of the transposed gradients
-//   adamw    master weights, moments, BF16 copies W and W^T for the next step
-// Every GEMM is D = A B^T with K-contiguous operands, so the epilogues also write the
-// transposed activations that the weight-gradient GEMMs read.
+//   stage    rows of X (double) -> BF16 X_s [B][256]; labels -> Y_s
+//   fwd 1,2  U = X W^T + b (FP32, kept for the backward pass), H = gelu(U) (BF16)
+//   fwd 3    out = H2 W3^T + b3; residual; loss; dO = 2 (out - y) / (6B) (BF16)
+//   dgrad    dU2 = (dO W3) * gelu'(U2);  dU1 = (dU2 W2) * gelu'(U1)   (BF16)
+//   wgrad    dW3 = dO^T H2, dW2 = dU2^T H1, dW1 = dU1^T X_s  (FP32 partials over row ranges, one launch)
+//   update   gradients (partials added and bias columns summed in a fixed order), AdamW, BF16 weights
+// The tensor cores take an operand with either its K or its rows contiguous, so the weight gradients
+// read the activations, and the data gradients the weights, as they lie: nothing is transposed.
+// A step of 8,192 rows: 175 -> 75 us (before: 16 launches, with transposed copies of every operand
+// written 2 bytes at a time, the sums over rows in three kernels of 11 us each, one atomic addition to
+// the loss a row).
 #include <math.h>
 #include <string.h>
 
@@ -34,7 +36,8 @@ struct Blob {
     // master | m | v | grad  (FP32), then BF16 copies, then feature stats, then counters
     static constexpr int64_t oM = nP, oV = 2 * nP, oG = 3 * nP;
     static constexpr int64_t oBf = 4 * nP;                                 // in floats
-    // BF16 region (in bf16 elements from oBf*2 bytes): W1, W2, W3p, W2t, W3t
+    // BF16 region (in bf16 elements from oBf*2 bytes): W1, W2, W3p; the rest is kept so that saved blobs
+    // stay readable (it held transposes of W2 and W3)
     static constexpr int64_t bW1 = 0, bW2 = bW1 + nW1, bW3 = bW2 + nW2, bW2t = bW3 + nW3,
                              bW3t = bW2t + nW2, bEnd = bW3t + (int64_t)kHid * kOutP;
     static constexpr int64_t oStats = oBf + (bEnd + 1) / 2 + 64;           // mean[256], std[256]
@@ -53,10 +56,6 @@ __device__ __forceinline__ float tanh_hw(float x) {
     asm("tanh.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-__device__ __forceinline__ float gelu_f(float u) {
-    const float t = tanh_hw(kGeluC * fmaf(kGeluA * u * u, u, u));
-    return 0.5f * u * (1.0f + t);
-}
 // d/du: (1 + t) / 2 + u (1 - t^2) c (1 + 3 a u^2) / 2
 __device__ __forceinline__ float gelu_grad_f(float u) {
     const float u2 = u * u;
@@ -65,54 +64,82 @@ __device__ __forceinline__ float gelu_grad_f(float u) {
 }
 
 // ---- epilogues ---------------------------------------------------------------------------------
-struct EpiHidden {           // U = acc + b (FP32, optional); H = gelu(U) (BF16); H^T (BF16, optional)
+// Two FP32 operations in one instruction, each rounded as by itself.
+__device__ __forceinline__ unsigned long long pk2(float a, float b) {
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void un2(unsigned long long v, float& a, float& b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+// gelu of two values as a BF16 pair.
+__device__ __forceinline__ unsigned gelu2(unsigned long long u) {
+    const unsigned long long x = mul2(pk2(kGeluC, kGeluC), fma2(mul2(mul2(pk2(kGeluA, kGeluA), u), u), u, u));
+    float x0, x1, y0, y1;
+    un2(x, x0, x1);
+    const unsigned long long y = mul2(mul2(pk2(0.5f, 0.5f), u), add2(pk2(1.0f, 1.0f), pk2(tanh_hw(x0), tanh_hw(x1))));
+    un2(y, y0, y1);
+    const __nv_bfloat162 h = __floats2bfloat162_rn(y0, y1);
+    return *reinterpret_cast<const unsigned*>(&h);
+}
+// 32 bytes in one store: a whole sector of L2 (16-byte halves of it cost a tag each).
+__device__ __forceinline__ void st32(void* p, const unsigned (&h)[8]) {
+    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+                 ::"l"(p), "r"(h[0]), "r"(h[1]), "r"(h[2]), "r"(h[3]), "r"(h[4]), "r"(h[5]), "r"(h[6]), "r"(h[7])
+                 : "memory");
+}
+struct EpiHidden {           // U = acc + b (FP32, [unit][B]: a warp's rows side by side); H = gelu(U) (BF16)
     const float* bias;
     float* U;
     __nv_bfloat16* H;
-    __nv_bfloat16* Ht;
-    int64_t ldt;             // rows of the batch (leading dimension of H^T)
+    int64_t ldu;             // rows of the batch
     __device__ void operator()(int row, int col0, const float (&v)[16]) const {
-        alignas(16) __nv_bfloat16 hb[16];
-        alignas(16) float u[16];
+        unsigned h[8];
         const float4* b4 = reinterpret_cast<const float4*>(bias + col0);
+        float* d = U + (int64_t)col0 * ldu + row;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const float4 b = __ldg(b4 + q);
-            u[4 * q] = v[4 * q] + b.x;
-            u[4 * q + 1] = v[4 * q + 1] + b.y;
-            u[4 * q + 2] = v[4 * q + 2] + b.z;
-            u[4 * q + 3] = v[4 * q + 3] + b.w;
+            const unsigned long long u0 = add2(pk2(v[4 * q], v[4 * q + 1]), pk2(b.x, b.y));
+            const unsigned long long u1 = add2(pk2(v[4 * q + 2], v[4 * q + 3]), pk2(b.z, b.w));
+            float x, y;
+            un2(u0, x, y);
+            d[(int64_t)(4 * q) * ldu] = x;
+            d[(int64_t)(4 * q + 1) * ldu] = y;
+            un2(u1, x, y);
+            d[(int64_t)(4 * q + 2) * ldu] = x;
+            d[(int64_t)(4 * q + 3) * ldu] = y;
+            h[2 * q] = gelu2(u0);
+            h[2 * q + 1] = gelu2(u1);
         }
-        if (U) {
-            float4* d = reinterpret_cast<float4*>(U + (int64_t)row * kHid + col0);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) d[q] = reinterpret_cast<const float4*>(u)[q];
-        }
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            hb[i] = __float2bfloat16(gelu_f(u[i]));
-            if (Ht) Ht[(int64_t)(col0 + i) * ldt + row] = hb[i];
-        }
-        uint4* dst = reinterpret_cast<uint4*>(H + (int64_t)row * kHid + col0);
-        dst[0] = reinterpret_cast<const uint4*>(hb)[0];
-        dst[1] = reinterpret_cast<const uint4*>(hb)[1];
+        st32(H + (int64_t)row * kHid + col0, h);
     }
 };
 
-struct EpiOutput {           // out = acc + b3; training: residual, loss, dO, dO^T; inference: pred
+struct EpiInfer {            // inference: out = acc + b3 and its ranking
     const float* bias;
-    const float* Y;          // [B][16] (training) or null
-    float* loss;             // accumulator (training)
-    __nv_bfloat16* dO;       // [B][16]
-    __nv_bfloat16* dOt;      // [16][B]
-    int64_t ldt;
-    float scale;             // 2 / (6 B)
-    float* pred;             // [B][6] (inference) or null
-    // inference ranking (Sec. 2 tier 3 on the surrogate's predictions), optional
-    const uint8_t* masks;    // [B] version masks (candidates: optimizations not applied)
-    int flags, k;
+    float* pred;             // nullable: [B][6]
+    const uint8_t* masks;    // the settings of the rows already enabled (null: none)
+    int flags;
+    int k;
     float log_tau;
-    uint32_t* rec_code;      // [B]
+    uint32_t* rec_code;      // [B], nullable: no ranking
     double* rec_pred;        // [B][k]
     __device__ void rank_row(int64_t row, const float (&o)[16]) const {
         const int cand = (flags & RS_RANK_ALL) || !masks ? 63 : (~masks[row] & 63);
@@ -151,230 +178,308 @@ struct EpiOutput {           // out = acc + b3; training: residual, loss, dO, dO
             for (int x = 0; x < kOut; ++x)
                 if (x < k) rec_pred[(int64_t)row * k + x] = rp[x];
     }
-    __device__ void operator()(int64_t row, int col0, const float (&v)[16]) const {
+    __device__ void operator()(int64_t row, const float (&v)[16]) const {
+        float o[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) o[i] = v[i] + bias[i];
+        if (rec_code) rank_row(row, o);
+        if (pred)
+#pragma unroll
+            for (int i = 0; i < kOut; ++i) pred[row * kOut + i] = o[i];
+    }
+};
+
+struct EpiLoss {             // training: out = acc + b3; dO = scale (out - y) and the loss
+    static constexpr bool kWarp = true;
+    const float* bias;
+    const float* Y;          // [B][16]
+    __nv_bfloat16* dO;       // [B][16]
+    float* part;             // [B / 32]: the minibatch MSE's sums over 32 rows
+    float scale;
+    __device__ void operator()(int row, bool in, int col0, const float (&v)[16]) const {
         if (col0 != 0) return;
-        if (rec_code) {
-            float o[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) o[i] = v[i] + bias[i];
-            rank_row(row, o);
-        }
         float l = 0.f;
-        alignas(16) __nv_bfloat16 g[16];
+        unsigned h[8] = {};
+        if (in) {
+            float g[kOut];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const float out = v[i] + bias[i];
-            float d = 0.f;
-            if (i < kOut) {
-                if (pred) pred[(int64_t)row * kOut + i] = out;
-                if (Y) {
-                    const float r = out - Y[(int64_t)row * kOutP + i];
-                    l += 0.5f * scale * r * r;      // r^2 / (6 B): the minibatch MSE
-                    d = scale * r;
-                }
+            for (int i = 0; i < kOut; ++i) {
+                const float r = v[i] + bias[i] - Y[(int64_t)row * kOutP + i];
+                l += 0.5f * scale * r * r;          // r^2 / (6 B)
+                g[i] = scale * r;
             }
-            g[i] = __float2bfloat16(d);
-            if (dOt) dOt[(int64_t)i * ldt + row] = g[i];
+#pragma unroll
+            for (int i = 0; i < kOut / 2; ++i) {
+                const __nv_bfloat162 p = __floats2bfloat162_rn(g[2 * i], g[2 * i + 1]);
+                h[i] = *reinterpret_cast<const unsigned*>(&p);
+            }
+            st32(dO + (int64_t)row * kOutP, h);
         }
-        if (dO) {
-            uint4* dst = reinterpret_cast<uint4*>(dO + (int64_t)row * kOutP);
-            dst[0] = reinterpret_cast<const uint4*>(g)[0];
-            dst[1] = reinterpret_cast<const uint4*>(g)[1];
-        }
-        if (loss) atomicAdd(loss, l);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if ((threadIdx.x & 31) == 0) part[row >> 5] = l;
     }
 };
 
-struct EpiGeluGrad {         // dU = acc * gelu'(U): BF16 dU (optional) and dU^T
-    const float* U;
+struct EpiGeluGrad {         // dU = acc * gelu'(U) (BF16)
+    const float* U;          // [unit][B]
     __nv_bfloat16* dU;
-    __nv_bfloat16* dUt;
-    int64_t ldt;
+    int64_t ldu;
     __device__ void operator()(int row, int col0, const float (&v)[16]) const {
-        alignas(16) __nv_bfloat16 g[16];
-        alignas(16) float u[16];
-        const float4* u4 = reinterpret_cast<const float4*>(U + (int64_t)row * kHid + col0);
+        const float* u = U + (int64_t)col0 * ldu + row;
+        float g[16];
+        unsigned h[8];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) reinterpret_cast<float4*>(u)[q] = u4[q];
+        for (int i = 0; i < 16; ++i) g[i] = u[(int64_t)i * ldu];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            g[i] = __float2bfloat16(v[i] * gelu_grad_f(u[i]));
-            dUt[(int64_t)(col0 + i) * ldt + row] = g[i];
+        for (int i = 0; i < 8; ++i) {
+            const __nv_bfloat162 p = __floats2bfloat162_rn(v[2 * i] * gelu_grad_f(g[2 * i]),
+                                                           v[2 * i + 1] * gelu_grad_f(g[2 * i + 1]));
+            h[i] = *reinterpret_cast<const unsigned*>(&p);
         }
-        if (dU) {
-            uint4* dst = reinterpret_cast<uint4*>(dU + (int64_t)row * kHid + col0);
-            dst[0] = reinterpret_cast<const uint4*>(g)[0];
-            dst[1] = reinterpret_cast<const uint4*>(g)[1];
-        }
-    }
-};
-
-struct EpiF32Part {          // split-K partial of a weight gradient: slice z -> D + z * zstride
-                             // (N, ldd, zstride multiples of 16: whole 16-column chunks)
-    float* D;
-    int64_t ldd;
-    int64_t zstride;
-    int N;
-    __device__ void operator()(int z, int row, int col0, const float (&v)[16]) const {
-        float4* d = reinterpret_cast<float4*>(D + (int64_t)z * zstride + (int64_t)row * ldd + col0);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) d[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-    }
-};
-
-struct EpiF32 {              // plain FP32 store (weight gradients; N, ldd multiples of 16)
-    float* D;
-    int64_t ldd;
-    int N;
-    __device__ void operator()(int row, int col0, const float (&v)[16]) const {
-        float4* d = reinterpret_cast<float4*>(D + (int64_t)row * ldd + col0);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) d[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+        st32(dU + (int64_t)row * kHid + col0, h);
     }
 };
 
 // Pipeline depth of the persistent GEMM (one CTA per SM): four 32 KB stages (BN = 128).
 constexpr int kStages = 4;
 
-template <int BN, int S, class Epi>
-cudaError_t gemm_attr();
-
-template <int BN, class Epi, bool BATCHED = false>
-cudaError_t gemm_attr() {
-    return cudaFuncSetAttribute(tc::gemm_kernel<BN, kStages, Epi, BATCHED>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, tc::Layout<BN, kStages>::kBytes);
+// The three weight gradients as one problem: each D = A^T B over a range of the batch's rows, A and B
+// row-major, D's partial sums (one per range) in FP32.  28 tiles of 128 x 128 a range.
+struct Wgrad {
+    float* d[3];             // of W1, W2, W3; range z at + z * zstride
+    int64_t zstride;
+    int slices, rows;        // ranges, rows of each
+};
+struct WgradProb {
+    static constexpr bool kAmn = true, kBmn = true;
+    struct Tile { int w, m0, n0, z, N, nk; };
+    const CUtensorMap *dU1, *X, *dU2, *H1, *dO, *H2;
+    const Wgrad& g;
+    __device__ long long tiles() const { return 28ll * g.slices; }
+    __device__ Tile tile(long long t) const {
+        const int z = (int)(t / 28), j = (int)(t % 28), nk = (g.rows + 63) / 64;
+        if (j < 16) return Tile{1, (j >> 2) * 128, (j & 3) * 128, z, kHid, nk};
+        if (j < 24) return Tile{0, ((j - 16) >> 1) * 128, (j & 1) * 128, z, kIn, nk};
+        return Tile{2, 0, (j - 24) * 128, z, kHid, nk};
+    }
+    __device__ void load(const Tile& t, int kb, uint32_t sa, uint32_t sb, uint32_t bar) const {
+        const int y = t.z * g.rows + kb * 64;
+        const CUtensorMap *a = t.w == 0 ? dU1 : t.w == 1 ? dU2 : dO, *b = t.w == 0 ? X : t.w == 1 ? H1 : H2;
+        tc::tma_load_2d(sa, a, bar, t.m0, y);
+        tc::tma_load_2d(sa + 8192, a, bar, t.m0 + 64, y);            // (dO: beyond its 16 columns, zeros)
+        tc::tma_load_2d(sb, b, bar, t.n0, y);
+        tc::tma_load_2d(sb + 8192, b, bar, t.n0 + 64, y);
+    }
+    __device__ void emit(const Tile& t, int row, int col0, const float (&v)[16]) const {
+        if (t.w == 2 && row >= kOutP) return;
+        float* d = (t.w == 0 ? g.d[0] : t.w == 1 ? g.d[1] : g.d[2]) + t.z * g.zstride + (int64_t)row * t.N + col0;
+        unsigned h[2][8];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) h[i >> 3][i & 7] = __float_as_uint(v[i]);
+        st32(d, h[0]);
+        st32(d + 8, h[1]);
+    }
+};
+__global__ void __launch_bounds__(tc::kGemmThreads, 1)
+wgrad_kernel(const __grid_constant__ CUtensorMap dU1, const __grid_constant__ CUtensorMap X,
+             const __grid_constant__ CUtensorMap dU2, const __grid_constant__ CUtensorMap H1,
+             const __grid_constant__ CUtensorMap dO, const __grid_constant__ CUtensorMap H2,
+             const __grid_constant__ Wgrad g, int* err) {
+    const WgradProb p{&dU1, &X, &dU2, &H1, &dO, &H2, g};
+    tc::gemm_core<128, kStages>(p, err);
 }
 
 // The function attributes of every product of a training step, set before a graph capture.
+template <int BN, class Epi, bool BMN = false>
+cudaError_t gemm_attr() {
+    return cudaFuncSetAttribute(tc::gemm_kernel<BN, kStages, Epi, false, BMN>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize, tc::Layout<BN, kStages>::kBytes);
+}
 cudaError_t all_attrs() {
     cudaError_t e = gemm_attr<128, EpiHidden>();
-    if (e == cudaSuccess) e = gemm_attr<32, EpiOutput>();
-    if (e == cudaSuccess) e = gemm_attr<128, EpiGeluGrad>();
-    if (e == cudaSuccess) e = gemm_attr<128, EpiF32>();
-    if (e == cudaSuccess) e = gemm_attr<128, EpiF32Part, true>();
+    if (e == cudaSuccess) e = gemm_attr<32, EpiLoss>();
+    if (e == cudaSuccess) e = gemm_attr<128, EpiGeluGrad, true>();
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(wgrad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::Layout<128, kStages>::kBytes);
     return e;
 }
 
-// Split-K product over `slices` K ranges (rank-3 maps from rs_make_tmap_bf16_kslices): batch z
-// is range z; the epilogue gets z.
-template <int BN, class Epi>
-cudaError_t gemm_slices(const CUtensorMap& ta, const CUtensorMap& tb, int M, int N, int Kslice, int slices,
-                        const Epi& epi, int* err, cudaStream_t st) {
-    return tc::gemm_launch<BN, kStages, Epi, true>(ta, tb, M, N, Kslice, slices, epi, err, st);
-}
-
-template <int BN, class Epi>
+template <int BN, bool BMN = false, class Epi>
 cudaError_t gemm(const CUtensorMap& ta, const CUtensorMap& tb, int M, int N, int K, const Epi& epi, int* err,
                  cudaStream_t st) {
-    return tc::gemm_launch<BN, kStages, Epi>(ta, tb, M, N, K, 1, epi, err, st);
+    return tc::gemm_launch<BN, kStages, Epi, false, BMN>(ta, tb, M, N, K, 1, epi, err, st);
 }
 
 // ---- small kernels -----------------------------------------------------------------------------
-// Stage a minibatch: rows (r0 + i) mod n of X (double [n][256]) -> BF16 X_s and X_s^T, labels
-// (double [n][6], NaN treated as 0 with zero weight) -> Y_s [B][16].  r0 = step * B, with the
-// step read from the device counter so the same launch serves every step of a graph.
+// A double as the nearest float (ties to even), by integer operations in the normal float range: a
+// conversion instruction takes the narrow FP64 pipe.
+__device__ __forceinline__ float f32_of(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    if ((hi & 0x7fffffffu) - (898u << 20) >= (252u << 20)) return (float)x;
+    const unsigned l = lo + 0x0fffffffu + ((lo >> 29) & 1u), h = hi + (l < lo);
+    return __uint_as_float(((__funnelshift_l(l, h, 3) - (896u << 23)) & 0x7fffffffu) | (hi & 0x80000000u));
+}
+// Stage a minibatch, a warp a row: rows (r0 + i) mod n of X (double [n][256]) -> BF16 X_s, labels
+// (double [n][6], NaN treated as 0 with zero weight) -> Y_s [B][16].  r0 = minibatch * B, read from the
+// device counter so that the same launch serves every step of a graph.  Also counts the step: Adam's,
+// and the call's (run).
 __global__ void __launch_bounds__(256)
-stage_kernel(const double* __restrict__ X, const double* __restrict__ Yin, int64_t n, int B, const int* step,
-             int64_t fixed_r0, __nv_bfloat16* Xs, __nv_bfloat16* Xt, float* Ys) {
-    const int64_t r0 = step ? (int64_t)(*step) * B : fixed_r0;
-    const int i = blockIdx.x;                   // batch row
+stage_kernel(const double* __restrict__ X, const double* __restrict__ Yin, int64_t n, int B, int* counters,
+             int* run, __nv_bfloat16* Xs, float* Ys) {
+    const int lane = threadIdx.x & 31, i = blockIdx.x * 8 + (threadIdx.x >> 5);     // batch row
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        counters[1] += 1;
+        *run += 1;
+    }
     if (i >= B) return;
-    const int64_t src = (r0 + i) % n;
-    for (int f = threadIdx.x; f < kIn; f += blockDim.x) {
-        const __nv_bfloat16 v = __float2bfloat16((float)X[src * kIn + f]);
-        Xs[(int64_t)i * kIn + f] = v;
-        if (Xt) Xt[(int64_t)f * B + i] = v;
-    }
-    if (Ys && threadIdx.x < kOutP) {
-        float y = 0.f;
-        if (threadIdx.x < kOut) {
-            const double d = Yin[src * kOut + threadIdx.x];
-            y = isfinite(d) ? (float)d : 0.f;
-        }
-        Ys[(int64_t)i * kOutP + threadIdx.x] = y;
-    }
+    const int64_t src = ((int64_t)counters[0] * B + i) % n;
+    double x[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) x[e] = X[src * kIn + 32 * e + lane];
+    double y = 0.0;
+    if (lane < kOut) y = Yin[src * kOut + lane];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) Xs[(int64_t)i * kIn + 32 * e + lane] = __float2bfloat16(f32_of(x[e]));
+    if (lane < kOutP) Ys[(int64_t)i * kOutP + lane] = isfinite(y) ? (float)y : 0.f;
 }
 
 #include "k_mlp_infer.cuh"
 
-// Row sums of a transposed gradient [rows][B] (BF16) -> FP32 bias gradient; one warp per row.
-__global__ void __launch_bounds__(256)
-rowsum_kernel(const __nv_bfloat16* __restrict__ T, int rows, int B, float* out) {
-    const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-    if (w >= rows) return;
-    float s = 0.f;
-    for (int i = lane; i < B; i += 32) s += __bfloat162float(T[(int64_t)w * B + i]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) out[w] = s;
-}
-
-// Sum of the split-K partials of the three weight gradients, slice 0 first (a fixed order,
-// so every step and every graph replay adds the same numbers the same way).  The partials
-// of one slice are laid out [W1 | W2 | W3] (nW1 + nW2 + nW3 floats).
-__global__ void __launch_bounds__(256)
-reduce_wgrad_kernel(const float* __restrict__ part, int slices, float* G) {
-    constexpr int64_t n = Blob::nW1 + Blob::nW2 + Blob::nW3;
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    float s = 0.f;
-    for (int z = 0; z < slices; ++z) s += part[(int64_t)z * n + i];
-    const int64_t o = i < Blob::nW1 ? Blob::oW1 + i
-                    : i < Blob::nW1 + Blob::nW2 ? Blob::oW2 + (i - Blob::nW1)
-                                                : Blob::oW3 + (i - Blob::nW1 - Blob::nW2);
-    G[o] = s;
-}
-
-// BF16 copies of the master weights: W1, W2, W3 (padded rows) and the transposes W2^T, W3^T.
+// BF16 copies of the master weights: W1, W2, W3 (padded rows).
 __global__ void __launch_bounds__(256)
 sync_bf16_kernel(const float* __restrict__ P, __nv_bfloat16* bf) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < Blob::nW1) bf[Blob::bW1 + i] = __float2bfloat16(P[Blob::oW1 + i]);
-    if (i < Blob::nW2) {
-        const float w = P[Blob::oW2 + i];
-        bf[Blob::bW2 + i] = __float2bfloat16(w);
-        const int64_t r = i / kHid, c = i % kHid;
-        bf[Blob::bW2t + c * kHid + r] = __float2bfloat16(w);
-    }
-    if (i < Blob::nW3) {
-        const int64_t r = i / kHid, c = i % kHid;           // r < 16 (rows >= 6 stay zero)
-        const float w = r < kOut ? P[Blob::oW3 + i] : 0.f;
-        bf[Blob::bW3 + i] = __float2bfloat16(w);
-        bf[Blob::bW3t + c * kOutP + r] = __float2bfloat16(w);
-    }
+    if (i < Blob::nW2) bf[Blob::bW2 + i] = __float2bfloat16(P[Blob::oW2 + i]);
+    if (i < Blob::nW3)                                      // rows >= 6 stay zero
+        bf[Blob::bW3 + i] = __float2bfloat16(i < (int64_t)kOut * kHid ? P[Blob::oW3 + i] : 0.f);
 }
 
-// AdamW over every parameter (padded output rows keep zero gradient and stay zero).
+// The step's last kernel: gradients from their partial sums (range 0 first, a fixed order, so that every
+// step and every graph replay adds the same numbers the same way), AdamW over every parameter (padded
+// output rows keep zero gradient and stay zero), the BF16 weights, the loss and the minibatch position.
+// The first kBBlocks blocks take 16 columns each of [b1 | b2 | b3]: a bias gradient sums its column of dU in
+// 32 chains (rows of one remainder mod 32 in order) and those as a tree, two columns a thread.  Then
+// four weights a thread.
+constexpr int kWBlocks = (int)((Blob::nW1 + Blob::nW2 + Blob::nW3) / 4 + 255) / 256, kBBlocks = 2 * kHid / 16 + 1;
+struct Update {
+    float* blob;
+    __nv_bfloat16* bf;
+    const float* w[3];       // partial sums of dW1, dW2, dW3, ranges zstride apart
+    int64_t zstride;
+    int slices;
+    const __nv_bfloat16* d[3];       // dU1, dU2 [B][512] and dO [B][16]
+    int B;
+    const float* loss_part;  // [rows of 32]
+    float lr, wd;
+    int* counters;
+    int64_t steps_per_epoch;
+    const int* run;
+    float* loss_curve;
+};
+__device__ __forceinline__ float adamw(const Update& a, float p, float g, float& m, float& v, float c1, float c2) {
+    constexpr float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+    m = b1 * m + (1.f - b1) * g;
+    v = b2 * v + (1.f - b2) * g * g;
+    const float mh = m / c1;
+    const float vh = v / c2;
+    return p - a.lr * (mh / (sqrtf(vh) + eps) + a.wd * p);
+}
 __global__ void __launch_bounds__(256)
-adamw_kernel(float* blob, float lr, float b1, float b2, float eps, float wd, int* counters) {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const int t = counters[1] + 1;              // this step's index (1-based)
-    if (i < Blob::nP) {
-        float* P = blob;
-        float* m = blob + Blob::oM;
-        float* v = blob + Blob::oV;
-        const float g = blob[Blob::oG + i];
-        const float mi = b1 * m[i] + (1.f - b1) * g;
-        const float vi = b2 * v[i] + (1.f - b2) * g * g;
-        m[i] = mi;
-        v[i] = vi;
-        const float mh = mi / (1.f - powf(b1, (float)t));
-        const float vh = vi / (1.f - powf(b2, (float)t));
-        P[i] = P[i] - lr * (mh / (sqrtf(vh) + eps) + wd * P[i]);
+update_kernel(const __grid_constant__ Update a) {
+    __shared__ float corr[2], red[32][17];
+    const int tid = threadIdx.x;
+    if (tid < 2) corr[tid] = 1.f - powf(tid ? 0.999f : 0.9f, (float)a.counters[1]);
+    if ((int)blockIdx.x >= kBBlocks) {
+        const int64_t i = ((int64_t)(blockIdx.x - kBBlocks) * 256 + tid) * 4;
+        const int k = i < Blob::nW1 ? 0 : i < Blob::nW1 + Blob::nW2 ? 1 : 2;
+        const int64_t j = i - (k == 0 ? 0 : k == 1 ? Blob::nW1 : Blob::nW1 + Blob::nW2);      // within its matrix
+        const bool in = i < Blob::nW1 + Blob::nW2 + Blob::nW3;
+        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (in) {
+            const float* src = (k == 0 ? a.w[0] : k == 1 ? a.w[1] : a.w[2]) + j;
+#pragma unroll 8
+            for (int z = 0; z < a.slices; ++z) {
+                const float4 p = *reinterpret_cast<const float4*>(src + z * a.zstride);
+                s.x += p.x;
+                s.y += p.y;
+                s.z += p.z;
+                s.w += p.w;
+            }
+        }
+        __syncthreads();
+        if (in) {
+            const int64_t o = (k == 0 ? Blob::oW1 : k == 1 ? Blob::oW2 : Blob::oW3) + j;
+            float4* P = reinterpret_cast<float4*>(a.blob + o);
+            float4 *M = P + Blob::oM / 4, *V = P + Blob::oV / 4, *G = P + Blob::oG / 4;
+            float4 q = *P, m = *M, v = *V;
+            q.x = adamw(a, q.x, s.x, m.x, v.x, corr[0], corr[1]);
+            q.y = adamw(a, q.y, s.y, m.y, v.y, corr[0], corr[1]);
+            q.z = adamw(a, q.z, s.z, m.z, v.z, corr[0], corr[1]);
+            q.w = adamw(a, q.w, s.w, m.w, v.w, corr[0], corr[1]);
+            *P = q;
+            *M = m;
+            *V = v;
+            *G = s;
+            if (k == 2 && j >= (int64_t)kOut * kHid) q = make_float4(0.f, 0.f, 0.f, 0.f);
+            const __nv_bfloat162 h[2] = {__floats2bfloat162_rn(q.x, q.y), __floats2bfloat162_rn(q.z, q.w)};
+            __nv_bfloat16* d = a.bf + (k == 0 ? Blob::bW1 : k == 1 ? Blob::bW2 : Blob::bW3) + j;
+            *reinterpret_cast<uint2*>(d) = *reinterpret_cast<const uint2*>(h);
+        }
+        return;
+    }
+    const int q = blockIdx.x, k = q < kHid / 16 ? 0 : q < 2 * kHid / 16 ? 1 : 2, ld = k == 2 ? kOutP : kHid;
+    const int c0 = k == 2 ? 0 : (q - k * (kHid / 16)) * 16;
+    float s0 = 0.f, s1 = 0.f;
+    const __nv_bfloat16* src = (k == 0 ? a.d[0] : k == 1 ? a.d[1] : a.d[2]) + c0 + 2 * (tid & 7);
+#pragma unroll 32
+    for (int r = tid >> 3; r < a.B; r += 32) {
+        const unsigned p = *reinterpret_cast<const unsigned*>(src + (int64_t)r * ld);
+        s0 += __uint_as_float(p << 16);
+        s1 += __uint_as_float(p & 0xffff0000u);
+    }
+    red[tid >> 3][2 * (tid & 7)] = s0;
+    red[tid >> 3][2 * (tid & 7) + 1] = s1;
+    __syncthreads();
+    const int lane = tid & 31;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int c = c0 + 2 * (tid >> 5) + h;
+        float g = red[lane][c - c0];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+        if (lane == 0) {
+            if (k == 2 && c >= kOut) g = 0.f;
+            float* P = a.blob + (k == 0 ? Blob::ob1 : k == 1 ? Blob::ob2 : Blob::ob3) + c;
+            *P = adamw(a, *P, g, P[Blob::oM], P[Blob::oV], corr[0], corr[1]);
+            P[Blob::oG] = g;
+        }
+    }
+    if (k == 2) {
+        float l = 0.f;
+        for (int r = tid; r * 32 < a.B; r += 256) l += a.loss_part[r];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        __syncthreads();
+        if (lane == 0) red[0][tid >> 5] = l;
+        __syncthreads();
+        if (tid == 0) {
+            for (int w = 1; w < 8; ++w) l += red[0][w];
+            if (a.loss_curve) a.loss_curve[*a.run] = l;
+            a.counters[0] = (int)((a.counters[0] + 1) % a.steps_per_epoch);
+        }
     }
 }
 
 // A call continues from the blob's counters (a restored checkpoint resumes the same sequence
 // of minibatches and Adam steps); the minibatch position wraps into this call's rows.
-__global__ void wrap_counters_kernel(int* counters, int64_t steps_per_epoch) {
+__global__ void wrap_counters_kernel(int* counters, int64_t steps_per_epoch, int* run) {
     int64_t q = counters[0] % steps_per_epoch;
     if (q < 0) q += steps_per_epoch;                         // (a blob not zeroed by its owner)
     counters[0] = (int)q;
     if (counters[1] < 0) counters[1] = 0;
-}
-__global__ void bump_counters_kernel(int* counters, int64_t steps_per_epoch) {
-    counters[1] += 1;                                        // Adam t
-    counters[0] = (int)((counters[0] + 1) % steps_per_epoch); // minibatch index
+    *run = -1;                                               // this call's step, counted by stage_kernel
 }
 
 // Feature mean / std over the training rows (for the out-of-distribution score): each
@@ -401,10 +506,12 @@ __global__ void feature_stats_finish(const double* acc, int64_t n, float* mean, 
 
 // ---- training workspace --------------------------------------------------------------------------
 struct TrainWs {
-    __nv_bfloat16 *Xs, *Xt, *H1, *H1t, *H2, *H2t, *dO, *dOt, *dU2, *dU2t, *dU1t;
+    __nv_bfloat16 *Xs, *H1, *H2, *dO, *dU2, *dU1;
     float *Ys, *U1, *U2;
     double* stats_acc;
+    int* run;                 // the call's step (in stats_acc, once the statistics are finished)
     float* part;              // split-K partials of the weight gradients (slices > 1)
+    float* loss_part;         // sums over 32 rows
     int slices;
     size_t bytes;
 };
@@ -427,20 +534,17 @@ TrainWs carve_train(void* base, int B) {
     auto take = [&](size_t b) { char* p = c ? c + o : nullptr; o += a256(b); return p; };
     const size_t bf = sizeof(__nv_bfloat16);
     w.Xs = (__nv_bfloat16*)take((size_t)B * kIn * bf);
-    w.Xt = (__nv_bfloat16*)take((size_t)B * kIn * bf);
     w.H1 = (__nv_bfloat16*)take((size_t)B * kHid * bf);
-    w.H1t = (__nv_bfloat16*)take((size_t)B * kHid * bf);
     w.H2 = (__nv_bfloat16*)take((size_t)B * kHid * bf);
-    w.H2t = (__nv_bfloat16*)take((size_t)B * kHid * bf);
     w.dO = (__nv_bfloat16*)take((size_t)B * kOutP * bf);
-    w.dOt = (__nv_bfloat16*)take((size_t)B * kOutP * bf);
     w.dU2 = (__nv_bfloat16*)take((size_t)B * kHid * bf);
-    w.dU2t = (__nv_bfloat16*)take((size_t)B * kHid * bf);
-    w.dU1t = (__nv_bfloat16*)take((size_t)B * kHid * bf);
+    w.dU1 = (__nv_bfloat16*)take((size_t)B * kHid * bf);
     w.Ys = (float*)take((size_t)B * kOutP * sizeof(float));
     w.U1 = (float*)take((size_t)B * kHid * sizeof(float));
     w.U2 = (float*)take((size_t)B * kHid * sizeof(float));
     w.stats_acc = (double*)take(2 * kIn * sizeof(double));
+    w.run = (int*)w.stats_acc;
+    w.loss_part = (float*)take((size_t)((B + 127) / 128 * 4) * sizeof(float));
     w.slices = wgrad_slices(B);
     w.part = w.slices > 1 ? (float*)take((size_t)w.slices * (Blob::nW1 + Blob::nW2 + Blob::nW3) * sizeof(float))
                           : nullptr;
@@ -449,9 +553,8 @@ TrainWs carve_train(void* base, int B) {
 }
 
 struct Maps {
-    CUtensorMap Xs, W1, H1, W2, H2, W3, dO, W3t, dU2, W2t, dOt, H2t, dU2t, H1t, dU1t, Xt;
-    // split-K views of the transposed operands of the weight gradients (slices > 1)
-    CUtensorMap sdOt, sH2t, sdU2t, sH1t, sdU1t, sXt;
+    CUtensorMap Xs, W1, H1, W2, H2, W3, dO, dU2;             // K-major operands
+    CUtensorMap tW3, tW2, tdO, tH2, tdU2, tH1, tdU1, tX;     // the same matrices by boxes of 64 rows
 };
 
 cudaError_t make_maps(Maps& m, const TrainWs& w, const __nv_bfloat16* bf, int B) {
@@ -466,78 +569,49 @@ cudaError_t make_maps(Maps& m, const TrainWs& w, const __nv_bfloat16* bf, int B)
     mk(&m.H2, w.H2, B, kHid, 128);
     mk(&m.W3, bf + Blob::bW3, kOutP, kHid, 32);
     mk(&m.dO, w.dO, B, kOutP, 128);
-    mk(&m.W3t, bf + Blob::bW3t, kHid, kOutP, 128);
     mk(&m.dU2, w.dU2, B, kHid, 128);
-    mk(&m.W2t, bf + Blob::bW2t, kHid, kHid, 128);
-    mk(&m.dOt, w.dOt, kOutP, B, 128);
-    mk(&m.H2t, w.H2t, kHid, B, 128);
-    mk(&m.dU2t, w.dU2t, kHid, B, 128);
-    mk(&m.H1t, w.H1t, kHid, B, 128);
-    mk(&m.dU1t, w.dU1t, kHid, B, 128);
-    mk(&m.Xt, w.Xt, kIn, B, 128);
-    if (w.slices > 1) {
-        auto ks = [&](CUtensorMap* t, const void* p, int64_t rows, int box) {
-            if (e == cudaSuccess) e = rs_make_tmap_bf16_kslices(t, p, rows, B, B, w.slices, box);
-        };
-        ks(&m.sdOt, w.dOt, kOutP, 128);
-        ks(&m.sH2t, w.H2t, kHid, 128);
-        ks(&m.sdU2t, w.dU2t, kHid, 128);
-        ks(&m.sH1t, w.H1t, kHid, 128);
-        ks(&m.sdU1t, w.dU1t, kHid, 128);
-        ks(&m.sXt, w.Xt, kIn, 128);
-    }
+    mk(&m.tW3, bf + Blob::bW3, kOutP, kHid, 64);
+    mk(&m.tW2, bf + Blob::bW2, kHid, kHid, 64);
+    mk(&m.tdO, w.dO, B, kOutP, 64);
+    mk(&m.tH2, w.H2, B, kHid, 64);
+    mk(&m.tdU2, w.dU2, B, kHid, 64);
+    mk(&m.tH1, w.H1, B, kHid, 64);
+    mk(&m.tdU1, w.dU1, B, kHid, 64);
+    mk(&m.tX, w.Xs, B, kIn, 64);
     return e;
 }
 
-// Forward + backward for the staged minibatch: gradients into the blob's grad region.
-cudaError_t step_body(float* blob, const TrainWs& w, const Maps& m, int B, float* loss_slot, int* err,
-                      cudaStream_t st) {
+// Forward + backward for the staged minibatch: the weight gradients' partial sums (straight into the
+// blob's gradients when the rows are one range).
+cudaError_t step_body(float* blob, const TrainWs& w, const Maps& m, int B, int* err, cudaStream_t st) {
     float* G = blob + Blob::oG;
     const float* P = blob;
-    cudaError_t e;
     const float sc = 2.0f / (6.0f * (float)B);
-    e = gemm<128>(m.Xs, m.W1, B, kHid, kIn, EpiHidden{P + Blob::ob1, w.U1, w.H1, w.H1t, B}, err, st);
+    cudaError_t e = gemm<128>(m.Xs, m.W1, B, kHid, kIn, EpiHidden{P + Blob::ob1, w.U1, w.H1, B}, err, st);
     if (e == cudaSuccess)
-        e = gemm<128>(m.H1, m.W2, B, kHid, kHid, EpiHidden{P + Blob::ob2, w.U2, w.H2, w.H2t, B}, err, st);
+        e = gemm<128>(m.H1, m.W2, B, kHid, kHid, EpiHidden{P + Blob::ob2, w.U2, w.H2, B}, err, st);
     if (e == cudaSuccess)
-        e = gemm<32>(m.H2, m.W3, B, kOutP, kHid,
-                     EpiOutput{P + Blob::ob3, w.Ys, loss_slot, w.dO, w.dOt, B, sc, nullptr, nullptr, 0, 0, 0.f,
-                               nullptr, nullptr}, err, st);
+        e = gemm<32>(m.H2, m.W3, B, kOutP, kHid, EpiLoss{P + Blob::ob3, w.Ys, w.dO, w.loss_part, sc}, err, st);
     if (e == cudaSuccess)      // dU2 = (dO W3) * gelu'(U2)
-        e = gemm<128>(m.dO, m.W3t, B, kHid, kOutP, EpiGeluGrad{w.U2, w.dU2, w.dU2t, B}, err, st);
+        e = gemm<128, true>(m.dO, m.tW3, B, kHid, kOutP, EpiGeluGrad{w.U2, w.dU2, B}, err, st);
     if (e == cudaSuccess)      // dU1 = (dU2 W2) * gelu'(U1)
-        e = gemm<128>(m.dU2, m.W2t, B, kHid, kHid, EpiGeluGrad{w.U1, nullptr, w.dU1t, B}, err, st);
-    if (w.slices > 1) {        // weight gradients split over K ranges, then summed in order
-        constexpr int64_t nPart = Blob::nW1 + Blob::nW2 + Blob::nW3;
-        const int S = w.slices, ks = B / S;
-        if (e == cudaSuccess)  // dW3 = dO^T H2
-            e = gemm_slices<128>(m.sdOt, m.sH2t, kOutP, kHid, ks, S,
-                                                EpiF32Part{w.part + Blob::nW1 + Blob::nW2, kHid, nPart, kHid}, err, st);
-        if (e == cudaSuccess)  // dW2 = dU2^T H1
-            e = gemm_slices<128>(m.sdU2t, m.sH1t, kHid, kHid, ks, S,
-                                                EpiF32Part{w.part + Blob::nW1, kHid, nPart, kHid}, err, st);
-        if (e == cudaSuccess)  // dW1 = dU1^T X
-            e = gemm_slices<128>(m.sdU1t, m.sXt, kHid, kIn, ks, S,
-                                                EpiF32Part{w.part, kIn, nPart, kIn}, err, st);
-        if (e == cudaSuccess) {
-            reduce_wgrad_kernel<<<(unsigned)((nPart + 255) / 256), 256, 0, st>>>(w.part, S, G);
-            e = cudaGetLastError();
-        }
-    } else {
-        if (e == cudaSuccess)  // dW3 = dO^T H2
-            e = gemm<128>(m.dOt, m.H2t, kOutP, kHid, B, EpiF32{G + Blob::oW3, kHid, kHid}, err, st);
-        if (e == cudaSuccess)  // dW2 = dU2^T H1
-            e = gemm<128>(m.dU2t, m.H1t, kHid, kHid, B, EpiF32{G + Blob::oW2, kHid, kHid}, err, st);
-        if (e == cudaSuccess)  // dW1 = dU1^T X
-            e = gemm<128>(m.dU1t, m.Xt, kHid, kIn, B, EpiF32{G + Blob::oW1, kIn, kIn}, err, st);
-    }
-    if (e == cudaSuccess) {
-        rowsum_kernel<<<(kOut * 32 + 255) / 256, 256, 0, st>>>(w.dOt, kOut, B, G + Blob::ob3);
-        rowsum_kernel<<<(kHid * 32 + 255) / 256, 256, 0, st>>>(w.dU2t, kHid, B, G + Blob::ob2);
-        rowsum_kernel<<<(kHid * 32 + 255) / 256, 256, 0, st>>>(w.dU1t, kHid, B, G + Blob::ob1);
-        e = cudaGetLastError();
-    }
-    return e;
+        e = gemm<128, true>(m.dU2, m.tW2, B, kHid, kHid, EpiGeluGrad{w.U1, w.dU1, B}, err, st);
+    if (e != cudaSuccess) return e;
+    Wgrad g{};
+    g.d[0] = w.slices > 1 ? w.part : G + Blob::oW1;
+    g.d[1] = w.slices > 1 ? w.part + Blob::nW1 : G + Blob::oW2;
+    g.d[2] = w.slices > 1 ? w.part + Blob::nW1 + Blob::nW2 : G + Blob::oW3;
+    g.zstride = Blob::nW1 + Blob::nW2 + Blob::nW3;
+    g.slices = w.slices;
+    g.rows = B / w.slices;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const int tiles = 28 * w.slices;
+    wgrad_kernel<<<tiles < sms ? tiles : sms, tc::kGemmThreads, tc::Layout<128, kStages>::kBytes, st>>>(
+        m.tdU1, m.tX, m.tdU2, m.tH1, m.tdO, m.tH2, g, err);
+    return cudaGetLastError();
 }
 
 }  // namespace
@@ -583,29 +657,27 @@ cudaError_t rs_launch_surrogate_train(float* blob, const double* X, const double
     feature_stats_kernel<<<(unsigned)(n < 1024 ? n : 1024), kIn, 0, st>>>(X, n, w.stats_acc);
     feature_stats_finish<<<1, kIn, 0, st>>>(w.stats_acc, n, blob + Blob::oStats, blob + Blob::oStats + kIn);
     sync_bf16_kernel<<<(unsigned)((Blob::nW2 + 255) / 256), 256, 0, st>>>(blob, bf);
-    wrap_counters_kernel<<<1, 1, 0, st>>>(counters, spe);
+    wrap_counters_kernel<<<1, 1, 0, st>>>(counters, spe, w.run);
     e = cudaGetLastError();
-    if (e == cudaSuccess && loss_curve) e = cudaMemsetAsync(loss_curve, 0, steps * sizeof(float), st);
     if (e != cudaSuccess) return e;
-    // one step; the loss goes to loss_curve[t - 1] through a device-side pointer bump
-    float* loss_dev = nullptr;     // loss slot is chosen per step below
-    auto one_step = [&](int64_t s, cudaStream_t q) -> cudaError_t {
-        stage_kernel<<<B, 256, 0, q>>>(X, Y, n, B, counters, 0, w.Xs, w.Xt, w.Ys);
-        cudaError_t e2 = step_body(blob, w, m, B, loss_curve ? loss_curve + s : loss_dev, err, q);
+    const bool split = w.slices > 1;
+    const float* G = blob + Blob::oG;
+    const Update u{blob, bf,
+                   {split ? w.part : G + Blob::oW1, split ? w.part + Blob::nW1 : G + Blob::oW2,
+                    split ? w.part + Blob::nW1 + Blob::nW2 : G + Blob::oW3},
+                   Blob::nW1 + Blob::nW2 + Blob::nW3, w.slices, {w.dU1, w.dU2, w.dO}, B, w.loss_part, lr, wd, counters, spe,
+                   w.run, loss_curve};
+    auto one_step = [&](cudaStream_t q) -> cudaError_t {
+        stage_kernel<<<(unsigned)((B + 7) / 8), 256, 0, q>>>(X, Y, n, B, counters, w.run, w.Xs, w.Ys);
+        cudaError_t e2 = step_body(blob, w, m, B, err, q);
         if (e2 != cudaSuccess) return e2;
-        adamw_kernel<<<(unsigned)((Blob::nP + 255) / 256), 256, 0, q>>>(blob, lr, 0.9f, 0.999f, 1e-8f, wd, counters);
-        sync_bf16_kernel<<<(unsigned)((Blob::nW2 + 255) / 256), 256, 0, q>>>(blob, bf);
-        bump_counters_kernel<<<1, 1, 0, q>>>(counters, spe);
+        update_kernel<<<kWBlocks + kBBlocks, 256, 0, q>>>(u);
         return cudaGetLastError();
     };
     if (!use_graph || !loss_curve) {
-        for (int64_t s = 0; s < steps && e == cudaSuccess; ++s) e = one_step(s, st);
+        for (int64_t s = 0; s < steps && e == cudaSuccess; ++s) e = one_step(st);
         return e;
     }
-    // The loss slot differs per step, so capture one graph per distinct slot would defeat the
-    // purpose: capture with the slot of step 0 and accumulate into a scratch float that a tiny
-    // copy kernel moves to loss_curve[s] after each replay.
-    float* slot = blob + Blob::oCount + 8;
     cudaStream_t cap;
     e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
     if (e != cudaSuccess) return e;
@@ -613,12 +685,7 @@ cudaError_t rs_launch_surrogate_train(float* blob, const double* X, const double
     cudaGraphExec_t ge = nullptr;
     e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        cudaError_t eb = cudaMemsetAsync(slot, 0, sizeof(float), cap);
-        stage_kernel<<<B, 256, 0, cap>>>(X, Y, n, B, counters, 0, w.Xs, w.Xt, w.Ys);
-        if (eb == cudaSuccess) eb = step_body(blob, w, m, B, slot, err, cap);
-        adamw_kernel<<<(unsigned)((Blob::nP + 255) / 256), 256, 0, cap>>>(blob, lr, 0.9f, 0.999f, 1e-8f, wd, counters);
-        sync_bf16_kernel<<<(unsigned)((Blob::nW2 + 255) / 256), 256, 0, cap>>>(blob, bf);
-        bump_counters_kernel<<<1, 1, 0, cap>>>(counters, spe);
+        const cudaError_t eb = one_step(cap);
         e = cudaStreamEndCapture(cap, &g);
         if (eb != cudaSuccess) e = eb;
     }
@@ -629,11 +696,7 @@ cudaError_t rs_launch_surrogate_train(float* blob, const double* X, const double
         // order the graph after the setup work on st
         cudaEventRecord(ev, st);
         cudaStreamWaitEvent(cap, ev, 0);
-        for (int64_t s = 0; s < steps && e == cudaSuccess; ++s) {
-            e = cudaGraphLaunch(ge, cap);
-            if (e == cudaSuccess)
-                e = cudaMemcpyAsync(loss_curve + s, slot, sizeof(float), cudaMemcpyDeviceToDevice, cap);
-        }
+        for (int64_t s = 0; s < steps && e == cudaSuccess; ++s) e = cudaGraphLaunch(ge, cap);
         cudaEventRecord(ev, cap);
         cudaStreamWaitEvent(st, ev, 0);
         cudaEventDestroy(ev);
@@ -672,8 +735,7 @@ cudaError_t rs_launch_surrogate_infer(const float* blob, const double* X, int64_
     a.thr = ood_thr;
     a.score = score;
     a.fallback = fallback;
-    a.out = EpiOutput{blob + Blob::ob3, nullptr, nullptr, nullptr, nullptr, 0, 0.f, pred, masks, flags, k,
-                      (float)log(tau), rec_code, rec_pred};
+    a.out = EpiInfer{blob + Blob::ob3, pred, masks, flags, k, (float)log(tau), rec_code, rec_pred};
     a.err = err;
     const int64_t tiles = (n + 127) / 128;
     mlp_infer_kernel<<<(unsigned)(tiles < sms ? tiles : sms), kInfThreads, kInfSmem, st>>>(tW1, tW2, tW3, a);

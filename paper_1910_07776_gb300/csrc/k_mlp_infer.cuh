@@ -48,7 +48,7 @@ struct InferArgs {
     float thr;
     float* score;
     uint8_t* fallback;
-    EpiOutput out;           // rows from 0
+    EpiInfer out;            // rows from 0
     int* err;
 };
 
@@ -59,42 +59,6 @@ __device__ __forceinline__ unsigned trunc_bits(double x, unsigned& range) {
     const unsigned d = (hi & 0x7fffffffu) - (898u << 20);
     range = range > d ? range : d;
     return ((__funnelshift_l(lo, hi, 3) - (896u << 23)) & 0x7fffffffu) | (hi & 0x80000000u);
-}
-
-// Two FP32 operations in one instruction, each rounded as by itself.
-__device__ __forceinline__ unsigned long long pk2(float a, float b) {
-    unsigned long long r;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-    return r;
-}
-__device__ __forceinline__ void un2(unsigned long long v, float& a, float& b) {
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
-    unsigned long long r;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ unsigned long long mul2(unsigned long long a, unsigned long long b) {
-    unsigned long long r;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-    return r;
-}
-__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
-    unsigned long long r;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-    return r;
-}
-// gelu_f of two values v + bias, in its operations and order, as a BF16 pair.
-__device__ __forceinline__ unsigned gelu2(unsigned v0, unsigned v1, float b0, float b1) {
-    const unsigned long long u = add2(pk2(__uint_as_float(v0), __uint_as_float(v1)), pk2(b0, b1));
-    const unsigned long long x = mul2(pk2(kGeluC, kGeluC), fma2(mul2(mul2(pk2(kGeluA, kGeluA), u), u), u, u));
-    float x0, x1, y0, y1;
-    un2(x, x0, x1);
-    const unsigned long long y = mul2(mul2(pk2(0.5f, 0.5f), u), add2(pk2(1.0f, 1.0f), pk2(tanh_hw(x0), tanh_hw(x1))));
-    un2(y, y0, y1);
-    const __nv_bfloat162 h = __floats2bfloat162_rn(y0, y1);
-    return *reinterpret_cast<const unsigned*>(&h);
 }
 
 // tcgen05.mma of BF16 tiles whose 128-byte-swizzle descriptors differ only in the start address: the
@@ -329,8 +293,8 @@ mlp_infer_kernel(const __grid_constant__ CUtensorMap tW1, const __grid_constant_
                 for (int c = 0; c < 8; ++c) {
                     const float4 bv = bias[c];
                     const int q = c >> 2, j = c & 3;
-                    h[q][2 * j] = gelu2(r[q][4 * j], r[q][4 * j + 1], bv.x, bv.y);
-                    h[q][2 * j + 1] = gelu2(r[q][4 * j + 2], r[q][4 * j + 3], bv.z, bv.w);
+                    h[q][2 * j] = gelu2(add2(pk2(__uint_as_float(r[q][4 * j]), __uint_as_float(r[q][4 * j + 1])), pk2(bv.x, bv.y)));
+                    h[q][2 * j + 1] = gelu2(add2(pk2(__uint_as_float(r[q][4 * j + 2]), __uint_as_float(r[q][4 * j + 3])), pk2(bv.z, bv.w)));
                 }
                 if (x < 8) {
                     tmem_st8(trow + k * 32 + half * 16, h[0]);
@@ -377,7 +341,7 @@ mlp_infer_kernel(const __grid_constant__ CUtensorMap tW1, const __grid_constant_
             __syncwarp();
             if (lane == 0) mbar_arrive(d3empty);
             const int64_t r = ((int64_t)blockIdx.x + (int64_t)it * gridDim.x) * 128 + quarter * 32 + lane;
-            if (r < a.n) a.out(r, 0, v);
+            if (r < a.n) a.out(r, v);
         };
         uint32_t it = 0;
         for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x, ++it) {

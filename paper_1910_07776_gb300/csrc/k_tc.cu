@@ -71,24 +71,6 @@ cudaError_t rs_make_tmap_bf16_3d(CUtensorMap* map, const void* ptr, int64_t batc
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-cudaError_t rs_make_tmap_bf16_kslices(CUtensorMap* map, const void* ptr, int64_t rows, int64_t K, int64_t ld,
-                                      int slices, int box_rows) {
-    std::call_once(g_encode_once, load_encode);
-    if (!g_encode) return cudaErrorNotSupported;
-    if (slices < 1 || rows < 1 || K < slices || K % slices || ld < K || (ld * 2) % 16 != 0 ||
-        ((K / slices) * 2) % 16 != 0 || ((uintptr_t)ptr % 16) != 0)
-        return cudaErrorInvalidValue;
-    const int64_t ks = K / slices;
-    cuuint64_t dims[3] = {(cuuint64_t)ks, (cuuint64_t)rows, (cuuint64_t)slices};
-    cuuint64_t strides[2] = {(cuuint64_t)(ld * 2), (cuuint64_t)(ks * 2)};
-    cuuint32_t box[3] = {(cuuint32_t)tc::BK, (cuuint32_t)box_rows, 1};
-    cuuint32_t estr[3] = {1, 1, 1};
-    CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(ptr), dims, strides, box,
-                          estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
-}
-
 template <int BN>
 static cudaError_t launch_store(const CUtensorMap& ta, const CUtensorMap& tb, int M, int N, int K, float* D,
                                 int64_t ldd, int* err, cudaStream_t st) {

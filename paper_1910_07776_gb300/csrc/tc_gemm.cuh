@@ -96,9 +96,22 @@ __device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
     d |= (uint64_t)2 << 61;                           // 128-byte swizzle
     return d;
 }
-// Instruction descriptor: BF16 x BF16 -> FP32, both operands K-major, M x N.
-__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+// The same of an MN-major tile (a row-major [K][units] matrix taken over its units): boxes of 64 units x
+// 64 of K, one after the other, each as a TMA load with the 128-byte swizzle writes it.  Units 64 apart
+// lie one box (8192 B) apart, groups of 8 of K 1024 B.
+__device__ __forceinline__ uint64_t sw128_desc_mn(uint32_t saddr) {
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)(8192 >> 4) << 16;                 // leading byte offset: the next 64 units
+    d |= (uint64_t)(1024 >> 4) << 32;                 // stride byte offset: the next 8 of K
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)2 << 61;
+    return d;
+}
+// Instruction descriptor: BF16 x BF16 -> FP32, M x N, each operand K-major or (mn) MN-major.
+__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, bool a_mn = false, bool b_mn = false) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)a_mn << 15) | ((uint32_t)b_mn << 16) |
+           ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 template <int BN, int STAGES>
@@ -113,10 +126,8 @@ struct Layout {
 constexpr int kEpiWarps = 8;                          // two per TMEM lane quarter
 constexpr int kGemmThreads = (2 + kEpiWarps) * 32;    // producer, MMA issuer, epilogue
 
-// Persistent, warp-specialised GEMM over all 128 x BN output tiles of all batches (tile t of
-// the CTA's static round-robin: t = blockIdx.x, + gridDim.x, ...; N-blocks fastest, so the
-// CTAs working at the same time share their A tiles -- the large, streamed operand -- in L2
-// and each is read from DRAM once; the B operands here are weights, L2-resident).
+// Persistent, warp-specialised product over the tiles of a problem (tile t of the CTA's static
+// round-robin: t = blockIdx.x, + gridDim.x, ...), D = A B^T.
 //   warp 0 (one thread): TMA producer -- a STAGES-deep shared-memory ring of 128 x 64 A and
 //     BN x 64 B slices (128-byte swizzle) running ahead across tile boundaries;
 //   warp 1 (one thread): MMA issuer -- tcgen05.mma (M = 128, N = BN, K = 16) into one of two
@@ -129,14 +140,12 @@ constexpr int kGemmThreads = (2 + kEpiWarps) * 32;    // producer, MMA issuer, e
 // (barriers, tensor-memory allocation) is paid once.  Every mbarrier wait is bounded (1 s);
 // a wait that gives up sets RS_ETIMEOUT, the role leaves its loop, the producer waits
 // (bounded) for its loads still in flight, and the CTA frees its tensor memory and returns.
-// Epi: __device__ void operator()(int row, int col0, const float (&v)[16]) const, called for
-// every row < M with the 16 accumulator columns starting at col0 (col0 < N).  BATCHED: the
-// operands are rank-3 tensor maps [batch][rows][K] and the functor is called as
-// epi(z, row, col0, v).
-template <int BN, int STAGES, class Epi, bool BATCHED = false>
-__global__ void __launch_bounds__(kGemmThreads, 1)
-gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb, int M, int N,
-            int K, int batch, Epi epi, int* err) {
+// Prob: kAmn, kBmn (operands MN-major), tiles(), tile(t) -> a Tile with m0, n0 (the tile's first row
+// and column), N (columns of its product) and nk (k-blocks), load(tile, kb, a, b, bar) (the TMA loads of
+// one stage) and emit(tile, row, col0, v), called by whole warps for the 16 accumulator columns from
+// col0 < N (rows may lie beyond the product).
+template <int BN, int STAGES, class Prob>
+__device__ __forceinline__ void gemm_core(const Prob& prob, int* err) {
     using L = Layout<BN, STAGES>;
     static_assert(BN % 16 == 0 && BN >= 32 && BN <= 256 && (BN & (BN - 1)) == 0, "BN: 32..256, power of 2");
     extern __shared__ uint8_t smem_raw[];
@@ -146,15 +155,13 @@ gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUte
     // barriers: full[S], empty[S], tfull[2], tempty[2], drain; then the tensor-memory slot
     const uint32_t bars = base + STAGES * L::kStage;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(gbase + STAGES * L::kStage + 8 * (2 * STAGES + 5));
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     auto full = [&](int s) { return bars + 8u * s; };
     auto empty = [&](int s) { return bars + 8u * (STAGES + s); };
     auto tfull = [&](int a) { return bars + 8u * (2 * STAGES + a); };
     auto tempty = [&](int a) { return bars + 8u * (2 * STAGES + 2 + a); };
     const uint32_t drain = bars + 8u * (2 * STAGES + 4);
-    const int mt = (M + BM - 1) / BM, nt = (N + BN - 1) / BN;
-    const long long tiles = (long long)mt * nt * batch;
-    const int nk = (K + BK - 1) / BK;
+    const long long tiles = prob.tiles();
 
     if (tid == 0) {
         for (int s = 0; s < STAGES; ++s) {
@@ -178,14 +185,12 @@ gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUte
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {                             // ---- TMA producer
+        if (elect_one()) {                           // ---- TMA producer
             long long kg = 0;                        // k-blocks issued by this CTA
             bool ok = true;
             for (long long t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
-                const int z = (int)(t / ((long long)mt * nt));
-                const int rem = (int)(t - (long long)z * mt * nt);
-                const int m0 = (rem / nt) * BM, n0 = (rem % nt) * BN;
-                for (int kb = 0; kb < nk; ++kb, ++kg) {
+                const auto tile = prob.tile(t);
+                for (int kb = 0; kb < tile.nk; ++kb, ++kg) {
                     const int s = (int)(kg % STAGES);
                     const long long j = kg / STAGES;
                     if (j >= 1 && !mbar_wait(empty(s), (uint32_t)((j - 1) & 1), err, 11)) {
@@ -194,13 +199,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUte
                     }
                     const uint32_t a = base + s * L::kStage, b = a + L::kA;
                     mbar_expect_tx(full(s), L::kStage);
-                    if (BATCHED) {
-                        tma_load_3d(a, &ta, full(s), kb * BK, m0, z);
-                        tma_load_3d(b, &tb, full(s), kb * BK, n0, z);
-                    } else {
-                        tma_load_2d(a, &ta, full(s), kb * BK, m0);
-                        tma_load_2d(b, &tb, full(s), kb * BK, n0);
-                    }
+                    prob.load(tile, kb, a, b, full(s));
                 }
             }
             if (!ok)   // wait (bounded) for this CTA's loads that may still be in flight
@@ -208,8 +207,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUte
                     mbar_wait(full((int)(q % STAGES)), (uint32_t)((q / STAGES) & 1), err, 12);
         }
     } else if (warp == 1) {
-        if (lane == 0) {                             // ---- MMA issuer
-            const uint32_t idesc = idesc_bf16(BM, BN);
+        if (elect_one()) {                           // ---- MMA issuer
+            constexpr uint32_t idesc = idesc_bf16(BM, BN, Prob::kAmn, Prob::kBmn);
             long long kg = 0;
             int tl = 0;
             bool ok = true;
@@ -221,6 +220,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUte
                 }
                 fence_after();
                 const uint32_t d = tmem + (uint32_t)(acc * BN);
+                const int nk = prob.tile(t).nk;
                 for (int kb = 0; kb < nk; ++kb, ++kg) {
                     const int s = (int)(kg % STAGES);
                     if (!mbar_wait(full(s), (uint32_t)((kg / STAGES) & 1), err, 14)) {
@@ -231,7 +231,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUte
                     const uint32_t a = base + s * L::kStage, b = a + L::kA;
 #pragma unroll
                     for (int kk = 0; kk < BK / 16; ++kk)
-                        mma_bf16(d, sw128_desc(a + kk * 32), sw128_desc(b + kk * 32), idesc, (kb | kk) != 0);
+                        mma_bf16(d, Prob::kAmn ? sw128_desc_mn(a + kk * 2048) : sw128_desc(a + kk * 32),
+                                 Prob::kBmn ? sw128_desc_mn(b + kk * 2048) : sw128_desc(b + kk * 32), idesc,
+                                 (kb | kk) != 0);
                     mma_commit(empty(s));
                 }
                 if (ok) mma_commit(tfull(acc));
@@ -251,10 +253,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUte
             ok = __shfl_sync(0xffffffffu, ok, 0);
             if (!ok) break;
             fence_after();
-            const int z = (int)(t / ((long long)mt * nt));
-            const int rem = (int)(t - (long long)z * mt * nt);
-            const int m0 = (rem / nt) * BM, n0 = (rem % nt) * BN;
-            const int row = m0 + quarter * 32 + lane;
+            const auto tile = prob.tile(t);
+            const int n0 = tile.n0, N = tile.N, row = tile.m0 + quarter * 32 + lane;
             const uint32_t trow = tmem + (uint32_t)(acc * BN) + ((uint32_t)(quarter * 32) << 16);
             // this warp's columns: all their tensor-memory loads in flight, then one wait
             constexpr int kChunks = BN / 32;
@@ -274,10 +274,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUte
                 float v[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[q][i]);
-                if (row < M) {
-                    if constexpr (BATCHED) epi(z, row, n0 + c0 + 16 * q, v);
-                    else epi(row, n0 + c0 + 16 * q, v);
-                }
+                prob.emit(tile, row, n0 + c0 + 16 * q, v);
             }
         }
     }
@@ -286,13 +283,73 @@ gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUte
     if (warp == 0) tmem_dealloc(tmem, 2 * BN);
 }
 
+// All 128 x BN output tiles of all batches of one product (N-blocks fastest, so the CTAs working at the
+// same time share their A tiles -- the large, streamed operand -- in L2 and each is read from DRAM
+// once; the B operands here are weights, L2-resident).  Epi: __device__ void operator()(int row,
+// int col0, const float (&v)[16]) const, called for every row < M; BATCHED: the operands are rank-3
+// tensor maps [batch][rows][K] and the functor is called as epi(z, row, col0, v).  BMN: B is a row-major
+// [K][N] matrix with boxes of 64 rows (BN 64 or 128).  An Epi with kWarp = true is called by whole warps,
+// as epi(row, row < M, col0, v).
+template <class Epi, class = void>
+struct WholeWarp { static constexpr bool value = false; };
+template <class Epi>
+struct WholeWarp<Epi, decltype((void)Epi::kWarp)> { static constexpr bool value = Epi::kWarp; };
+
+template <int BN, class Epi, bool BATCHED, bool BMN>
+struct PlainProb {
+    static constexpr bool kAmn = false, kBmn = BMN;
+    struct Tile { int m0, n0, z, N, nk; };
+    const CUtensorMap* ta;
+    const CUtensorMap* tb;
+    int M, N, K, batch;
+    const Epi& epi;
+    __device__ long long tiles() const { return (long long)((M + BM - 1) / BM) * ((N + BN - 1) / BN) * batch; }
+    __device__ Tile tile(long long t) const {
+        const int mt = (M + BM - 1) / BM, nt = (N + BN - 1) / BN;
+        const int z = BATCHED ? (int)(t / ((long long)mt * nt)) : 0;
+        const int rem = (int)(t - (long long)z * mt * nt);
+        return Tile{(rem / nt) * BM, (rem % nt) * BN, z, N, (K + BK - 1) / BK};
+    }
+    __device__ void load(const Tile& t, int kb, uint32_t a, uint32_t b, uint32_t bar) const {
+        if constexpr (BATCHED) {
+            tma_load_3d(a, ta, bar, kb * BK, t.m0, t.z);
+            tma_load_3d(b, tb, bar, kb * BK, t.n0, t.z);
+        } else {
+            tma_load_2d(a, ta, bar, kb * BK, t.m0);
+            if constexpr (BMN) {
+#pragma unroll
+                for (int q = 0; q < BN / 64; ++q) tma_load_2d(b + q * 8192, tb, bar, t.n0 + 64 * q, kb * BK);
+            } else {
+                tma_load_2d(b, tb, bar, kb * BK, t.n0);
+            }
+        }
+    }
+    __device__ void emit(const Tile& t, int row, int col0, const float (&v)[16]) const {
+        if constexpr (WholeWarp<Epi>::value) {
+            epi(row, row < M, col0, v);
+        } else if (row < M) {
+            if constexpr (BATCHED) epi(t.z, row, col0, v);
+            else epi(row, col0, v);
+        }
+    }
+};
+
+template <int BN, int STAGES, class Epi, bool BATCHED = false, bool BMN = false>
+__global__ void __launch_bounds__(kGemmThreads, 1)
+gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb, int M, int N,
+            int K, int batch, const __grid_constant__ Epi epi, int* err) {
+    static_assert(!BMN || (!BATCHED && BN >= 64), "MN-major B: boxes of 64 columns");
+    const PlainProb<BN, Epi, BATCHED, BMN> p{&ta, &tb, M, N, K, batch, epi};
+    gemm_core<BN, STAGES>(p, err);
+}
+
 // Launches gemm_kernel over all tiles of `batch` products, one persistent CTA per SM (at most
 // one per tile).  The function attribute (dynamic shared memory) is set unless the stream is
 // capturing a graph (the callers set it once beforehand).
-template <int BN, int STAGES, class Epi, bool BATCHED = false>
+template <int BN, int STAGES, class Epi, bool BATCHED = false, bool BMN = false>
 cudaError_t gemm_launch(const CUtensorMap& ta, const CUtensorMap& tb, int M, int N, int K, int batch,
                         const Epi& epi, int* err, cudaStream_t st) {
-    auto kern = gemm_kernel<BN, STAGES, Epi, BATCHED>;
+    auto kern = gemm_kernel<BN, STAGES, Epi, BATCHED, BMN>;
     const int smem = Layout<BN, STAGES>::kBytes;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     cudaError_t e = cudaStreamIsCapturing(st, &cs);
@@ -324,8 +381,3 @@ cudaError_t rs_make_tmap_bf16(CUtensorMap* map, const void* ptr, int64_t rows, i
 // box = 64 columns x box_rows rows x 1 batch; rows beyond `rows` read as zero.
 cudaError_t rs_make_tmap_bf16_3d(CUtensorMap* map, const void* ptr, int64_t batch, int64_t rows, int64_t cols,
                                  int64_t ld, int box_rows);
-// A [rows][K] BF16 operand (row stride ld) seen as `slices` consecutive K ranges of K / slices
-// columns: a rank-3 map (K / slices, rows, slices) whose third coordinate selects the range
-// (split-K with the batched GEMM kernel).  K / slices * 2 bytes must be a multiple of 16.
-cudaError_t rs_make_tmap_bf16_kslices(CUtensorMap* map, const void* ptr, int64_t rows, int64_t K, int64_t ld,
-                                      int slices, int box_rows);

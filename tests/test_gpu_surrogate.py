@@ -249,3 +249,48 @@ def test_inference_at_the_edges_of_its_tiles(env, n):
     eps = 2.0 ** -23
     tol = (2 * np.abs(d) * (2 * np.abs(X[fine]) + 2 * np.abs(mean)) / sd).mean(1) * eps + (2 * 4 + 14) * eps * ref
     assert (np.abs(score[fine] - ref) <= tol).all()
+
+
+@pytest.mark.parametrize("B", [16, 40, 128, 136, 504, 512, 1000, 1024])
+def test_a_step_at_the_edges_of_its_tiles(env, B):
+    # Gradients, loss and the AdamW update at batches around the 32, 64 and 128 rows of the kernels'
+    # tiles and at one and several row ranges of the weight gradients; the minibatch wraps around.
+    # BF16 operands (relative error 2^-9 each, tanh 2^-11) in chains of up to three layers: 3e-2.
+    rs, ctx = env
+    n = B + 24
+    X, Y, Xd, Yd = data(n, B)
+    Y[3, 2] = np.nan
+    X[5, :4] = [0.0, 1e-310, -1e-40, 3e20]
+    X[6, 7] = -0.0
+    Xd, Yd = torch.from_numpy(X).cuda(), torch.from_numpy(Y).cuda()
+    p = mlp.init_params(3)
+    p["W1"][:, 3] = 0.0                                   # (the large value meets no weight)
+    sur = rs.Surrogate(ctx, B)
+    sur.load(p)
+    lc = torch.zeros(2, dtype=torch.float32, device="cuda")
+    sur.train(Xd, Yd, steps=1, lr=0.0, use_graph=False, loss_curve=lc)
+    torch.cuda.synchronize()
+    ctx.check_device_status()
+    Yz = np.where(np.isfinite(Y), Y, 0.0)
+    loss, g = mlp.loss_and_grads(ref_params(p), bf16(X[:B]), Yz[:B])
+    assert abs(float(lc[0]) - loss) <= 2e-2 * loss
+    for k in mlp.NAMES:
+        gg = sur.view(k, "grad").cpu().numpy().astype(np.float64)
+        if k in ("W3", "b3"):
+            assert np.all(gg[6:] == 0)
+            gg = gg[:6]
+        if k == "W1":                                     # (its input is 1e20 times the others')
+            gg, g[k] = np.delete(gg, 3, axis=1), np.delete(g[k], 3, axis=1)
+        c, r = cos_rel(gg, g[k])
+        assert c >= 0.999 and r <= 3e-2, (k, c, r)
+    # a second call continues: graph replays equal eager steps, bit for bit
+    other = rs.Surrogate(ctx, B)
+    other.load(p)
+    other.train(Xd, Yd, steps=1, lr=0.0, use_graph=False)
+    la, lb = torch.zeros(3, device="cuda"), torch.zeros(3, device="cuda")
+    sur.train(Xd, Yd, steps=3, lr=1e-3, use_graph=True, loss_curve=la)
+    other.train(Xd, Yd, steps=3, lr=1e-3, use_graph=False, loss_curve=lb)
+    torch.cuda.synchronize()
+    np.testing.assert_array_equal(la.cpu().numpy(), lb.cpu().numpy())
+    for k in mlp.NAMES:
+        np.testing.assert_array_equal(sur.view(k).cpu().numpy(), other.view(k).cpu().numpy())
