@@ -4,7 +4,7 @@
 // FP32 accumulation; FP32 master weights with AdamW.
 //
 // One training step (a fixed sequence, captured once in a CUDA graph and replayed):
-//   stage    rows of X (double) -> BF16 X_s [B][256]; labels -> Y_s
+//   stage    rows of X (double) -> BF16 X_s [B][256]; labels -> Y_s  (within the step before's update)
 //   fwd 1,2  U = X W^T + b (FP32, kept for the backward pass), H = gelu(U) (BF16)
 //   fwd 3    out = H2 W3^T + b3; residual; loss; dO = 2 (out - y) / (6B) (BF16)
 //   dgrad    dU2 = (dO W3) * gelu'(U2);  dU1 = (dU2 W2) * gelu'(U1)   (BF16)
@@ -12,7 +12,7 @@
 //   update   gradients (partials added and bias columns summed in a fixed order), AdamW, BF16 weights
 // The tensor cores take an operand with either its K or its rows contiguous, so the weight gradients
 // read the activations, and the data gradients the weights, as they lie: nothing is transposed.
-// A step of 8,192 rows: 175 -> 75 us (before: 16 launches, with transposed copies of every operand
+// A step of 8,192 rows: 175 -> 61 us (before: 16 launches, with transposed copies of every operand
 // written 2 bytes at a time, the sums over rows in three kernels of 11 us each, one atomic addition to
 // the loss a row).
 #include <math.h>
@@ -225,16 +225,20 @@ struct EpiGeluGrad {         // dU = acc * gelu'(U) (BF16)
     const float* U;          // [unit][B]
     __nv_bfloat16* dU;
     int64_t ldu;
-    __device__ void operator()(int row, int col0, const float (&v)[16]) const {
+    struct Fetched { float u[16]; };
+    __device__ Fetched fetch(int row, bool in, int col0) const {
         const float* u = U + (int64_t)col0 * ldu + row;
-        float g[16];
+        Fetched f;
+#pragma unroll
+        for (int i = 0; i < 16; ++i) f.u[i] = in ? u[(int64_t)i * ldu] : 0.f;
+        return f;
+    }
+    __device__ void operator()(int row, int col0, const float (&v)[16], const Fetched& f) const {
         unsigned h[8];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) g[i] = u[(int64_t)i * ldu];
-#pragma unroll
         for (int i = 0; i < 8; ++i) {
-            const __nv_bfloat162 p = __floats2bfloat162_rn(v[2 * i] * gelu_grad_f(g[2 * i]),
-                                                           v[2 * i + 1] * gelu_grad_f(g[2 * i + 1]));
+            const __nv_bfloat162 p = __floats2bfloat162_rn(v[2 * i] * gelu_grad_f(f.u[2 * i]),
+                                                           v[2 * i + 1] * gelu_grad_f(f.u[2 * i + 1]));
             h[i] = *reinterpret_cast<const unsigned*>(&p);
         }
         st32(dU + (int64_t)row * kHid + col0, h);
@@ -245,11 +249,19 @@ struct EpiGeluGrad {         // dU = acc * gelu'(U) (BF16)
 constexpr int kStages = 4;
 
 // The three weight gradients as one problem: each D = A^T B over a range of the batch's rows, A and B
-// row-major, D's partial sums (one per range) in FP32.  28 tiles of 128 x 128 a range.
+// row-major, D's partial sums (one per range) in FP32.  28 tiles of 128 x 128 a range.  Four further
+// warps a CTA start the bias gradients: a column of dU in 32 chains, chain l the rows l, l + 32, ... in
+// order, two columns a lane (in the update kernel the chains took 20 us, the weights beside them 10).
+constexpr int kWgradExtra = 4;
 struct Wgrad {
     float* d[3];             // of W1, W2, W3; range z at + z * zstride
     int64_t zstride;
     int slices, rows;        // ranges, rows of each
+    const __nv_bfloat16* du[3];      // dU1, dU2 [B][512], dO [B][16]
+    float* chain[3];         // [min(B, 32)][512], the same, [min(B, 32)][16]
+    int B;
+    int* counters;           // minibatch, Adam's step, and at 8 the call's: counted here
+    int64_t steps_per_epoch;
 };
 struct WgradProb {
     static constexpr bool kAmn = true, kBmn = true;
@@ -271,7 +283,32 @@ struct WgradProb {
         tc::tma_load_2d(sb, b, bar, t.n0, y);
         tc::tma_load_2d(sb + 8192, b, bar, t.n0 + 64, y);
     }
-    __device__ void emit(const Tile& t, int row, int col0, const float (&v)[16]) const {
+    using Fetched = tc::Nothing;
+    __device__ Fetched fetch(const Tile&, int, int) const { return Fetched{}; }
+    __device__ void extra(int warp, int lane) const {
+        const int chains = g.B < 32 ? g.B : 32;
+        if (blockIdx.x == 0 && warp == 0 && lane == 0) {
+            g.counters[0] = (int)((g.counters[0] + 1) % g.steps_per_epoch);
+            g.counters[1] += 1;
+            g.counters[8] += 1;
+        }
+        for (int w = blockIdx.x + gridDim.x * warp; w < 17 * chains; w += gridDim.x * kWgradExtra) {
+            const int l = w / 17, j = w % 17;              // 64 columns of dU1, of dU2; dO's 16
+            if (j == 16 && lane >= kOutP / 2) continue;
+            const int ld = j == 16 ? kOutP : kHid, c = (j & 7) * 64 * (j < 16) + 2 * lane;
+            const __nv_bfloat16* src = (j < 8 ? g.du[0] : j < 16 ? g.du[1] : g.du[2]) + c;
+            float s0 = 0.f, s1 = 0.f;
+#pragma unroll 32
+            for (int r = l; r < g.B; r += 32) {
+                const unsigned p = *reinterpret_cast<const unsigned*>(src + (int64_t)r * ld);
+                s0 += __uint_as_float(p << 16);
+                s1 += __uint_as_float(p & 0xffff0000u);
+            }
+            float* d = (j < 8 ? g.chain[0] : j < 16 ? g.chain[1] : g.chain[2]) + l * ld + c;
+            *reinterpret_cast<float2*>(d) = make_float2(s0, s1);
+        }
+    }
+    __device__ void emit(const Tile& t, int row, int col0, const float (&v)[16], const Fetched&) const {
         if (t.w == 2 && row >= kOutP) return;
         float* d = (t.w == 0 ? g.d[0] : t.w == 1 ? g.d[1] : g.d[2]) + t.z * g.zstride + (int64_t)row * t.N + col0;
         unsigned h[2][8];
@@ -281,7 +318,8 @@ struct WgradProb {
         st32(d + 8, h[1]);
     }
 };
-__global__ void __launch_bounds__(tc::kGemmThreads, 1)
+constexpr int kWgradThreads = tc::kGemmThreads<128> + 32 * kWgradExtra;
+__global__ void __launch_bounds__(kWgradThreads, 1)
 wgrad_kernel(const __grid_constant__ CUtensorMap dU1, const __grid_constant__ CUtensorMap X,
              const __grid_constant__ CUtensorMap dU2, const __grid_constant__ CUtensorMap H1,
              const __grid_constant__ CUtensorMap dO, const __grid_constant__ CUtensorMap H2,
@@ -320,28 +358,35 @@ __device__ __forceinline__ float f32_of(double x) {
     const unsigned l = lo + 0x0fffffffu + ((lo >> 29) & 1u), h = hi + (l < lo);
     return __uint_as_float(((__funnelshift_l(l, h, 3) - (896u << 23)) & 0x7fffffffu) | (hi & 0x80000000u));
 }
-// Stage a minibatch, a warp a row: rows (r0 + i) mod n of X (double [n][256]) -> BF16 X_s, labels
-// (double [n][6], NaN treated as 0 with zero weight) -> Y_s [B][16].  r0 = minibatch * B, read from the
-// device counter so that the same launch serves every step of a graph.  Also counts the step: Adam's,
-// and the call's (run).
-__global__ void __launch_bounds__(256)
-stage_kernel(const double* __restrict__ X, const double* __restrict__ Yin, int64_t n, int B, int* counters,
-             int* run, __nv_bfloat16* Xs, float* Ys) {
-    const int lane = threadIdx.x & 31, i = blockIdx.x * 8 + (threadIdx.x >> 5);     // batch row
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        counters[1] += 1;
-        *run += 1;
+// Stage a minibatch, a warp a row (eight a block): rows (q B + i) mod n of X (double [n][256]) -> BF16 X_s,
+// labels (double [n][6], NaN treated as 0 with zero weight) -> Y_s [B][16].  q is read from the device
+// counter, so that the same launch serves every step of a graph.
+struct Stage {
+    const double* X;
+    const double* Y;
+    int64_t n;
+    int B;
+    const int* counters;
+    __nv_bfloat16* Xs;
+    float* Ys;
+    int blocks() const { return (B + 7) / 8; }
+    __device__ void operator()(int block) const {
+        const int lane = threadIdx.x & 31, i = block * 8 + (threadIdx.x >> 5);      // batch row
+        if (i >= B) return;
+        const int64_t src = ((int64_t)counters[0] * B + i) % n;
+        double x[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) x[e] = X[src * kIn + 32 * e + lane];
+        double y = 0.0;
+        if (lane < kOut) y = Y[src * kOut + lane];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) Xs[(int64_t)i * kIn + 32 * e + lane] = __float2bfloat16(f32_of(x[e]));
+        if (lane < kOutP) Ys[(int64_t)i * kOutP + lane] = isfinite(y) ? (float)y : 0.f;
     }
-    if (i >= B) return;
-    const int64_t src = ((int64_t)counters[0] * B + i) % n;
-    double x[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) x[e] = X[src * kIn + 32 * e + lane];
-    double y = 0.0;
-    if (lane < kOut) y = Yin[src * kOut + lane];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) Xs[(int64_t)i * kIn + 32 * e + lane] = __float2bfloat16(f32_of(x[e]));
-    if (lane < kOutP) Ys[(int64_t)i * kOutP + lane] = isfinite(y) ? (float)y : 0.f;
+};
+__global__ void __launch_bounds__(256)
+stage_kernel(const __grid_constant__ Stage s) {
+    s(blockIdx.x);
 }
 
 #include "k_mlp_infer.cuh"
@@ -358,10 +403,10 @@ sync_bf16_kernel(const float* __restrict__ P, __nv_bfloat16* bf) {
 
 // The step's last kernel: gradients from their partial sums (range 0 first, a fixed order, so that every
 // step and every graph replay adds the same numbers the same way), AdamW over every parameter (padded
-// output rows keep zero gradient and stay zero), the BF16 weights, the loss and the minibatch position.
-// The first kBBlocks blocks take 16 columns each of [b1 | b2 | b3]: a bias gradient sums its column of dU in
-// 32 chains (rows of one remainder mod 32 in order) and those as a tree, two columns a thread.  Then
-// four weights a thread.
+// output rows keep zero gradient and stay zero), the BF16 weights and the loss; and beside these, as they
+// share nothing, the next minibatch's staging (the call's last step stages one that a later call stages
+// again).  The first kBBlocks blocks take 16 columns each of [b1 | b2 | b3], adding their chains as a
+// tree; kWBlocks four weights a thread; the others stage.
 constexpr int kWBlocks = (int)((Blob::nW1 + Blob::nW2 + Blob::nW3) / 4 + 255) / 256, kBBlocks = 2 * kHid / 16 + 1;
 struct Update {
     float* blob;
@@ -369,14 +414,13 @@ struct Update {
     const float* w[3];       // partial sums of dW1, dW2, dW3, ranges zstride apart
     int64_t zstride;
     int slices;
-    const __nv_bfloat16* d[3];       // dU1, dU2 [B][512] and dO [B][16]
+    const float* chain[3];   // of the columns of dU1, dU2 and dO
     int B;
     const float* loss_part;  // [rows of 32]
     float lr, wd;
-    int* counters;
-    int64_t steps_per_epoch;
-    const int* run;
+    const int* counters;
     float* loss_curve;
+    Stage next;
 };
 __device__ __forceinline__ float adamw(const Update& a, float p, float g, float& m, float& v, float c1, float c2) {
     constexpr float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
@@ -390,16 +434,28 @@ __global__ void __launch_bounds__(256)
 update_kernel(const __grid_constant__ Update a) {
     __shared__ float corr[2], red[32][17];
     const int tid = threadIdx.x;
+    tc::let_successor();
+    tc::after_predecessor();
+    if ((int)blockIdx.x >= kBBlocks + kWBlocks) {
+        a.next(blockIdx.x - kBBlocks - kWBlocks);
+        return;
+    }
     if (tid < 2) corr[tid] = 1.f - powf(tid ? 0.999f : 0.9f, (float)a.counters[1]);
     if ((int)blockIdx.x >= kBBlocks) {
         const int64_t i = ((int64_t)(blockIdx.x - kBBlocks) * 256 + tid) * 4;
         const int k = i < Blob::nW1 ? 0 : i < Blob::nW1 + Blob::nW2 ? 1 : 2;
         const int64_t j = i - (k == 0 ? 0 : k == 1 ? Blob::nW1 : Blob::nW1 + Blob::nW2);      // within its matrix
         const bool in = i < Blob::nW1 + Blob::nW2 + Blob::nW3;
-        float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+        const int64_t o = (k == 0 ? Blob::oW1 : k == 1 ? Blob::oW2 : Blob::oW3) + j;
+        float4* P = reinterpret_cast<float4*>(a.blob + o);
+        float4 *M = P + Blob::oM / 4, *V = P + Blob::oV / 4, *G = P + Blob::oG / 4;
+        float4 s = make_float4(0.f, 0.f, 0.f, 0.f), q = s, m = s, v = s;
         if (in) {
+            q = *P;
+            m = *M;
+            v = *V;
             const float* src = (k == 0 ? a.w[0] : k == 1 ? a.w[1] : a.w[2]) + j;
-#pragma unroll 8
+#pragma unroll 16
             for (int z = 0; z < a.slices; ++z) {
                 const float4 p = *reinterpret_cast<const float4*>(src + z * a.zstride);
                 s.x += p.x;
@@ -410,10 +466,6 @@ update_kernel(const __grid_constant__ Update a) {
         }
         __syncthreads();
         if (in) {
-            const int64_t o = (k == 0 ? Blob::oW1 : k == 1 ? Blob::oW2 : Blob::oW3) + j;
-            float4* P = reinterpret_cast<float4*>(a.blob + o);
-            float4 *M = P + Blob::oM / 4, *V = P + Blob::oV / 4, *G = P + Blob::oG / 4;
-            float4 q = *P, m = *M, v = *V;
             q.x = adamw(a, q.x, s.x, m.x, v.x, corr[0], corr[1]);
             q.y = adamw(a, q.y, s.y, m.y, v.y, corr[0], corr[1]);
             q.z = adamw(a, q.z, s.z, m.z, v.z, corr[0], corr[1]);
@@ -431,16 +483,11 @@ update_kernel(const __grid_constant__ Update a) {
     }
     const int q = blockIdx.x, k = q < kHid / 16 ? 0 : q < 2 * kHid / 16 ? 1 : 2, ld = k == 2 ? kOutP : kHid;
     const int c0 = k == 2 ? 0 : (q - k * (kHid / 16)) * 16;
-    float s0 = 0.f, s1 = 0.f;
-    const __nv_bfloat16* src = (k == 0 ? a.d[0] : k == 1 ? a.d[1] : a.d[2]) + c0 + 2 * (tid & 7);
-#pragma unroll 32
-    for (int r = tid >> 3; r < a.B; r += 32) {
-        const unsigned p = *reinterpret_cast<const unsigned*>(src + (int64_t)r * ld);
-        s0 += __uint_as_float(p << 16);
-        s1 += __uint_as_float(p & 0xffff0000u);
-    }
-    red[tid >> 3][2 * (tid & 7)] = s0;
-    red[tid >> 3][2 * (tid & 7) + 1] = s1;
+    const float* src = (k == 0 ? a.chain[0] : k == 1 ? a.chain[1] : a.chain[2]) + c0 + 2 * (tid & 7);
+    float2 s = make_float2(0.f, 0.f);
+    if ((tid >> 3) < a.B) s = *reinterpret_cast<const float2*>(src + (tid >> 3) * ld);
+    red[tid >> 3][2 * (tid & 7)] = s.x;
+    red[tid >> 3][2 * (tid & 7) + 1] = s.y;
     __syncthreads();
     const int lane = tid & 31;
 #pragma unroll
@@ -464,22 +511,21 @@ update_kernel(const __grid_constant__ Update a) {
         __syncthreads();
         if (lane == 0) red[0][tid >> 5] = l;
         __syncthreads();
-        if (tid == 0) {
+        if (tid == 0 && a.loss_curve) {
             for (int w = 1; w < 8; ++w) l += red[0][w];
-            if (a.loss_curve) a.loss_curve[*a.run] = l;
-            a.counters[0] = (int)((a.counters[0] + 1) % a.steps_per_epoch);
+            a.loss_curve[a.counters[8]] = l;
         }
     }
 }
 
 // A call continues from the blob's counters (a restored checkpoint resumes the same sequence
 // of minibatches and Adam steps); the minibatch position wraps into this call's rows.
-__global__ void wrap_counters_kernel(int* counters, int64_t steps_per_epoch, int* run) {
+__global__ void wrap_counters_kernel(int* counters, int64_t steps_per_epoch) {
     int64_t q = counters[0] % steps_per_epoch;
     if (q < 0) q += steps_per_epoch;                         // (a blob not zeroed by its owner)
     counters[0] = (int)q;
     if (counters[1] < 0) counters[1] = 0;
-    *run = -1;                                               // this call's step, counted by stage_kernel
+    counters[8] = -1;                                        // this call's step
 }
 
 // Feature mean / std over the training rows (for the out-of-distribution score): each
@@ -509,9 +555,10 @@ struct TrainWs {
     __nv_bfloat16 *Xs, *H1, *H2, *dO, *dU2, *dU1;
     float *Ys, *U1, *U2;
     double* stats_acc;
-    int* run;                 // the call's step (in stats_acc, once the statistics are finished)
     float* part;              // split-K partials of the weight gradients (slices > 1)
     float* loss_part;         // sums over 32 rows
+    float* chain[3];          // bias gradients' chains: [min(B, 32)][512] where U1 and U2 were (read
+                              // before), [32][16]
     int slices;
     size_t bytes;
 };
@@ -543,7 +590,9 @@ TrainWs carve_train(void* base, int B) {
     w.U1 = (float*)take((size_t)B * kHid * sizeof(float));
     w.U2 = (float*)take((size_t)B * kHid * sizeof(float));
     w.stats_acc = (double*)take(2 * kIn * sizeof(double));
-    w.run = (int*)w.stats_acc;
+    w.chain[0] = w.U1;
+    w.chain[1] = w.U2;
+    w.chain[2] = (float*)take(32 * kOutP * sizeof(float));
     w.loss_part = (float*)take((size_t)((B + 127) / 128 * 4) * sizeof(float));
     w.slices = wgrad_slices(B);
     w.part = w.slices > 1 ? (float*)take((size_t)w.slices * (Blob::nW1 + Blob::nW2 + Blob::nW3) * sizeof(float))
@@ -583,7 +632,8 @@ cudaError_t make_maps(Maps& m, const TrainWs& w, const __nv_bfloat16* bf, int B)
 
 // Forward + backward for the staged minibatch: the weight gradients' partial sums (straight into the
 // blob's gradients when the rows are one range).
-cudaError_t step_body(float* blob, const TrainWs& w, const Maps& m, int B, int* err, cudaStream_t st) {
+cudaError_t step_body(float* blob, const TrainWs& w, const Maps& m, int B, int* counters, int64_t spe, int* err,
+                      cudaStream_t st) {
     float* G = blob + Blob::oG;
     const float* P = blob;
     const float sc = 2.0f / (6.0f * (float)B);
@@ -604,14 +654,20 @@ cudaError_t step_body(float* blob, const TrainWs& w, const Maps& m, int B, int* 
     g.zstride = Blob::nW1 + Blob::nW2 + Blob::nW3;
     g.slices = w.slices;
     g.rows = B / w.slices;
+    g.du[0] = w.dU1;
+    g.du[1] = w.dU2;
+    g.du[2] = w.dO;
+    for (int k = 0; k < 3; ++k) g.chain[k] = w.chain[k];
+    g.B = B;
+    g.counters = counters;
+    g.steps_per_epoch = spe;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     const int tiles = 28 * w.slices;
-    wgrad_kernel<<<tiles < sms ? tiles : sms, tc::kGemmThreads, tc::Layout<128, kStages>::kBytes, st>>>(
-        m.tdU1, m.tX, m.tdU2, m.tH1, m.tdO, m.tH2, g, err);
-    return cudaGetLastError();
+    return tc::launch_after(wgrad_kernel, tiles < sms ? tiles : sms, kWgradThreads, tc::Layout<128, kStages>::kBytes, st,
+                            m.tdU1, m.tX, m.tdU2, m.tH1, m.tdO, m.tH2, g, err);
 }
 
 }  // namespace
@@ -657,7 +713,9 @@ cudaError_t rs_launch_surrogate_train(float* blob, const double* X, const double
     feature_stats_kernel<<<(unsigned)(n < 1024 ? n : 1024), kIn, 0, st>>>(X, n, w.stats_acc);
     feature_stats_finish<<<1, kIn, 0, st>>>(w.stats_acc, n, blob + Blob::oStats, blob + Blob::oStats + kIn);
     sync_bf16_kernel<<<(unsigned)((Blob::nW2 + 255) / 256), 256, 0, st>>>(blob, bf);
-    wrap_counters_kernel<<<1, 1, 0, st>>>(counters, spe, w.run);
+    wrap_counters_kernel<<<1, 1, 0, st>>>(counters, spe);
+    const Stage stage{X, Y, n, B, counters, w.Xs, w.Ys};
+    stage_kernel<<<stage.blocks(), 256, 0, st>>>(stage);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     const bool split = w.slices > 1;
@@ -665,14 +723,12 @@ cudaError_t rs_launch_surrogate_train(float* blob, const double* X, const double
     const Update u{blob, bf,
                    {split ? w.part : G + Blob::oW1, split ? w.part + Blob::nW1 : G + Blob::oW2,
                     split ? w.part + Blob::nW1 + Blob::nW2 : G + Blob::oW3},
-                   Blob::nW1 + Blob::nW2 + Blob::nW3, w.slices, {w.dU1, w.dU2, w.dO}, B, w.loss_part, lr, wd, counters, spe,
-                   w.run, loss_curve};
+                   Blob::nW1 + Blob::nW2 + Blob::nW3, w.slices, {w.chain[0], w.chain[1], w.chain[2]}, B, w.loss_part, lr, wd, counters,
+                   loss_curve, stage};
     auto one_step = [&](cudaStream_t q) -> cudaError_t {
-        stage_kernel<<<(unsigned)((B + 7) / 8), 256, 0, q>>>(X, Y, n, B, counters, w.run, w.Xs, w.Ys);
-        cudaError_t e2 = step_body(blob, w, m, B, err, q);
-        if (e2 != cudaSuccess) return e2;
-        update_kernel<<<kWBlocks + kBBlocks, 256, 0, q>>>(u);
-        return cudaGetLastError();
+        cudaError_t e2 = step_body(blob, w, m, B, counters, spe, err, q);
+        if (e2 == cudaSuccess) e2 = tc::launch_after(update_kernel, kBBlocks + kWBlocks + stage.blocks(), 256, 0, q, u);
+        return e2;
     };
     if (!use_graph || !loss_curve) {
         for (int64_t s = 0; s < steps && e == cudaSuccess; ++s) e = one_step(st);

@@ -10,6 +10,8 @@
 // Every mbarrier wait is bounded (1 s of %globaltimer); a wait that gives up sets
 // RS_ETIMEOUT in the device status word and the CTA winds down without hanging.
 #pragma once
+#include <type_traits>
+
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -123,8 +125,12 @@ struct Layout {
     static constexpr int kBytes = STAGES * kStage + kBars + 1024;   // + alignment slack
 };
 
-constexpr int kEpiWarps = 8;                          // two per TMEM lane quarter
-constexpr int kGemmThreads = (2 + kEpiWarps) * 32;    // producer, MMA issuer, epilogue
+// Epilogue warps: four per TMEM lane quarter, two where a tile has 32 columns.  (Eight in all took
+// 10 to 15 us for the surrogate's 8,192 x 512 layers, sixteen 10 to 12: their loads and stores are latency.)
+template <int BN>
+constexpr int kEpiWarps = BN >= 64 ? 16 : 8;
+template <int BN>
+constexpr int kGemmThreads = (2 + kEpiWarps<BN>) * 32;    // producer, MMA issuer, epilogue
 
 // Persistent, warp-specialised product over the tiles of a problem (tile t of the CTA's static
 // round-robin: t = blockIdx.x, + gridDim.x, ...), D = A B^T.
@@ -133,17 +139,19 @@ constexpr int kGemmThreads = (2 + kEpiWarps) * 32;    // producer, MMA issuer, e
 //   warp 1 (one thread): MMA issuer -- tcgen05.mma (M = 128, N = BN, K = 16) into one of two
 //     tensor-memory accumulators, tcgen05.commit frees each stage and, after a tile's last
 //     k-block, hands the accumulator to the epilogue;
-//   warps 2..9: epilogue -- warp w reads TMEM lane quarter (w mod 4) (rows 32 (w mod 4) ..+31),
-//     half of the columns each, 16 at a time with tcgen05.ld, calls the epilogue functor and
-//     returns the accumulator to the MMA issuer.
+//   kEpiWarps from warp 2: epilogue -- warp w reads TMEM lane quarter (w mod 4) (rows 32 (w mod 4)
+//     ..+31), its part of the columns, 16 at a time with tcgen05.ld, returns the accumulator to the
+//     MMA issuer and calls the epilogue functor;
+//   any further warps: prob.extra(warp, lane), warp from 0.
 // Two accumulators let a tile's epilogue overlap the next tile's MMAs; the CTA's set-up
 // (barriers, tensor-memory allocation) is paid once.  Every mbarrier wait is bounded (1 s);
 // a wait that gives up sets RS_ETIMEOUT, the role leaves its loop, the producer waits
 // (bounded) for its loads still in flight, and the CTA frees its tensor memory and returns.
 // Prob: kAmn, kBmn (operands MN-major), tiles(), tile(t) -> a Tile with m0, n0 (the tile's first row
 // and column), N (columns of its product) and nk (k-blocks), load(tile, kb, a, b, bar) (the TMA loads of
-// one stage) and emit(tile, row, col0, v), called by whole warps for the 16 accumulator columns from
-// col0 < N (rows may lie beyond the product).
+// one stage), fetch(tile, row, col0) -> what an epilogue needs from memory, started before the wait for
+// the accumulator, and emit(tile, row, col0, v, fetched), both called by whole warps for the 16
+// accumulator columns from col0 < N (rows may lie beyond the product).
 template <int BN, int STAGES, class Prob>
 __device__ __forceinline__ void gemm_core(const Prob& prob, int* err) {
     using L = Layout<BN, STAGES>;
@@ -170,7 +178,7 @@ __device__ __forceinline__ void gemm_core(const Prob& prob, int* err) {
         }
         for (int a = 0; a < 2; ++a) {
             mbar_init(tfull(a), 1);
-            mbar_init(tempty(a), kEpiWarps);
+            mbar_init(tempty(a), kEpiWarps<BN>);
         }
         mbar_init(drain, 1);
         fence_barrier_init();
@@ -183,6 +191,8 @@ __device__ __forceinline__ void gemm_core(const Prob& prob, int* err) {
     __syncthreads();
     fence_after();
     const uint32_t tmem = *tmem_slot;
+    let_successor();
+    after_predecessor();
 
     if (warp == 0) {
         if (elect_one()) {                           // ---- TMA producer
@@ -242,23 +252,26 @@ __device__ __forceinline__ void gemm_core(const Prob& prob, int* err) {
             mma_commit(drain);
             mbar_wait(drain, 0, err, 16);
         }
-    } else {                                         // ---- epilogue
+    } else if (warp < 2 + kEpiWarps<BN>) {           // ---- epilogue
         const int quarter = warp & 3;
-        const int half = (warp - 2) >> 2;
         int tl = 0;
         for (long long t = blockIdx.x; t < tiles; t += gridDim.x, ++tl) {
             const int acc = tl & 1, u = tl >> 1;
+            const auto tile = prob.tile(t);
+            const int n0 = tile.n0, N = tile.N, row = tile.m0 + quarter * 32 + lane;
+            constexpr int kCols = BN / (kEpiWarps<BN> / 4), kChunks = kCols / 16;
+            const int c0 = ((warp - 2) >> 2) * kCols;
+            typename Prob::Fetched f[kChunks];
+#pragma unroll
+            for (int q = 0; q < kChunks; ++q)
+                if (n0 + c0 + 16 * q < N) f[q] = prob.fetch(tile, row, n0 + c0 + 16 * q);
             int ok = 1;
             if (lane == 0) ok = mbar_wait(tfull(acc), (uint32_t)(u & 1), err, 15) ? 1 : 0;
             ok = __shfl_sync(0xffffffffu, ok, 0);
             if (!ok) break;
             fence_after();
-            const auto tile = prob.tile(t);
-            const int n0 = tile.n0, N = tile.N, row = tile.m0 + quarter * 32 + lane;
             const uint32_t trow = tmem + (uint32_t)(acc * BN) + ((uint32_t)(quarter * 32) << 16);
             // this warp's columns: all their tensor-memory loads in flight, then one wait
-            constexpr int kChunks = BN / 32;
-            const int c0 = half * (BN / 2);
             uint32_t r[kChunks][16];
 #pragma unroll
             for (int q = 0; q < kChunks; ++q)
@@ -274,9 +287,11 @@ __device__ __forceinline__ void gemm_core(const Prob& prob, int* err) {
                 float v[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[q][i]);
-                prob.emit(tile, row, n0 + c0 + 16 * q, v);
+                prob.emit(tile, row, n0 + c0 + 16 * q, v, f[q]);
             }
         }
+    } else {
+        prob.extra(warp - 2 - kEpiWarps<BN>, lane);
     }
     fence_before();
     __syncthreads();
@@ -295,8 +310,17 @@ struct WholeWarp { static constexpr bool value = false; };
 template <class Epi>
 struct WholeWarp<Epi, decltype((void)Epi::kWarp)> { static constexpr bool value = Epi::kWarp; };
 
+// An Epi with a type Fetched has fetch(row, row < M, col0) -> Fetched and is called with it as last argument.
+struct Nothing {};
+template <class Epi, class = void>
+struct FetchedOf { using type = Nothing; };
+template <class Epi>
+struct FetchedOf<Epi, decltype((void)sizeof(typename Epi::Fetched))> { using type = typename Epi::Fetched; };
+
 template <int BN, class Epi, bool BATCHED, bool BMN>
 struct PlainProb {
+    using Fetched = typename FetchedOf<Epi>::type;
+    static constexpr bool kFetch = !std::is_same<Fetched, Nothing>::value;
     static constexpr bool kAmn = false, kBmn = BMN;
     struct Tile { int m0, n0, z, N, nk; };
     const CUtensorMap* ta;
@@ -324,9 +348,16 @@ struct PlainProb {
             }
         }
     }
-    __device__ void emit(const Tile& t, int row, int col0, const float (&v)[16]) const {
+    __device__ void extra(int, int) const {}
+    __device__ Fetched fetch(const Tile&, int row, int col0) const {
+        if constexpr (kFetch) return epi.fetch(row, row < M, col0);
+        else return Fetched{};
+    }
+    __device__ void emit(const Tile& t, int row, int col0, const float (&v)[16], const Fetched& f) const {
         if constexpr (WholeWarp<Epi>::value) {
             epi(row, row < M, col0, v);
+        } else if constexpr (kFetch) {
+            if (row < M) epi(row, col0, v, f);
         } else if (row < M) {
             if constexpr (BATCHED) epi(t.z, row, col0, v);
             else epi(row, col0, v);
@@ -335,7 +366,7 @@ struct PlainProb {
 };
 
 template <int BN, int STAGES, class Epi, bool BATCHED = false, bool BMN = false>
-__global__ void __launch_bounds__(kGemmThreads, 1)
+__global__ void __launch_bounds__(kGemmThreads<BN>, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb, int M, int N,
             int K, int batch, const __grid_constant__ Epi epi, int* err) {
     static_assert(!BMN || (!BATCHED && BN >= 64), "MN-major B: boxes of 64 columns");
@@ -365,8 +396,7 @@ cudaError_t gemm_launch(const CUtensorMap& ta, const CUtensorMap& tb, int M, int
     const long long tiles = (long long)((M + BM - 1) / BM) * ((N + BN - 1) / BN) * batch;
     const long long grid = tiles < sms ? tiles : sms;
     if (grid < 1) return cudaSuccess;
-    kern<<<(unsigned)grid, kGemmThreads, smem, st>>>(ta, tb, M, N, K, batch, epi, err);
-    return cudaGetLastError();
+    return launch_after(kern, (unsigned)grid, kGemmThreads<BN>, smem, st, ta, tb, M, N, K, batch, epi, err);
 }
 
 }  // namespace tc
