@@ -48,3 +48,21 @@ def test_reciprocal_and_rsqrt_within_one_ulp_of_cuda_and_exact():
         t_q = float(Decimal(1) / Decimal(float(x)).sqrt())
         assert _ulp_diff(np.array([r]), np.array([t_r]))[0] <= 1
         assert _ulp_diff(np.array([q]), np.array([t_q]))[0] <= 1
+
+
+@pytest.mark.parametrize("exponent", [-100, -1, 0, 1, 99])
+def test_reciprocal_is_rounded_once(exponent):
+    # Mantissas around the powers of two, the 24 bits of the seed and the 32-bit halves of the products:
+    # the series leaves less than 2^-63 of the value before the one rounding, so the result is the
+    # correctly rounded one but for ties that close (2^-10 of a unit: one in 500 at random).
+    from paper_1910_07776_gb300 import build, rs
+    build.build()
+    k = np.arange(2048, dtype=np.uint64)
+    top = np.uint64((1 << 52) - 1)
+    m = np.concatenate([k, top - k, (k << np.uint64(29)) | np.uint64((1 << 29) - 1), k << np.uint64(29),
+                        np.uint64(1 << 51) + k, (k << np.uint64(21)) | np.uint64((1 << 21) - 1),
+                        np.random.default_rng(3).integers(0, 1 << 52, size=1 << 16, dtype=np.uint64)])
+    d = (m | np.uint64((1023 + exponent) << 52)).view(np.float64)
+    r = rs.check_reciprocals(torch.from_numpy(d).cuda()).cpu().numpy()[:, 0]
+    assert _ulp_diff(r, 1.0 / d).max() <= 1
+    assert (r != 1.0 / d).mean() <= 1 / 500
