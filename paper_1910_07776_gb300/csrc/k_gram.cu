@@ -262,9 +262,15 @@ transfer_tile_kernel(const int64_t* __restrict__ group_off, int max_runs, int64_
 
 cudaError_t rs_launch_transfer_blocks(const rs_batch* train_std, const rs_batch* test_std, const int64_t* group_off,
                                       int max_runs, int stat_stride, int ld, double* KA, double* Kx, int dist,
-                                      cudaStream_t st) {
+                                      int* dstatus, cudaStream_t st) {
     const unsigned Q = (unsigned)test_std->n_programs;
     const int n = RS_MAXV * max_runs;
+    // The tensor-core form (k_gram_split.cu) is the faster one from 32 features on: 90 problems of 192 + 64
+    // rows x 96 features 527 (the tiles below, two launches) against 108 us, x 32 185 against 82; 6 problems
+    // of 64 + 64 rows x 64 features 55 against 17, x 32 32 against 18.  Below that the rounding of its digits is
+    // no longer below that of an FP64 sum.
+    if (KA && !dist && stat_stride >= 32)
+        return rs_launch_transfer_split(train_std, test_std, group_off, max_runs, stat_stride, ld, KA, Kx, dstatus, st);
     const double* ZA = (const double*)train_std->X;
     const double* ZB = (const double*)test_std->X;
     const int nt = (n + kTT - 1) / kTT;        // tiles along the group's versions

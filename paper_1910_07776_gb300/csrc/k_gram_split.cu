@@ -49,13 +49,14 @@ static_assert((kSplBlock * kSplChunk * 4) << 14 <= 1 << 24, "sums of one accumul
 
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// 2^52 z rounded to nearest, plus 128 in every digit's place: byte k of the result is digit 7 - k
-// plus 128.  |z| < 7.95; false otherwise.
+// 2^(52 - W) z rounded to nearest, plus 128 in every digit's place: byte k of the result is digit 7 - k
+// plus 128.  |z| < 7.95 2^W; false otherwise.
+template <int W>
 __device__ __forceinline__ unsigned long long digits_of(double z, bool& ok) {
     const unsigned hi = (unsigned)__double2hiint(z), lo = (unsigned)__double2loint(z);
-    ok = ok && (hi & 0x7fffffffu) < kSplHi;
+    ok = ok && (hi & 0x7fffffffu) < kSplHi + ((unsigned)W << 20);
     const int ex = (int)(hi >> 20) & 0x7ff;
-    int s = 1025 - ex;
+    int s = 1025 + W - ex;
     s = s > 60 ? 60 : (s < 0 ? 0 : s);                    // (a subnormal's spurious bit is shifted out)
     const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32 | lo) << 2;
     const unsigned long long x = (m + ((1ull << s) >> 1)) >> s;
@@ -113,6 +114,7 @@ __device__ __forceinline__ void spl_load(const SplItem& it, double (&v)[16]) {
 
 // The digits of the block into a stage: task (row, chunk of 8 features) writes 16 bytes of each
 // slice at the swizzled place of that chunk.
+template <int W>
 __device__ __forceinline__ bool spl_store(const double (&v)[16], unsigned char* stage) {
     bool ok = true;
 #pragma unroll
@@ -121,7 +123,7 @@ __device__ __forceinline__ bool spl_store(const double (&v)[16], unsigned char* 
         unsigned ylo[8], yhi[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-            const unsigned long long y = digits_of(v[8 * i + e], ok);
+            const unsigned long long y = digits_of<W>(v[8 * i + e], ok);
             ylo[e] = (unsigned)y;
             yhi[e] = (unsigned)(y >> 32);
         }
@@ -146,7 +148,8 @@ __device__ __forceinline__ bool spl_store(const double (&v)[16], unsigned char* 
     return ok;
 }
 
-// 2^-64 (hi 2^32 + lo) as a double, rounded to nearest, by integer operations (|hi|, |lo| < 2^62).
+// 2^(2 W - 64) (hi 2^32 + lo) as a double, rounded to nearest, by integer operations (|hi|, |lo| < 2^62).
+template <int W>
 __device__ __forceinline__ double spl_double(long long hi, long long lo) {
     hi += lo >> 32;
     unsigned l = (unsigned)lo;
@@ -169,7 +172,7 @@ __device__ __forceinline__ double spl_double(long long hi, long long lo) {
         m |= e >= 32 ? (unsigned long long)l << (e - 32) : (unsigned long long)l >> (32 - e);
     }
     // m in [2^63, 2^64) stands for m 2^(32 - e) 2^-64: its leading bit is 2^(31 - e)
-    const unsigned long long b = ((unsigned long long)(1023 + 31 - e - 1) << 52) + (m >> 11) + ((m >> 10) & 1ull);
+    const unsigned long long b = ((unsigned long long)(1023 + 31 + 2 * W - e - 1) << 52) + (m >> 11) + ((m >> 10) & 1ull);
     return __longlong_as_double((long long)(b | (neg ? 0x8000000000000000ull : 0ull)));
 }
 
@@ -180,6 +183,87 @@ __device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, uint32_t (&r)[8]
 }
 
 __device__ __forceinline__ void split_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
+
+// The eight warps' reading of the four accumulators: rows x cols sums of digits' products as doubles into
+// out (row stride ld), added to what is there or not.  xch: two buffers of kXchBytes.
+template <int W>
+__device__ __forceinline__ void spl_sums(uint32_t tmem, longlong2* xch, double* out, int ld, int rows, int cols, bool add) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int quarter = warp & 3, half = warp >> 2;          // TMEM lanes, columns 32 half ..
+    const int row = (quarter & 1) * 32 + lane;
+    const bool upper = quarter >= 2;
+    const int mine = upper ? 4 : 0;            // of 8 columns: the four this warp finishes
+    const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16);
+    for (int c0 = 0; c0 < 32; c0 += 8) {
+        const int col = half * 32 + c0;
+        if (col >= cols) {                    // (uniform over the half's four warps)
+            split_sync();
+            continue;
+        }
+        double* o = out + (int64_t)row * ld + col + mine;
+        const bool whole = (reinterpret_cast<uintptr_t>(o) & 15) == 0 && row < rows && col + mine + 4 <= cols;
+        double old[4] = {0.0, 0.0, 0.0, 0.0};
+        if (add) {
+            if (whole) {
+                *reinterpret_cast<double2*>(old) = *reinterpret_cast<const double2*>(o);
+                *reinterpret_cast<double2*>(old + 2) = *reinterpret_cast<const double2*>(o + 2);
+            } else {
+#pragma unroll
+                for (int c = 0; c < 4; ++c)
+                    if (row < rows && col + mine + c < cols) old[c] = o[c];
+            }
+        }
+        uint32_t r[8][8];                      // weights t + (upper) + (right half): t = 2, 4, 6, 8
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            tmem_ld8_nowait(trow + (uint32_t)(t * 128 + col), r[2 * t]);
+            tmem_ld8_nowait(trow + (uint32_t)(t * 128 + 64 + col), r[2 * t + 1]);
+        }
+        tc::tmem_wait_ld();
+        // lower lanes: r[k] has weight k + 2, upper lanes: k + 3 (weight 10 is left out);
+        // hi collects weights 2 .. 5 (in the place of 5), lo 6 .. 9 (in the place of 9).
+        // A lower and an upper lane share a row: each finishes four of the columns and
+        // sends its sums of the other four (two buffers, one barrier a round)
+        longlong2* xb = xch + ((c0 >> 3) & 1) * (kXchBytes / 16);
+        long long hi[4], lo[4];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) {
+            int x[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) x[k] = __float2int_rn(__uint_as_float(r[k][c]));
+            long long h, l;
+            if (!upper) {
+                h = ((long long)x[0] << 24) + ((long long)x[1] << 16) + ((long long)x[2] << 8) + x[3];
+                l = ((long long)x[4] << 24) + ((long long)x[5] << 16) + ((long long)x[6] << 8) + x[7];
+            } else {
+                h = ((long long)x[0] << 16) + ((long long)x[1] << 8) + x[2];
+                l = ((long long)x[3] << 24) + ((long long)x[4] << 16) + ((long long)x[5] << 8) + x[6];
+            }
+            if ((c >= 4) == upper) {
+                hi[c & 3] = h;
+                lo[c & 3] = l;
+            } else {
+                xb[(half * 8 + c) * 64 + row] = make_longlong2(h, l);
+            }
+        }
+        split_sync();
+        double d[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const longlong2 u = xb[(half * 8 + mine + c) * 64 + row];
+            d[c] = spl_double<W>(hi[c] + u.x, lo[c] + u.y);
+            if (add) d[c] += old[c];
+        }
+        if (whole) {
+            *reinterpret_cast<double2*>(o) = make_double2(d[0], d[1]);
+            *reinterpret_cast<double2*>(o + 2) = make_double2(d[2], d[3]);
+        } else {
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+                if (row < rows && col + mine + c < cols) o[c] = d[c];
+        }
+    }
+}
 
 __global__ void __launch_bounds__(kSplThreads + 32, 1) gram_split_kernel(const SplArgs a) {
     extern __shared__ uint8_t smem_raw[];
@@ -268,7 +352,7 @@ __global__ void __launch_bounds__(kSplThreads + 32, 1) gram_split_kernel(const S
         double v[16];
         if (alive) {
             spl_load(cur, v);
-            if (!spl_store(v, g)) outside[0] = 1;
+            if (!spl_store<0>(v, g)) outside[0] = 1;
             stage_full(0);
         }
         while (alive) {
@@ -284,7 +368,7 @@ __global__ void __launch_bounds__(kSplThreads + 32, 1) gram_split_kernel(const S
                 spl_load(nxt, v);
                 // the products that read the other stage have completed
                 if (it >= 1) wait(done + 8 * (buf ^ 1), (uint32_t)(((it - 1) >> 1) & 1), -31);
-                if (!spl_store(v, g + (buf ^ 1) * kStageBytes)) outside[nxt.n & 3] = 1;
+                if (!spl_store<0>(v, g + (buf ^ 1) * kStageBytes)) outside[nxt.n & 3] = 1;
                 stage_full(buf ^ 1);
             }
             const bool last = cur.kb + 1 == cur.nk;
@@ -293,81 +377,7 @@ __global__ void __launch_bounds__(kSplThreads + 32, 1) gram_split_kernel(const S
                 __syncwarp();
                 tc::fence_after();
                 double* Kp = a.K + cur.p * (RS_GRAM_LD * RS_GRAM_LD);
-                const int quarter = warp & 3, half = warp >> 2;          // TMEM lanes, columns 32 half ..
-                const int row = (quarter & 1) * 32 + lane;
-                const bool upper = quarter >= 2;
-                const int mine = upper ? 4 : 0;            // of 8 columns: the four this warp finishes
-                const bool vec = (reinterpret_cast<uintptr_t>(a.K) & 15) == 0;
-                const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16);
-                for (int c0 = 0; c0 < 32; c0 += 8) {
-                    const int col = half * 32 + c0;
-                    if (col >= cur.V) {                    // (uniform over the half's four warps)
-                        split_sync();
-                        continue;
-                    }
-                    double* o = Kp + row * RS_GRAM_LD + col + mine;
-                    const bool whole = vec && row < cur.V && col + mine + 4 <= cur.V;
-                    double old[4] = {0.0, 0.0, 0.0, 0.0};
-                    if (cur.kb >= kSplChunk) {
-                        if (whole) {
-                            *reinterpret_cast<double2*>(old) = *reinterpret_cast<const double2*>(o);
-                            *reinterpret_cast<double2*>(old + 2) = *reinterpret_cast<const double2*>(o + 2);
-                        } else {
-#pragma unroll
-                            for (int c = 0; c < 4; ++c)
-                                if (row < cur.V && col + mine + c < cur.V) old[c] = o[c];
-                        }
-                    }
-                    uint32_t r[8][8];                      // weights t + (upper) + (right half): t = 2, 4, 6, 8
-#pragma unroll
-                    for (int t = 0; t < 4; ++t) {
-                        tmem_ld8_nowait(trow + (uint32_t)(t * 128 + col), r[2 * t]);
-                        tmem_ld8_nowait(trow + (uint32_t)(t * 128 + 64 + col), r[2 * t + 1]);
-                    }
-                    tc::tmem_wait_ld();
-                    // lower lanes: r[k] has weight k + 2, upper lanes: k + 3 (weight 10 is left out);
-                    // hi collects weights 2 .. 5 (in the place of 5), lo 6 .. 9 (in the place of 9).
-                    // A lower and an upper lane share a row: each finishes four of the columns and
-                    // sends its sums of the other four (two buffers, one barrier a round)
-                    longlong2* xb = xch + ((c0 >> 3) & 1) * (kXchBytes / 16);
-                    long long hi[4], lo[4];
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        int x[8];
-#pragma unroll
-                        for (int k = 0; k < 8; ++k) x[k] = __float2int_rn(__uint_as_float(r[k][c]));
-                        long long h, l;
-                        if (!upper) {
-                            h = ((long long)x[0] << 24) + ((long long)x[1] << 16) + ((long long)x[2] << 8) + x[3];
-                            l = ((long long)x[4] << 24) + ((long long)x[5] << 16) + ((long long)x[6] << 8) + x[7];
-                        } else {
-                            h = ((long long)x[0] << 16) + ((long long)x[1] << 8) + x[2];
-                            l = ((long long)x[3] << 24) + ((long long)x[4] << 16) + ((long long)x[5] << 8) + x[6];
-                        }
-                        if ((c >= 4) == upper) {
-                            hi[c & 3] = h;
-                            lo[c & 3] = l;
-                        } else {
-                            xb[(half * 8 + c) * 64 + row] = make_longlong2(h, l);
-                        }
-                    }
-                    split_sync();
-                    double d[4];
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const longlong2 u = xb[(half * 8 + mine + c) * 64 + row];
-                        d[c] = spl_double(hi[c] + u.x, lo[c] + u.y);
-                        if (cur.kb >= kSplChunk) d[c] += old[c];
-                    }
-                    if (whole) {
-                        *reinterpret_cast<double2*>(o) = make_double2(d[0], d[1]);
-                        *reinterpret_cast<double2*>(o + 2) = make_double2(d[2], d[3]);
-                    } else {
-#pragma unroll
-                        for (int c = 0; c < 4; ++c)
-                            if (row < cur.V && col + mine + c < cur.V) o[c] = d[c];
-                    }
-                }
+                spl_sums<0>(tmem, xch, Kp, RS_GRAM_LD, cur.V, cur.V, cur.kb >= kSplChunk);
                 tc::fence_before();
                 __syncwarp();
                 if (lane == 0) tc::mbar_arrive(drained);
@@ -398,7 +408,244 @@ __global__ void __launch_bounds__(kSplThreads + 32, 1) gram_split_kernel(const S
     if (warp == 0) tc::tmem_dealloc(tmem, 512);
 }
 
+// The dot products of a transfer (k_gram.cu: transfer_tile_kernel) by the same splitting: 64 x 64 blocks of
+// the group's Gram (lower triangle of blocks) and of the test rows against the group's.  The group's
+// z-scores are below sqrt(64 runs - 1), the test rows' unbounded, so the digits start at 2^4 (|z| <
+// 15.9; a block with an element outside takes plain FP64 multiply-adds in feature order), X = round(2^51
+// z).  A CTA takes a block at a time; a stage holds 64 features of its rows' digits and one those of its
+// columns (a diagonal block's are the same), so splitting waits for the products before it; loads
+// and, across blocks, nothing else overlap them.  Per block: the sums 20,000 cycles, per 64 features 4,400
+// for splitting and 2,600 for products.
+// 90 problems of 192 + 64 rows x 96 features: 108 us (FP64 tiles: 527).
+struct TrSplArgs {
+    const int64_t* group_off;
+    int max_runs;
+    int64_t n_runs;
+    int stat_stride;
+    const int64_t* a_row;
+    const int32_t* a_fw;
+    const int64_t* a_xo;
+    const double* ZA;
+    const int64_t* b_row;
+    const int32_t* b_fw;
+    const int64_t* b_xo;
+    const double* ZB;
+    int ld;
+    double* KA;                // null: only Kx
+    double* Kx;
+    int64_t Q;
+    int* dstatus;
+};
+
+struct TrBlock {
+    const double* rowp[4];     // this thread's two rows of the block's rows and two of its columns (null: none)
+    double* out;
+    int rows, cols, F, nk;
+    bool same;                 // a diagonal block
+};
+
+// Block t of the launch: false if it does not exist (the same for every thread).
+__device__ __forceinline__ bool tr_block(const TrSplArgs& a, int64_t t, TrBlock& b) {
+    const int nb = a.max_runs, ng = a.KA ? nb * (nb + 1) / 2 : 0;
+    const int64_t q = t / (ng + nb);
+    int k = (int)(t - q * (ng + nb));
+    int start[RS_MAXRUNS + 1];
+    const int N = rs_group_layout((int)q, a.group_off, a.max_runs, a.n_runs, a.a_row, a.a_fw, a.b_fw, a.stat_stride, start, b.F);
+    if (N < 0 || N > a.ld) return false;
+    const bool cross = k >= ng;
+    int bi = 0, bu;
+    if (cross) {
+        bu = k - ng;
+    } else {                                   // k = bi (bi + 1) / 2 + bu, bu <= bi
+        while ((bi + 1) * (bi + 2) / 2 <= k) ++bi;
+        bu = k - bi * (bi + 1) / 2;
+    }
+    const int64_t VB = a.b_row[q + 1] - a.b_row[q];
+    if (cross && (VB < 1 || VB > RS_MAXV)) return false;
+    const int i0 = bi * 64, u0 = bu * 64, rows = cross ? (int)VB : N;
+    if (i0 >= rows || u0 >= N) return false;
+    b.rows = rows - i0 < 64 ? rows - i0 : 64;
+    b.cols = N - u0 < 64 ? N - u0 : 64;
+    b.nk = (b.F + kSplBlock - 1) / kSplBlock;
+    b.same = !cross && bi == bu;
+    b.out = (cross ? a.Kx + q * RS_MAXV * a.ld : a.KA + q * a.ld * a.ld) + (int64_t)i0 * a.ld + u0;
+    const int64_t g0 = a.group_off[q];
+    auto group_row = [&](int v) -> const double* {
+        int r = 0;
+        while (v >= start[r + 1]) ++r;
+        return a.ZA + a.a_xo[g0 + r] + (int64_t)(v - start[r]) * b.F;
+    };
+    if (threadIdx.x < kSplThreads) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int v = (threadIdx.x >> 3) + 32 * i;
+            b.rowp[i] = v >= b.rows ? nullptr : cross ? a.ZB + a.b_xo[q] + (int64_t)v * b.F : group_row(i0 + v);
+            b.rowp[2 + i] = v >= b.cols ? nullptr : group_row(u0 + v);
+        }
+    }
+    return true;
+}
+
+// This thread's two tasks of 64 features from f0: eight consecutive features of a row each.
+__device__ __forceinline__ void tr_load(const double* const (&rowp)[4], int first, int f0, int F, double (&v)[16]) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int f = f0 + (threadIdx.x & 7) * 8;
+        const double* s = rowp[first + i] + f;
+        const bool row = rowp[first + i] != nullptr;
+        if (row && f + 8 <= F && (reinterpret_cast<uintptr_t>(s) & 15) == 0) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const double2 d = __ldg(reinterpret_cast<const double2*>(s) + e);
+                v[8 * i + 2 * e] = d.x;
+                v[8 * i + 2 * e + 1] = d.y;
+            }
+        } else {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[8 * i + e] = row && f + e < F ? __ldg(s + e) : 0.0;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kSplThreads + 32, 1) transfer_split_kernel(const TrSplArgs a) {
+    constexpr int W = 1;
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ uint32_t tmem_slot;
+    __shared__ int outside;                                // an element outside the range
+    __shared__ const double* plain_rows[2][64];
+    __shared__ volatile int gave_up;
+    const uint32_t raw = tc::smem_u32(smem_raw), base = (raw + 1023u) & ~1023u;
+    uint8_t* g = smem_raw + (base - raw);
+    longlong2* xch = reinterpret_cast<longlong2*>(g + 2 * kStageBytes);
+    // barriers: stages written (8 warps), their products complete, accumulators read (8 warps)
+    const uint32_t full = base + 2 * kStageBytes + 2 * kXchBytes, done = full + 8, drained = full + 16;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    if (tid == 0) {
+        tc::mbar_init(full, 8);
+        tc::mbar_init(done, 1);
+        tc::mbar_init(drained, 8);
+        tc::fence_barrier_init();
+        outside = 0;
+        gave_up = 0;
+    }
+    for (int i = tid; i < (int)(2 * kSliceBytes / 16); i += kSplThreads + 32)      // the zero slices
+        *reinterpret_cast<uint4*>(g + (i >= (int)(kSliceBytes / 16) ? kStageBytes : 0) + 7 * kSliceBytes +
+                                  (i % (kSliceBytes / 16)) * 16) = make_uint4(0u, 0u, 0u, 0u);
+    fence_async_smem();
+    if (warp == 0) {
+        tc::tmem_alloc(tc::smem_u32(&tmem_slot), 512);
+        tc::tmem_relinquish();
+    }
+    tc::fence_before();
+    __syncthreads();
+    tc::fence_after();
+    const uint32_t tmem = tmem_slot;
+    // a wait that gives up (RS_ETIMEOUT) ends all waiting, as above
+    auto wait = [&](uint32_t bar, uint32_t phase, int site) {
+        if (!gave_up && !tc::mbar_wait(bar, phase & 1u, a.dstatus, site)) gave_up = 1;
+    };
+    const int64_t total = a.Q * (a.max_runs + (a.KA ? a.max_runs * (a.max_runs + 1) / 2 : 0));
+    uint32_t it = 0, chunk = 0;                            // stages and chunks of 256 features so far
+    TrBlock b;
+    if (warp == 8) {                                       // ---- the products
+        constexpr uint32_t idesc = (1u << 4) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
+        if (tc::elect_one()) {
+            for (int64_t t = blockIdx.x; t < total; t += gridDim.x) {
+                if (!tr_block(a, t, b)) continue;
+                const uint32_t sb = base + (b.same ? 0 : kStageBytes);
+                for (int kb = 0; kb < b.nk; ++kb, ++it) {
+                    const bool first = kb % kSplChunk == 0;
+                    if (first && chunk > 0) wait(drained, chunk - 1, -36);
+                    chunk += first;
+                    wait(full, it, -37);
+                    tc::fence_after();
+#pragma unroll 1
+                    for (int k = 0; k < kSplBlock / 16; ++k)
+#pragma unroll
+                        for (int u = 2; u <= 8; u += 2)
+#pragma unroll
+                            for (int i = 1; i < u; i += 2)
+                                tc::mma_bf16(tmem + (uint32_t)((u / 2 - 1) * 128),
+                                             tc::sw128_desc(base + (i - 1) * kSliceBytes + k * 32),
+                                             tc::sw128_desc(sb + (u - i - 1) * kSliceBytes + k * 32), idesc,
+                                             !(first && k == 0 && i == 1));
+                    tc::mma_commit(done);
+                }
+            }
+            // every product has completed before the tensor memory is freed
+            if (it > 0) tc::mbar_wait(done, (it - 1) & 1u, a.dstatus, -38);
+        }
+    } else {                                               // ---- digits, and the sums
+        for (int64_t t = blockIdx.x; t < total; t += gridDim.x) {
+            if (!tr_block(a, t, b)) continue;
+            bool ok = true;
+            for (int kb = 0; kb < b.nk; ++kb, ++it) {
+                double v[16];
+                tr_load(b.rowp, 0, kb * kSplBlock, b.F, v);
+                // the products that read the stages have completed
+                if (it >= 1) wait(done, it - 1, -39);
+                ok = spl_store<W>(v, g) && ok;
+                if (!b.same) {
+                    tr_load(b.rowp, 2, kb * kSplBlock, b.F, v);
+                    ok = spl_store<W>(v, g + kStageBytes) && ok;
+                }
+                fence_async_smem();
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(full);
+                if (kb + 1 == b.nk || kb % kSplChunk == kSplChunk - 1) {
+                    wait(done, it, -40);
+                    __syncwarp();
+                    tc::fence_after();
+                    spl_sums<W>(tmem, xch, b.out, a.ld, b.rows, b.cols, kb >= kSplChunk);
+                    tc::fence_before();
+                    __syncwarp();
+                    if (lane == 0) tc::mbar_arrive(drained);
+                }
+            }
+            if (!ok) outside = 1;
+            if ((tid & 7) == 0)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) plain_rows[i >> 1][(tid >> 3) + 32 * (i & 1)] = b.rowp[i];
+            split_sync();
+            if (outside) {                                 // plain FP64, uniform
+                for (int e = tid; e < b.rows * 64; e += kSplThreads) {
+                    const int i = e >> 6, u = e & 63;
+                    if (u >= b.cols) continue;
+                    const double *zi = plain_rows[0][i], *zu = plain_rows[1][u];
+                    double acc = 0.0;
+                    for (int f = 0; f < b.F; ++f) acc = fma(__ldg(zi + f), __ldg(zu + f), acc);
+                    b.out[(int64_t)i * a.ld + u] = acc;
+                }
+            }
+            split_sync();
+            if (tid == 0) outside = 0;
+            split_sync();
+        }
+    }
+    tc::fence_before();
+    __syncthreads();
+    if (warp == 0) tc::tmem_dealloc(tmem, 512);
+}
+
 }  // namespace
+
+cudaError_t rs_launch_transfer_split(const rs_batch* train_std, const rs_batch* test_std, const int64_t* group_off,
+                                     int max_runs, int stat_stride, int ld, double* KA, double* Kx, int* dstatus,
+                                     cudaStream_t st) {
+    cudaError_t e = cudaFuncSetAttribute(transfer_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSplSmem);
+    if (e != cudaSuccess) return e;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const TrSplArgs a{group_off, max_runs, train_std->n_programs, stat_stride, train_std->row_offsets, train_std->feat_width,
+                      train_std->x_offsets, (const double*)train_std->X, test_std->row_offsets, test_std->feat_width,
+                      test_std->x_offsets, (const double*)test_std->X, ld, KA, Kx, test_std->n_programs, dstatus};
+    const int64_t total = a.Q * (max_runs + (KA ? max_runs * (max_runs + 1) / 2 : 0));
+    if (total < 1) return cudaSuccess;
+    transfer_split_kernel<<<(unsigned)(total < sms ? total : sms), kSplThreads + 32, kSplSmem, st>>>(a);
+    return cudaGetLastError();
+}
 
 cudaError_t rs_launch_gram_split(const rs_batch* b, double* K, int* dstatus, cudaStream_t st) {
     cudaError_t e = cudaFuncSetAttribute(gram_split_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSplSmem);

@@ -836,7 +836,7 @@ rs_status rs_transfer(rs_ctx* c, const rs_batch* train, const rs_batch* test, co
     zb.dtype = RS_F64;
     if (!m5p) {                 // the model tree reads the standardized rows themselves
         e = rs_launch_transfer_blocks(&za, &zb, goff, max_runs, stride, ld, ibk ? nullptr : w.KA, w.Kx, ibk ? 1 : 0,
-                                      c->stream);
+                                      c->dstatus, c->stream);
         if (e != cudaSuccess) return cuda_fail(c, e, "rs_transfer (blocks)");
     }
     rs_transfer_args t{};

@@ -107,7 +107,10 @@ cudaError_t rs_launch_transfer_standardize(const rs_batch* train, const rs_batch
 // test row t against group version u, dot products or, with dist, squared distances).
 cudaError_t rs_launch_transfer_blocks(const rs_batch* train_std, const rs_batch* test_std, const int64_t* group_off,
                                       int max_runs, int stat_stride, int ld, double* KA, double* Kx, int dist,
-                                      cudaStream_t st);
+                                      int* dstatus, cudaStream_t st);
+cudaError_t rs_launch_transfer_split(const rs_batch* train_std, const rs_batch* test_std, const int64_t* group_off,
+                                     int max_runs, int stat_stride, int ld, double* KA, double* Kx, int* dstatus,
+                                     cudaStream_t st);
 size_t rs_gram_tc_workspace_bytes(int64_t P, int max_feat);
 // tile_n: 32 or 64 output columns per tile; ksplit: 1 or 3 (see k_gram_tc.cu).
 cudaError_t rs_launch_gram_bf16x3_ws(const rs_batch* b, double* K, void* ws, size_t ws_bytes, int* dstatus,

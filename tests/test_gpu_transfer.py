@@ -189,3 +189,27 @@ def test_m5p_at_its_edges(rs, ctx, feat, runs_per, versions, case):
     test = synth.take_programs(b, list(range(4 * runs_per, 4 * runs_per + 4)))
     g, r = _both(rs, ctx, train, test, groups, "m5p", flags=oracle.RANK_ALL)
     _check(g, r, "m5p")
+
+
+@pytest.mark.parametrize("feat,runs_per,versions,case", [
+    (64, 1, (64, 64), "plain"), (72, 1, (2, 40), "plain"), (257, 1, (50, 64), "plain"), (33, 3, (64, 64), "plain"),
+    (64, 2, (33, 64), "plain"), (129, 3, (1, 64), "plain"), (321, 4, (60, 64), "plain"), (96, 3, (64, 64), "far"),
+    (96, 2, (40, 64), "nan")])
+def test_ridge_blocks_at_the_edges_of_their_tiles(rs, ctx, feat, runs_per, versions, case):
+    """Dot products by the tensor cores' blocks of 64 x 64 entries: part blocks, one and several stages of 64
+    features and sums of 256, one to four runs; a test version far outside the training range (a counter
+    e^40 times the others': its block takes plain FP64), and one whose counter is not a number."""
+    Q = 6
+    b = synth.make_batch(Q * runs_per + Q, versions=versions, feat=feat, dtype=np.float64, seed=900 + feat)
+    train = synth.take_programs(b, list(range(Q * runs_per)))
+    test = synth.take_programs(b, list(range(Q * runs_per, Q * runs_per + Q)))
+    if case != "plain":
+        for p in (1, 4):
+            test.program_X(p)[-1, feat // 2] *= np.exp(40.0) if case == "far" else np.nan
+    g, r = _both(rs, ctx, train, test, np.arange(Q + 1, dtype=np.int64) * runs_per, "ridge", flags=oracle.RANK_ALL)
+    if case == "nan":             # that version's predictions alone are lost
+        bad = [int(test.row_offsets[p + 1]) - 1 for p in (1, 4)]
+        keep = np.setdiff1d(np.arange(test.row_offsets[-1]), bad)
+        close(np.asarray(g["pred_all"]).reshape(-1, 6)[keep], np.asarray(r.pred_all).reshape(-1, 6)[keep], abs_=g["abs_tol"])
+        return
+    _check(g, r, "ridge", abs_tol=g["abs_tol"])
