@@ -117,8 +117,11 @@ __device__ __forceinline__ double rcp_newton_any(double d) {
 }
 
 // One block per (problem, optimization): the ridge fit of that optimization's pairs.  The
-// factor lives in shared memory (nmax rows of nmax + 1 doubles); right-looking LDL^T whose
-// trailing update of each step is spread over all threads (16 row groups x 8 column lanes),
+// factor lives in shared memory (the lower triangle, packed: five blocks of 96 pairs an SM where a
+// full square left room for two); right-looking LDL^T whose
+// trailing update of each step is spread over all threads (16 row groups x 8 column lanes); the FP64
+// pipe bounds it (540 fits of 96 pairs 374 -> 276 us, of which 200 are its instructions; two columns a
+// step, with half the barriers, 273),
 // reciprocal pivots from rcp_newton kept for the solves, then the two forward solves and the
 // back solve of the bordered system, one thread per row.
 __global__ void __launch_bounds__(kTrThreads)
@@ -131,9 +134,9 @@ transfer_fit_kernel(const TransferArgs a, int nmax) {
     __shared__ double bval;
     __shared__ double red[8];
     const int q = blockIdx.x, j = blockIdx.y, tid = threadIdx.x;
-    const int ldm = nmax + 1;
+    auto tri = [](int i) { return i * (i + 1) / 2; };         // row i of the packed lower triangle
     double* M = fsm;
-    double* col = M + (size_t)nmax * ldm;
+    double* col = M + tri(nmax);
     double* lrow = col + nmax;
     double* ty = lrow + nmax;
     double* t1 = ty + nmax;
@@ -167,13 +170,13 @@ transfer_fit_kernel(const TransferArgs a, int nmax) {
     const double* KAq = a.KA + (int64_t)q * a.ld * a.ld;
     for (int e = tid; e < n * n; e += kTrThreads) {
         const int i = e / n, c = e - i * n;
-        if (c <= i) M[i * ldm + c] = __ldg(KAq + (int64_t)pu[i] * a.ld + pu[c]) + (i == c ? a.lambda : 0.0);
+        if (c <= i) M[tri(i) + c] = __ldg(KAq + (int64_t)pu[i] * a.ld + pu[c]) + (i == c ? a.lambda : 0.0);
     }
     __syncthreads();
     const int ty8 = tid >> 3, tx8 = tid & 7;
     int st = RS_FIT_OK;
     for (int k = 0; k < n; ++k) {
-        const double d = M[k * ldm + k];
+        const double d = M[tri(k) + k];
         if (!pos_finite(d)) {                      // every thread read the same pivot
             st = RS_FIT_NOTPD;
             break;
@@ -181,15 +184,15 @@ transfer_fit_kernel(const TransferArgs a, int nmax) {
         const double di = rcp_newton(d);
         if (tid == 0) dinv[k] = di;
         for (int i = k + 1 + tid; i < n; i += kTrThreads) {
-            const double c = M[i * ldm + k];
+            const double c = M[tri(i) + k];
             col[i] = c;
             lrow[i] = c * di;
-            M[i * ldm + k] = c * di;
+            M[tri(i) + k] = c * di;
         }
         __syncthreads();
         for (int i = k + 1 + ty8; i < n; i += 16) {
             const double l = lrow[i];
-            for (int c = k + 1 + tx8; c <= i; c += 8) M[i * ldm + c] = fma(-l, col[c], M[i * ldm + c]);
+            for (int c = k + 1 + tx8; c <= i; c += 8) M[tri(i) + c] = fma(-l, col[c], M[tri(i) + c]);
         }
         __syncthreads();
     }
@@ -201,7 +204,7 @@ transfer_fit_kernel(const TransferArgs a, int nmax) {
         __syncthreads();
         for (int k = 0; k < n - 1; ++k) {
             if (tid > k && tid < n) {
-                const double l = M[tid * ldm + k];
+                const double l = M[tri(tid) + k];
                 ty[tid] = fma(-l, ty[k], ty[tid]);
                 t1[tid] = fma(-l, t1[k], t1[tid]);
             }
@@ -231,7 +234,7 @@ transfer_fit_kernel(const TransferArgs a, int nmax) {
         if (tid < n) ty[tid] = fma(-b, t1[tid], ty[tid]) * dinv[tid];
         __syncthreads();
         for (int k = n - 1; k > 0; --k) {          // L^T alpha = D^-1 (t_y - b t_1)
-            if (tid < k) ty[tid] = fma(-M[k * ldm + tid], ty[k], ty[tid]);
+            if (tid < k) ty[tid] = fma(-M[tri(k) + tid], ty[k], ty[tid]);
             __syncthreads();
         }
         bool fin = true;
@@ -1373,7 +1376,7 @@ cudaError_t rs_launch_transfer(const rs_transfer_args& t, cudaStream_t st) {
         if (e != cudaSuccess) return e;
     } else if (!t.ibk) {
         const int nmax = RS_MAXPAIRS * t.max_runs;
-        const size_t fsmem = ((size_t)nmax * (nmax + 1) + 5 * (size_t)nmax) * sizeof(double);
+        const size_t fsmem = ((size_t)nmax * (nmax + 1) / 2 + 5 * (size_t)nmax) * sizeof(double);
         e = cudaFuncSetAttribute(transfer_fit_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fsmem);
         if (e != cudaSuccess) return e;
         transfer_fit_kernel<<<dim3((unsigned)t.Q, RS_NOPT), kTrThreads, fsmem, st>>>(a, nmax);
