@@ -710,11 +710,16 @@ rs_status rs_cv_step(rs_ctx* c, const rs_batch* b, const rs_splits* sp, double l
     if (s != RS_OK) return s;
     cudaSetDevice(c->device);
     cudaError_t e = cudaSuccess;
+    auto gram = [&]() -> rs_status {     // the learner IBK compares distances only: any that order alike will do
+        if (!(flags & RS_MODEL_IBK)) return rs_gram(c, &zb, precision, K, fws, fbytes);
+        const cudaError_t eg = rs_launch_dist2_order(&zb, K, c->dstatus, c->stream);
+        return eg == cudaSuccess ? RS_OK : cuda_fail(c, eg, "rs_gram");
+    };
     if (!c->side || !c->fork || !c->join || precision == RS_GRAM_BF16X3) {
         // one stream, in order: the tensor-core Gram's scratch is the fit workspace, which the
         // planning fills afterwards
         s = rs_standardize(c, b, Z, nullptr, nullptr);
-        if (s == RS_OK) s = rs_gram(c, &zb, precision, K, fws, fbytes);
+        if (s == RS_OK) s = gram();
         if (s != RS_OK) return s;
         e = rs_launch_rec_offsets(&zb, sp, rec_offsets, c->scan, c->dstatus, c->stream);
         if (e == cudaSuccess) e = rs_launch_fit_predict(a, c->stream);
@@ -733,7 +738,7 @@ rs_status rs_cv_step(rs_ctx* c, const rs_batch* b, const rs_splits* sp, double l
     if (e == cudaSuccess) e = cudaEventRecord(c->join, c->side);
     if (e != cudaSuccess) return cuda_fail(c, e, "rs_cv_step (planning)");
     s = rs_standardize(c, b, Z, nullptr, nullptr);
-    if (s == RS_OK) s = rs_gram(c, &zb, precision, K, fws, fbytes);
+    if (s == RS_OK) s = gram();
     e = cudaStreamWaitEvent(c->stream, c->join, 0);   // joined whatever happened above
     if (s != RS_OK) return s;
     if (e != cudaSuccess) return cuda_fail(c, e, "rs_cv_step (join)");

@@ -100,6 +100,8 @@ cudaError_t rs_launch_standardize(const rs_batch* b, double* Z, double* mu, doub
 cudaError_t rs_launch_gram_f64(const rs_batch* b, double* K, int* dstatus, cudaStream_t st);
 cudaError_t rs_launch_gram_split(const rs_batch* b, double* K, int* dstatus, cudaStream_t st);
 cudaError_t rs_launch_dist2_f64(const rs_batch* b, double* K, int* dstatus, cudaStream_t st);
+// Distances that compare within each row like those of rs_launch_dist2_f64 (nearest neighbours).
+cudaError_t rs_launch_dist2_order(const rs_batch* b, double* K, int* dstatus, cudaStream_t st);
 cudaError_t rs_launch_transfer_standardize(const rs_batch* train, const rs_batch* test, const int64_t* group_off,
                                            int max_runs, int stat_stride, double* ZA, double* ZB, double* mu,
                                            double* sigma, int* dstatus, cudaStream_t st);

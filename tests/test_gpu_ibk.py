@@ -123,3 +123,39 @@ def test_ibk_argument_errors(rs, ctx):
         flags = kw.pop("flags", rs.RS_MODEL_IBK)
         with pytest.raises(rs.RsError):
             ctx.predict_rank(zb, D, ds, ro, out.rec_code, flags=flags, **kw)
+
+
+@pytest.mark.parametrize("case", ["plain", "wide", "ragged", "repeated", "few_values", "near", "constant", "nan"])
+def test_ibk_over_batches_exact(rs, ctx, case):
+    # Batches whose distances come from the tensor cores' Gram: every comparison, ties and near-ties
+    # included, as by the plain definition (which the entry points take).
+    P = 24
+    versions, feat = ((2, 64), [33, 96, 257]) if case == "ragged" else ((64, 64), [300 if case == "wide" else 64])
+    batch = synth.make_batch(P, versions=versions, feat_choices=feat, dtype=np.float64, seed=71)
+    rng = np.random.default_rng(71)
+    for p in range(P):
+        X, cyc = batch.program_X(p), batch.cycles[batch.program_rows(p)][:, None]
+        if case == "repeated":               # rows equal to one another: tied distances
+            X[:] = (X / cyc)[rng.integers(0, 9, size=len(X))] * cyc
+        if case == "few_values":             # counters of three values: ties between different sums
+            X[:] = np.exp(rng.integers(0, 3, size=X.shape)) * cyc
+        if case == "near":                   # pairs of rows a few units in the last place apart
+            X[1::2] = (X / cyc)[::2][:len(X[1::2])] * cyc[1::2] * (1 + 1e-15 * rng.integers(-4, 5, size=X[1::2].shape))
+        if case == "constant":               # most features without spread
+            X[:, 2:] = 3.0 * cyc
+        if case == "nan":
+            X[5 % len(X), 1] = np.nan
+    splits = synth.make_splits(batch, "half" if case == "ragged" else "lovo", 40)
+    db = rs.DeviceBatch.from_host(batch)
+    ds = rs.DeviceSplits.from_host(splits, batch=batch)
+    g = rs.cv_run(ctx, db, ds, flags=rs.RS_MODEL_IBK)    # the entry points: the plain definition
+    ws = ctx.workspace(ctx.cv_workspace_bytes(db, ds))
+    ro = torch.empty(ds.n_splits + 1, dtype=torch.int64, device="cuda")
+    out = rs.alloc_outputs(int(g["rec_offsets"][-1]), ds.n_splits, 3, "cuda")
+    ctx.cv_step(db, ds, ws, ro, out.rec_code, flags=rs.RS_MODEL_IBK, rec_pred=out.rec_pred, pred_all=out.pred_all,
+                counters=out.counters)
+    torch.cuda.synchronize()
+    ctx.check_device_status()
+    np.testing.assert_array_equal(out.rec_code.cpu().numpy().view(np.uint32), g["rec_code"])
+    np.testing.assert_array_equal(out.pred_all.cpu().numpy().reshape(-1), np.asarray(g["pred_all"]).reshape(-1))
+    np.testing.assert_array_equal(out.counters.cpu().numpy().view(np.uint64), g["counters"])
