@@ -33,6 +33,7 @@ WORKLOAD = "batched_cv: 64 programs x U{16..64} versions x 256 f32 features, 409
 LAUNCHES_PER_STEP = 13
 CFG = dict(programs=64, versions=(16, 64), feat=256, splits=4096, lam=1e-3, k=3, tau=1.05, seed=0)
 FP64_PEAK_NOMINAL_GFLOPS = 152 * 4 * 2.07   # 152 SMs x 2 FP64 FMA/clk x 2 flops x 2.07 GHz
+BF16_PEAK_TFLOPS = 1922.0              # measured cuBLAS burst
 
 
 def source_sha():
@@ -582,17 +583,20 @@ def main():
     # the whole step against the sum of its stages' roofline times (HBM bytes at the measured
     # copy bandwidth, FP64 flops at the FP64 peak), on the executed (dual) form
     bounds = {"standardize": work["std_bytes"] / (hbm_peak * 1e6),
-              "gram": work["gram_flops"] / (fp64_peak * 1e9),
+              # 30 products of digits for each of the full block's (twice the upper triangle's)
+              "gram": work["gram_flops"] * 60 / (BF16_PEAK_TFLOPS * 1e9),
               "plan": work["mask_bytes"] / (hbm_peak * 1e6),
               "solve": work["solve_group"] / (fp64_peak * 1e9),
               "rank": work["rank_bytes"] / (hbm_peak * 1e6)}
     # the stages before the solvers, from their stand-alone times
     roof["stages"]["gram_alone"] = {"ms": alone["gram_f64"], "flops": work["gram_flops"],
-                                    "frac_fp64": work["gram_flops"] / (alone["gram_f64"] * 1e-3) / 1e12 / fp64_peak}
+                                    "frac_fp64": work["gram_flops"] / (alone["gram_f64"] * 1e-3) / 1e12 / fp64_peak,
+                                    "note": "exact digit products on the tensor cores where the batch is large "
+                                            "enough: the fraction of the FP64 pipe's peak may pass 1"}
     roof["stages"]["standardize_alone"] = {
         "ms": alone["standardize"], "bytes": work["std_bytes"],
         "frac_hbm": work["std_bytes"] / (alone["standardize"] * 1e-3) / 1e9 / hbm_peak,
-        "note": "bound by the FP64 logarithm (9 FP64 instructions per element), not by HBM"}
+        "note": "bound by the integer instructions of its fixed-point logarithms, not by HBM"}
     roof["stages"]["step"] = {"ms": ms_step, "bound_ms": sum(bounds.values()),
                               "frac": sum(bounds.values()) / ms_step,
                               "bound_ms_parts": bounds,
@@ -807,11 +811,11 @@ def run_lovo(rs, ctx, dev, stream, flush, args, programs=256):
     """Leave-one-version-out (the paper's protocol over all 64 masks, Sec. 5) at the
     precision form's shape: 256 programs x 64 versions x 1024 FP64 features, 16,384 splits,
     98,304 ridge fits of 31 pairs each, every stage in FP64 through the one-call step.  The
-    fits of more than 16 pairs run in solve_wide_kernel; its stage time (from the end of the
-    planning to the join of the solver streams) against its FP64 flops gives its roofline
-    fraction, and the Gram (1.07 GFLOP) is timed alone beside it.  The same step with
-    RS_LOO_CLOSED (one inverse per program and optimization, every fit from it in O(n)) is
-    timed beside it, with its largest prediction difference from the direct solves."""
+    step recognises the splits and takes the fits in closed form (one inverse per program and
+    optimization, every fit from it in O(n)); the fit stage (from the end of the planning to the
+    join of the solver streams) against the inverses' FP64 flops gives its roofline fraction, and
+    the Gram (1.07 GFLOP) is timed alone beside it.  The same step asked for the closed form
+    (RS_LOO_CLOSED) is timed beside it, with its largest prediction difference."""
     import torch
     from paper_1910_07776_gb300 import synth
     b = synth.make_batch_fast(programs, versions=64, feat=1024, dtype=np.float64, seed=43)
@@ -862,25 +866,24 @@ def run_lovo(rs, ctx, dev, stream, flush, args, programs=256):
     work = algorithmic_work(b, sp, CFG["k"])
     fp64_peak = FP64_PEAK_NOMINAL_GFLOPS / 1e3
     solve_ms = stages.get("solve", 0.0) + stages.get("solve_join", 0.0)
-    flops = work["solve_small"] + work["solve_large"]
     c = o.counters.cpu().numpy().view(np.uint64).astype(np.float64)
     cc = oc.counters.cpu().numpy().view(np.uint64).astype(np.float64)
     pa, pc = o.pred_all.cpu().numpy(), oc.pred_all.cpu().numpy()
     fin = ~np.isnan(pa)
     same_nan = bool(np.array_equal(np.isnan(pa), np.isnan(pc)))
     diff = np.abs(pa[fin] - pc[fin])
-    # the closed form's FP64 work: one Gauss-Jordan inverse per (program, optimization) with at
-    # least one pair, padded to 32 x 32 with two right-hand sides (2 flops per FMA)
+    # the closed form's FP64 work: one inverse by 32 symmetric sweeps per (program, optimization) with
+    # at least one pair: the lower triangle of 32 x 32 and two right-hand sides (2 flops per FMA)
     n_inv = 0
     for p_ in range(b.n_programs):
         m_ = set(int(x) for x in b.masks[b.program_rows(p_)])
         n_inv += sum(1 for j in range(6) if any(not (x >> j) & 1 and (x | 1 << j) in m_ for x in m_))
-    inv_flops = n_inv * 2.0 * 32 * 32 * (32 + 2)
+    inv_flops = n_inv * 2.0 * 32 * (32 * 33 / 2 + 2 * 32)
     fit_ms_c = stages_c.get("solve", 0.0) + stages_c.get("solve_join", 0.0)
     closed = {"ms_per_step": ms_c, "value": R / (ms_c * 1e-3), "unit": UNIT, "stages_ms": stages_c,
               "fit_ms": fit_ms_c, "inverses": n_inv, "inverse_flops": inv_flops,
               "fit_stage_frac_fp64": inv_flops / (fit_ms_c * 1e-3) / 1e12 / fp64_peak if fit_ms_c > 0 else None,
-              "fit_stage_note": "the inverses' FMAs (1,536 x 32 x 32 x 34 at 256 programs) over the stage time, "
+              "fit_stage_note": "the inverses' FMAs (1,536 x 32 sweeps x 592 at 256 programs) over the stage time, "
                                 "which also holds the diagonal kernel and the O(1) per-fit kernel",
               "sign_accuracy": cc[3] / max(cc[2], 1), "top1_hit_rate": cc[8] / max(cc[7], 1),
               "fits_ok": int(cc[9]),
@@ -893,9 +896,9 @@ def run_lovo(rs, ctx, dev, stream, flush, args, programs=256):
             "ms_per_step": ms, "value": R / (ms * 1e-3), "unit": UNIT, "recs_per_step": R,
             "sign_accuracy": c[3] / max(c[2], 1), "top1_hit_rate": c[8] / max(c[7], 1),
             "stages_ms": stages,
-            "roofline": {"bound": "alu", "kernel": "solve_wide_kernel (fits of 17..32 pairs)",
-                         "achieved": flops / (solve_ms * 1e-3) / 1e12, "peak": fp64_peak, "unit": "TFLOP/s",
-                         "frac": flops / (solve_ms * 1e-3) / 1e12 / fp64_peak, "flops_per_launch": flops,
+            "roofline": {"bound": "alu", "kernel": "loo_inv_kernel and loo_fit_kernel (fits of 31 pairs)",
+                         "achieved": inv_flops / (solve_ms * 1e-3) / 1e12, "peak": fp64_peak, "unit": "TFLOP/s",
+                         "frac": inv_flops / (solve_ms * 1e-3) / 1e12 / fp64_peak, "flops_per_launch": inv_flops,
                          "ms": solve_ms,
                          "peak_source": "FP64 1.25 TFLOP/s nominal (152 SMs x 2 FMA/clk x 2.07 GHz)"},
             "closed_form": closed,

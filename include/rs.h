@@ -47,7 +47,8 @@ typedef enum {
 
 enum { RS_FIT_OK = 0, RS_FIT_EMPTY = 1, RS_FIT_NOTPD = 2, RS_FIT_NONFINITE = 3 };
 enum { RS_F32 = 0, RS_F64 = 1 };
-/* Gram precision: plain FP64 FMAs, or the BF16 hi/lo split on the tensor cores (three
+/* Gram precision: FP64 (FMAs, or for larger batches exact products of digits on the tensor
+ * cores, with smaller errors), or the BF16 hi/lo split on the tensor cores (three
  * BF16 products per term, FP32 accumulation in tensor memory).  RS_GRAM_DIST2 makes the
  * block of squared Euclidean distances instead, for the instance-based learner.         */
 enum { RS_GRAM_F64 = 0, RS_GRAM_BF16X3 = 1, RS_GRAM_DIST2 = 2 };
@@ -151,7 +152,8 @@ rs_status rs_standardize(rs_ctx* ctx, const rs_batch* batch, double* Z, double* 
 /* ---- A3: per-program Gram of the standardized feature vectors -------------------------
  * K_p[a][b] = sum_f Z[a][f] * Z[b][f] for a, b < V_p, written to
  * K[p * 64 * 64 + a * 64 + b] (double; entries outside V_p x V_p are left untouched).
- * std: a batch whose X is Z (double).  precision: RS_GRAM_F64 (FP64 FMAs, no workspace) or
+ * std: a batch whose X is Z (double).  precision: RS_GRAM_F64 (FP64 FMAs, or exact
+ * digit products summed in integers; no workspace) or
  * RS_GRAM_BF16X3 (tcgen05 tensor cores: z = hi + lo with hi = bf16(z), lo = bf16(z - hi),
  * K ~ hi hi^T + hi lo^T + lo hi^T accumulated in FP32 -- relative error about 2^-16 per
  * entry; symmetric; needs rs_gram_workspace_bytes(std, precision) bytes of workspace,
@@ -249,8 +251,8 @@ rs_status rs_predict_rank(rs_ctx* ctx, const rs_batch* std, const double* K,
  * device memory of at least rs_cv_workspace_bytes(batch, splits) bytes, 256-byte
  * aligned, owned by the caller and used as scratch (Z, the Gram blocks and the fit
  * workspace).  Outputs as in rs_predict_rank, equal bit for bit to those of the individual
- * calls.  With RS_MODEL_IBK the block is the distance block (precision RS_GRAM_F64 or
- * RS_GRAM_DIST2).  Ordering: the row planning and the fit plan (they read only masks, times
+ * calls.  With RS_MODEL_IBK the block is one of distances (precision RS_GRAM_F64 or
+ * RS_GRAM_DIST2) that order in each row as those of RS_GRAM_DIST2 do.  Ordering: the row planning and the fit plan (they read only masks, times
  * and splits) run on the context's internal second stream beside the standardization and
  * the Gram, forked from and joined back into the context's stream with events, so the call
  * is still ordered on the context's stream as a whole; with RS_GRAM_BF16X3 (whose scratch is
