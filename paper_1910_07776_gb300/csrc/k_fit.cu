@@ -104,6 +104,7 @@ pairs_kernel(int P, const int64_t* __restrict__ row_off, const uint8_t* __restri
              const double* __restrict__ log_time, uint8_t* pb, uint8_t* pa, double* ylab,
              int* npair, uint64_t* cand, uint32_t* rowinfo, uint64_t* pset, uint8_t* psorted,
              int* dstatus) {
+    tc::in_sequence();
     __shared__ int8_t slot_of[RS_MAXV];
     __shared__ uint8_t msk[RS_MAXV];
     __shared__ double lt[RS_MAXV];
@@ -176,6 +177,7 @@ pairs_kernel(int P, const int64_t* __restrict__ row_off, const uint8_t* __restri
 // dlam[p][t] = K_p[t][t] + lambda, the diagonal the solvers factor (one block per program).
 __global__ void __launch_bounds__(64)
 dlam_kernel(const int64_t* __restrict__ row_off, const double* __restrict__ K, double lambda, double* dlam) {
+    tc::in_sequence();
     const int p = blockIdx.x, t = threadIdx.x;
     const int V = (int)(row_off[p + 1] - row_off[p]);
     if (V >= 1 && V <= RS_MAXV && t < V)
@@ -199,6 +201,7 @@ plan_fits_kernel(int P, const int64_t* __restrict__ row_off, const int64_t* __re
                  const uint32_t* __restrict__ rowinfo, const uint64_t* __restrict__ cand, int cand_all,
                  int count_preds, const uint64_t* __restrict__ pset, const uint8_t* __restrict__ psorted,
                  int* dstatus) {
+    tc::in_sequence();
     __shared__ unsigned h[kHist];
     // the tables of the block's first kPlanProgs programs (its splits' programs are
     // consecutive): pair slots [program][before / after][optimization][32], pair counts,
@@ -602,6 +605,7 @@ bucket_fits_kernel(int64_t S6, const uint16_t* __restrict__ fit_key, const unsig
                    unsigned* cursor, uint4* recs, int64_t* fit_off, uint8_t* status, double* coef_user,
                    unsigned long long* counters, const uint32_t* __restrict__ fit_pm,
                    const int* __restrict__ split_prog, const int64_t* __restrict__ row_off) {
+    tc::in_sequence();
     __shared__ long long start[kHist], cstart[kHist];
     __shared__ unsigned lcount[kKeys];       // fits per (n, c); then their offsets inside n's range
     __shared__ unsigned lbase[kHist];
@@ -717,7 +721,14 @@ template <int NLO, int NHI, int MINB>
 __global__ void __launch_bounds__(128, MINB)
 solve_small_kernel(const SolveArgs a, unsigned long long* work) {
     __shared__ long long start[kHist], cstart[kHist];
-    if (none_left(a)) return;
+    // The solver of the larger fits shares no fit with the one launched before it, whose inputs are its
+    // own: it begins on the SMs that one's tail leaves, and waits for it at its end.
+    if constexpr (NLO == 1) tc::in_sequence();
+    else tc::let_successor();
+    if (none_left(a)) {
+        if constexpr (NLO > 1) tc::after_predecessor();
+        return;
+    }
     bucket_tables(a.hist, start, cstart);
     const long long lo = start[NLO], hi = start[NHI + 1];
     const int lane = threadIdx.x & 31;
@@ -765,6 +776,7 @@ solve_small_kernel(const SolveArgs a, unsigned long long* work) {
         base = next;
         rec = nrec;
     }
+    if constexpr (NLO > 1) tc::after_predecessor();
 }
 
 // ====================================================================== IBK (Sec. 3.4)
@@ -802,6 +814,7 @@ __device__ __forceinline__ double ibk_nearest_mean(uint32_t pm, const double* __
 // the mean is formed once.
 __global__ void __launch_bounds__(128)
 ibk_kernel(const SolveArgs a, int nmax, unsigned long long* work) {
+    tc::in_sequence();
     __shared__ long long start[kHist], cstart[kHist];
     bucket_tables(a.hist, start, cstart);
     const long long lo = start[1], hi = start[nmax + 1];
@@ -935,6 +948,7 @@ __host__ __device__ constexpr size_t mid_warp_bytes(int nmax) {
 // Fits with kNReg < n, one per thread (solve_var), dynamic work distribution.
 __global__ void __launch_bounds__(128)
 solve_mid_kernel(const SolveArgs a, int nmax, unsigned long long* work) {
+    tc::in_sequence();
     extern __shared__ __align__(16) double dsm[];
     __shared__ long long start[kHist], cstart[kHist];
     if (none_left(a)) return;
@@ -1347,6 +1361,7 @@ __device__ __forceinline__ void tri_step(int& i, int& j) {
 
 __global__ void __launch_bounds__(kWideWarps * 32)
 solve_wide_kernel(const SolveArgs a, unsigned long long* work) {
+    tc::in_sequence();
     __shared__ long long start[kHist], cstart[kHist];
     __shared__ uint16_t tri_rc[tri(RS_MAXPAIRS - 1)];         // packed-triangle entry -> row, column
     extern __shared__ __align__(16) double wsm[];
@@ -1571,6 +1586,7 @@ loo_inv_kernel(const int64_t* __restrict__ row_off, const double* __restrict__ K
                const uint8_t* __restrict__ pb, const double* __restrict__ ylab,
                const int* __restrict__ npair, const double* __restrict__ dlam, float limit, double* tab,
                uint8_t* ok, uint32_t* bad) {
+    tc::in_sequence();
     __shared__ double col[2][RS_MAXPAIRS + 2];                  // column k as it stands, by row
     __shared__ double w[RS_MAXPAIRS + 2];                       // the column / d
     __shared__ double rk;                                       // 1 / d of the next pivot; 0: not positive
@@ -1730,6 +1746,7 @@ __global__ void __launch_bounds__(kLooFitThreads)
 loo_fit_kernel(const SolveArgs a, int64_t S6, const int* __restrict__ npair,
                const double* __restrict__ tab, const uint8_t* __restrict__ tab_ok,
                const uint32_t* __restrict__ tab_bad) {
+    tc::in_sequence();
     const int64_t f = (int64_t)blockIdx.x * kLooFitThreads + threadIdx.x;
     const int n = f < S6 ? a.fit_key[f] / kCntBins : 0;
     const bool active = n > 0;
@@ -1856,6 +1873,7 @@ static_assert(kRankTile % 32 == 0, "whole warps of rows");
 template <bool PACK>
 __global__ void __launch_bounds__(kRankThreads, RS_RANK_MINB)
 rank_pass_kernel(const RankPassArgs a) {
+    tc::in_sequence();
     extern __shared__ __align__(128) unsigned char rsm[];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t total = a.rec_offsets[a.S];
@@ -2486,7 +2504,7 @@ FitWs carve(void* base, int64_t P, int64_t S, int nmax, int64_t Rcap) {
 }
 
 template <int NLO, int NHI, int MINB>
-cudaError_t launch_small(const SolveArgs& sa, int sms, int64_t S6, unsigned long long* work, cudaStream_t st) {
+cudaError_t launch_small(const SolveArgs& sa, int sms, int64_t S6, unsigned long long* work, cudaStream_t st, bool early) {
     auto kern = solve_small_kernel<NLO, NHI, MINB>;
     int per_sm = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 128, 0);
@@ -2495,13 +2513,12 @@ cudaError_t launch_small(const SolveArgs& sa, int sms, int64_t S6, unsigned long
     const int64_t need = (S6 + 127) / 128;
     if (grid > need) grid = need;
     if (grid < 1) grid = 1;
-    kern<<<(unsigned)grid, 128, 0, st>>>(sa, work);
-    return cudaGetLastError();
+    return tc::launch_when(early, kern, (unsigned)grid, 128, 0, st, sa, work);
 }
 
 // The one-fit-per-thread solver of kNReg < n <= nmax: as many warps per block as fit in
 // 200 KB of shared memory (1..4), as many blocks as can be resident.
-cudaError_t launch_mid(const SolveArgs& sa, int sms, int nmax, unsigned long long* work, cudaStream_t st) {
+cudaError_t launch_mid(const SolveArgs& sa, int sms, int nmax, unsigned long long* work, cudaStream_t st, bool early) {
     const size_t per_warp = mid_warp_bytes(nmax);
     int warps = (int)((size_t)200 * 1024 / per_warp);
     if (warps > 4) warps = 4;
@@ -2513,8 +2530,7 @@ cudaError_t launch_mid(const SolveArgs& sa, int sms, int nmax, unsigned long lon
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, solve_mid_kernel, warps * 32, smem);
     if (e != cudaSuccess) return e;
     const int64_t grid = (int64_t)sms * (per_sm > 0 ? per_sm : 1);
-    solve_mid_kernel<<<(unsigned)grid, warps * 32, smem, st>>>(sa, nmax, work);
-    return cudaGetLastError();
+    return tc::launch_when(early, solve_mid_kernel, (unsigned)grid, warps * 32, smem, st, sa, nmax, work);
 }
 
 int nmax_of(int max_train) {
@@ -2556,18 +2572,20 @@ cudaError_t rs_launch_fit_predict(const rs_fit_args& a, cudaStream_t st) {
         pairs_kernel<<<a.P, 64, 0, st>>>(a.P, a.row_offsets, a.masks, a.log_time, w.pb, w.pa, w.ylab,
                                          w.npair, w.cand, w.rowinfo, w.pset, w.psorted, a.dstatus);
         mark(1);
-        plan_fits_kernel<<<(unsigned)((a.S + 255) / 256), 256, 0, st>>>(a.P, a.row_offsets, a.split_offsets, a.train_masks,
+        e = tc::launch_after(plan_fits_kernel, (unsigned)((a.S + 255) / 256), 256, 0, st, a.P, a.row_offsets, a.split_offsets, a.train_masks,
                                                     a.S, w.pb, w.pa, w.npair, w.fit_pm, w.fit_key, w.hist,
                                                     nmax, w.split_prog, a.rec_offsets,
                                                     a.rec_code ? a.rows_cap : 0,
                                                     a.rec_code ? w.row_info : nullptr,
                                                     a.masks, w.rowinfo, w.cand, (a.flags & RS_RANK_ALL) ? 1 : 0,
                                                     a.rec_code ? 1 : 0, w.pset, w.psorted, a.dstatus);
+        if (e != cudaSuccess) return e;
         mark(2);
-        bucket_fits_kernel<<<bucket_blocks, kBucketThreads, 0, st>>>(S6, w.fit_key, w.hist, w.cursor, w.recs,
+        e = tc::launch_after(bucket_fits_kernel, bucket_blocks, kBucketThreads, 0, st, S6, w.fit_key, w.hist, w.cursor, w.recs,
                                                       need_off ? w.fit_off : nullptr,
                                                       status, user ? a.coef_out : nullptr, a.counters,
                                                       w.fit_pm, w.split_prog, a.row_offsets);
+        if (e != cudaSuccess) return e;
         mark(3);
     }
     if (!solve) return cudaGetLastError();
@@ -2583,6 +2601,11 @@ cudaError_t rs_launch_fit_predict(const rs_fit_args& a, cudaStream_t st) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const bool refine = (a.flags & RS_REFINE_X) != 0;
+    // Solvers on both streams start by plain launches, in their order: begun early, the register solver
+    // took every register before solve_mid came, which then ran alone after it (64 programs x 4,096
+    // half splits 584 -> 693 us).  On one stream every kernel begins early (2 programs, leave one
+    // version out: 102 -> 74 us; 256 x 1024 features 418 -> 402).
+    bool fork = false;
     if (a.flags & RS_MODEL_IBK) {
         int per_sm = 0;
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ibk_kernel, 128, 0);
@@ -2591,19 +2614,17 @@ cudaError_t rs_launch_fit_predict(const rs_fit_args& a, cudaStream_t st) {
         const int64_t need = (S6 + 127) / 128;
         if (grid > need) grid = need;
         if (grid < 1) grid = 1;
-        ibk_kernel<<<(unsigned)grid, 128, 0, st>>>(sa, nmax, w.work + 3);
-        e = cudaGetLastError();
+        e = tc::launch_after(ibk_kernel, (unsigned)grid, 128, 0, st, sa, nmax, w.work + 3);
         if (e != cudaSuccess) return e;
         mark(4);
     } else if (a.flags & RS_LOO_CLOSED) {
         // one inverse per (program, optimization), then every fit in closed form
-        loo_inv_kernel<<<(unsigned)(a.P * RS_NOPT), kLooThreads, 0, st>>>(a.row_offsets, a.K, w.pb, w.ylab, w.npair,
-                                                                 w.dlam, 0.f, w.loo_tab, w.loo_ok, w.loo_bad);
-        e = cudaGetLastError();
+        e = tc::launch_after(loo_inv_kernel, (unsigned)(a.P * RS_NOPT), kLooThreads, 0, st, a.row_offsets, a.K, w.pb, w.ylab,
+                             w.npair, w.dlam, 0.f, w.loo_tab, w.loo_ok, w.loo_bad);
         if (e != cudaSuccess) return e;
         const int64_t grid = (S6 + kLooFitThreads - 1) / kLooFitThreads;
-        loo_fit_kernel<false><<<(unsigned)grid, kLooFitThreads, 0, st>>>(sa, S6, w.npair, w.loo_tab, w.loo_ok, w.loo_bad);
-        e = cudaGetLastError();
+        e = tc::launch_after(loo_fit_kernel<false>, (unsigned)grid, kLooFitThreads, 0, st, sa, S6, w.npair, w.loo_tab,
+                             w.loo_ok, w.loo_bad);
         if (e != cudaSuccess) return e;
         mark(4);
     } else if (!refine) {
@@ -2630,21 +2651,21 @@ cudaError_t rs_launch_fit_predict(const rs_fit_args& a, cudaStream_t st) {
         const bool lovo = a.lovo && nmax > kNMid && (user || rank) && a.lambda > 0.0;
         if (lovo) {
             sa.left = w.work + 5;
-            loo_inv_kernel<<<(unsigned)(a.P * RS_NOPT), kLooThreads, 0, st>>>(a.row_offsets, a.K, w.pb, w.ylab, w.npair,
-                                                                     w.dlam, kLooLimit, w.loo_tab, w.loo_ok, w.loo_bad);
+            e = tc::launch_after(loo_inv_kernel, (unsigned)(a.P * RS_NOPT), kLooThreads, 0, st, a.row_offsets, a.K, w.pb,
+                                 w.ylab, w.npair, w.dlam, kLooLimit, w.loo_tab, w.loo_ok, w.loo_bad);
+            if (e != cudaSuccess) return e;
             const int64_t grid = (S6 + kLooFitThreads - 1) / kLooFitThreads;
-            loo_fit_kernel<true><<<(unsigned)grid, kLooFitThreads, 0, st>>>(sa, S6, w.npair, w.loo_tab, w.loo_ok,
-                                                                            w.loo_bad);
-            e = cudaGetLastError();
+            e = tc::launch_after(loo_fit_kernel<true>, (unsigned)grid, kLooFitThreads, 0, st, sa, S6, w.npair, w.loo_tab,
+                                 w.loo_ok, w.loo_bad);
             if (e != cudaSuccess) return e;
         }
-        const bool fork = mid && !lovo && a.side && a.fork && a.join;
+        fork = mid && !lovo && a.side && a.fork && a.join;
         cudaStream_t s2 = fork ? a.side : st;
         if (fork) {
             e = cudaEventRecord(a.fork, st);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(a.side, a.fork, 0);
         }
-        if (e == cudaSuccess && mid) e = launch_mid(sa, sms, nmax < kNMid ? nmax : kNMid, w.work + 2, s2);
+        if (e == cudaSuccess && mid) e = launch_mid(sa, sms, nmax < kNMid ? nmax : kNMid, w.work + 2, s2, !fork);
         if (e == cudaSuccess && nmax > kNMid) {
             // kWideGroups fits per warp, persistent blocks taking their fits dynamically
             e = cudaFuncSetAttribute(solve_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWideSmem);
@@ -2656,8 +2677,7 @@ cudaError_t rs_launch_fit_predict(const rs_fit_args& a, cudaStream_t st) {
                 const int64_t need = (S6 + kWideWarps * kWideGroups - 1) / (kWideWarps * kWideGroups);
                 if (grid > need) grid = need;
                 if (grid < 1) grid = 1;
-                solve_wide_kernel<<<(unsigned)grid, kWideWarps * 32, kWideSmem, s2>>>(sa, w.work + 4);
-                e = cudaGetLastError();
+                e = tc::launch_when(!fork, solve_wide_kernel, (unsigned)grid, kWideWarps * 32, kWideSmem, s2, sa, w.work + 4);
             }
         }
         if (e == cudaSuccess && fork) e = cudaEventRecord(a.join, a.side);
@@ -2665,16 +2685,16 @@ cudaError_t rs_launch_fit_predict(const rs_fit_args& a, cudaStream_t st) {
         unsigned long long* w0 = w.work;
         unsigned long long* w1 = w.work + 1;
         switch (a.tune_split) {
-            case 4: e = launch_small<1, 4, 4>(sa, sms, S6, w0, st);
-                    if (e == cudaSuccess) e = launch_small<5, kNReg, 2>(sa, sms, S6, w1, st); break;
-            case 5: e = launch_small<1, 5, 4>(sa, sms, S6, w0, st);
-                    if (e == cudaSuccess) e = launch_small<6, kNReg, 2>(sa, sms, S6, w1, st); break;
-            case 7: e = launch_small<1, 7, 3>(sa, sms, S6, w0, st);
-                    if (e == cudaSuccess) e = launch_small<8, kNReg, 2>(sa, sms, S6, w1, st); break;
-            case 8: e = launch_small<1, 8, 3>(sa, sms, S6, w0, st);
-                    if (e == cudaSuccess) e = launch_small<9, kNReg, 2>(sa, sms, S6, w1, st); break;
-            default: e = launch_small<1, 6, 4>(sa, sms, S6, w0, st);
-                    if (e == cudaSuccess) e = launch_small<7, kNReg, 2>(sa, sms, S6, w1, st); break;
+            case 4: e = launch_small<1, 4, 4>(sa, sms, S6, w0, st, !fork);
+                    if (e == cudaSuccess) e = launch_small<5, kNReg, 2>(sa, sms, S6, w1, st, !fork); break;
+            case 5: e = launch_small<1, 5, 4>(sa, sms, S6, w0, st, !fork);
+                    if (e == cudaSuccess) e = launch_small<6, kNReg, 2>(sa, sms, S6, w1, st, !fork); break;
+            case 7: e = launch_small<1, 7, 3>(sa, sms, S6, w0, st, !fork);
+                    if (e == cudaSuccess) e = launch_small<8, kNReg, 2>(sa, sms, S6, w1, st, !fork); break;
+            case 8: e = launch_small<1, 8, 3>(sa, sms, S6, w0, st, !fork);
+                    if (e == cudaSuccess) e = launch_small<9, kNReg, 2>(sa, sms, S6, w1, st, !fork); break;
+            default: e = launch_small<1, 6, 4>(sa, sms, S6, w0, st, !fork);
+                    if (e == cudaSuccess) e = launch_small<7, kNReg, 2>(sa, sms, S6, w1, st, !fork); break;
         }
         if (e != cudaSuccess) return e;
         mark(4);
@@ -2717,7 +2737,8 @@ cudaError_t rs_launch_fit_predict(const rs_fit_args& a, cudaStream_t st) {
         const int64_t tiles = (a.rows_cap + kRankTile - 1) / kRankTile;
         if (blocks > tiles) blocks = tiles;
         if (blocks < 1) blocks = 1;
-        rank_kern<<<(unsigned)blocks, kRankThreads, kRankSmem, st>>>(ra);
+        e = tc::launch_when(!fork, rank_kern, (unsigned)blocks, kRankThreads, kRankSmem, st, ra);
+        if (e != cudaSuccess) return e;
         if (packed && tiles_cap > 0) {
             e = cudaGetLastError();
             if (e != cudaSuccess) return e;

@@ -2,6 +2,7 @@
 // and their exclusive prefix sum, which indexes every per-row output.  Three launches:
 // per-block counts + block sums, a single-block scan of the block sums, and the final
 // per-block scan.  Integer work only; bit-exact by construction.
+#include "mbar.cuh"
 #include "rs_internal.cuh"
 
 namespace {
@@ -42,6 +43,7 @@ __device__ int64_t block_exclusive_scan(int64_t v, int64_t* total) {
 __global__ void __launch_bounds__(kScanThreads)
 count_kernel(int P, const int64_t* row_off, const int64_t* split_off, const uint64_t* tm,
              int64_t S, int64_t* out, int64_t* block_sums) {
+    tc::in_sequence();
     const int64_t base = (int64_t)blockIdx.x * kPerBlock + (int64_t)threadIdx.x * kItems;
     int64_t local = 0;
     // one search for the thread's first split; its next splits are in the same program or
@@ -65,6 +67,7 @@ count_kernel(int P, const int64_t* row_off, const int64_t* split_off, const uint
 
 __global__ void __launch_bounds__(kScanThreads)
 scan_block_sums_kernel(int64_t* block_sums, int nblocks, int64_t* grand_total) {
+    tc::in_sequence();
     int64_t v[kItems];
     int64_t local = 0;
 #pragma unroll
@@ -86,6 +89,7 @@ scan_block_sums_kernel(int64_t* block_sums, int nblocks, int64_t* grand_total) {
 
 __global__ void __launch_bounds__(kScanThreads)
 finish_kernel(int64_t* out, int64_t S, const int64_t* block_sums) {
+    tc::in_sequence();
     const int64_t base = (int64_t)blockIdx.x * kPerBlock + (int64_t)threadIdx.x * kItems;
     int64_t v[kItems];
     int64_t local = 0;
@@ -121,7 +125,9 @@ cudaError_t rs_launch_rec_offsets(const rs_batch* b, const rs_splits* s, int64_t
     count_kernel<<<(unsigned)nb, kScanThreads, 0, st>>>(b->n_programs, b->row_offsets,
                                                         s->split_offsets, s->train_masks, S,
                                                         rec_offsets, scratch);
-    scan_block_sums_kernel<<<1, kScanThreads, 0, st>>>(scratch, (int)nb, rec_offsets + S);
-    finish_kernel<<<(unsigned)nb, kScanThreads, 0, st>>>(rec_offsets, S, scratch);
+    cudaError_t e = tc::launch_after(scan_block_sums_kernel, 1, kScanThreads, 0, st, scratch, (int)nb, rec_offsets + S);
+    if (e != cudaSuccess) return e;
+    e = tc::launch_after(finish_kernel, (unsigned)nb, kScanThreads, 0, st, rec_offsets, S, scratch);
+    if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }

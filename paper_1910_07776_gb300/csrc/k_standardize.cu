@@ -7,6 +7,7 @@
 // and the product that scales it.  log(x / c) is log x - log c, the second taken once per version.
 // 256 programs x 64 versions x 1024 FP64 counters: 562 -> 149 us (the two passes over
 // memory alone take 40 us); 64 programs x 40 x 256 FP32: 41 -> 16 us.
+#include "mbar.cuh"
 #include "rank_row.cuh"
 #include "rs_internal.cuh"
 #include "rs_log_table.h"

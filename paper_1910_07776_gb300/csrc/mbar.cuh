@@ -35,22 +35,33 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 }
 // Programmatic dependent launch: a kernel launched by launch_after may begin (set up its barriers and
 // tensor memory) while its predecessor's last blocks run; after_predecessor() waits for those and their
-// writes, and comes before the first access to memory that another kernel writes or reads.  Each such kernel lets its own successor in at once.
+// writes, and comes before the first access to memory that another kernel writes or reads (a kernel
+// that shares nothing with its predecessor, and whose inputs that one has waited for, may wait at its
+// end).  let_successor() comes after the wait where a successor relies on that.
 __device__ __forceinline__ void let_successor() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void after_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void in_sequence() {      // the plain case, at a kernel's start
+    after_predecessor();
+    let_successor();
+}
+// early = false: a plain launch.
 template <class... P, class... A>
-cudaError_t launch_after(void (*kern)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A&&... args) {
+cudaError_t launch_when(bool early, void (*kern)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, A&&... args) {
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t c{};
-    c.gridDim = dim3(grid);
+    c.gridDim = grid;
     c.blockDim = dim3(block);
     c.dynamicSmemBytes = smem;
     c.stream = st;
     c.attrs = &at;
-    c.numAttrs = 1;
+    c.numAttrs = early ? 1 : 0;
     return cudaLaunchKernelEx(&c, kern, P(args)...);
+}
+template <class... P, class... A>
+cudaError_t launch_after(void (*kern)(P...), dim3 grid, unsigned block, size_t smem, cudaStream_t st, A&&... args) {
+    return launch_when(true, kern, grid, block, smem, st, args...);
 }
 
 // True in one thread of a converged warp.  Branching on it (rather than on the lane) tells the compiler
