@@ -265,7 +265,12 @@ transfer_fit_kernel(const TransferArgs a, int nmax) {
 // Greedy elimination keeps the inverse H of the normal equations, the residuals and T = C H (C the
 // centred attributes): dropping attribute d changes every residual by (w_d / H_dd) T_ad, so all the
 // drop-one errors of a round cost m ns operations, and the round's winner is taken out by rank-one
-// updates of H, w and T; the model that stays is solved again from scratch.  (Before: one thread per
+// updates of H, w and T; the model that stays is solved again from scratch.  Where taking d out would
+// shrink a diagonal entry of H by more than 2^kM5Shrink since H was last formed (d and another attribute
+// nearly agree: what the subtraction leaves of their large entries is rounding), the attributes that stay
+// are solved from their own normal equations at once, and the elimination goes on from there: with pairs
+// of attributes 1e-5 of a deviation apart the updates alone chose wrong drops in 25 of 60 models, this
+// form, as an inverse a round, in none.  (Before: one thread per
 // attribute walking every candidate's SDR, an inverse per round and every drop-one model applied to
 // every instance, all serial over the nodes.)  Small nodes' models take one warp each.
 // 36 problems x 3 runs x 37 attributes (96 instances a fit): 5532 -> 1351 us.
@@ -281,6 +286,7 @@ constexpr int kM5WarpBuf = kM5WarpTerms * kM5WarpLd + kM5WarpN * kM5WarpLd +
                            (kM5WarpN * kM5WarpLd + 1) / 2;                   // H, C, T (FP32)
 constexpr int kM5Surv = 1024;                     // candidate splits listed for exact evaluation, per level
 constexpr double kM5SdFrac = 0.05, kM5Smooth = 15.0, kM5Ridge = 1e-8;
+constexpr int kM5Shrink = 6;                      // bits that rank-one updates may take off an entry H_kk
 
 struct M5Tree {
     int n_nodes;
@@ -296,7 +302,8 @@ struct M5Tree {
 template <int N>
 struct M5Vec {
     double colk[N], rowk[N], zbar[N], r[N], w[N], wt[N], fac[N];
-    float fac32[N], rowk32[N];
+    int h0[N];                                    // H_kk when H was last formed (high word)
+    float fac32[N], rowk32[N], t32[N], e32[N];    // bounds of |T_ak|, and of the error of T in FP32
     int16_t cand[N];
     uint8_t sel[N];
     double e_cur, b;
@@ -449,6 +456,11 @@ struct M5Group {
         if (WARP) __syncwarp();
         else __syncthreads();
     }
+    static __device__ __forceinline__ bool any(bool x) {      // (also a barrier)
+        if (!WARP) return __syncthreads_or(x) != 0;
+        __syncwarp();
+        return __any_sync(0xffffffffu, x) != 0;
+    }
 };
 
 // In-place inverse of the nb x nb leading block of M (row stride ld) by Gauss-Jordan elimination
@@ -582,26 +594,36 @@ __device__ __noinline__ void m5_model(M5Smem& S, Vec& V, M5Tree* T, int t, int F
     int ns = nc;
     bool dropped = false;
     if (nc > 0 && m > nc) {                        // else no model with one attribute fewer has an estimate
-        // residuals (lane = instance, kept by the warp that owns its 32 instances) and T = C H in FP32
         const int row = WARP ? lane : (int)threadIdx.x;
-        double res = 0.0;
-        if (row < m) {
-            double p = ybar;
-            for (int i = 0; i < nc; ++i) p = fma(C[row * ld + i], V.w[i], p);
-            res = S.y[S.ids[lo + row]] - p;
-        }
-        for (int e = tid; e < m * nc; e += Gp::kNT) {
-            const int a = e / nc, k = e - a * nc;
-            double s = 0.0;
-            for (int i = 0; i < nc; ++i) s = fma(C[a * ld + i], H[i * ld + k], s);
-            T32[a * ld + k] = (float)s;
-        }
         float* res32 = S.res32 + (WARP ? 32 * (int)(threadIdx.x >> 5) : 0);
-        if (row < m) res32[row] = (float)res;
-        Gp::sync();
+        double res = 0.0;
+        bool formed = true;                        // H, w are those of the nc attributes' normal equations
         for (;;) {
-            // w_d / H_dd, then sum_a |res_a + fac_d T_ad| of every attribute still there, in FP32
-            // with the size of its terms
+            if (formed) {
+                // residuals (lane = instance, kept by the warp that owns its 32 instances) and T = C H in FP32
+                formed = false;
+                if (row < m) {
+                    double p = ybar;
+                    for (int i = 0; i < nc; ++i) p = fma(C[row * ld + i], V.w[i], p);
+                    res = S.y[S.ids[lo + row]] - p;
+                    res32[row] = (float)res;
+                }
+                for (int e = tid; e < m * nc; e += Gp::kNT) {
+                    const int a = e / nc, k = e - a * nc;
+                    double s = 0.0;
+                    for (int i = 0; i < nc; ++i) s = fma(C[a * ld + i], H[i * ld + k], s);
+                    T32[a * ld + k] = (float)s;
+                }
+                // column k of T has the norm sqrt(H_kk) at most, and no update makes it longer
+                for (int k = tid; k < nc; k += Gp::kNT) {
+                    V.h0[k] = __double2hiint(H[k * ld + k]);
+                    V.t32[k] = 1.01f * sqrtf(fabsf((float)H[k * ld + k]));
+                    V.e32[k] = 6e-8f * V.t32[k];
+                }
+                Gp::sync();
+            }
+            // w_d / H_dd, then sum_a |res_a + fac_d T_ad| of every attribute still there, in FP32: off by
+            // less than 1e-4 of the sizes of its terms, and by what T has lost in the updates
             for (int d = tid; d < nc; d += Gp::kNT) {
                 V.fac[d] = (alive >> d) & 1ull ? V.w[d] * rcp_newton_any(H[d * ld + d]) : 0.0;
                 V.fac32[d] = (float)V.fac[d];
@@ -649,15 +671,16 @@ __device__ __noinline__ void m5_model(M5Smem& S, Vec& V, M5Tree* T, int t, int F
                                 z += S.errp[1][w][d];
                             }
                         }
-                        lo32[h] = s - 1e-4f * z;
-                        best = fminf(best, s + 1e-4f * z);
+                        const float off = 1e-4f * z + 1.01f * (float)m * fabsf(V.fac32[d]) * V.e32[d];
+                        lo32[h] = s - off;
+                        best = fminf(best, s + off);
                         on[h] = s < 1e30f;         // (not for an estimate that is not finite)
                     }
                 }
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
-                const unsigned b0 = __ballot_sync(0xffffffffu, on[0] && lo32[0] <= best);
-                const unsigned b1 = __ballot_sync(0xffffffffu, on[1] && lo32[1] <= best);
+                const unsigned b0 = __ballot_sync(0xffffffffu, on[0] && !(lo32[0] > best));
+                const unsigned b1 = __ballot_sync(0xffffffffu, on[1] && !(lo32[1] > best));
                 if (tid == 0) {
                     V.reach = (unsigned long long)b1 << 32 | b0;
                     V.drop = -1;
@@ -702,12 +725,10 @@ __device__ __noinline__ void m5_model(M5Smem& S, Vec& V, M5Tree* T, int t, int F
             // estimate with ns - 1 terms (v = ns)
             const double est = drop < 0 ? DBL_MAX : be * S.rcp[m] * ((double)(m + ns) * rcp_newton((double)(m - ns)));
             if (m <= ns || drop < 0 || !(est <= V.e_cur)) break;
-            Gp::sync();                            // (every thread has compared with e_cur)
             const int d = drop;
             dropped = true;
             --ns;
             alive &= ~(1ull << d);
-            if (tid == 0) V.e_cur = est;
             if (ns == 0) break;
             // take d out: w and the residuals as just computed, H -= H_d H_d^T / H_dd, T -= T_d H_d^T / H_dd
             const double fd = V.fac[d], hi = rcp_newton_any(H[d * ld + d]);
@@ -715,20 +736,49 @@ __device__ __noinline__ void m5_model(M5Smem& S, Vec& V, M5Tree* T, int t, int F
                 V.colk[i] = H[i * ld + d];
                 V.rowk[i] = H[i * ld + d] * hi;
                 V.rowk32[i] = (float)V.rowk[i];
+                if (i != d) V.e32[i] += fabsf(V.rowk32[i]) * V.e32[d] + 1.3e-7f * V.t32[i];
                 V.w[i] = i != d && ((alive >> i) & 1ull) ? fma(-H[i * ld + d], fd, V.w[i]) : 0.0;
             }
             res = bres;
             if (row < m) res32[row] = (float)res;
             Gp::sync();
+            if (tid == 0) V.e_cur = est;           // (every thread has compared with it)
+            bool lost = false;                     // an entry H_ii of which too little is left
             for (int e = tid; e < nc * nc; e += Gp::kNT) {
                 const int i = e / nc, j = e - i * nc;
-                if (i != d && j != d) H[i * ld + j] = fma(-V.colk[i], V.rowk[j], H[i * ld + j]);
+                if (i == d || j == d) continue;
+                const double h = fma(-V.colk[i], V.rowk[j], H[i * ld + j]);
+                H[i * ld + j] = h;
+                if (i == j && ((alive >> i) & 1ull)) lost = lost || __double2hiint(h) + (kM5Shrink << 20) < V.h0[i];
             }
             for (int e = tid; e < m * nc; e += Gp::kNT) {
                 const int a = e / nc, k = e - a * nc;
                 if (k != d) T32[a * ld + k] = fmaf(-T32[a * ld + d], V.rowk32[k], T32[a * ld + k]);
             }
-            Gp::sync();
+            if (Gp::any(lost)) {
+                // C and the attributes' lists without the dropped columns (a thread a row, ascending), and
+                // the model of those that stay
+                const int at = tid < nc && ((alive >> tid) & 1ull) ? __popcll(alive & ((1ull << tid) - 1ull)) : -1;
+                const int16_t cand = at >= 0 ? V.cand[tid] : (int16_t)0;
+                const double zbar = at >= 0 ? V.zbar[tid] : 0.0, r = at >= 0 ? V.r[tid] : 0.0;
+                Gp::sync();
+                if (at >= 0) {
+                    V.cand[at] = cand;
+                    V.zbar[at] = zbar;
+                    V.r[at] = r;
+                    V.sel[at] = (uint8_t)at;
+                }
+                if (row < m) {
+                    int k = 0;
+                    for (unsigned long long x = alive; x; x &= x - 1) C[row * ld + k++] = C[row * ld + __ffsll((long long)x) - 1];
+                }
+                Gp::sync();
+                nc = ns;
+                alive = (1ull << nc) - 1ull;       // (nc < kM5MaxTerms: one has gone)
+                m5_solve<WARP>(S, V, C, H, ld, nc, lo, m, ybar);
+                dropped = false;                   // (solved already)
+                formed = true;
+            }
         }
         Gp::sync();
     }

@@ -191,6 +191,31 @@ def test_m5p_at_its_edges(rs, ctx, feat, runs_per, versions, case):
     _check(g, r, "m5p")
 
 
+@pytest.mark.parametrize("gap", [1e-3, 1e-4, 1e-5, 1e-6])
+@pytest.mark.parametrize("seed", [600, 601, 602])
+def test_m5p_pairs_of_nearly_equal_counters(rs, ctx, gap, seed):
+    """Counters in pairs that agree to `gap` of a deviation, on a few levels, so that a tree splits on both
+    of a pair and its models drop one of them.  The versions predicted are training instances, where a
+    model's values do not hang on the difference within a pair.  Tolerance: 100 kappa eps, kappa the
+    condition of a pair's normal equations, at most 4 / gap^2 and, by the ridge of 1e-8, 2 x 96 / 1e-8 (the
+    factor: the terms of a model and the deviations of the labels); a wrong drop moves predictions by up
+    to tenths."""
+    feat, runs_per = 16, 3
+    b = synth.make_batch(4 * runs_per, versions=64, feat=feat, dtype=np.float64, seed=seed)
+    rng = np.random.default_rng(seed)
+    w = rng.standard_normal(feat // 2)
+    for p in range(b.n_programs):
+        level = np.round(1.5 * rng.standard_normal((64, feat // 2))) / 1.5
+        b.program_X(p)[:] = np.exp(np.repeat(level, 2, axis=1) + gap * rng.standard_normal((64, feat)))
+        b.log_time[b.program_rows(p)] = level @ w * 0.3 + 0.1 * rng.standard_normal(64)
+    b.cycles = np.ones_like(b.cycles)
+    test = synth.take_programs(b, [q * runs_per for q in range(4)])
+    g, r = _both(rs, ctx, b, test, np.arange(5, dtype=np.int64) * runs_per, "m5p")
+    tol = 100 * min(4 / gap ** 2, 2 * 96 / 1e-8) * np.finfo(np.float64).eps
+    np.testing.assert_array_equal(g["fit_status"], r.fit_status)
+    close(g["pred_all"], r.pred_all, rel=max(1e-7, tol), abs_=max(1e-9, tol))
+
+
 @pytest.mark.parametrize("feat,runs_per,versions,case", [
     (64, 1, (64, 64), "plain"), (72, 1, (2, 40), "plain"), (257, 1, (50, 64), "plain"), (33, 3, (64, 64), "plain"),
     (64, 2, (33, 64), "plain"), (129, 3, (1, 64), "plain"), (321, 4, (60, 64), "plain"), (96, 3, (64, 64), "far"),
