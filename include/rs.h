@@ -48,7 +48,7 @@ typedef enum {
 enum { RS_FIT_OK = 0, RS_FIT_EMPTY = 1, RS_FIT_NOTPD = 2, RS_FIT_NONFINITE = 3 };
 enum { RS_F32 = 0, RS_F64 = 1 };
 /* Gram precision: FP64 (FMAs, or for larger batches exact products of digits on the tensor
- * cores, with smaller errors), or the BF16 hi/lo split on the tensor cores (three
+ * cores, whose errors stay within those of an FMA chain), or the BF16 hi/lo split on the tensor cores (three
  * BF16 products per term, FP32 accumulation in tensor memory).  RS_GRAM_DIST2 makes the
  * block of squared Euclidean distances instead, for the instance-based learner.         */
 enum { RS_GRAM_F64 = 0, RS_GRAM_BF16X3 = 1, RS_GRAM_DIST2 = 2 };
@@ -153,7 +153,9 @@ rs_status rs_standardize(rs_ctx* ctx, const rs_batch* batch, double* Z, double* 
  * K_p[a][b] = sum_f Z[a][f] * Z[b][f] for a, b < V_p, written to
  * K[p * 64 * 64 + a * 64 + b] (double; entries outside V_p x V_p are left untouched).
  * std: a batch whose X is Z (double).  precision: RS_GRAM_F64 (FP64 FMAs, or exact
- * digit products summed in integers; no workspace) or
+ * digit products summed in integers; no workspace; which of the two depends on the batch's
+ * sizes, and a program with a value outside +-7.95 or a row of norm in (0, 1) always takes
+ * the FMAs, so any double values keep an FMA chain's accuracy) or
  * RS_GRAM_BF16X3 (tcgen05 tensor cores: z = hi + lo with hi = bf16(z), lo = bf16(z - hi),
  * K ~ hi hi^T + hi lo^T + lo hi^T accumulated in FP32 -- relative error about 2^-16 per
  * entry; symmetric; needs rs_gram_workspace_bytes(std, precision) bytes of workspace,

@@ -26,7 +26,10 @@
 // four accumulators: the quadrant (lane half h, column half w) of accumulator t holds digit sums of
 // weight t + h + w.
 // A program with an element outside +-7.95, or not finite (not z-scores, then), is redone by plain
-// FP64 multiply-adds in feature order.
+// FP64 multiply-adds in feature order; so is one with a row whose norm is below 1 but not 0, as the digits
+// hold an element to 2^-53, whatever its size: sum over f of 2^-53 (|z_a| + |z_b|) <= 2^-53 sqrt(F) (|Z_a| +
+// |Z_b|) is within 2^-52 sqrt(F) |Z_a| |Z_b| for norms from 1 up, and so within what F roundings of an FP64
+// chain may come to (F 2^-53 |Z_a| |Z_b|).
 // Per block of 64 features the products take 2600 cycles and the splitting 2200, per 256 features
 // the sums 20000 (64 conversions and 64-bit sums per thread and 8 columns).
 // 256 programs x 1024 features 952 -> 137 us, 64 x 256 37 -> 22 us.
@@ -185,9 +188,11 @@ __device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, uint32_t (&r)[8]
 __device__ __forceinline__ void split_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 
 // The eight warps' reading of the four accumulators: rows x cols sums of digits' products as doubles into
-// out (row stride ld), added to what is there or not.  xch: two buffers of kXchBytes.
+// out (row stride ld), added to what is there or not.  xch: two buffers of kXchBytes.  last: true if
+// this thread wrote an entry (i, i) below 1.
 template <int W>
-__device__ __forceinline__ void spl_sums(uint32_t tmem, longlong2* xch, double* out, int ld, int rows, int cols, bool add) {
+__device__ __forceinline__ bool spl_sums(uint32_t tmem, longlong2* xch, double* out, int ld, int rows, int cols, bool add, bool last) {
+    bool low = false;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int quarter = warp & 3, half = warp >> 2;          // TMEM lanes, columns 32 half ..
     const int row = (quarter & 1) * 32 + lane;
@@ -254,6 +259,10 @@ __device__ __forceinline__ void spl_sums(uint32_t tmem, longlong2* xch, double* 
             d[c] = spl_double<W>(hi[c] + u.x, lo[c] + u.y);
             if (add) d[c] += old[c];
         }
+        if (last && (unsigned)(row - col - mine) < 4u && row < rows) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) low = low || (row == col + mine + c && __double2hiint(d[c]) < 0x3ff00000);
+        }
         if (whole) {
             *reinterpret_cast<double2*>(o) = make_double2(d[0], d[1]);
             *reinterpret_cast<double2*>(o + 2) = make_double2(d[2], d[3]);
@@ -263,12 +272,57 @@ __device__ __forceinline__ void spl_sums(uint32_t tmem, longlong2* xch, double* 
                 if (row < rows && col + mine + c < cols) o[c] = d[c];
         }
     }
+    return low;
+}
+
+// K of one program by plain FP64 multiply-adds in feature order (the eight warps; buf: 64 x 33 doubles): 32
+// features of its rows at a time in shared memory, nine entries of the triangle a thread.  256 programs x 64
+// versions x 1024 features of small values: 1309 us for the call (gram_f64_kernel: 949).
+constexpr int kPlainLd = 33;
+static_assert(RS_MAXV * kPlainLd * sizeof(double) <= 2 * kXchBytes, "the rows' slice fits the exchange buffers");
+__device__ __noinline__ void spl_plain(const double* z, int V, int F, double* Kp, double* buf) {
+    const int tid = threadIdx.x, E = V * (V + 1) / 2;
+    constexpr int kPer = (RS_MAXV * (RS_MAXV + 1) / 2 + kSplThreads - 1) / kSplThreads;
+    int at[kPer];                                          // row << 8 | column <= row; past the last: row 0
+    double acc[kPer];
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+        const int e = tid + kSplThreads * q;
+        int i = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
+        if (i * (i + 1) / 2 > e) --i;
+        if ((i + 1) * (i + 2) / 2 <= e) ++i;
+        at[q] = e < E ? i << 8 | (e - i * (i + 1) / 2) : 0;
+        acc[q] = 0.0;
+    }
+    for (int f0 = 0; f0 < F; f0 += 32) {
+        split_sync();
+        for (int e = tid; e < V * 32; e += kSplThreads) {
+            const int r = e >> 5, f = f0 + (e & 31);
+            buf[r * kPlainLd + (e & 31)] = f < F ? __ldg(z + (int64_t)r * F + f) : 0.0;
+        }
+        split_sync();
+        const int w = F - f0 < 32 ? F - f0 : 32;
+        for (int c = 0; c < w; ++c)
+#pragma unroll
+            for (int q = 0; q < kPer; ++q)
+                if (tid + kSplThreads * q < E)
+                    acc[q] = fma(buf[(at[q] >> 8) * kPlainLd + c], buf[(at[q] & 0xff) * kPlainLd + c], acc[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < kPer; ++q)
+        if (tid + kSplThreads * q < E) {
+            const int i = at[q] >> 8, j = at[q] & 0xff;
+            Kp[i * RS_GRAM_LD + j] = acc[q];
+            Kp[j * RS_GRAM_LD + i] = acc[q];
+        }
+    split_sync();
 }
 
 __global__ void __launch_bounds__(kSplThreads + 32, 1) gram_split_kernel(const SplArgs a) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint32_t tmem_slot;
     __shared__ int outside[4];                             // an element outside the range, by program (mod 4)
+    __shared__ int low[4], anew;                           // a row's norm below 1; such a row is not 0
     __shared__ volatile int gave_up;
     const uint32_t raw = tc::smem_u32(smem_raw), base = (raw + 1023u) & ~1023u;
     uint8_t* g = smem_raw + (base - raw);
@@ -284,6 +338,7 @@ __global__ void __launch_bounds__(kSplThreads + 32, 1) gram_split_kernel(const S
         tc::mbar_init(drained, 8);
         tc::fence_barrier_init();
         outside[0] = outside[1] = outside[2] = outside[3] = 0;
+        low[0] = low[1] = low[2] = low[3] = anew = 0;
         gave_up = 0;
     }
     for (int i = tid; i < (int)(2 * kSliceBytes / 16); i += kSplThreads + 32)      // the zero slices
@@ -377,24 +432,26 @@ __global__ void __launch_bounds__(kSplThreads + 32, 1) gram_split_kernel(const S
                 __syncwarp();
                 tc::fence_after();
                 double* Kp = a.K + cur.p * (RS_GRAM_LD * RS_GRAM_LD);
-                spl_sums<0>(tmem, xch, Kp, RS_GRAM_LD, cur.V, cur.V, cur.kb >= kSplChunk);
+                if (spl_sums<0>(tmem, xch, Kp, RS_GRAM_LD, cur.V, cur.V, cur.kb >= kSplChunk, last)) low[cur.n & 3] = 1;
                 tc::fence_before();
                 __syncwarp();
                 if (lane == 0) tc::mbar_arrive(drained);
                 if (last) {
                     split_sync();                          // (also: the flags of every warp are in)
-                    if (outside[cur.n & 3]) {              // plain FP64, uniform
-                        for (int e = tid; e < cur.V * RS_MAXV; e += kSplThreads) {
-                            const int i = e >> 6, j = e & 63;
-                            if (j > i) continue;
-                            const double *zi = cur.z + (int64_t)i * cur.F, *zj = cur.z + (int64_t)j * cur.F;
-                            double acc = 0.0;
-                            for (int f = 0; f < cur.F; ++f) acc = fma(__ldg(zi + f), __ldg(zj + f), acc);
-                            Kp[i * RS_GRAM_LD + j] = acc;
-                            Kp[j * RS_GRAM_LD + i] = acc;
+                    const bool far = outside[cur.n & 3];   // (these are uniform)
+                    if (far || low[cur.n & 3]) {
+                        if (!far) {                        // a warp a row: is a short one all zeros?
+                            for (int r = warp; r < cur.V; r += kSplThreads / 32) {
+                                if (!(Kp[r * (RS_GRAM_LD + 1)] < 1.0)) continue;
+                                bool some = false;
+                                for (int f = lane; f < cur.F; f += 32) some = some || __ldg(cur.z + (int64_t)r * cur.F + f) != 0.0;
+                                if (some) anew = 1;
+                            }
+                            split_sync();
                         }
+                        if (far || anew) spl_plain(cur.z, cur.V, cur.F, Kp, reinterpret_cast<double*>(xch));
                         split_sync();
-                        if (tid == 0) outside[cur.n & 3] = 0;
+                        if (tid == 0) outside[cur.n & 3] = low[cur.n & 3] = anew = 0;
                     }
                 }
             }
@@ -596,7 +653,7 @@ __global__ void __launch_bounds__(kSplThreads + 32, 1) transfer_split_kernel(con
                     wait(done, it, -40);
                     __syncwarp();
                     tc::fence_after();
-                    spl_sums<W>(tmem, xch, b.out, a.ld, b.rows, b.cols, kb >= kSplChunk);
+                    spl_sums<W>(tmem, xch, b.out, a.ld, b.rows, b.cols, kb >= kSplChunk, false);
                     tc::fence_before();
                     __syncwarp();
                     if (lane == 0) tc::mbar_arrive(drained);

@@ -91,3 +91,48 @@ def test_programs_of_other_values_take_plain_fp64(env):
         assert np.array_equal(np.isinf(K[p]), np.isinf(ref.astype(np.float64)) & ~nan)
         a = np.abs(np.where(np.isfinite(Z[p]), Z[p], 0))
         assert np.all(np.abs(K[p][fin] - ref[fin]) <= (F * U * (a @ a.T))[fin])
+
+
+def test_programs_of_small_rows_keep_their_accuracy(env):
+    """Digits hold an element to 2^-53 whatever its size, so a program with a row of norm below 1 (but not
+    0) takes plain FP64 multiply-adds: the chain's bound, F roundings of at most sum |z_a z_b| (below the
+    normal range of half the smallest subnormal), for it."""
+    rs, ctx = env
+    P, V, F = 40, 64, 130
+    rng = np.random.default_rng(6)
+    Z = rng.standard_normal((P, V, F)).clip(-6, 6)
+    Z[3] *= 1e-8
+    Z[5, 17] *= 1e-9                                         # one row of a program
+    Z[7, 63] = 0.0                                           # a row of zeros: exact either way
+    Z[9, 0] = rng.choice([-1.0, 1.0], F) * 2.0 ** -60        # digits of nothing
+    Z[11] *= 1e-200
+    Z[13, 40] /= 1.001 * np.linalg.norm(Z[13, 40])           # just below 1
+    Z[15, 40] /= 0.999 * np.linalg.norm(Z[15, 40])           # just above: digits
+    Z[17] = 0.0
+    Z[19, 5] = 0.0
+    Z[19, 5, 129] = 1e-3                                     # one element, the last
+    K = _gram(rs, ctx, Z, P, V, F)
+    _check(K, Z, [0, 2, 4, 6, 7, 8, 10, 12, 14, 15, 16, 17, 18, 20, 39])
+    for p in (3, 5, 9, 11, 13, 19):
+        z, a = Z[p].astype(np.longdouble), np.abs(Z[p])
+        assert np.all(np.abs(K[p] - z @ z.T) <= F * (U * (a @ a.T) + 2.0 ** -1074)), p
+        assert np.array_equal(K[p], K[p].T)
+
+
+def test_ragged_programs(env):
+    """1 to 64 versions and several widths in one batch, their z-scores."""
+    from paper_1910_07776_gb300 import synth
+    rs, ctx = env
+    h = synth.make_batch(200, versions=(1, 64), feat_choices=[5, 64, 131, 300], dtype=np.float64, seed=8)
+    b = rs.DeviceBatch.from_host(h)
+    z = b.with_X(ctx.standardize(b))
+    K = ctx.gram(z, rs.RS_GRAM_F64)
+    torch.cuda.synchronize()
+    ctx.check_device_status()
+    K, Z = K.cpu().numpy().reshape(-1, 64, 64), z.X.cpu().numpy()
+    for p in range(0, 200, 9):
+        V, F, x0 = h.versions(p), int(h.feat_width[p]), int(h.x_offsets[p])
+        a = Z[x0:x0 + V * F].reshape(V, F).astype(np.longdouble)
+        row = np.abs(a).sum(axis=1)
+        bound = U * (row[:, None] + row[None]) + F * U * (np.abs(a) @ np.abs(a).T + 0.5)
+        assert np.all(np.abs(K[p, :V, :V] - a @ a.T) <= bound), p
