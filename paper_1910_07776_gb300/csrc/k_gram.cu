@@ -328,6 +328,32 @@ transfer_tile_kernel(const int64_t* __restrict__ group_off, int max_runs, int64_
         }
 }
 
+// Whether the Gram (with dist, the distances that only have to order) goes through the products of digits
+// (k_gram_split.cu).  That form takes a program an SM: 10 + 0.05 F us alone, and with several programs an SM
+// 4.5 + 0.09 V + 0.033 F us each; the multiply-adds 32 F ns per block of 128 entries and SM plus 6 us, in
+// the long run 8 F ns per warp of entries and 0.25 us per block.  So the multiply-adds keep the grids that
+// fit the SMs once and small products (64 versions x 96 features: 26 programs 14.7 against 16.4 us, 40
+// programs 22.6 against 16.4; 256 features: 8 programs 18.6 against 20.0, 12 programs 22.6 against 20.5; 30
+// versions x 96: 76 programs 12.9 against 14.5, 300 programs 30.9 against 24.7), and many programs of few
+// versions or features (3,000 programs of 20 versions x 48 features 91 against 146 us, x 256 313 against
+// 264; of 45 x 24 173 against 187, of 64 x 24 303 against 199).  From a mean of 256 features up the digits
+// stay for those too, as a chain of multiply-adds rounds at every feature (3,000 x 10 versions x 256: 119
+// against 205 us).
+// The differences of distances cost three times the multiply-adds and more, the ordering 20 us a wave of
+// programs, about 2 us each in the long run: 64 versions, 9 programs x 300 features 55 (differences)
+// against 49 us, 40 x 96 58 against 36, 64 x 48 48 against 34; the whole step of 3,000 programs of 20
+// versions x 24 features 216 against 259 us, x 48 337 against 286.
+bool by_digits(const rs_batch* b, bool dist) {
+    const int64_t P = b->n_programs, v = b->n_rows / P < RS_MAXV ? b->n_rows / P : RS_MAXV;
+    const int64_t entries = v * (v + 1) / 2, per = (entries + kGramThreads - 1) / kGramThreads;
+    if (P * per <= 152 || P * per * b->max_feat < 44000 || (dist && b->max_feat < 16)) return false;
+    const int64_t mean = b->n_rows > 0 ? b->x_elems / b->n_rows : 1;
+    const int64_t f = mean < 1 ? 1 : mean < b->max_feat ? mean : b->max_feat;
+    if (P <= 152 || (f >= 256 && !dist)) return true;
+    const int64_t warps = (entries + 31) / 32, plain = (dist ? 30 : 8) * f * warps + 250 * per;      // ns
+    return plain > 4500 + 90 * v + 33 * f + (dist ? 2000 : 0);
+}
+
 }  // namespace
 
 cudaError_t rs_launch_transfer_blocks(const rs_batch* train_std, const rs_batch* test_std, const int64_t* group_off,
@@ -369,15 +395,7 @@ cudaError_t rs_launch_transfer_blocks(const rs_batch* train_std, const rs_batch*
 #define RS_GRAM_MAXB 4
 #endif
 cudaError_t rs_launch_gram_f64(const rs_batch* b, double* K, int* dstatus, cudaStream_t st) {
-    // The tensor-core form (k_gram_split.cu) takes about 10 + 0.05 F us per program and SM whatever
-    // its versions; this one 32 F ns per block of 128 entries and SM, plus 6 us.  So the latter keeps
-    // the grids that fit the SMs once, and small products (64 versions x 96 features: 26 programs
-    // 14.7 against 16.4 us, 40 programs 22.6 against 16.4; 256 features: 8 programs 18.6 against
-    // 20.0, 12 programs 22.6 against 20.5; 30 versions x 96: 76 programs 12.9 against 14.5, 300
-    // programs 30.9 against 24.7).
-    const int64_t v = b->n_rows / b->n_programs < RS_MAXV ? b->n_rows / b->n_programs : RS_MAXV;
-    const int64_t blocks = b->n_programs * ((v * (v + 1) / 2 + kGramThreads - 1) / kGramThreads);
-    if (blocks > 152 && blocks * b->max_feat >= 44000) return rs_launch_gram_split(b, K, dstatus, st);
+    if (by_digits(b, false)) return rs_launch_gram_split(b, K, dstatus, st);
     dim3 grid((unsigned)b->n_programs, kGramChunks);
     const size_t pad = rs_residency_pad(RS_GRAM_MAXB, sizeof(double) * 2 * RS_MAXV * kGramLd);
     if (pad) cudaFuncSetAttribute(gram_f64_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pad);
@@ -394,12 +412,7 @@ cudaError_t rs_launch_dist2_f64(const rs_batch* b, double* K, int* dstatus, cuda
 }
 
 cudaError_t rs_launch_dist2_order(const rs_batch* b, double* K, int* dstatus, cudaStream_t st) {
-    // The line is the Gram's (rs_launch_gram_f64): the differences cost three times its multiply-adds, the
-    // ordering 20 us a wave of programs.  64 versions: 9 programs x 300 features 55 (differences) against
-    // 49 us, 40 x 96 58 against 36, 64 x 48 48 against 34; but 2,600 x 8 257 against 300.
-    const int64_t v = b->n_rows / b->n_programs < RS_MAXV ? b->n_rows / b->n_programs : RS_MAXV;
-    const int64_t blocks = b->n_programs * ((v * (v + 1) / 2 + kGramThreads - 1) / kGramThreads);
-    if (blocks <= 152 || blocks * b->max_feat < 44000 || b->max_feat < 16) return rs_launch_dist2_f64(b, K, dstatus, st);
+    if (!by_digits(b, true)) return rs_launch_dist2_f64(b, K, dstatus, st);
     const cudaError_t e = rs_launch_gram_split(b, K, dstatus, st);
     if (e != cudaSuccess) return e;
     dist_order_kernel<<<(unsigned)b->n_programs, kOrderThreads, 0, st>>>(b->row_offsets, b->feat_width, b->x_offsets,
