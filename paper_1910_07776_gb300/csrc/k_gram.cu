@@ -394,8 +394,8 @@ cudaError_t rs_launch_transfer_blocks(const rs_batch* train_std, const rs_batch*
 #ifndef RS_GRAM_MAXB
 #define RS_GRAM_MAXB 4
 #endif
-cudaError_t rs_launch_gram_f64(const rs_batch* b, double* K, int* dstatus, cudaStream_t st) {
-    if (by_digits(b, false)) return rs_launch_gram_split(b, K, dstatus, st);
+cudaError_t rs_launch_gram_f64(const rs_batch* b, double* K, int* dstatus, cudaStream_t st, const rs_batch* sizes) {
+    if (by_digits(sizes, false)) return rs_launch_gram_split(b, K, dstatus, st);
     dim3 grid((unsigned)b->n_programs, kGramChunks);
     const size_t pad = rs_residency_pad(RS_GRAM_MAXB, sizeof(double) * 2 * RS_MAXV * kGramLd);
     if (pad) cudaFuncSetAttribute(gram_f64_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pad);

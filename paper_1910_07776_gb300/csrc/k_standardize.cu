@@ -111,9 +111,13 @@ __device__ __forceinline__ long long fix_mean(long long hs, long long ls, int n)
     return (q << 24) + (rem + (rem >= 0 ? n / 2 : -(n / 2))) / n;
 }
 
-// What the two kernels below do once a thread holds its ROWS logarithms of feature fl (rows g,
-// g + GROUPS, ..., those below n): the mean and the deviation over the n rows of the block's
-// feature, then the centred values (as doubles) and 1 / sigma (0: a constant or non-finite feature).
+// What the two kernels below do once a thread holds its ROWS logarithms of feature fl (rows r0,
+// r0 + GROUPS, ..., those below n; r0 = g, the thread's row group): the mean and the deviation over the
+// n rows of the block's feature, then the centred values (as doubles) and 1 / sigma (0: a constant or
+// non-finite feature).
+// PAIR (16 groups, two a warp): r0 = pair_row(g), and the squares are added in the order of eight groups,
+// so that a program's outputs do not depend on the form that the rest of its batch asks for (one chain of
+// eight rows in two lanes, but half the sums to add at the end).
 template <int FEAT, int ROWS>
 struct StdSmem {
     static constexpr int kGroups = kThreads / FEAT;
@@ -125,16 +129,18 @@ struct StdSmem {
     uint16_t tc[256];
 };
 
-template <int FEAT, int ROWS>
+__device__ __forceinline__ int pair_row(int g) { return (g >> 1) + 8 * (g & 1); }
+
+template <int FEAT, int ROWS, bool PAIR = false>
 __device__ __forceinline__ double centre(StdSmem<FEAT, ROWS>& S, const long long (&l)[ROWS], double (&d)[ROWS], int n,
                                          bool active, double* mu, double* sigma) {
-    constexpr int G = kThreads / FEAT;
-    const int fl = threadIdx.x % FEAT, g = threadIdx.x / FEAT;
+    constexpr int G = kThreads / FEAT, kSums = PAIR ? G / 2 : G;
+    const int fl = threadIdx.x % FEAT, g = threadIdx.x / FEAT, r0 = PAIR ? pair_row(g) : g;
     long long hs = 0;
     unsigned ls = 0;
 #pragma unroll
     for (int q = 0; q < ROWS; ++q)
-        if (active && g + G * q < n) {
+        if (active && r0 + G * q < n) {
             if (l[q] == kFixInf) S.inf[fl] = 1;
             hs += l[q] >> 24;
             ls += (unsigned)l[q] & 0xffffffu;
@@ -158,9 +164,17 @@ __device__ __forceinline__ double centre(StdSmem<FEAT, ROWS>& S, const long long
 #pragma unroll
     for (int q = 0; q < ROWS; ++q) {
         d[q] = 0.0;
-        if (active && g + G * q < n) {
+        if (active && r0 + G * q < n) {
             d[q] = fix_double(l[q] - m);
-            q2 = fma(d[q], d[q], q2);
+            if constexpr (!PAIR) q2 = fma(d[q], d[q], q2);
+        }
+    }
+    if constexpr (PAIR) {                      // rows g / 2, g / 2 + 8, ... of both lanes, in order
+#pragma unroll
+        for (int q = 0; q < ROWS; ++q) {
+            const double e = __shfl_xor_sync(0xffffffffu, d[q], 16);
+            const double a = g & 1 ? e : d[q], b = g & 1 ? d[q] : e;
+            q2 = fma(b, b, fma(a, a, q2));
         }
     }
     S.pq[g][fl] = q2;
@@ -168,7 +182,7 @@ __device__ __forceinline__ double centre(StdSmem<FEAT, ROWS>& S, const long long
     if (threadIdx.x < FEAT) {
         double t = 0.0;
 #pragma unroll
-        for (int q = 0; q < G; ++q) t += S.pq[q][fl];
+        for (int q = 0; q < kSums; ++q) t += S.pq[q * (G / kSums)][fl];
         t = t * rcp_newton((double)n);
         const bool inf = S.inf[fl] != 0;
         const bool ok = !inf && t > 1e-24;                   // sigma > 1e-12
@@ -195,6 +209,8 @@ standardize_kernel(int P, const int64_t* __restrict__ row_off, const int32_t* __
                    double* __restrict__ Z, double* __restrict__ mu, double* __restrict__ sigma,
                    int* dstatus) {
     constexpr int G = kThreads / FEAT, ROWS = RS_MAXV / G;
+    constexpr bool PAIR = G == 16;
+    static_assert(G == 8 || G == 16, "the squares are added as by eight groups");
     __shared__ StdSmem<FEAT, ROWS> S;
     __shared__ double cyc_s[RS_MAXV];
     __shared__ long long lc_s[RS_MAXV];
@@ -202,7 +218,7 @@ standardize_kernel(int P, const int64_t* __restrict__ row_off, const int32_t* __
     const int64_t r0 = row_off[p];
     const int V = (int)(row_off[p + 1] - r0);
     const int F = fw[p];
-    const int fl = threadIdx.x % FEAT, g = threadIdx.x / FEAT;
+    const int fl = threadIdx.x % FEAT, g = PAIR ? pair_row(threadIdx.x / FEAT) : threadIdx.x / FEAT;
     const int f = blockIdx.y * FEAT + fl;
     if (blockIdx.y * FEAT >= F) return;
     if (V < 1 || V > RS_MAXV) {
@@ -230,7 +246,7 @@ standardize_kernel(int P, const int64_t* __restrict__ row_off, const int32_t* __
         l[q] = r < V ? elem_log(x[q], cycles != nullptr, cyc_s[r], lc_s[r], S.tl, S.tc) : 0;
     }
     double d[ROWS];
-    const double rs = centre(S, l, d, V, active, mu && active ? mu + fo[p] + f : nullptr,
+    const double rs = centre<FEAT, ROWS, PAIR>(S, l, d, V, active, mu && active ? mu + fo[p] + f : nullptr,
                              sigma && active ? sigma + fo[p] + f : nullptr);
     if (!active) return;
 #pragma unroll

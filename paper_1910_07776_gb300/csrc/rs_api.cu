@@ -205,15 +205,16 @@ size_t rs_gram_workspace_bytes(const rs_batch* b, int precision) {
     return precision == RS_GRAM_BF16X3 ? rs_gram_tc_workspace_bytes(b->n_programs, b->max_feat) : 0;
 }
 
-rs_status rs_gram(rs_ctx* c, const rs_batch* b, int precision, double* K, void* ws, size_t ws_bytes) {
-    if (!c) return RS_EINVAL;
+// rs_gram; sizes as in rs_launch_gram_f64.
+static rs_status gram(rs_ctx* c, const rs_batch* b, const rs_batch* sizes, int precision, double* K, void* ws,
+                      size_t ws_bytes) {
     rs_status s = check_batch(c, b, false);
     if (s != RS_OK) return s;
     if (!K) return fail(c, RS_EINVAL, "K is NULL");
     cudaSetDevice(c->device);
     cudaError_t e;
     if (precision == RS_GRAM_F64) {
-        e = rs_launch_gram_f64(b, K, c->dstatus, c->stream);
+        e = rs_launch_gram_f64(b, K, c->dstatus, c->stream, sizes);
     } else if (precision == RS_GRAM_DIST2) {
         e = rs_launch_dist2_f64(b, K, c->dstatus, c->stream);
     } else if (precision == RS_GRAM_BF16X3) {
@@ -231,6 +232,10 @@ rs_status rs_gram(rs_ctx* c, const rs_batch* b, int precision, double* K, void* 
     return e == cudaSuccess ? RS_OK : cuda_fail(c, e, "rs_gram");
 }
 
+rs_status rs_gram(rs_ctx* c, const rs_batch* b, int precision, double* K, void* ws, size_t ws_bytes) {
+    return c ? gram(c, b, b, precision, K, ws, ws_bytes) : RS_EINVAL;
+}
+
 }  // extern "C"
 
 extern "C" {
@@ -245,6 +250,9 @@ rs_status rs_rec_offsets(rs_ctx* c, const rs_batch* b, const rs_splits* sp, int6
     cudaError_t e = rs_launch_rec_offsets(b, sp, ro, c->scan, c->dstatus, c->stream);
     return e == cudaSuccess ? RS_OK : cuda_fail(c, e, "rs_rec_offsets");
 }
+
+// Splits that by their number are leave-one-version-out (rs_launch_fit_predict looks for its closed form).
+static int lovo_sizes(const rs_batch* b, const rs_splits* sp) { return sp->n_splits == b->n_rows; }
 
 static rs_status fit_common(rs_ctx* c, const rs_batch* b, const double* K, const rs_splits* sp,
                             double lambda, int form, rs_fit_args& a) {
@@ -269,7 +277,7 @@ static rs_status fit_common(rs_ctx* c, const rs_batch* b, const double* K, const
     a.lambda = lambda;
     a.form = form;
     a.max_feat = b->max_feat;
-    a.lovo = sp->n_splits == b->n_rows;
+    a.lovo = lovo_sizes(b, sp);
     a.dstatus = c->dstatus;
     a.queue = (unsigned int*)(c->dstatus + RS_DST_QUEUE);
     a.ev = c->profiling ? c->ev : nullptr;
@@ -607,6 +615,11 @@ size_t rs_fallback_workspace_bytes(const rs_batch* b, const rs_splits* sp) {
     return carve_fallback(nullptr, b, sp).bytes;
 }
 
+static rs_status cv_step(rs_ctx* c, const rs_batch* b, const rs_splits* sp, const rs_batch* all,
+                         const rs_splits* all_sp, double lambda, int k, double tau, int flags, int precision, void* ws,
+                         size_t ws_bytes, int64_t* rec_offsets, uint32_t* rec_code, double* rec_pred,
+                         double* pred_all, uint64_t* counters);
+
 rs_status rs_surrogate_fallback(rs_ctx* c, const rs_batch* b, const rs_splits* sp, const uint8_t* used_fallback,
                                 double lambda, int k, double tau, int flags, void* ws, size_t ws_bytes,
                                 uint32_t* rec_code, double* rec_pred, int64_t* refit) {
@@ -652,8 +665,8 @@ rs_status rs_surrogate_fallback(rs_ctx* c, const rs_batch* b, const rs_splits* s
         ss.n_test_rows = tot[4];
         ss.split_offsets = w.sub_split_off;
         ss.train_masks = w.s_train;
-        s = rs_cv_step(c, &sb, &ss, lambda, k, tau, flags, RS_GRAM_F64, w.cv_ws, w.cv_ws_bytes, w.s_rec_off,
-                       w.s_code, w.s_pred, nullptr, nullptr);
+        s = cv_step(c, &sb, &ss, b, sp, lambda, k, tau, flags, RS_GRAM_F64, w.cv_ws, w.cv_ws_bytes, w.s_rec_off,
+                    w.s_code, w.s_pred, nullptr, nullptr);
         if (s != RS_OK) return s;
         e = rs_launch_fallback_merge(b, used_fallback, w, k, rec_code, rec_pred, c->stream);
         if (e != cudaSuccess) return cuda_fail(c, e, "rs_surrogate_fallback (merge)");
@@ -674,10 +687,12 @@ size_t rs_cv_workspace_bytes(const rs_batch* b, const rs_splits* sp) {
     return z + k + (f > g ? f : g);     // the Gram's scratch is free again when the fits start
 }
 
-rs_status rs_cv_step(rs_ctx* c, const rs_batch* b, const rs_splits* sp, double lambda, int k,
-                     double tau, int flags, int precision, void* ws, size_t ws_bytes,
-                     int64_t* rec_offsets, uint32_t* rec_code, double* rec_pred,
-                     double* pred_all, uint64_t* counters) {
+// rs_cv_step.  all, all_sp: the batch and splits whose sizes choose between forms that round differently
+// (of the Gram and of the fits) -- b and sp, or those that they are a part of.
+static rs_status cv_step(rs_ctx* c, const rs_batch* b, const rs_splits* sp, const rs_batch* all,
+                         const rs_splits* all_sp, double lambda, int k, double tau, int flags, int precision, void* ws,
+                         size_t ws_bytes, int64_t* rec_offsets, uint32_t* rec_code, double* rec_pred,
+                         double* pred_all, uint64_t* counters) {
     if (!c) return RS_EINVAL;
     rs_status s = check_batch(c, b, true);
     if (s != RS_OK) return s;
@@ -708,10 +723,11 @@ rs_status rs_cv_step(rs_ctx* c, const rs_batch* b, const rs_splits* sp, double l
     s = predict_args(c, &zb, K, sp, lambda, nullptr, k, tau, flags, RS_FORM_BATCHED, fws, fbytes,
                      rec_offsets, rec_code, rec_pred, pred_all, counters, a);
     if (s != RS_OK) return s;
+    a.lovo = lovo_sizes(all, all_sp);
     cudaSetDevice(c->device);
     cudaError_t e = cudaSuccess;
-    auto gram = [&]() -> rs_status {     // the learner IBK compares distances only: any that order alike will do
-        if (!(flags & RS_MODEL_IBK)) return rs_gram(c, &zb, precision, K, fws, fbytes);
+    auto block = [&]() -> rs_status {    // the learner IBK compares distances only: any that order alike will do
+        if (!(flags & RS_MODEL_IBK)) return gram(c, &zb, all, precision, K, fws, fbytes);
         const cudaError_t eg = rs_launch_dist2_order(&zb, K, c->dstatus, c->stream);
         return eg == cudaSuccess ? RS_OK : cuda_fail(c, eg, "rs_gram");
     };
@@ -719,7 +735,7 @@ rs_status rs_cv_step(rs_ctx* c, const rs_batch* b, const rs_splits* sp, double l
         // one stream, in order: the tensor-core Gram's scratch is the fit workspace, which the
         // planning fills afterwards
         s = rs_standardize(c, b, Z, nullptr, nullptr);
-        if (s == RS_OK) s = gram();
+        if (s == RS_OK) s = block();
         if (s != RS_OK) return s;
         e = rs_launch_rec_offsets(&zb, sp, rec_offsets, c->scan, c->dstatus, c->stream);
         if (e == cudaSuccess) e = rs_launch_fit_predict(a, c->stream);
@@ -738,13 +754,21 @@ rs_status rs_cv_step(rs_ctx* c, const rs_batch* b, const rs_splits* sp, double l
     if (e == cudaSuccess) e = cudaEventRecord(c->join, c->side);
     if (e != cudaSuccess) return cuda_fail(c, e, "rs_cv_step (planning)");
     s = rs_standardize(c, b, Z, nullptr, nullptr);
-    if (s == RS_OK) s = gram();
+    if (s == RS_OK) s = block();
     e = cudaStreamWaitEvent(c->stream, c->join, 0);   // joined whatever happened above
     if (s != RS_OK) return s;
     if (e != cudaSuccess) return cuda_fail(c, e, "rs_cv_step (join)");
     a.phase = 2;
     e = rs_launch_fit_predict(a, c->stream);
     return e == cudaSuccess ? RS_OK : cuda_fail(c, e, "rs_cv_step");
+}
+
+rs_status rs_cv_step(rs_ctx* c, const rs_batch* b, const rs_splits* sp, double lambda, int k,
+                     double tau, int flags, int precision, void* ws, size_t ws_bytes,
+                     int64_t* rec_offsets, uint32_t* rec_code, double* rec_pred,
+                     double* pred_all, uint64_t* counters) {
+    return cv_step(c, b, sp, b, sp, lambda, k, tau, flags, precision, ws, ws_bytes, rec_offsets, rec_code, rec_pred,
+                   pred_all, counters);
 }
 
 

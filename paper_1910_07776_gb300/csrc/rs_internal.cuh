@@ -97,7 +97,9 @@ __device__ __forceinline__ int rs_group_layout(int q, const int64_t* group_off, 
 // ---- launchers (defined in the kernel translation units) -------------------------------
 cudaError_t rs_launch_standardize(const rs_batch* b, double* Z, double* mu, double* sigma,
                                   int* dstatus, cudaStream_t st);
-cudaError_t rs_launch_gram_f64(const rs_batch* b, double* K, int* dstatus, cudaStream_t st);
+// sizes: the batch whose sizes choose the form (k_gram.cu) -- b, or the one that b is a part of: the two
+// forms round differently, and a part has to come out as in the whole.
+cudaError_t rs_launch_gram_f64(const rs_batch* b, double* K, int* dstatus, cudaStream_t st, const rs_batch* sizes);
 cudaError_t rs_launch_gram_split(const rs_batch* b, double* K, int* dstatus, cudaStream_t st);
 cudaError_t rs_launch_dist2_f64(const rs_batch* b, double* K, int* dstatus, cudaStream_t st);
 // Distances that compare within each row like those of rs_launch_dist2_f64 (nearest neighbours).

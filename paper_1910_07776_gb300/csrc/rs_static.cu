@@ -148,7 +148,7 @@ extern "C" rs_status rs_cv_step_static(void* cuda_stream, const rs_batch* b, con
     rs_batch zb = *b;
     zb.X = Z;
     zb.dtype = RS_F64;
-    if (e == cudaSuccess) e = rs_launch_gram_f64(&zb, K, dstatus, st);
+    if (e == cudaSuccess) e = rs_launch_gram_f64(&zb, K, dstatus, st, &zb);
     if (e == cudaSuccess) e = rs_launch_rec_offsets(&zb, sp, rec_offsets, scan, dstatus, st);
     if (e == cudaSuccess && sp->n_splits > 0) {
         rs_fit_args a;
