@@ -1555,6 +1555,11 @@ constexpr int kLooFitThreads = 256;
 // it: the condition number is then at most n^2 q = 4e6, an error of the inverse below 5e-10 even
 // at that bound.  (Typical systems: q of tens; it passes the limit near as many features as pairs.)
 constexpr float kLooLimit = 4096.f;
+// Systems of n pairs with F < n features are not tried: K_PP has n - F eigenvalues 0, M those of lambda, and q
+// comes to about F / lambda (z-scores: M_ii about F), unless lambda is large enough for that.
+__host__ __device__ __forceinline__ bool loo_narrow(int F, int n, double lambda) {
+    return F < n && (double)F > (double)kLooLimit * lambda;
+}
 
 // One block per (program, optimization): the symmetric sweep operator over the lower triangle of
 //   [ M  . ]        with M = K_PP + lambda I of its n pairs (symmetric positive definite, no
@@ -1582,9 +1587,9 @@ constexpr int kLooPer = 5;
 static_assert(kLooEntries <= 4 * kLooThreads + (kLooThreads - 32), "4 entries in warp 0's threads, 5 in the others'");
 
 __global__ void __launch_bounds__(kLooThreads)
-loo_inv_kernel(const int64_t* __restrict__ row_off, const double* __restrict__ K,
+loo_inv_kernel(const int64_t* __restrict__ row_off, const int32_t* __restrict__ fw, const double* __restrict__ K,
                const uint8_t* __restrict__ pb, const double* __restrict__ ylab,
-               const int* __restrict__ npair, const double* __restrict__ dlam, float limit, double* tab,
+               const int* __restrict__ npair, const double* __restrict__ dlam, double lambda, float limit, double* tab,
                uint8_t* ok, uint32_t* bad) {
     tc::in_sequence();
     __shared__ double col[2][RS_MAXPAIRS + 2];                  // column k as it stands, by row
@@ -1595,7 +1600,7 @@ loo_inv_kernel(const int64_t* __restrict__ row_off, const double* __restrict__ K
     const int pj = blockIdx.x, p = pj / RS_NOPT, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int V = (int)(row_off[p + 1] - row_off[p]);
     const int n = V >= 1 && V <= RS_MAXV ? npair[pj] : 0;
-    if (n < 1 || n > RS_MAXPAIRS) {
+    if (n < 1 || n > RS_MAXPAIRS || (limit > 0.f && loo_narrow(fw[p], n, lambda))) {
         if (tid == 0) {
             ok[pj] = 0;
             bad[pj] = 0;
@@ -2619,8 +2624,8 @@ cudaError_t rs_launch_fit_predict(const rs_fit_args& a, cudaStream_t st) {
         mark(4);
     } else if (a.flags & RS_LOO_CLOSED) {
         // one inverse per (program, optimization), then every fit in closed form
-        e = tc::launch_after(loo_inv_kernel, (unsigned)(a.P * RS_NOPT), kLooThreads, 0, st, a.row_offsets, a.K, w.pb, w.ylab,
-                             w.npair, w.dlam, 0.f, w.loo_tab, w.loo_ok, w.loo_bad);
+        e = tc::launch_after(loo_inv_kernel, (unsigned)(a.P * RS_NOPT), kLooThreads, 0, st, a.row_offsets, a.feat_width, a.K,
+                             w.pb, w.ylab, w.npair, w.dlam, a.lambda, 0.f, w.loo_tab, w.loo_ok, w.loo_bad);
         if (e != cudaSuccess) return e;
         const int64_t grid = (S6 + kLooFitThreads - 1) / kLooFitThreads;
         e = tc::launch_after(loo_fit_kernel<false>, (unsigned)grid, kLooFitThreads, 0, st, sa, S6, w.npair, w.loo_tab,
@@ -2648,11 +2653,15 @@ cudaError_t rs_launch_fit_predict(const rs_fit_args& a, cudaStream_t st) {
         // own rounding while the condition bound q stays below the limit (relative prediction
         // errors within 0.9-1.3 of each other, 48..1024 features: equal).  256 programs x 64
         // versions x 1024 features: the fit stage 1.95 -> 0.15 ms.
-        const bool lovo = a.lovo && nmax > kNMid && (user || rank) && a.lambda > 0.0;
+        // Not looked for where the programs have fewer features than pairs (loo_narrow): every fit would be left,
+        // after the inverses and without the second stream (2 programs x 64 versions x 24 features 180 us
+        // where 110 do, 256 programs 1889 and 1801).
+        const bool lovo = a.lovo && nmax > kNMid && (user || rank) && a.lambda > 0.0 &&
+                          !loo_narrow(a.max_feat, (a.max_train + 1) / 2, a.lambda);
         if (lovo) {
             sa.left = w.work + 5;
-            e = tc::launch_after(loo_inv_kernel, (unsigned)(a.P * RS_NOPT), kLooThreads, 0, st, a.row_offsets, a.K, w.pb,
-                                 w.ylab, w.npair, w.dlam, kLooLimit, w.loo_tab, w.loo_ok, w.loo_bad);
+            e = tc::launch_after(loo_inv_kernel, (unsigned)(a.P * RS_NOPT), kLooThreads, 0, st, a.row_offsets, a.feat_width,
+                                 a.K, w.pb, w.ylab, w.npair, w.dlam, a.lambda, kLooLimit, w.loo_tab, w.loo_ok, w.loo_bad);
             if (e != cudaSuccess) return e;
             const int64_t grid = (S6 + kLooFitThreads - 1) / kLooFitThreads;
             e = tc::launch_after(loo_fit_kernel<true>, (unsigned)grid, kLooFitThreads, 0, st, sa, S6, w.npair, w.loo_tab,

@@ -251,9 +251,6 @@ rs_status rs_rec_offsets(rs_ctx* c, const rs_batch* b, const rs_splits* sp, int6
     return e == cudaSuccess ? RS_OK : cuda_fail(c, e, "rs_rec_offsets");
 }
 
-// Splits that by their number are leave-one-version-out (rs_launch_fit_predict looks for its closed form).
-static int lovo_sizes(const rs_batch* b, const rs_splits* sp) { return sp->n_splits == b->n_rows; }
-
 static rs_status fit_common(rs_ctx* c, const rs_batch* b, const double* K, const rs_splits* sp,
                             double lambda, int form, rs_fit_args& a) {
     rs_status s = check_batch(c, b, false);
@@ -277,7 +274,7 @@ static rs_status fit_common(rs_ctx* c, const rs_batch* b, const double* K, const
     a.lambda = lambda;
     a.form = form;
     a.max_feat = b->max_feat;
-    a.lovo = lovo_sizes(b, sp);
+    a.lovo = rs_lovo_sizes(b, sp);
     a.dstatus = c->dstatus;
     a.queue = (unsigned int*)(c->dstatus + RS_DST_QUEUE);
     a.ev = c->profiling ? c->ev : nullptr;
@@ -723,7 +720,7 @@ static rs_status cv_step(rs_ctx* c, const rs_batch* b, const rs_splits* sp, cons
     s = predict_args(c, &zb, K, sp, lambda, nullptr, k, tau, flags, RS_FORM_BATCHED, fws, fbytes,
                      rec_offsets, rec_code, rec_pred, pred_all, counters, a);
     if (s != RS_OK) return s;
-    a.lovo = lovo_sizes(all, all_sp);
+    a.lovo = rs_lovo_sizes(all, all_sp);
     cudaSetDevice(c->device);
     cudaError_t e = cudaSuccess;
     auto block = [&]() -> rs_status {    // the learner IBK compares distances only: any that order alike will do

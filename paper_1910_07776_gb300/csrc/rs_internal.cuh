@@ -159,6 +159,12 @@ cudaError_t rs_launch_fallback_gather(const rs_batch* b, const rs_splits* sp, in
 cudaError_t rs_launch_fallback_merge(const rs_batch* b, const uint8_t* used, const rs_fallback_ws& w, int k,
                                      uint32_t* rec_code, double* rec_pred, cudaStream_t st);
 
+// Splits that by the host's sizes may be leave-one-version-out: as many as versions, and the largest training
+// set at least the mean program's versions but one (half splits in the same number are not).
+inline int rs_lovo_sizes(const rs_batch* b, const rs_splits* sp) {
+    return sp->n_splits == b->n_rows && (sp->max_train + 1) * (int64_t)b->n_programs >= b->n_rows;
+}
+
 struct rs_fit_args {
     // batch (standardized)
     int P;

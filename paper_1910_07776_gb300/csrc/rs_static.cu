@@ -177,7 +177,7 @@ extern "C" rs_status rs_cv_step_static(void* cuda_stream, const rs_batch* b, con
         a.dstatus = dstatus;
         a.queue = (unsigned int*)(dstatus + RS_DST_QUEUE);
         a.max_train = sp->max_train;
-        a.lovo = sp->n_splits == b->n_rows;
+        a.lovo = rs_lovo_sizes(b, sp);
         a.rows_cap = rows_cap;
         a.workspace = fws;
         a.workspace_bytes = f_bytes;

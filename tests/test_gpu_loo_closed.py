@@ -324,3 +324,23 @@ def test_coefficients_without_the_flag_equal_the_direct_fits(rs, ctx):
     ok = sg == 0
     scale = np.abs(cp[ok]).max(axis=1, keepdims=True)
     assert np.all(np.abs(cg[ok] - cp[ok]) <= 1e-9 * scale + 1e-11)
+
+
+@pytest.mark.parametrize("feat,lam,held_out", [(24, 1e-3, 1), (31, 1e-3, 1), (32, 1e-3, 1), (24, 1.0, 1), (64, 1e-3, 9)])
+def test_as_many_splits_as_versions_where_the_closed_form_is_not_looked_for(rs, ctx, feat, lam, held_out):
+    """Fewer features than pairs (unless lambda is large), and several versions held out in as many splits
+    as versions: the direct fits, against the plain form.  Tolerance as above."""
+    batch = synth.make_batch(3, versions=64, feat=feat, dtype=np.float64, seed=95)
+    rng, full, tm = np.random.default_rng(95), (1 << 64) - 1, []
+    for p in range(3):
+        for r in range(64):
+            out = [r] + list(rng.choice([v for v in range(64) if v != r], held_out - 1, replace=False))
+            tm.append(full & ~sum(1 << int(v) for v in out))
+    splits = synth.Splits(split_offsets=batch.row_offsets.copy(), train_masks=np.array(tm, dtype=np.uint64))
+    db, ds = rs.DeviceBatch.from_host(batch), rs.DeviceSplits.from_host(splits, batch=batch)
+    g = rs.cv_run(ctx, db, ds, lam=lam)
+    r = rs.cv_run(ctx, db, ds, lam=lam, form=rs.RS_FORM_PLAIN)
+    np.testing.assert_array_equal(g["rec_offsets"], r["rec_offsets"])
+    close(g["pred_all"], r["pred_all"], abs_=4e6 * 2.0 ** -53)
+    _, nnear = compare_rankings(g["rec_code"], r["rec_code"], r["pred_all"], math.log(1.05))
+    compare_counters(g["counters"], r["counters"], slack=nnear)
