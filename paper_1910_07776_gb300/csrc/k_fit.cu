@@ -193,13 +193,13 @@ constexpr int kPlanProgs = 8;                // programs whose pair tables a pla
 // the row's scoring summary | version mask << 30 | mask of the split's empty fits << 36.
 __global__ void __launch_bounds__(256)
 plan_fits_kernel(int P, const int64_t* __restrict__ row_off, const int64_t* __restrict__ split_off,
-                 const uint64_t* __restrict__ tm, int64_t S, const uint8_t* __restrict__ pb,
-                 const uint8_t* __restrict__ pa, const int* __restrict__ npair, uint32_t* fit_pm,
+                 const uint64_t* __restrict__ tm, int64_t S, const uint8_t* pb,
+                 const uint8_t* pa, const int* npair, uint32_t* fit_pm,
                  uint16_t* fit_key, unsigned* hist, int nmax, int* split_prog,
                  const int64_t* __restrict__ rec_offsets, int64_t rows_cap,
                  unsigned long long* row_info, const uint8_t* __restrict__ masks,
-                 const uint32_t* __restrict__ rowinfo, const uint64_t* __restrict__ cand, int cand_all,
-                 int count_preds, const uint64_t* __restrict__ pset, const uint8_t* __restrict__ psorted,
+                 const uint32_t* rowinfo, const uint64_t* cand, int cand_all,
+                 int count_preds, const uint64_t* pset, const uint8_t* psorted,
                  int* dstatus) {
     tc::in_sequence();
     __shared__ unsigned h[kHist];
@@ -226,7 +226,7 @@ plan_fits_kernel(int P, const int64_t* __restrict__ row_off, const int64_t* __re
             const int t = w / words, r = w - t * words;               // table (before / after), word
             const int q = r / (RS_NOPT * RS_MAXPAIRS / 16), k = r - q * (RS_NOPT * RS_MAXPAIRS / 16);
             const uint8_t* src = (t ? pa : pb) + (int64_t)(p0 + q) * RS_NOPT * RS_MAXPAIRS;
-            reinterpret_cast<uint4*>(&tab[q][t][0][0])[k] = __ldg(reinterpret_cast<const uint4*>(src) + k);
+            reinterpret_cast<uint4*>(&tab[q][t][0][0])[k] = reinterpret_cast<const uint4*>(src)[k];
         }
         for (int i = threadIdx.x; i < np_tab * RS_MAXV; i += blockDim.x) {
             const int q = i / RS_MAXV, t = i - q * RS_MAXV, pq = p0 + q;
@@ -372,7 +372,7 @@ struct PredTarget {
 template <int N>
 __device__ __forceinline__ int fit_fixed(const double* __restrict__ Kp, const uint8_t* __restrict__ pb,
                                          const double* __restrict__ yl, uint32_t pm,
-                                         const double* __restrict__ dl, double* out, double (&ty)[N],
+                                         const double* dl, double* out, double (&ty)[N],
                                          double& b, int (&vb)[N]) {
     double t1[N], L[tri(N)], dinv[N];
     uint32_t x = pm;
@@ -385,7 +385,7 @@ __device__ __forceinline__ int fit_fixed(const double* __restrict__ Kp, const ui
     }
     if constexpr (N == 1) {
         // one pair: 1^T alpha = 0 forces alpha = 0, so b = y and every prediction is b
-        if (!pos_finite(__ldg(dl + vb[0]))) return RS_FIT_NOTPD;
+        if (!pos_finite(dl[vb[0]])) return RS_FIT_NOTPD;
         b = ty[0];
         ty[0] = 0.0;
         if (out) {
@@ -405,7 +405,7 @@ __device__ __forceinline__ int fit_fixed(const double* __restrict__ Kp, const ui
             c[k] = s;
             L[tri(i) + k] = s * dinv[k];
         }
-        double d = __ldg(dl + vb[i]);      // K[v][v] + lambda
+        double d = dl[vb[i]];      // K[v][v] + lambda
 #pragma unroll
         for (int m = 0; m < i; ++m) d = fma(-c[m], L[tri(i) + m], d);
         if (!pos_finite(d)) return RS_FIT_NOTPD;
@@ -450,7 +450,7 @@ __device__ __forceinline__ int fit_fixed(const double* __restrict__ Kp, const ui
 template <int N>
 __device__ __forceinline__ int solve_fixed(const double* __restrict__ Kp, const uint8_t* __restrict__ pb,
                                            const double* __restrict__ yl, uint32_t pm,
-                                           const double* __restrict__ dl, double* out,
+                                           const double* dl, double* out,
                                            const PredTarget* pt) {
     double al[N], b = 0.0;
     int vb[N];
@@ -601,10 +601,10 @@ __device__ __forceinline__ double* coef_out(const SolveArgs& a, int64_t f) {
 // A fit without a training pair (n = 0) is finished here (status RS_FIT_EMPTY); the rank
 // pass knows it from the row records.
 __global__ void __launch_bounds__(kBucketThreads, 2)
-bucket_fits_kernel(int64_t S6, const uint16_t* __restrict__ fit_key, const unsigned* __restrict__ hist,
+bucket_fits_kernel(int64_t S6, const uint16_t* fit_key, const unsigned* hist,
                    unsigned* cursor, uint4* recs, int64_t* fit_off, uint8_t* status, double* coef_user,
-                   unsigned long long* counters, const uint32_t* __restrict__ fit_pm,
-                   const int* __restrict__ split_prog, const int64_t* __restrict__ row_off) {
+                   unsigned long long* counters, const uint32_t* fit_pm,
+                   const int* split_prog, const int64_t* __restrict__ row_off) {
     tc::in_sequence();
     __shared__ long long start[kHist], cstart[kHist];
     __shared__ unsigned lcount[kKeys];       // fits per (n, c); then their offsets inside n's range
@@ -869,7 +869,7 @@ ibk_kernel(const SolveArgs a, int nmax, unsigned long long* work) {
 // across the 32 lanes of the warp (element e of this lane at W[32 e]): every access of a
 // warp touches 32 distinct banks.  Layout per lane: L (tri(nmax)), D^-1, t_y, t_1 (nmax each).
 __device__ int solve_var(int n, int nmax, const double* __restrict__ Kp, const uint8_t* __restrict__ pb,
-                         const double* __restrict__ yl, uint32_t pm, const double* __restrict__ dl,
+                         const double* __restrict__ yl, uint32_t pm, const double* dl,
                          double* out, const PredTarget* pt, double* W, int* VB) {
     const int oD = tri(nmax), oY = oD + nmax, oT = oY + nmax;
 #define LW(e) W[(size_t)(e) * 32]
@@ -887,7 +887,7 @@ __device__ int solve_var(int n, int nmax, const double* __restrict__ Kp, const u
             for (int m = 0; m < k; ++m) s = fma(-LW(tri(i) + m), LW(tri(k) + m), s);
             LW(tri(i) + k) = s;
         }
-        double d = __ldg(dl + VB[i * 32]);
+        double d = dl[VB[i * 32]];
         for (int m = 0; m < i; ++m) {          // L(i, m) = c_m / d_m; d_i = M_ii - sum c_m L(i, m)
             const double c = LW(tri(i) + m);
             const double l = c * LW(oD + m);
@@ -1196,7 +1196,7 @@ __device__ int fit_warp_ldl(int n, uint32_t pm, const uint8_t* pair_b, const dou
     for (int jj = 0; jj < n; ++jj) {
         double sv = 0.0;
         if (act && lane >= jj) {
-            sv = lane == jj ? __ldg(dl + v) : Lsh[lane * 33 + jj];
+            sv = lane == jj ? dl[v] : Lsh[lane * 33 + jj];
             for (int m = 0; m < jj; ++m) sv = fma(-Lsh[lane * 33 + m], Ush[jj * 33 + m], sv);
         }
         const double d = __shfl_sync(0xffffffffu, sv, jj);
@@ -1415,7 +1415,7 @@ solve_wide_kernel(const SolveArgs a, unsigned long long* work) {
             int i, jj;
             tri_pos(l, i, jj);
             for (int e = l; e < tri(n); e += kWideLanes, tri_step(i, jj))
-                A[e] = i == jj ? __ldg(dl + VS[i]) : __ldg(Kp + VS[i] * RS_GRAM_LD + VS[jj]);
+                A[e] = i == jj ? dl[VS[i]] : __ldg(Kp + VS[i] * RS_GRAM_LD + VS[jj]);
         }
         __syncwarp();
         // Right-looking LDL^T with a one-pivot lookahead, and the forward substitution of both
@@ -1589,7 +1589,7 @@ static_assert(kLooEntries <= 4 * kLooThreads + (kLooThreads - 32), "4 entries in
 __global__ void __launch_bounds__(kLooThreads)
 loo_inv_kernel(const int64_t* __restrict__ row_off, const int32_t* __restrict__ fw, const double* __restrict__ K,
                const uint8_t* __restrict__ pb, const double* __restrict__ ylab,
-               const int* __restrict__ npair, const double* __restrict__ dlam, double lambda, float limit, double* tab,
+               const int* __restrict__ npair, const double* dlam, double lambda, float limit, double* tab,
                uint8_t* ok, uint32_t* bad) {
     tc::in_sequence();
     __shared__ double col[2][RS_MAXPAIRS + 2];                  // column k as it stands, by row
@@ -1749,8 +1749,8 @@ loo_inv_kernel(const int64_t* __restrict__ row_off, const int32_t* __restrict__ 
 template <bool AUTO>
 __global__ void __launch_bounds__(kLooFitThreads)
 loo_fit_kernel(const SolveArgs a, int64_t S6, const int* __restrict__ npair,
-               const double* __restrict__ tab, const uint8_t* __restrict__ tab_ok,
-               const uint32_t* __restrict__ tab_bad) {
+               const double* tab, const uint8_t* tab_ok,
+               const uint32_t* tab_bad) {
     tc::in_sequence();
     const int64_t f = (int64_t)blockIdx.x * kLooFitThreads + threadIdx.x;
     const int n = f < S6 ? a.fit_key[f] / kCntBins : 0;

@@ -112,10 +112,11 @@ struct EpiHidden {           // U = acc + b (FP32, [unit][B]: a warp's rows side
     __device__ void operator()(int row, int col0, const float (&v)[16]) const {
         unsigned h[8];
         const float4* b4 = reinterpret_cast<const float4*>(bias + col0);
-        float* d = U + (int64_t)col0 * ldu + row;
+        const float4 bias4[4] = {b4[0], b4[1], b4[2], b4[3]};      // (before the stores; the step before may
+        float* d = U + (int64_t)col0 * ldu + row;                   // still be writing: no read-only loads)
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            const float4 b = __ldg(b4 + q);
+            const float4 b = bias4[q];
             const unsigned long long u0 = add2(pk2(v[4 * q], v[4 * q + 1]), pk2(b.x, b.y));
             const unsigned long long u1 = add2(pk2(v[4 * q + 2], v[4 * q + 3]), pk2(b.z, b.w));
             float x, y;

@@ -37,7 +37,9 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
 // tensor memory) while its predecessor's last blocks run; after_predecessor() waits for those and their
 // writes, and comes before the first access to memory that another kernel writes or reads (a kernel
 // that shares nothing with its predecessor, and whose inputs that one has waited for, may wait at its
-// end).  let_successor() comes after the wait where a successor relies on that.
+// end).  let_successor() comes after the wait where a successor relies on that.  What a kernel still running
+// at the launch may write is read by plain loads: no __ldg, no const __restrict__ (read-only loads ask that
+// their data stay as they are for the kernel's whole life).
 __device__ __forceinline__ void let_successor() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void after_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void in_sequence() {      // the plain case, at a kernel's start
