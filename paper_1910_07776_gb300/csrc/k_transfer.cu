@@ -324,7 +324,8 @@ struct M5Smem {
     int nn, task, nsurv;
     double sd_root;
     // the level's nodes (at most kM5MaxN / 2 that split), by node - first of the level
-    float mean[kM5MaxN], tot[kM5MaxN], tot2[kM5MaxN], amax2[kM5MaxN], sda[kM5MaxN];
+    float mean[kM5MaxN], tot[kM5MaxN], tot2[kM5MaxN], amax2[kM5MaxN], sda[kM5MaxN], ymax[kM5MaxN];
+    float mean0;                                  // magnitude of the root's mean
     unsigned best_hi[kM5MaxN];                    // smallest upper bound of Q, as FP32 bits
     unsigned long long best_red[kM5MaxN];         // largest exact SDR, as FP64 bits
     unsigned best_key[kM5MaxN];                   // attribute << 8 | count of the chosen split
@@ -372,6 +373,8 @@ __device__ __forceinline__ double m5_warp_sum(double x) {
 // Bounds of Q = sqrt(c l2 - l1^2) + sqrt((m - c) r2 - r1^2) (SDR = sd - Q / m) from FP32 prefix
 // sums.  Each radicand's error is below 1e-5 n^2 A^2 for n labels of magnitude at most A: labels
 // rounded to FP32 and shifted (1.8e-7 A each), sums by at most 12 additions (7e-7 each way), products.
+// The exact evaluation works on the labels themselves, of magnitude up to Y: its own rounding, up to
+// 6 c m^2 2^-53 Y^2 in a radicand, counts as well, as 6e-7 Y^2 in a2 (a2 = A^2 + 6e-7 Y^2; c >= 2, m <= 128).
 __device__ __forceinline__ void m5_bounds(int c, int m, float l1, float l2, float t1, float t2, float a2, float& lo,
                                           float& hi) {
     const float cl = (float)c, cr = (float)(m - c);
@@ -911,6 +914,7 @@ m5p_fit_kernel(const TransferArgs a, int fmax) {
             S.parent[0] = -1;
         }
         const double mean = s1 / n;
+        if (lane == 0) S.mean0 = fabsf((float)mean);
         for (int i = lane; i < n; i += 32) S.yf[i] = (float)(S.y[i] - mean);
     }
     __syncthreads();
@@ -954,7 +958,8 @@ m5p_fit_kernel(const TransferArgs a, int fmax) {
             bool leaf = m < 4;
             const float sda = sqrtf(t2 / (float)m), lim = (float)(kM5SdFrac * S.sd_root);
             const bool fp32 = t2 < 1e30f && am < 1e15f && lim > 1e-15f;
-            const float slack = 1e-3f * lim + 4e-6f * am;
+            // (the exact deviation's rounding: below sqrt(4e-14) of the labels' magnitude)
+            const float ymax = am + 1.001f * S.mean0, slack = 1e-3f * lim + 4e-6f * am + 3e-7f * ymax;
             if (!leaf && fp32 && sda < lim - slack) leaf = true;
             int cnt = leaf ? -1 : 0;
             if (!leaf) {
@@ -978,7 +983,8 @@ m5p_fit_kernel(const TransferArgs a, int fmax) {
                 S.mean[k] = mean;
                 S.tot[k] = t1;
                 S.tot2[k] = t2;
-                S.amax2[k] = am * am;
+                S.amax2[k] = am * am + 6e-7f * ymax * ymax;
+                S.ymax[k] = ymax;
                 S.sda[k] = sda;
                 S.best_hi[k] = 0x7f800000u;
                 S.best_red[k] = 0ull;
@@ -1016,7 +1022,7 @@ m5p_fit_kernel(const TransferArgs a, int fmax) {
             const bool here = x < nsv && S.surv[x] != 0xffffffffu;
             const int k = (int)(sv >> 16), f = (int)(sv >> 8) & 0xff, c = (int)(sv & 0xff);
             const int t = n0 + k, lo = S.lo[t], m = S.hi[t] - lo;
-            const bool sure = here && S.cnt[k] == 1 && __uint_as_float(S.best_hi[k]) < 0.999f * (float)m * S.sda[k] - 1e-5f * (float)m * sqrtf(S.amax2[k]);
+            const bool sure = here && S.cnt[k] == 1 && __uint_as_float(S.best_hi[k]) < 0.999f * (float)m * S.sda[k] - (float)m * (1e-5f * sqrtf(S.amax2[k]) + 3e-7f * S.ymax[k]);
             const bool work = here && !sure;
             double sdx = 0.0;
             if (work) {

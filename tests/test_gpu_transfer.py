@@ -216,6 +216,23 @@ def test_m5p_pairs_of_nearly_equal_counters(rs, ctx, gap, seed):
     close(g["pred_all"], r.pred_all, rel=max(1e-7, tol), abs_=max(1e-9, tol))
 
 
+@pytest.mark.parametrize("spread", [1e-2, 1e-4, 1e-5, 1e-6])
+def test_m5p_labels_close_to_a_common_value(rs, ctx, spread):
+    """Every optimization's speedup near one value: what the deviations of labels 1 +- spread are by the
+    reference's arithmetic (sums of squares) is more and more its rounding, and its decisions are
+    followed all the same."""
+    runs_per = 3
+    b = synth.make_batch(4 * runs_per + 4, versions=64, feat=24, dtype=np.float64, seed=610)
+    bits = (np.arange(64)[:, None] >> np.arange(6)) & 1
+    for p in range(b.n_programs):
+        rows = b.program_rows(p)
+        b.log_time[rows] = spread * b.log_time[rows] - bits[b.masks[rows]].sum(axis=1)
+    train = synth.take_programs(b, list(range(4 * runs_per)))
+    test = synth.take_programs(b, list(range(4 * runs_per, 4 * runs_per + 4)))
+    g, r = _both(rs, ctx, train, test, np.arange(5, dtype=np.int64) * runs_per, "m5p", flags=oracle.RANK_ALL)
+    _check(g, r, "m5p")
+
+
 @pytest.mark.parametrize("feat,runs_per,versions,case", [
     (64, 1, (64, 64), "plain"), (72, 1, (2, 40), "plain"), (257, 1, (50, 64), "plain"), (33, 3, (64, 64), "plain"),
     (64, 2, (33, 64), "plain"), (129, 3, (1, 64), "plain"), (321, 4, (60, 64), "plain"), (96, 3, (64, 64), "far"),
