@@ -807,6 +807,16 @@ def run_ibk(rs, ctx, batch, splits, dev, stream, flush, args):
     return out
 
 
+def with_one_more_split(splits):
+    """The splits and a copy of the last one.  As they are then not as many as versions, the closed form of
+    leave-one-version-out fits is not looked for: every fit is the direct solvers', and the rows of the
+    splits proper come first and in the same order."""
+    from paper_1910_07776_gb300 import synth
+    offs = splits.split_offsets.copy()
+    offs[-1] += 1
+    return synth.Splits(split_offsets=offs, train_masks=np.concatenate([splits.train_masks, splits.train_masks[-1:]]))
+
+
 def run_lovo(rs, ctx, dev, stream, flush, args, programs=256):
     """Leave-one-version-out (the paper's protocol over all 64 masks, Sec. 5) at the
     precision form's shape: 256 programs x 64 versions x 1024 FP64 features, 16,384 splits,
@@ -815,19 +825,21 @@ def run_lovo(rs, ctx, dev, stream, flush, args, programs=256):
     optimization, every fit from it in O(n)); the fit stage (from the end of the planning to the
     join of the solver streams) against the inverses' FP64 flops gives its roofline fraction, and
     the Gram (1.07 GFLOP) is timed alone beside it.  The same step asked for the closed form
-    (RS_LOO_CLOSED) is timed beside it, with its largest prediction difference."""
+    (RS_LOO_CLOSED) is timed beside it, and by the direct solvers (with_one_more_split), with the closed
+    form's largest prediction difference from those."""
     import torch
     from paper_1910_07776_gb300 import synth
     b = synth.make_batch_fast(programs, versions=64, feat=1024, dtype=np.float64, seed=43)
     sp = synth.make_splits(b, "lovo")
     db = rs.DeviceBatch.from_host(b, dev)
     ds = rs.DeviceSplits.from_host(sp, dev, b)
+    dd = rs.DeviceSplits.from_host(with_one_more_split(sp), dev, b)
     R = ds.n_test_rows
-    ws = ctx.workspace(ctx.cv_workspace_bytes(db, ds))
+    ws = ctx.workspace(ctx.cv_workspace_bytes(db, dd))
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
 
-    def timed(flags):
-        o = rs.alloc_outputs(R, ds.n_splits, CFG["k"], dev)
+    def timed(flags, ds):
+        o = rs.alloc_outputs(ds.n_test_rows, ds.n_splits, CFG["k"], dev)
         step = lambda: ctx.cv_step(db, ds, ws, o.rec_offsets, o.rec_code, lam=CFG["lam"], k=CFG["k"],
                                    tau=CFG["tau"], flags=flags, rec_pred=o.rec_pred, pred_all=o.pred_all,
                                    counters=o.counters)
@@ -850,8 +862,9 @@ def run_lovo(rs, ctx, dev, stream, flush, args, programs=256):
         ctx.check_device_status()
         return tot / reps, stages, o
 
-    ms, stages, o = timed(0)
-    ms_c, stages_c, oc = timed(rs.RS_LOO_CLOSED)
+    ms, stages, o = timed(0, ds)
+    ms_c, stages_c, oc = timed(rs.RS_LOO_CLOSED, ds)
+    ms_d, stages_d, od = timed(0, dd)
     Z = torch.empty(db.x_elems, dtype=torch.float64, device=dev)
     K = torch.zeros(db.n_programs * 64 * 64, dtype=torch.float64, device=dev)
     ctx.standardize(db, Z)
@@ -868,7 +881,7 @@ def run_lovo(rs, ctx, dev, stream, flush, args, programs=256):
     solve_ms = stages.get("solve", 0.0) + stages.get("solve_join", 0.0)
     c = o.counters.cpu().numpy().view(np.uint64).astype(np.float64)
     cc = oc.counters.cpu().numpy().view(np.uint64).astype(np.float64)
-    pa, pc = o.pred_all.cpu().numpy(), oc.pred_all.cpu().numpy()
+    pa, pc = od.pred_all.cpu().numpy().reshape(-1)[:6 * R], oc.pred_all.cpu().numpy().reshape(-1)[:6 * R]
     fin = ~np.isnan(pa)
     same_nan = bool(np.array_equal(np.isnan(pa), np.isnan(pc)))
     diff = np.abs(pa[fin] - pc[fin])
@@ -890,7 +903,7 @@ def run_lovo(rs, ctx, dev, stream, flush, args, programs=256):
               "max_abs_pred_diff_vs_direct": float(diff.max()) if diff.size else 0.0,
               "max_rel_pred_diff_vs_direct": float((diff / np.maximum(np.abs(pa[fin]), 1e-300)).max()) if diff.size else 0.0,
               "nan_pattern_equal": same_nan,
-              "rec_code_rows_differing": int((o.rec_code != oc.rec_code).sum().item())}
+              "rec_code_rows_differing": int((od.rec_code[:R] != oc.rec_code[:R]).sum().item())}
     return {"workload": f"{programs} programs x 64 versions (all masks) x 1024 f64 features, "
                         f"leave-one-version-out ({64 * programs:,} splits, {384 * programs:,} fits of 31 pairs)",
             "ms_per_step": ms, "value": R / (ms * 1e-3), "unit": UNIT, "recs_per_step": R,
@@ -902,6 +915,7 @@ def run_lovo(rs, ctx, dev, stream, flush, args, programs=256):
                          "ms": solve_ms,
                          "peak_source": "FP64 1.25 TFLOP/s nominal (152 SMs x 2 FMA/clk x 2.07 GHz)"},
             "closed_form": closed,
+            "direct": {"ms_per_step": ms_d, "stages_ms": stages_d},
             "gram_alone": {"ms": g_ms, "flops": work["gram_flops"],
                            "frac_fp64": work["gram_flops"] / (g_ms * 1e-3) / 1e12 / fp64_peak}}
 
@@ -1147,7 +1161,7 @@ def _rel_stats(d, ref):
 
 
 def precision_coef_errors(rs, ctx, batch, dev, programs=4):
-    """Per-coefficient errors of the BF16x3 forms (raw, refined) against the FP64 GPU path on
+    """Per-coefficient errors of the BF16x3 forms (raw, refined) against the FP64 GPU path's direct fits on
     the first `programs` programs of a leave-one-version-out batch: the dual alpha and b of
     every fit and the primal beta = sum_a alpha_a z_a it implies (computed on the host in FP64
     from the standardized features), each as elementwise relative error (median, 99th
@@ -1161,14 +1175,15 @@ def precision_coef_errors(rs, ctx, batch, dev, programs=4):
     Z = ctx.standardize(db)
     zb = db.with_X(Z)
     Zh = Z.cpu().numpy()
+    dd = rs.DeviceSplits.from_host(with_one_more_split(sp), dev, sub)
     S = ds.n_splits
     coefs = {}
     for name, prec, flags in (("f64", rs.RS_GRAM_F64, 0), ("bf16x3", rs.RS_GRAM_BF16X3, 0),
                               ("bf16x3_refined", rs.RS_GRAM_BF16X3, rs.RS_REFINE_X)):
         K = ctx.gram(zb, prec)
-        c = torch.zeros(S * 6 * 33, dtype=torch.float64, device=dev)
-        ctx.fit_batched(zb, K, ds, CFG["lam"], rs.RS_FORM_BATCHED | flags, c)
-        coefs[name] = c.cpu().numpy().reshape(S, 6, 33)
+        c = torch.zeros((S + 1) * 6 * 33, dtype=torch.float64, device=dev)
+        ctx.fit_batched(zb, K, dd if name == "f64" else ds, CFG["lam"], rs.RS_FORM_BATCHED | flags, c)
+        coefs[name] = c.cpu().numpy().reshape(S + 1, 6, 33)
     beta = {k: [] for k in coefs}
     alpha = {k: [] for k in coefs}
     bias = {k: [] for k in coefs}
@@ -1203,9 +1218,10 @@ def precision_coef_errors(rs, ctx, batch, dev, programs=4):
 def run_precision(rs, ctx, dev, stream, flush, args):
     """Precision form: 256 programs x 64 versions x 1024 FP64 features, leave-one-version-out,
     a condition-number sweep by random mixing; BF16-split tensor-core Gram + FP64 factorisation
-    + one refinement step through Z, against the FP64 path (itself within 1e-9 of the CPU
+    + one refinement step through Z, against the FP64 path with direct fits (itself within 1e-9 of the CPU
     reference).  Reports errors of the raw and refined forms per kappa and their timings, and
-    those of the FP64 and the tensor-core paths with their fits in closed form (RS_LOO_CLOSED)."""
+    those of the FP64 and the tensor-core paths with their fits in closed form (RS_LOO_CLOSED; all calls
+    without it but f64_direct take that form by themselves where the systems allow it)."""
     import torch
     from paper_1910_07776_gb300 import synth
     base = synth.make_batch_fast(256, versions=64, feat=1024, dtype=np.float64, seed=21)
@@ -1217,40 +1233,43 @@ def run_precision(rs, ctx, dev, stream, flush, args):
         b = synth.apply_mixing(base, kappa, seed=21)
         db = rs.DeviceBatch.from_host(b, dev)
         ds = rs.DeviceSplits.from_host(splits, dev, b)
+        dd = rs.DeviceSplits.from_host(with_one_more_split(splits), dev, b)
         R = ds.n_test_rows
-        ws = ctx.workspace(ctx.cv_workspace_bytes(db, ds))
+        ws = ctx.workspace(ctx.cv_workspace_bytes(db, dd))
         if "gram_autotune" not in res:              # the tensor-core Gram's tile shape, 1024 features
             res["gram_autotune"] = ctx.autotune_gram(db, ws)
         outs = {}
         times = {}
-        for name, prec, flags in (("f64", rs.RS_GRAM_F64, 0), ("bf16x3", rs.RS_GRAM_BF16X3, 0),
+        for name, prec, flags in (("f64_direct", rs.RS_GRAM_F64, 0), ("f64", rs.RS_GRAM_F64, 0),
+                                  ("bf16x3", rs.RS_GRAM_BF16X3, 0),
                                   ("bf16x3_refined", rs.RS_GRAM_BF16X3, rs.RS_REFINE_X),
                                   ("f64_closed_form", rs.RS_GRAM_F64, rs.RS_LOO_CLOSED),
                                   ("bf16x3_closed_form", rs.RS_GRAM_BF16X3, rs.RS_LOO_CLOSED)):
-            o = rs.alloc_outputs(R, ds.n_splits, CFG["k"], dev)
-            ctx.cv_step(db, ds, ws, o.rec_offsets, o.rec_code, lam=CFG["lam"], k=CFG["k"], tau=CFG["tau"],
+            sd = dd if name == "f64_direct" else ds
+            o = rs.alloc_outputs(sd.n_test_rows, sd.n_splits, CFG["k"], dev)
+            ctx.cv_step(db, sd, ws, o.rec_offsets, o.rec_code, lam=CFG["lam"], k=CFG["k"], tau=CFG["tau"],
                         flags=flags, precision=prec, rec_pred=o.rec_pred, pred_all=o.pred_all)
             torch.cuda.synchronize()
             flush.fill_(1)
             e0.record(stream)
-            ctx.cv_step(db, ds, ws, o.rec_offsets, o.rec_code, lam=CFG["lam"], k=CFG["k"], tau=CFG["tau"],
+            ctx.cv_step(db, sd, ws, o.rec_offsets, o.rec_code, lam=CFG["lam"], k=CFG["k"], tau=CFG["tau"],
                         flags=flags, precision=prec, rec_pred=o.rec_pred, pred_all=o.pred_all)
             e1.record(stream)
             torch.cuda.synchronize()
             times[name] = e0.elapsed_time(e1)
-            outs[name] = (o.pred_all.cpu().numpy().reshape(R, 6), o.rec_code.cpu().numpy())
-        ref, rcode = outs["f64"]
+            outs[name] = (o.pred_all.cpu().numpy().reshape(-1, 6)[:R], o.rec_code.cpu().numpy()[:R])
+        ref, rcode = outs["f64_direct"]
         ok = ~np.isnan(ref)
         sc = float(np.abs(ref[ok]).max())
         ent = {}
-        for name in ("bf16x3", "bf16x3_refined", "f64_closed_form", "bf16x3_closed_form"):
+        for name in ("f64", "bf16x3", "bf16x3_refined", "f64_closed_form", "bf16x3_closed_form"):
             pa, code = outs[name]
             d = np.abs(pa[ok] - ref[ok])
             ent[name] = {"max_rel_err_pred": float(d.max() / sc), "median_rel_err_pred": float(np.median(d) / sc),
                          "pred_elementwise": _rel_stats(pa[ok] - ref[ok], ref[ok]),
                          "ranking_rows_changed": int(np.sum(code != rcode)), "ms": times[name],
                          "recs_per_s": R / (times[name] * 1e-3)}
-        ent["f64"] = {"ms": times["f64"], "recs_per_s": R / (times["f64"] * 1e-3)}
+        ent["f64_direct"] = {"ms": times["f64_direct"], "recs_per_s": R / (times["f64_direct"] * 1e-3)}
         ent["coefficients_vs_f64_path"] = precision_coef_errors(rs, ctx, b, dev, programs=4)
         # achieved condition number of one training system (program 0, split 0, optimization 0)
         Zp = np.log(b.program_X(0) / b.cycles[b.program_rows(0)][:, None])

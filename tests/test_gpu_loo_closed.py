@@ -344,3 +344,51 @@ def test_as_many_splits_as_versions_where_the_closed_form_is_not_looked_for(rs, 
     close(g["pred_all"], r["pred_all"], abs_=4e6 * 2.0 ** -53)
     _, nnear = compare_rankings(g["rec_code"], r["rec_code"], r["pred_all"], math.log(1.05))
     compare_counters(g["counters"], r["counters"], slack=nnear)
+
+
+def _one_more(splits):
+    """The splits and a copy of the last one: not as many as versions, so every fit is the direct solvers'."""
+    offs, tm = splits.split_offsets.copy(), splits.train_masks
+    offs[-1] += 1
+    return synth.Splits(split_offsets=offs, train_masks=np.concatenate([tm, tm[-1:]]))
+
+
+@pytest.mark.parametrize("name", ["ragged", "inf_label", "wide"])
+def test_closed_form_coefficients_against_the_direct_solvers(rs, ctx, name):
+    # as test_closed_form_coefficients_equal_the_direct_fits, whose call without the flag takes the
+    # closed form by itself where the sizes allow it
+    batch, splits = _case(name)
+    db = rs.DeviceBatch.from_host(batch)
+    zb = db.with_X(ctx.standardize(db))
+    K = ctx.gram(zb)
+    S = splits.n_splits
+    res = []
+    for sp, form in ((_one_more(splits), rs.RS_FORM_BATCHED), (splits, rs.RS_FORM_BATCHED | rs.RS_LOO_CLOSED)):
+        ds = rs.DeviceSplits.from_host(sp, batch=batch)
+        coef = torch.full((ds.n_splits * 6 * 33,), 7.0, dtype=torch.float64, device="cuda")
+        st = torch.full((ds.n_splits * 6,), 9, dtype=torch.uint8, device="cuda")
+        ctx.fit_batched(zb, K, ds, 1e-3, form, coef, st)
+        torch.cuda.synchronize()
+        ctx.check_device_status()
+        res.append((coef.cpu().numpy().reshape(-1, 33)[:6 * S], st.cpu().numpy()[:6 * S]))
+    (cd, sd), (cc, sc) = res
+    np.testing.assert_array_equal(sc, sd)
+    ok = sd == 0
+    assert ok.any()
+    scale = np.abs(cd[ok]).max(axis=1, keepdims=True)
+    assert np.all(np.abs(cc[ok] - cd[ok]) <= 1e-9 * scale + 1e-11)
+    assert not np.array_equal(cc[ok], cd[ok])                # two computations
+    np.testing.assert_array_equal(np.isnan(cc[~ok, 0]), np.isnan(cd[~ok, 0]))
+
+
+def test_closed_form_on_the_tensor_core_gram_against_the_direct_solvers(rs, ctx):
+    batch = synth.make_batch(4, versions=64, feat=256, dtype=np.float64, seed=82, mixing_kappa=1e4)
+    splits = synth.make_splits(batch, "lovo")
+    db = rs.DeviceBatch.from_host(batch)
+    d = rs.cv_run(ctx, db, rs.DeviceSplits.from_host(_one_more(splits), batch=batch), precision=rs.RS_GRAM_BF16X3)
+    for flags in (0, rs.RS_LOO_CLOSED):
+        c = rs.cv_run(ctx, db, rs.DeviceSplits.from_host(splits, batch=batch), precision=rs.RS_GRAM_BF16X3, flags=flags)
+        R = len(c["rec_code"])
+        pd = np.asarray(d["pred_all"]).reshape(-1, 6)[:R]
+        close(np.asarray(c["pred_all"]).reshape(-1, 6), pd)
+        compare_rankings(c["rec_code"], d["rec_code"][:R], pd, math.log(1.05))

@@ -74,6 +74,15 @@ def test_leave_one_out_at_a_wide_feature_width(rs, ctx):
     _check(rs, ctx, batch, splits)
 
 
+def test_leave_one_out_by_the_direct_solvers_at_a_wide_feature_width(rs, ctx):
+    # one split more than versions: the closed form is not looked for
+    batch = synth.make_batch(3, versions=64, feat=512, dtype=np.float64, seed=67)
+    sp = synth.make_splits(batch, "lovo")
+    offs = sp.split_offsets.copy()
+    offs[-1] += 1
+    _check(rs, ctx, batch, synth.Splits(split_offsets=offs, train_masks=np.concatenate([sp.train_masks, sp.train_masks[-1:]])))
+
+
 def test_wide_fit_coefficients_give_the_reference_primal_solution(rs, ctx):
     # dual alpha, b from the GPU; beta = sum_a alpha_a z_{v_a} must equal the reference's
     # primal ridge coefficients of the same fit (push-through identity)
