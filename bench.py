@@ -8,7 +8,8 @@ train/test splits per program (262,144 splits, about 1.57 M ridge fits), lambda 
 top-3, threshold 1.05.  A step = one whole pass: standardize, Gram, test-row planning and
 the fused fit / predict / rank / score kernel, all in the sm_103a library.
 
-Prints ONE JSON line (rank 0).  --impl reference times the FP64 CPU reference on the
+Prints ONE JSON line (rank 0); the stages and the other forms go to standard error, as a second one.
+--impl reference times the FP64 CPU reference on the
 host cores instead (bounded samples of the same workload).
 """
 import argparse
@@ -687,7 +688,8 @@ def main():
         "gpu_launches": LAUNCHES_PER_STEP * args.steps,
     }
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        print(json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(short_line(line)), flush=True)
     if world > 1:
         dist.destroy_process_group()
     ctx.close()
@@ -805,6 +807,21 @@ def run_ibk(rs, ctx, batch, splits, dev, stream, flush, args):
     out["lovo"] = {"workload": "256 programs x 64 versions (all masks) x 256 f32 features, leave-one-"
                                "version-out (16,384 splits, 98,304 fits of 31 pairs)", **measure(b, sp, 20, loo=True)}
     return out
+
+
+def short_line(line):
+    """The line for standard output: the headline and what explains it, short enough (under 2,000
+    characters) to be read whole from the end of a log.  The whole of `line` goes to standard error."""
+    def some(d, *keys):
+        return {k: d[k] for k in keys if k in d} if d else None
+    keys = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+            "vs_baseline", "dtype", "data", "config", "gpu_launches")
+    return {**{k: line[k] for k in keys},
+            "e2e": some(line["e2e"], "value", "unit", "ms_per_step", "steps", "h2d_bytes_per_step", "d2h_bytes_per_step"),
+            "clocks": some(line["clocks"], "sm_mhz", "sm_max_mhz", "reasons", "samples"),
+            "roofline": some(line["roofline"], "bound", "kernel", "achieved", "peak", "unit", "frac"),
+            "accuracy": line["accuracy"], "cpu_baseline": some(line["cpu_baseline"], "value", "unit", "cores"),
+            "plain_form": some(line["plain_form"], "value", "unit"), "details": "JSON line on standard error"}
 
 
 def with_one_more_split(splits):

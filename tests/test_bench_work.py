@@ -108,3 +108,27 @@ def test_algorithmic_work_matches_brute_force_and_the_oracle():
     Z = np.empty(batch.X.shape[0], dtype=np.float64)
     assert w["std_bytes"] == batch.X.nbytes + Z.nbytes
     assert w["mask_bytes"] == splits.train_masks.nbytes
+
+
+def test_the_short_line_is_short_and_whole():
+    # the contract's keys, in under 2,000 characters whatever the details hold
+    import json
+    long = {"note": "x" * 5000}
+    line = {"metric": bench.METRIC, "value": 9115799556.140308, "unit": bench.UNIT, "n_gpus": 1, "steps": 200, "warmup": 3,
+            "ms_per_step": 0.5895206412672996, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
+            "dtype": "f64", "data": "synthetic",
+            "config": {"workload": bench.WORKLOAD, "programs": 64, "l2": "flushed", "parallelism": "1 GPU"},
+            "e2e": {"value": 7.3e9, "unit": bench.UNIT, "h2d_bytes_per_step": 1, "d2h_bytes_per_step": 2, "path": "x" * 3000},
+            "clocks": {"sm_mhz": 2070.0, "sm_max_mhz": 2070.0, "reasons": [], "samples": 900, **long},
+            "roofline": {"bound": "alu", "kernel": "k", "achieved": 0.5, "peak": 1.25, "unit": "TFLOP/s", "frac": 0.4, "stages": long},
+            "accuracy": {"sign_accuracy": 0.9}, "cpu_baseline": {"value": 3e4, "unit": bench.UNIT, "sample": "x" * 3000},
+            "plain_form": None, "surrogate_form": long, "precision_form": long, "gpu_launches": 2600}
+    out = json.dumps(bench.short_line(line))
+    assert len(out) < 2000
+    back = json.loads(out)
+    for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better", "scaling",
+              "vs_baseline", "dtype", "data", "config", "e2e", "clocks", "gpu_launches"):
+        assert k in back
+    assert back["e2e"]["h2d_bytes_per_step"] == 1 and back["clocks"]["reasons"] == []
+    # the forms that a run leaves out are None
+    assert json.loads(json.dumps(bench.short_line({**line, "e2e": None, "cpu_baseline": None})))["e2e"] is None
