@@ -468,12 +468,13 @@ __global__ void __launch_bounds__(kSplThreads + 32, 1) gram_split_kernel(const S
 // The dot products of a transfer (k_gram.cu: transfer_tile_kernel) by the same splitting: 64 x 64 blocks of
 // the group's Gram (lower triangle of blocks) and of the test rows against the group's.  The group's
 // z-scores are below sqrt(64 runs - 1), the test rows' unbounded, so the digits start at 2^4 (|z| <
-// 15.9; a block with an element outside takes plain FP64 multiply-adds in feature order), X = round(2^51
-// z).  A CTA takes a block at a time; a stage holds 64 features of its rows' digits and one those of its
+// 15.9), X = round(2^51 z).  An element outside enters the digits as 0; its products are added in FP64, the
+// features that have one in order (tr_far).  A CTA takes a block at a time; a stage holds 64 features of its rows' digits and one those of its
 // columns (a diagonal block's are the same), so splitting waits for the products before it; loads
 // and, across blocks, nothing else overlap them.  Per block: the sums 20,000 cycles, per 64 features 4,400
 // for splitting and 2,600 for products.
-// 90 problems of 192 + 64 rows x 96 features: 108 us (FP64 tiles: 527).
+// 90 problems of 192 + 64 rows x 96 features: 108 us (FP64 tiles: 527).  The whole call 439 us, with a
+// counter of every test version outside 483, with all of them 816 (the block anew in plain FP64 for either: 1069).
 struct TrSplArgs {
     const int64_t* group_off;
     int max_runs;
@@ -564,12 +565,72 @@ __device__ __forceinline__ void tr_load(const double* const (&rowp)[4], int firs
     }
 }
 
+constexpr int kFarWords = 4096 / 8 / 32;       // a bit for eight features (max_feat is at most 4096)
+template <int W>
+__device__ __forceinline__ bool far_out(double z) {
+    return ((unsigned)__double2hiint(z) & 0x7fffffffu) >= kSplHi + ((unsigned)W << 20);
+}
+
+// This thread's elements outside the digits' range: their features marked, themselves 0.
+template <int W>
+__device__ __forceinline__ void tr_mark(double (&v)[16], int kb, unsigned* far, int& outside) {
+    const int ch = kb * 8 + (threadIdx.x & 7);
+#pragma unroll
+    for (int e = 0; e < 16; ++e)
+        if (far_out<W>(v[e])) v[e] = 0.0;
+    atomicOr(&far[ch >> 5], 1u << (ch & 31));
+    outside = 1;
+}
+
+// The products that the digits left out: entry (i, u) of the block takes z_if z_uf for the features f of which
+// one or the other is outside, in order.  By the eight warps, 4 x 4 entries a thread; buf: 2 x 64 x 9 doubles.
+constexpr int kFarLd = 9;
+static_assert(2 * 64 * kFarLd * sizeof(double) <= 2 * kXchBytes, "the rows of eight features fit the exchange buffers");
+template <int W>
+__device__ __noinline__ void tr_far(const double* const (*rows)[64], const unsigned* far, int F, int nrows, int ncols,
+                                    double* out, int ld, double* buf) {
+    const int tid = threadIdx.x, ti = tid >> 4, tu = tid & 15;
+    double acc[4][4] = {};
+    for (int ch = 0; ch * 8 < F; ++ch) {
+        if (!(far[ch >> 5] >> (ch & 31) & 1u)) continue;           // (uniform)
+        split_sync();
+        for (int e = tid; e < 2 * 64 * 8; e += kSplThreads) {
+            const int side = e >> 9, r = (e >> 3) & 63, f = ch * 8 + (e & 7);
+            const double* z = rows[side][r];
+            buf[(side * 64 + r) * kFarLd + (e & 7)] = z && f < F ? __ldg(z + f) : 0.0;
+        }
+        split_sync();
+        for (int c = 0; c < 8; ++c) {
+            double x[4], y[4];
+            bool xo[4], yo[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                x[q] = buf[(ti + 16 * q) * kFarLd + c];
+                y[q] = buf[(64 + tu + 16 * q) * kFarLd + c];
+                xo[q] = far_out<W>(x[q]);
+                yo[q] = far_out<W>(y[q]);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (xo[i] || yo[u]) acc[i][u] = fma(x[i], y[u], acc[i][u]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (ti + 16 * i < nrows && tu + 16 * u < ncols) out[(int64_t)(ti + 16 * i) * ld + tu + 16 * u] += acc[i][u];
+}
+
 __global__ void __launch_bounds__(kSplThreads + 32, 1) transfer_split_kernel(const TrSplArgs a) {
     constexpr int W = 1;
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint32_t tmem_slot;
     __shared__ int outside;                                // an element outside the range
-    __shared__ const double* plain_rows[2][64];
+    __shared__ unsigned far[kFarWords];                    // ... in these eight features
+    __shared__ const double* far_rows[2][64];
     __shared__ volatile int gave_up;
     const uint32_t raw = tc::smem_u32(smem_raw), base = (raw + 1023u) & ~1023u;
     uint8_t* g = smem_raw + (base - raw);
@@ -583,6 +644,7 @@ __global__ void __launch_bounds__(kSplThreads + 32, 1) transfer_split_kernel(con
         tc::mbar_init(drained, 8);
         tc::fence_barrier_init();
         outside = 0;
+        for (int i = 0; i < kFarWords; ++i) far[i] = 0u;
         gave_up = 0;
     }
     for (int i = tid; i < (int)(2 * kSliceBytes / 16); i += kSplThreads + 32)      // the zero slices
@@ -635,16 +697,20 @@ __global__ void __launch_bounds__(kSplThreads + 32, 1) transfer_split_kernel(con
     } else {                                               // ---- digits, and the sums
         for (int64_t t = blockIdx.x; t < total; t += gridDim.x) {
             if (!tr_block(a, t, b)) continue;
-            bool ok = true;
             for (int kb = 0; kb < b.nk; ++kb, ++it) {
                 double v[16];
+                auto store = [&](unsigned char* stage) {
+                    if (spl_store<W>(v, stage)) return;
+                    tr_mark<W>(v, kb, far, outside);
+                    spl_store<W>(v, stage);
+                };
                 tr_load(b.rowp, 0, kb * kSplBlock, b.F, v);
                 // the products that read the stages have completed
                 if (it >= 1) wait(done, it - 1, -39);
-                ok = spl_store<W>(v, g) && ok;
+                store(g);
                 if (!b.same) {
                     tr_load(b.rowp, 2, kb * kSplBlock, b.F, v);
-                    ok = spl_store<W>(v, g + kStageBytes) && ok;
+                    store(g + kStageBytes);
                 }
                 fence_async_smem();
                 __syncwarp();
@@ -659,23 +725,16 @@ __global__ void __launch_bounds__(kSplThreads + 32, 1) transfer_split_kernel(con
                     if (lane == 0) tc::mbar_arrive(drained);
                 }
             }
-            if (!ok) outside = 1;
             if ((tid & 7) == 0)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) plain_rows[i >> 1][(tid >> 3) + 32 * (i & 1)] = b.rowp[i];
+                for (int i = 0; i < 4; ++i) far_rows[i >> 1][(tid >> 3) + 32 * (i & 1)] = b.rowp[i];
             split_sync();
-            if (outside) {                                 // plain FP64, uniform
-                for (int e = tid; e < b.rows * 64; e += kSplThreads) {
-                    const int i = e >> 6, u = e & 63;
-                    if (u >= b.cols) continue;
-                    const double *zi = plain_rows[0][i], *zu = plain_rows[1][u];
-                    double acc = 0.0;
-                    for (int f = 0; f < b.F; ++f) acc = fma(__ldg(zi + f), __ldg(zu + f), acc);
-                    b.out[(int64_t)i * a.ld + u] = acc;
-                }
+            if (outside) {                                 // (uniform)
+                tr_far<W>(far_rows, far, b.F, b.rows, b.cols, b.out, a.ld, reinterpret_cast<double*>(xch));
+                split_sync();
+                if (tid < kFarWords) far[tid] = 0u;
+                if (tid == 0) outside = 0;
             }
-            split_sync();
-            if (tid == 0) outside = 0;
             split_sync();
         }
     }

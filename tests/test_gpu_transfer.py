@@ -255,3 +255,26 @@ def test_ridge_blocks_at_the_edges_of_their_tiles(rs, ctx, feat, runs_per, versi
         close(np.asarray(g["pred_all"]).reshape(-1, 6)[keep], np.asarray(r.pred_all).reshape(-1, 6)[keep], abs_=g["abs_tol"])
         return
     _check(g, r, "ridge", abs_tol=g["abs_tol"])
+
+
+@pytest.mark.parametrize("feat", [40, 100, 300])
+@pytest.mark.parametrize("case", ["one", "some", "all", "few_rows"])
+def test_ridge_with_counters_outside_the_training_range(rs, ctx, feat, case):
+    """Test versions whose counters lie far outside their training group's (z-scores beyond 15.9 enter the
+    digit products as 0 and are added in FP64): one counter of every version, some, all, and single
+    elements of a few versions; inside and outside values meet in one feature."""
+    Q, runs_per = 5, 2
+    b = synth.make_batch(Q * runs_per + Q, versions=(33, 64), feat=feat, dtype=np.float64, seed=950 + feat)
+    rng = np.random.default_rng(feat)
+    train = synth.take_programs(b, list(range(Q * runs_per)))
+    test = synth.take_programs(b, list(range(Q * runs_per, Q * runs_per + Q)))
+    for p in range(Q - 1):                       # (the last problem stays inside)
+        X = test.program_X(p)
+        if case == "few_rows":
+            for v in (0, 7, X.shape[0] - 1):
+                X[v, rng.integers(0, feat, size=3)] *= np.exp(rng.choice([-25.0, 30.0], size=3))
+        else:
+            cols = {"one": [feat - 1], "some": rng.choice(feat, feat // 3, replace=False), "all": np.arange(feat)}[case]
+            X[:, cols] *= np.exp(rng.uniform(10.0, 30.0, size=len(cols)))
+    g, r = _both(rs, ctx, train, test, np.arange(Q + 1, dtype=np.int64) * runs_per, "ridge", flags=oracle.RANK_ALL)
+    _check(g, r, "ridge", abs_tol=g["abs_tol"])
