@@ -81,15 +81,20 @@ __device__ __forceinline__ long long cycle_log(double c, const long long* tl, co
 __device__ __forceinline__ long long elem_log(double x, bool cyc, double c, long long lc, const long long* tl,
                                               const uint16_t* tc) {
     const unsigned hi = (unsigned)__double2hiint(x);
-    if (!fast_hi(hi) || (cyc && lc == kFixNone)) return fix_log_clamped(cyc ? x * (1.0 / c) : x, tl, tc);
+    if (!fast_hi(hi) || (cyc && lc == kFixNone)) {
+        if ((hi << 1 | (unsigned)__double2loint(x)) == 0u) return kFixClamp;      // 0 (by any c: no more, or NaN)
+        return fix_log_clamped(cyc ? x * (1.0 / c) : x, tl, tc);
+    }
     const long long l = fix_log(hi, (unsigned)__double2loint(x), tl, tc) - (cyc ? lc : 0ll);
     return l > kFixClamp ? l : kFixClamp;
 }
 __device__ __forceinline__ long long elem_log(float x, bool cyc, double c, long long lc, const long long* tl,
                                               const uint16_t* tc) {
     const unsigned u = __float_as_uint(x);
-    if (u - (1u << 23) >= (254u << 23) || (cyc && lc == kFixNone))     // not a positive normal number
+    if (u - (1u << 23) >= (254u << 23) || (cyc && lc == kFixNone)) {   // not a positive normal number
+        if (u << 1 == 0u) return kFixClamp;
         return fix_log_clamped(cyc ? (double)x * (1.0 / c) : (double)x, tl, tc);
+    }
     const long long l = fix_log((u >> 3) + (896u << 20), u << 29, tl, tc) - (cyc ? lc : 0ll);
     return l > kFixClamp ? l : kFixClamp;
 }
