@@ -2430,7 +2430,7 @@ cudaError_t launch_rank(const rs_fit_args& a, const int64_t* coef_off, const uin
 struct FitWs {
     unsigned* hist;      // [kHist] fits per n
     unsigned* cursor;    // [kHist]
-    unsigned long long* work;   // [4] work counters of the solve kernels
+    unsigned long long* work;   // [5] work counters of the solve kernels, [1] fits that the closed form left
     uint8_t* pb;         // [P][6][32]
     uint8_t* pa;         // [P][6][32]
     double* ylab;        // [P][6][32]
@@ -2451,7 +2451,7 @@ struct FitWs {
     double* predbuf;     // [6][Rcap]
     unsigned long long* tile_sum;   // [ceil(Rcap / 256)] recommendations per rank tile (packed output)
     unsigned long long* tile_off;   // [ceil(Rcap / 256)] their exclusive scan
-    double* loo_tab;     // [P][6][kLooTab] M^-1, w_y, w_1, sums (RS_LOO_CLOSED; aliases coef)
+    double* loo_tab;     // [P][6][kLooTab] M^-1, w_y, w_1, sums (the closed form, asked for or found; aliases coef)
     uint8_t* loo_ok;     // [P][6] 1 when that inverse exists
     uint32_t* loo_bad;   // [P][6] pairs whose label is not finite
     size_t bytes;
@@ -2492,8 +2492,8 @@ FitWs carve(void* base, int64_t P, int64_t S, int nmax, int64_t Rcap) {
     w.recs = (uint4*)take(S6 * sizeof(uint4));
     w.fit_off = (int64_t*)take(S6 * sizeof(int64_t));
     w.status = (uint8_t*)take(S6);
-    // compact records, or with RS_LOO_CLOSED (which keeps fits only in a caller's array) the
-    // tables of the inverses: one region serves both
+    // compact records, or with fits in closed form (RS_LOO_CLOSED, or found by a call that keeps no
+    // compact records) the tables of the inverses: one region serves both
     const size_t coef_bytes = S6 * (size_t)(nmax + 1) * sizeof(double);
     const size_t loo_bytes = (size_t)P * RS_NOPT * kLooTab * sizeof(double);
     w.coef = (double*)take(coef_bytes > loo_bytes ? coef_bytes : loo_bytes);

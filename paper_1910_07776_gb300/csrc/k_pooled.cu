@@ -37,7 +37,6 @@ struct PoolArgs {
     double* ybar;                // [6]
     double* G;                   // [6][F][F]
     double* r;                   // [6][F]
-    double* rho;                 // [6][F]
     double* s;                   // [6][NP]: c_a . beta during refinement
     double* coef;                // [6][F + 1]: b, beta
     uint8_t* status;             // [6]
@@ -642,7 +641,7 @@ struct PoolWs {
     int* counts;
     int64_t* offs;
     int64_t* zoff;
-    double *y, *zbar, *ybar, *G, *r, *rho, *s;
+    double *y, *zbar, *ybar, *G, *r, *s;
     __nv_bfloat16 *A, *B;
     size_t bytes;
 };
@@ -666,7 +665,6 @@ PoolWs carve_pool(void* base, int64_t P, int F) {
     w.ybar = (double*)take(RS_NOPT * sizeof(double));
     w.G = (double*)take((size_t)RS_NOPT * F * F * sizeof(double));
     w.r = (double*)take((size_t)RS_NOPT * F * sizeof(double));
-    w.rho = (double*)take((size_t)RS_NOPT * F * sizeof(double));
     const size_t ab = (size_t)RS_NOPT * F * 3 * Np * sizeof(__nv_bfloat16);
     const size_t sb = (size_t)RS_NOPT * pool_scratch_doubles(F) * sizeof(double);   // larger for F < 9 only
     w.A = (__nv_bfloat16*)take(ab > sb ? ab : sb);
@@ -704,7 +702,6 @@ cudaError_t rs_launch_fit_pooled(const rs_batch* b, const uint8_t* use, double l
     a.ybar = w.ybar;
     a.G = w.G;
     a.r = w.r;
-    a.rho = w.rho;
     a.s = w.s;
     a.coef = coef;
     a.status = status;

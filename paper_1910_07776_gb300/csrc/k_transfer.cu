@@ -308,7 +308,6 @@ struct M5Vec {
     uint8_t sel[N];
     double e_cur, b;
     unsigned long long reach;                     // attributes whose drop may be the best
-    int drop;
 };
 
 struct M5Smem {
@@ -321,7 +320,7 @@ struct M5Smem {
     uint8_t lo[kM5MaxNodes], hi[kM5MaxNodes];
     uint8_t ids[kM5MaxN], side[kM5MaxN];
     int level[kM5MaxN + 2];                       // first node of each level
-    int nn, task, nsurv;
+    int nn, nsurv;
     double sd_root;
     // the level's nodes (at most kM5MaxN / 2 that split), by node - first of the level
     float mean[kM5MaxN], tot[kM5MaxN], tot2[kM5MaxN], amax2[kM5MaxN], sda[kM5MaxN], ymax[kM5MaxN];
@@ -684,10 +683,7 @@ __device__ __noinline__ void m5_model(M5Smem& S, Vec& V, M5Tree* T, int t, int F
                 for (int o = 16; o > 0; o >>= 1) best = fminf(best, __shfl_xor_sync(0xffffffffu, best, o));
                 const unsigned b0 = __ballot_sync(0xffffffffu, on[0] && !(lo32[0] > best));
                 const unsigned b1 = __ballot_sync(0xffffffffu, on[1] && !(lo32[1] > best));
-                if (tid == 0) {
-                    V.reach = (unsigned long long)b1 << 32 | b0;
-                    V.drop = -1;
-                }
+                if (tid == 0) V.reach = (unsigned long long)b1 << 32 | b0;
             }
             Gp::sync();
             // the drops that may be the best, in FP64 from C (nearly always one): the lowest error
@@ -922,10 +918,7 @@ m5p_fit_kernel(const TransferArgs a, int fmax) {
     int depth = 0;
     for (;; ++depth) {
         const int n0 = S.level[depth], nl = S.level[depth + 1] - n0;
-        if (tid == 0) {
-            S.task = 0;
-            S.nsurv = 0;
-        }
+        if (tid == 0) S.nsurv = 0;
         // per node: FP32 statistics, and leaves by size or deviation (near the line, or with labels
         // that FP32 does not hold: by the exact deviation)
         for (int k = warp; k < nl; k += kM5Warps) {

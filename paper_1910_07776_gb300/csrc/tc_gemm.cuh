@@ -1,12 +1,13 @@
 // tc_gemm.cuh -- BF16 GEMM on the sm_103a tensor cores (tcgen05), used by the surrogate's
 // forward / backward kernels, the tensor-core Gram and rs_gemm_bf16.
 //
-//   D[M][N] (FP32, in tensor memory) = A[M][K] * B[N][K]^T,  A, B BF16, both K-contiguous.
+//   D[M][N] (FP32, in tensor memory) = A[M][K] * B[N][K]^T,  A, B BF16, each contiguous along K or
+//   along its rows (M, N).
 //
 // Persistent CTAs (one per SM) walk the 128 x BN output tiles; inside a CTA a TMA producer
-// warp, a single-thread MMA issuer and eight epilogue warps run concurrently, connected by
+// warp, a single-thread MMA issuer and 16 epilogue warps (8 for BN = 32) run concurrently, connected by
 // mbarriers (stage full / empty, accumulator full / empty), with two tensor-memory
-// accumulators so that a tile's epilogue overlaps the next tile's MMAs (see gemm_kernel).
+// accumulators so that a tile's epilogue overlaps the next tile's MMAs (see gemm_core).
 // Every mbarrier wait is bounded (1 s of %globaltimer); a wait that gives up sets
 // RS_ETIMEOUT in the device status word and the CTA winds down without hanging.
 #pragma once
