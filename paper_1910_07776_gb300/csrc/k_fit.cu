@@ -1611,6 +1611,15 @@ loo_inv_kernel(const int64_t* __restrict__ row_off, const int32_t* __restrict__ 
     if (tid < n) vs[tid] = pb[(int64_t)pj * RS_MAXPAIRS + tid];
     if (tid == 0) umax = 0;
     __syncthreads();
+    // With a limit: the largest 1 / d that a pivot may have.  1 / d_k is an entry of the inverse of the leading
+    // block, and so at most (M^-1)_kk: a pivot beyond ends it (nearly collinear counters, within a few pivots).
+    int dmax = 0, rmax = 0x7fe00000;
+    if (limit > 0.f) {
+        const double dii = lane < n ? dlam[(int64_t)p * RS_MAXV + vs[lane]] : 0.0;
+        dmax = __reduce_max_sync(0xffffffffu, pos_finite(dii) ? __double2hiint(dii) : 0);
+        const double most = (double)limit * rcp_newton(__hiloint2double(dmax, 0));
+        if (pos_finite(most)) rmax = __double2hiint(most) + 1;  // (rounded up)
+    }
     double A[kLooPer];
     int ri[kLooPer], ci[kLooPer];                               // row 0..33, column 0..31; -1: none
 #pragma unroll
@@ -1660,7 +1669,7 @@ loo_inv_kernel(const int64_t* __restrict__ row_off, const int32_t* __restrict__ 
     for (int k = 0; k < n; ++k) {
         const double* c = col[k & 1];
         const double r = rk;                                    // the same value in every thread
-        good = pos_finite(r);
+        good = pos_finite(r) && __double2hiint(r) <= rmax;
         if (!good) break;
         if (warp == 1) {
             if (lane < n) w[lane] = lane == k ? -r : c[lane] * r;
@@ -1693,9 +1702,6 @@ loo_inv_kernel(const int64_t* __restrict__ row_off, const int32_t* __restrict__ 
         atomicMax(&umax, um_bad ? 0x7ff00000 : um);
         __syncthreads();
         if (limit > 0.f) {
-            double dii = 0.0;
-            if (lane < n) dii = dlam[(int64_t)p * RS_MAXV + vs[lane]];
-            const int dmax = __reduce_max_sync(0xffffffffu, pos_finite(dii) ? __double2hiint(dii) : 0);
             good = umax < 0x7fe00000 &&
                    (double)limit >= __hiloint2double(dmax + 1, 0) * __hiloint2double(umax + 1, 0);
         }

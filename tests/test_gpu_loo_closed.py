@@ -392,3 +392,27 @@ def test_closed_form_on_the_tensor_core_gram_against_the_direct_solvers(rs, ctx)
         pd = np.asarray(d["pred_all"]).reshape(-1, 6)[:R]
         close(np.asarray(c["pred_all"]).reshape(-1, 6), pd)
         compare_rankings(c["rec_code"], d["rec_code"][:R], pd, math.log(1.05))
+
+
+@pytest.mark.parametrize("copies", [1, 3])
+def test_nearly_collinear_counters_take_the_direct_solvers(rs, ctx, copies):
+    """Counters of few independent directions plus little noise, as measured profiles have: a call without
+    the flag finds its systems beyond the condition limit, after a few pivots, beside programs whose systems
+    are not; against the plain form.  Tolerance: the parity bound with the absolute term of the worst
+    system, kappa <= 32 F / lambda (a program's K has a trace of 64 F), times u."""
+    feat, lam = 80, 1e-3
+    batch = synth.make_batch(3 * copies, versions=64, feat=feat, dtype=np.float64, seed=96)
+    rng = np.random.default_rng(96)
+    X = batch.X.copy()
+    for p in range(0, 3 * copies, 3):                        # six directions, noise of 1e-3
+        x0 = int(batch.x_offsets[p])
+        low = rng.standard_normal((64, 6)) @ rng.standard_normal((6, feat)) + 1e-3 * rng.standard_normal((64, feat))
+        X[x0:x0 + 64 * feat] = (np.exp(low) * batch.cycles[batch.program_rows(p)][:, None]).reshape(-1)
+    batch.X = X
+    db, ds = rs.DeviceBatch.from_host(batch), rs.DeviceSplits.from_host(synth.make_splits(batch, "lovo"), batch=batch)
+    g = rs.cv_run(ctx, db, ds, lam=lam)
+    r = rs.cv_run(ctx, db, ds, lam=lam, form=rs.RS_FORM_PLAIN)
+    tol = max(4e6, 64 * feat / lam) * 2.0 ** -53
+    close(g["pred_all"], r["pred_all"], abs_=tol)
+    _, nnear = compare_rankings(g["rec_code"], r["rec_code"], r["pred_all"], math.log(1.05), tol=max(1e-8, 4 * tol))
+    compare_counters(g["counters"], r["counters"], slack=nnear)
