@@ -2680,7 +2680,10 @@ cudaError_t rs_launch_fit_predict(const rs_fit_args& a, cudaStream_t st) {
             e = cudaEventRecord(a.fork, st);
             if (e == cudaSuccess) e = cudaStreamWaitEvent(a.side, a.fork, 0);
         }
-        if (e == cudaSuccess && mid) e = launch_mid(sa, sms, nmax < kNMid ? nmax : kNMid, w.work + 2, s2, !fork);
+        // On one stream the wide solver comes before solve_mid: begun while that one's blocks, which fill the
+        // SMs' shared memory, leave, its own crowd onto the first SMs to be free (a program of 64
+        // versions whose systems are beyond the limit, 384 wide fits: 158 us a call, this way 118).
+        if (e == cudaSuccess && mid && fork) e = launch_mid(sa, sms, nmax < kNMid ? nmax : kNMid, w.work + 2, s2, false);
         if (e == cudaSuccess && nmax > kNMid) {
             // kWideGroups fits per warp, persistent blocks taking their fits dynamically
             e = cudaFuncSetAttribute(solve_wide_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kWideSmem);
@@ -2695,6 +2698,7 @@ cudaError_t rs_launch_fit_predict(const rs_fit_args& a, cudaStream_t st) {
                 e = tc::launch_when(!fork, solve_wide_kernel, (unsigned)grid, kWideWarps * 32, kWideSmem, s2, sa, w.work + 4);
             }
         }
+        if (e == cudaSuccess && mid && !fork) e = launch_mid(sa, sms, nmax < kNMid ? nmax : kNMid, w.work + 2, s2, true);
         if (e == cudaSuccess && fork) e = cudaEventRecord(a.join, a.side);
         if (e != cudaSuccess) return e;
         unsigned long long* w0 = w.work;
