@@ -265,12 +265,13 @@ transfer_fit_kernel(const TransferArgs a, int nmax) {
 // Greedy elimination keeps the inverse H of the normal equations, the residuals and T = C H (C the
 // centred attributes): dropping attribute d changes every residual by (w_d / H_dd) T_ad, so all the
 // drop-one errors of a round cost m ns operations, and the round's winner is taken out by rank-one
-// updates of H, w and T; the model that stays is solved again from scratch.  Where taking d out would
-// shrink a diagonal entry of H by more than 2^kM5Shrink since H was last formed (d and another attribute
-// nearly agree: what the subtraction leaves of their large entries is rounding), the attributes that stay
-// are solved from their own normal equations at once, and the elimination goes on from there: with pairs
-// of attributes 1e-5 of a deviation apart the updates alone chose wrong drops in 25 of 60 models, this
-// form, as an inverse a round, in none.  (Before: one thread per
+// updates of H, w and T; the model that stays is solved again from scratch.  Not where attributes nearly
+// make up one another (an entry G_kk H_kk, the variance inflation, beyond 2^kM5Inflated), nor where taking d
+// out shrinks a diagonal entry of H by more than 2^kM5Shrink since H was last formed: what such updates
+// leave of large entries is rounding, so the attributes that stay are solved from their own normal
+// equations at once, and the elimination goes on from there.  With pairs of attributes 1e-5 of a deviation
+// apart the updates alone chose wrong drops in 25 of 60 models, this form, as an inverse a round, in none.
+// (Before: one thread per
 // attribute walking every candidate's SDR, an inverse per round and every drop-one model applied to
 // every instance, all serial over the nodes.)  Small nodes' models take one warp each.
 // 36 problems x 3 runs x 37 attributes (96 instances a fit): 5532 -> 1351 us.
@@ -287,6 +288,7 @@ constexpr int kM5WarpBuf = kM5WarpTerms * kM5WarpLd + kM5WarpN * kM5WarpLd +
 constexpr int kM5Surv = 1024;                     // candidate splits listed for exact evaluation, per level
 constexpr double kM5SdFrac = 0.05, kM5Smooth = 15.0, kM5Ridge = 1e-8;
 constexpr int kM5Shrink = 6;                      // bits that rank-one updates may take off an entry H_kk
+constexpr int kM5Inflated = 16;                   // G_kk H_kk beyond 2^this: no rank-one updates
 
 struct M5Tree {
     int n_nodes;
@@ -302,7 +304,7 @@ struct M5Tree {
 template <int N>
 struct M5Vec {
     double colk[N], rowk[N], zbar[N], r[N], w[N], wt[N], fac[N];
-    int h0[N];                                    // H_kk when H was last formed (high word)
+    int g0[N], h0[N];                             // G_kk and H_kk when H was last formed (high words)
     float fac32[N], rowk32[N], t32[N], e32[N];    // bounds of |T_ak|, and of the error of T in FP32
     int16_t cand[N];
     uint8_t sel[N];
@@ -520,7 +522,10 @@ __device__ void m5_solve(M5Smem& S, Vec& V, const double* C, double* H, int ld, 
         const int g = e - f * (f + 1) / 2, cf = V.sel[f], cg = V.sel[g];
         double s = 0.0;
         for (int a = 0; a < m; ++a) s = fma(C[a * ld + cf], C[a * ld + cg], s);
-        if (f == g) s += kM5Ridge;
+        if (f == g) {
+            s += kM5Ridge;
+            V.g0[f] = __double2hiint(s);
+        }
         H[f * ld + g] = s;
         H[g * ld + f] = s;
     }
@@ -600,6 +605,7 @@ __device__ __noinline__ void m5_model(M5Smem& S, Vec& V, M5Tree* T, int t, int F
         float* res32 = S.res32 + (WARP ? 32 * (int)(threadIdx.x >> 5) : 0);
         double res = 0.0;
         bool formed = true;                        // H, w are those of the nc attributes' normal equations
+        bool ill = false;                          // an attribute that the others nearly make up
         for (;;) {
             if (formed) {
                 // residuals (lane = instance, kept by the warp that owns its 32 instances) and T = C H in FP32
@@ -617,12 +623,14 @@ __device__ __noinline__ void m5_model(M5Smem& S, Vec& V, M5Tree* T, int t, int F
                     T32[a * ld + k] = (float)s;
                 }
                 // column k of T has the norm sqrt(H_kk) at most, and no update makes it longer
+                ill = false;
                 for (int k = tid; k < nc; k += Gp::kNT) {
                     V.h0[k] = __double2hiint(H[k * ld + k]);
+                    ill = ill || (V.g0[k] >> 20) + (V.h0[k] >> 20) > 2 * 1023 + kM5Inflated;
                     V.t32[k] = 1.01f * sqrtf(fabsf((float)H[k * ld + k]));
                     V.e32[k] = 6e-8f * V.t32[k];
                 }
-                Gp::sync();
+                ill = Gp::any(ill);
             }
             // w_d / H_dd, then sum_a |res_a + fac_d T_ad| of every attribute still there, in FP32: off by
             // less than 1e-4 of the sizes of its terms, and by what T has lost in the updates
@@ -742,7 +750,7 @@ __device__ __noinline__ void m5_model(M5Smem& S, Vec& V, M5Tree* T, int t, int F
             if (row < m) res32[row] = (float)res;
             Gp::sync();
             if (tid == 0) V.e_cur = est;           // (every thread has compared with it)
-            bool lost = false;                     // an entry H_ii of which too little is left
+            bool lost = ill;                       // or an entry H_ii of which too little is left
             for (int e = tid; e < nc * nc; e += Gp::kNT) {
                 const int i = e / nc, j = e - i * nc;
                 if (i == d || j == d) continue;

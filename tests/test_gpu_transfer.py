@@ -216,6 +216,64 @@ def test_m5p_pairs_of_nearly_equal_counters(rs, ctx, gap, seed):
     close(g["pred_all"], r.pred_all, rel=max(1e-7, tol), abs_=max(1e-9, tol))
 
 
+def _m5p_on_its_rows(rs, ctx, train, test, groups):
+    """rs_transfer's M5P predictions, and the reference's on the very rows that it standardized (they lie at
+    the front of the workspace: the training rows, then from the next 256-byte boundary the test rows), so
+    that only the trees are compared: {(problem, optimization): (got, reference, labels)}, all versions."""
+    a, b = rs.DeviceBatch.from_host(train), rs.DeviceBatch.from_host(test)
+    g = (torch.from_numpy(groups).cuda(), int(np.diff(groups).max()))
+    flags = rs.RS_MODEL_M5P | rs.RS_RANK_ALL
+    ws = ctx.workspace(ctx.transfer_workspace_bytes(a, b, g, flags))
+    out = rs.alloc_outputs(test.n_rows, 0, 3)
+    ctx.transfer(a, b, ws, out.rec_code, groups=g, flags=flags, pred_all=out.pred_all)
+    torch.cuda.synchronize()
+    ctx.check_device_status()
+    raw, n = ws.view(torch.uint8), 8 * train.X.size
+    ZA = raw[:n].view(torch.float64).cpu().numpy()
+    ZB = raw[(n + 255) // 256 * 256:][:8 * test.X.size].view(torch.float64).cpu().numpy()
+    pred, res = out.pred_all.cpu().numpy().reshape(-1, 6), {}
+    rows = lambda Z, bt, p: Z[int(bt.x_offsets[p]):][:bt.versions(p) * bt.feat_width[p]].reshape(bt.versions(p), -1)  # noqa: E731
+    for q in range(test.n_programs):
+        for j in range(6):
+            Zr, y = [], []
+            for p in range(int(groups[q]), int(groups[q + 1])):
+                m, lt = train.masks[train.program_rows(p)].astype(int), train.log_time[train.program_rows(p)]
+                slot = {x: v for v, x in enumerate(m)}
+                for v, x in enumerate(m):
+                    if not (x >> j) & 1 and x | 1 << j in slot:
+                        Zr.append(rows(ZA, train, p)[v])
+                        y.append(lt[v] - lt[slot[x | 1 << j]])
+            ref = oracle.m5p_fit_predict(np.array(Zr), np.array(y), rows(ZB, test, q))[0]
+            res[q, j] = pred[test.program_rows(q), j], ref, np.array(y)
+    return res
+
+
+@pytest.mark.parametrize("seed", [701, 703])
+def test_m5p_counters_that_nearly_make_up_one_another(rs, ctx, seed):
+    """Ten counters that are one of four others, or the sum of two, to 1e-6: every elimination starts from a
+    nearly singular system.  Versions predicted and tolerance as in the test of pairs (the condition at most
+    14 x 96 / 1e-8 by the ridge), and the trees are those of the same rows."""
+    feat, runs_per, Q = 14, 3, 4
+    b = synth.make_batch(Q * runs_per, versions=64, feat=feat, dtype=np.float64, seed=seed)
+    rng = np.random.default_rng(seed)
+    of, w = rng.integers(0, 4, size=(feat, 2)), rng.standard_normal(4)
+    for p in range(b.n_programs):
+        base = np.round(2 * rng.standard_normal((64, 4))) / 2
+        x = np.empty((64, feat))
+        x[:, :4] = base
+        for f in range(4, feat):
+            x[:, f] = x[:, of[f, 0]] + (x[:, of[f, 1]] if f % 2 else 0) + 1e-6 * rng.standard_normal(64)
+        b.program_X(p)[:] = np.exp(x)
+        b.log_time[b.program_rows(p)] = 0.3 * base @ w + 0.1 * rng.standard_normal(64)
+    b.cycles = np.ones_like(b.cycles)
+    test = synth.take_programs(b, [q * runs_per for q in range(Q)])
+    tol = 100 * 14 * 96 / 1e-8 * np.finfo(np.float64).eps
+    masks = test.masks.reshape(Q, 64).astype(int)
+    for (q, j), (got, ref, _) in _m5p_on_its_rows(rs, ctx, b, test, np.arange(Q + 1, dtype=np.int64) * runs_per).items():
+        trained = (masks[q] >> j) & 1 == 0
+        close(got[trained], ref[trained], rel=1e-7, abs_=tol)
+
+
 @pytest.mark.parametrize("spread", [1e-2, 1e-4, 1e-5, 1e-6])
 def test_m5p_labels_close_to_a_common_value(rs, ctx, spread):
     """Every optimization's speedup near one value: what the deviations of labels 1 +- spread are by the
