@@ -550,6 +550,49 @@ __device__ void m5_solve(M5Smem& S, Vec& V, const double* C, double* H, int ld, 
     Gp::sync();
 }
 
+// The estimated error of a node's model on attribute f (f < 0: none, the label mean) with the reference's
+// operations in its order (instances ascending: an inner node's lie by its children), one rounding each.
+// One thread.
+__device__ __noinline__ double m5_exact_err(const M5Smem& S, int f, int lo, int m) {
+    const double md = (double)m;
+    unsigned long long in[kM5MaxN / 64] = {};
+    for (int a = 0; a < m; ++a) {
+        const int i = S.ids[lo + a];
+#pragma unroll
+        for (int w = 0; w < kM5MaxN / 64; ++w)
+            if (i >> 6 == w) in[w] |= 1ull << (i & 63);
+    }
+    auto each = [&](auto&& take) {
+#pragma unroll
+        for (int w = 0; w < kM5MaxN / 64; ++w)
+            for (unsigned long long x = in[w]; x; x &= x - 1) {
+                const int i = 64 * w + __ffsll((long long)x) - 1;
+                take(S.y[i], f >= 0 ? __ldg(S.zp[i] + f) : 0.0);
+            }
+    };
+    double b = 0.0, w = 0.0;
+    each([&](double y, double) { b = __dadd_rn(b, y); });
+    b = __ddiv_rn(b, md);
+    if (f >= 0) {
+        double zbar = 0.0, g = 0.0, r = 0.0;
+        each([&](double, double z) { zbar = __dadd_rn(zbar, z); });
+        zbar = __ddiv_rn(zbar, md);
+        each([&](double y, double z) {
+            const double c = __dsub_rn(z, zbar);
+            g = __dadd_rn(g, __dmul_rn(c, c));
+            r = __dadd_rn(r, __dmul_rn(c, __dsub_rn(y, b)));
+        });
+        const double l = __dsqrt_rn(__dadd_rn(g, kM5Ridge));
+        w = __ddiv_rn(__ddiv_rn(r, l), l);
+        b = __dsub_rn(b, __dmul_rn(w, zbar));
+    }
+    const int v = f >= 0 ? 2 : 1;
+    if (m <= v) return DBL_MAX;
+    double e = 0.0;
+    each([&](double y, double z) { e = __dadd_rn(e, fabs(__dsub_rn(y, f >= 0 ? __dadd_rn(b, __dmul_rn(w, z)) : b))); });
+    return __dmul_rn(__ddiv_rn(e, md), __ddiv_rn((double)(m + v), (double)(m - v)));
+}
+
 // The model of internal node t on the attributes tested below it (the lowest kM5MaxTerms of them),
 // greedily simplified, and the pruning decision.  H: tmax x ld; C, T32: m x ld.
 template <bool WARP, class Vec>
@@ -803,10 +846,14 @@ __device__ __noinline__ void m5_model(M5Smem& S, Vec& V, M5Tree* T, int t, int F
         T->nterm[t] = ns;
         T->b[t] = V.b;
         T->count[t] = m;
-        const double e = V.e_cur;
+        double e = V.e_cur;
         const int l = S.left[t], r = S.right[t];
         const int ml = S.hi[l] - S.lo[l], mr = S.hi[r] - S.lo[r];
-        const double keep = (ml * S.est[l] + mr * S.est[r]) / m;
+        const double keep = __ddiv_rn(__dadd_rn(__dmul_rn((double)ml, S.est[l]), __dmul_rn((double)mr, S.est[r])), (double)m);
+        // A split into halves of two instances and a line through their means have the same estimated error
+        // (as have halves of any size on a two-valued attribute), so that their roundings decide: the
+        // reference's
+        if (ns <= 1 && fabs(e - keep) <= 1e-9 * keep) e = m5_exact_err(S, ns ? V.cand[V.sel[0]] : -1, lo, m);
         if (!(e <= keep)) {
             S.est[t] = keep;
         } else {                                   // a leaf: its parent's candidates get no test
@@ -1150,16 +1197,15 @@ m5p_fit_kernel(const TransferArgs a, int fmax) {
     for (int t = warp; t < nn; t += kM5Warps) {
         if (S.attr[t] >= 0) continue;
         const int lo = S.lo[t], m = S.hi[t] - lo;
-        double s = 0.0, e = 0.0;
-        for (int x = lane; x < m; x += 32) s += S.y[S.ids[lo + x]];
-        s = m5_warp_sum(s) / m;
-        for (int x = lane; x < m; x += 32) e += fabs(S.y[S.ids[lo + x]] - s);
-        e = m5_warp_sum(e);
+        double s = 0.0, e = 0.0;                   // (in instance order, by every lane: as the reference)
+        for (int x = 0; x < m; ++x) s = __dadd_rn(s, S.y[S.ids[lo + x]]);
+        s = __ddiv_rn(s, (double)m);
+        for (int x = 0; x < m; ++x) e = __dadd_rn(e, fabs(__dsub_rn(S.y[S.ids[lo + x]], s)));
         if (lane == 0) {
             T->nterm[t] = 0;
             T->b[t] = s;
             T->count[t] = m;
-            S.est[t] = m <= 1 ? DBL_MAX : e / m * ((double)(m + 1) / (double)(m - 1));
+            S.est[t] = m <= 1 ? DBL_MAX : __dmul_rn(__ddiv_rn(e, (double)m), __ddiv_rn((double)(m + 1), (double)(m - 1)));
             for (int k = 0; k < kM5MaxFeat / 64; ++k) S.tested[t][k] = 0;
         }
     }

@@ -243,8 +243,9 @@ def _m5p_on_its_rows(rs, ctx, train, test, groups):
                     if not (x >> j) & 1 and x | 1 << j in slot:
                         Zr.append(rows(ZA, train, p)[v])
                         y.append(lt[v] - lt[slot[x | 1 << j]])
-            ref = oracle.m5p_fit_predict(np.array(Zr), np.array(y), rows(ZB, test, q))[0]
-            res[q, j] = pred[test.program_rows(q), j], ref, np.array(y)
+            if y:
+                ref = oracle.m5p_fit_predict(np.array(Zr), np.array(y), rows(ZB, test, q))[0]
+                res[q, j] = pred[test.program_rows(q), j], ref, np.array(y)
     return res
 
 
@@ -272,6 +273,30 @@ def test_m5p_counters_that_nearly_make_up_one_another(rs, ctx, seed):
     for (q, j), (got, ref, _) in _m5p_on_its_rows(rs, ctx, b, test, np.arange(Q + 1, dtype=np.int64) * runs_per).items():
         trained = (masks[q] >> j) & 1 == 0
         close(got[trained], ref[trained], rel=1e-7, abs_=tol)
+
+
+def test_m5p_splits_that_a_line_ties_with(rs, ctx):
+    """Four instances, two on either value of the one counter: the split into halves and a line through
+    their means have the same estimated error, (|y1 - y2| + |y3 - y4|) 3 / 4, whatever the labels, so that the
+    roundings of both decide, and the tree follows the reference's.  The versions predicted lie between and
+    beyond the two values, where a line and a split differ."""
+    Q, masks = 200, np.arange(8, dtype=np.uint8)
+    rng = np.random.default_rng(11)
+    parity = (masks ^ masks >> 1 ^ masks >> 2) & 1           # 2 + 2 among the four before sides of each pair
+
+    def batch(x):
+        return synth.ProgramBatch(
+            X=np.exp(x).reshape(-1), x_offsets=np.arange(Q, dtype=np.int64) * 8, row_offsets=np.arange(Q + 1, dtype=np.int64) * 8,
+            feat_width=np.ones(Q, dtype=np.int32), masks=np.tile(masks, Q), log_time=rng.standard_normal(8 * Q), cycles=None)
+
+    train = batch(rng.standard_normal((Q, 1)) + rng.standard_normal((Q, 1)) * parity)
+    test = batch(rng.standard_normal((Q, 8)))
+    res = _m5p_on_its_rows(rs, ctx, train, test, np.arange(Q + 1, dtype=np.int64))
+    for q in range(Q):
+        for j in range(3):
+            got, ref, y = res[q, j]
+            assert len(y) == 4
+            close(got, ref, rel=1e-7, abs_=1e-7 * np.abs(ref).max())
 
 
 @pytest.mark.parametrize("spread", [1e-2, 1e-4, 1e-5, 1e-6])
