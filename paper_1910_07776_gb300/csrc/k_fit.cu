@@ -1573,7 +1573,8 @@ __host__ __device__ __forceinline__ bool loo_narrow(int F, int n, double lambda)
 // column by 1 / d; then every entry is updated, warp 0 first moving its copy of the diagonal ahead
 // so that the next pivot's reciprocal is ready when the column is.  Pivots past n are not swept.
 // (One warp per system with full rows in registers -- Gauss-Jordan, 38 instructions a pivot on one
-// scheduler: 256 programs 125 us, and the step of 2 programs 128 us; this form 115 and 104 us.)
+// scheduler: 256 programs 125 us, and the step of 2 programs 128 us; this form 97 and, with its kernels begun
+// early, 75 us.)
 // Writes the inverse, w_y, w_1 and their sums to tab, and
 // ok = 1 when every pivot was positive and finite -- and, with limit > 0, when q = max_i M_ii
 // max_i (M^-1)_ii is at most limit (q bounds the condition number: q <= cond(M) <= n^2 q for a
@@ -2658,7 +2659,7 @@ cudaError_t rs_launch_fit_predict(const rs_fit_args& a, cudaStream_t st) {
         // that keep compact records.  Against 64 bits the two forms differ by no more than their
         // own rounding while the condition bound q stays below the limit (relative prediction
         // errors within 0.9-1.3 of each other, 48..1024 features: equal).  256 programs x 64
-        // versions x 1024 features: the fit stage 1.95 -> 0.15 ms.
+        // versions x 1024 features: the fit stage 1.95 -> 0.11 ms.
         // Not looked for where the programs have fewer features than pairs (loo_narrow): every fit would be left,
         // after the inverses and without the second stream (2 programs x 64 versions x 24 features 180 us
         // where 110 do, 256 programs 1889 and 1801).
