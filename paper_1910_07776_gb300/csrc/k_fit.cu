@@ -1554,7 +1554,8 @@ constexpr int kLooFitThreads = 256;
 // Largest q = max M_ii max (M^-1)_ii for which a call that did not ask for the closed form takes
 // it: the condition number is then at most n^2 q = 4e6, an error of the inverse below 5e-10 even
 // at that bound.  (Typical systems: q of tens; it passes the limit near as many features as pairs.)
-constexpr float kLooLimit = 4096.f;
+constexpr int kLooLimitBits = 12;
+constexpr float kLooLimit = 1 << kLooLimitBits;
 // Systems of n pairs with F < n features are not tried: K_PP has n - F eigenvalues 0, M those of lambda, and q
 // comes to about F / lambda (z-scores: M_ii about F), unless lambda is large enough for that.
 __host__ __device__ __forceinline__ bool loo_narrow(int F, int n, double lambda) {
@@ -1612,15 +1613,7 @@ loo_inv_kernel(const int64_t* __restrict__ row_off, const int32_t* __restrict__ 
     if (tid < n) vs[tid] = pb[(int64_t)pj * RS_MAXPAIRS + tid];
     if (tid == 0) umax = 0;
     __syncthreads();
-    // With a limit: the largest 1 / d that a pivot may have.  1 / d_k is an entry of the inverse of the leading
-    // block, and so at most (M^-1)_kk: a pivot beyond ends it (nearly collinear counters, within a few pivots).
-    int dmax = 0, rmax = 0x7fe00000;
-    if (limit > 0.f) {
-        const double dii = lane < n ? dlam[(int64_t)p * RS_MAXV + vs[lane]] : 0.0;
-        dmax = __reduce_max_sync(0xffffffffu, pos_finite(dii) ? __double2hiint(dii) : 0);
-        const double most = (double)limit * rcp_newton(__hiloint2double(dmax, 0));
-        if (pos_finite(most)) rmax = __double2hiint(most) + 1;  // (rounded up)
-    }
+    const double dii = lane < n ? dlam[(int64_t)p * RS_MAXV + vs[lane]] : 0.0;      // (used behind the entries' loads)
     double A[kLooPer];
     int ri[kLooPer], ci[kLooPer];                               // row 0..33, column 0..31; -1: none
 #pragma unroll
@@ -1658,8 +1651,16 @@ loo_inv_kernel(const int64_t* __restrict__ row_off, const int32_t* __restrict__ 
             else if (ri[s] == k) col[k & 1][ci[s]] = A[s];
         }
     };
+    // With a limit: the largest 1 / d that a pivot may have (high word).  1 / d_k is an entry of the inverse of
+    // the leading block, and so at most (M^-1)_kk: 1 / d_k from limit / 2^floor(log2(max M_ii)) up proves q beyond
+    // it and ends the sweep (nearly collinear counters: within a few pivots).
+    int dmax = 0, rmax = 0x7fe00000;
+    if (limit > 0.f) {
+        dmax = __reduce_max_sync(0xffffffffu, pos_finite(dii) ? __double2hiint(dii) : 0);
+        rmax = min(2 * 1023 + kLooLimitBits - (dmax >> 20), rmax >> 20) << 20;
+    }
     // warp 0, lane i: A_ii (i < n), ahead of the entries by one reciprocal
-    double dg = warp == 0 && lane < n ? dlam[(int64_t)p * RS_MAXV + vs[lane]] : 1.0;
+    double dg = warp == 0 && lane < n ? dii : 1.0;
     auto next_pivot = [&](int k) {
         if (lane == k) rk = pos_finite(dg) ? rcp_newton(dg) : 0.0;
     };
@@ -1670,7 +1671,7 @@ loo_inv_kernel(const int64_t* __restrict__ row_off, const int32_t* __restrict__ 
     for (int k = 0; k < n; ++k) {
         const double* c = col[k & 1];
         const double r = rk;                                    // the same value in every thread
-        good = pos_finite(r) && __double2hiint(r) <= rmax;
+        good = pos_finite(r) && __double2hiint(r) < rmax;
         if (!good) break;
         if (warp == 1) {
             if (lane < n) w[lane] = lane == k ? -r : c[lane] * r;

@@ -330,8 +330,9 @@ transfer_tile_kernel(const int64_t* __restrict__ group_off, int max_runs, int64_
 
 // Whether the Gram (with dist, the distances that only have to order) goes through the products of digits
 // (k_gram_split.cu).  That form takes a program an SM: 10 + 0.05 F us alone, and with several programs an SM
-// 4.5 + 0.09 V + 0.033 F us each; the multiply-adds 32 F ns per block of 128 entries and SM plus 6 us, in
-// the long run 8 F ns per warp of entries and 0.25 us per block.  So the multiply-adds keep the grids that
+// 5.5 + 0.09 V + 0.033 F us each; the multiply-adds 32 F ns per block of 128 entries and SM plus 6 us, in
+// the long run 9 F ns per warp of entries and 0.25 us per block (over 100 batches of mixed sizes the choice
+// costs 0.3 % of the better form's time on the mean).  So the multiply-adds keep the grids that
 // fit the SMs once and small products (64 versions x 96 features: 26 programs 14.7 against 16.4 us, 40
 // programs 22.6 against 16.4; 256 features: 8 programs 18.6 against 20.0, 12 programs 22.6 against 20.5; 30
 // versions x 96: 76 programs 12.9 against 14.5, 300 programs 30.9 against 24.7), and many programs of few
@@ -340,7 +341,7 @@ transfer_tile_kernel(const int64_t* __restrict__ group_off, int max_runs, int64_
 // stay for those too, as a chain of multiply-adds rounds at every feature (3,000 x 10 versions x 256: 119
 // against 205 us).
 // The differences of distances cost three times the multiply-adds and more, the ordering 20 us a wave of
-// programs, about 2 us each in the long run: 64 versions, 9 programs x 300 features 55 (differences)
+// programs, about 1 us each in the long run: 64 versions, 9 programs x 300 features 55 (differences)
 // against 49 us, 40 x 96 58 against 36, 64 x 48 48 against 34; the whole step of 3,000 programs of 20
 // versions x 24 features 216 against 259 us, x 48 337 against 286.
 bool by_digits(const rs_batch* b, bool dist) {
@@ -350,8 +351,11 @@ bool by_digits(const rs_batch* b, bool dist) {
     const int64_t mean = b->n_rows > 0 ? b->x_elems / b->n_rows : 1;
     const int64_t f = mean < 1 ? 1 : mean < b->max_feat ? mean : b->max_feat;
     if (P <= 152 || (f >= 256 && !dist)) return true;
-    const int64_t warps = (entries + 31) / 32, plain = (dist ? 30 : 8) * f * warps + 250 * per;      // ns
-    return plain > 4500 + 90 * v + 33 * f + (dist ? 2000 : 0);
+    // twice the mean entries, versions spread evenly about their mean up to max_versions; ns
+    const int64_t top = b->max_versions < v ? v : b->max_versions < RS_MAXV ? b->max_versions : RS_MAXV;
+    const int64_t e2 = v * v + (top - v) * (top - v) / 3 + v;
+    const int64_t plain = (dist ? 30 : 9) * f * (e2 / 32 + 1) + 250 * (e2 / 128 + 1);
+    return plain > 2 * (5500 + 90 * v + 33 * f + (dist ? 1000 : 0));
 }
 
 }  // namespace
